@@ -73,22 +73,24 @@ int pack_weights(const float *w, int cin, int cout, int transpose, int cin_pad, 
 // Runs the convolution; returns SPP_OK or an SPP error code.
 int conv3x3(const ConvArgs &a, cudaStream_t stream);
 
-// Weight gradient (wgrad_tc.cu).  x describes the layer's input exactly as
-// the forward convolution reads it (B, H, W, cin_pad and the source mode);
-// g the gradient with respect to the layer's output before its ReLU
-// (kSrcNHWC with c0 = its channel count, or kSrcPlanarF32 with cf = cout),
-// on the same grid.  gw [cout][cin][3][3] and gb [cout] are overwritten.
+// Weight gradient (wgrad_tc.cu).  x0 is the layer's input BF16 [B][H][W][c0];
+// for a concatenating layer x1 [B][H][W][c1] holds its further channels at
+// full resolution (c0 a multiple of 32 then).  g is the gradient with respect
+// to the layer's output before its ReLU, BF16 [B][H][W][cg], cg >= cout.
+// Channel strides are multiples of 8.  gw [cout][cin][3][3] and gb [cout] (may
+// be null) are overwritten; ws holds wgrad_workspace_bytes.
 struct WgradArgs {
-    ConvArgs x;
-    ConvArgs g;
+    int B = 0, H = 0, W = 0;
+    const __nv_bfloat16 *x0 = nullptr;
+    int c0 = 0;
+    const __nv_bfloat16 *x1 = nullptr;
+    int c1 = 0;
+    const __nv_bfloat16 *g = nullptr;
+    int cg = 0;
     int cin = 0, cout = 0;  // real channel counts
-    int n = 0;              // cout padded: 32, 64 or 128 (the MMA N)
-    float *partial = nullptr;
-    float *pbias = nullptr;
     int32_t *status = nullptr;
 };
-int wgrad_splits(int B, int W, int H, int cin_pad);
-size_t wgrad_workspace_bytes(int B, int W, int H, int cin_pad, int n);
+size_t wgrad_workspace_bytes(int B, int W, int H, int cin, int cout);
 int wgrad(const WgradArgs &a, float *gw, float *gb, void *ws, cudaStream_t stream);
 
 // Supported MMA widths of conv3x3.

@@ -3,7 +3,10 @@
 // transposed weights; the ReLU mask of the layer below fused into the
 // epilogue), weight gradients through wgrad_tc.cu, the gradient junctions
 // of the pooling / upsampling / concatenation edges in one small kernel,
-// and AdamW on the FP32 master parameters.
+// and AdamW on the FP32 master parameters.  Both kinds of gradient read BF16
+// NHWC operands through TMA: the heads' FP32 planar gradients are converted
+// once, and the upsampled half of a decoder input is written out once for its
+// weight gradient.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -24,6 +27,8 @@ struct GradLayout {
     size_t d0b, d0a, cat0, e0b, e0a, gin;          // level 0 (gin: input gradient)
     size_t t1h, d1b, d1a, cat1, e1b, e1a, pool0;   // level 1
     size_t bth, e2b, e2a, pool1;                   // level 2
+    size_t gh[3];                                  // head gradients (round16(cout) channels)
+    size_t up;                                     // upsampled decoder input
     size_t wg;                                     // weight-gradient scratch
     size_t total;
 };
@@ -54,14 +59,17 @@ GradLayout grad_layout(int net, int B, int W, int H) {
     G.e2b = take(p2 * 128);
     G.e2a = take(p2 * 128);
     G.pool1 = take(p2 * 64);
+    G.gh[0] = take(p0 * round16(kNets[net].heads[0]));
+    G.gh[1] = take(p1 * round16(kNets[net].heads[1]));
+    G.gh[2] = take(p2 * round16(kNets[net].heads[2]));
+    G.up = take(std::max(p0 * 64, p1 * 128));
     G.wg = off;
     size_t wg = 0;
     for (int i = 0; i < kNumLayers; ++i) {
         if (!present(net, i)) continue;
         const int level = level_of(i);
-        const int cin_pad = i == E0A ? input_channels_padded(net) : round16(layer(net, i).cin);
-        wg = std::max(wg, conv::wgrad_workspace_bytes(B, W >> level, H >> level, cin_pad,
-                                                      fwd_n(net, i)));
+        wg = std::max(wg, conv::wgrad_workspace_bytes(B, W >> level, H >> level,
+                                                      layer(net, i).cin, layer(net, i).cout));
     }
     G.total = align256(off + wg);
     return G;
@@ -152,6 +160,54 @@ __global__ void nhwc_to_planar_kernel(const __nv_bfloat16 *__restrict__ src, int
     }
 }
 
+// FP32 planar [B][C][H][W] -> BF16 NHWC [B][H][W][CP] (rounded to nearest
+// even, padding channels zero), 16 channels per thread: plane reads are
+// coalesced along x and each thread writes one 32-byte sector.
+__global__ void __launch_bounds__(256)
+planar_to_nhwc_kernel(const float *__restrict__ src, int C, int CP, int64_t n, int64_t hw,
+                      __nv_bfloat16 *__restrict__ dst) {
+    pdl_wait();
+    pdl_trigger();
+    const int64_t p = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    if (p >= n) return;
+    const int c0 = blockIdx.y * 16;
+    const int64_t b = p / hw, i = p - b * hw;
+    const float *s = src + (b * C + c0) * hw + i;
+    uint32_t w[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const float lo = c0 + 2 * k < C ? __ldg(s + (2 * k) * hw) : 0.f;
+        const float hi = c0 + 2 * k + 1 < C ? __ldg(s + (2 * k + 1) * hw) : 0.f;
+        w[k] = conv::pack_bf16x2(lo, hi);
+    }
+    uint4 *o = reinterpret_cast<uint4 *>(dst + p * CP + c0);
+    o[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    o[1] = make_uint4(w[4], w[5], w[6], w[7]);
+}
+
+// BF16 NHWC [B][H][W][C] -> its nearest 2x upsampling [B][2H][2W][C], one
+// 16-byte piece per thread.
+__global__ void __launch_bounds__(256)
+upsample_kernel(const __nv_bfloat16 *__restrict__ src, int H, int W, int C, int64_t pieces,
+                __nv_bfloat16 *__restrict__ dst) {
+    pdl_wait();
+    pdl_trigger();
+    const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    if (k >= pieces) return;
+    const int c8 = C / 8;
+    const int c = static_cast<int>(k % c8) * 8;
+    const int64_t p = k / c8;
+    const int x = static_cast<int>(p % W);
+    const int64_t by = p / W;  // b H + y
+    const uint4 v = conv::ldg16(src + p * C + c);
+    __nv_bfloat16 *d = dst + ((2 * by) * (2 * W) + 2 * x) * static_cast<int64_t>(C) + c;
+    const int64_t row = static_cast<int64_t>(2 * W) * C;
+    *reinterpret_cast<uint4 *>(d) = v;
+    *reinterpret_cast<uint4 *>(d + C) = v;
+    *reinterpret_cast<uint4 *>(d + row) = v;
+    *reinterpret_cast<uint4 *>(d + row + C) = v;
+}
+
 int launch_junction(int B, int H, int W, int C, const __nv_bfloat16 *act, const __nv_bfloat16 *A,
                     int a_c, int a_off, const __nv_bfloat16 *F, int f_c, int f_off,
                     const __nv_bfloat16 *Cq, int c_c, __nv_bfloat16 *out, cudaStream_t stream) {
@@ -188,32 +244,49 @@ int backward(int net, const unsigned char *packed, int B, int W, int H, const un
                                G.d1a, G.d1b, 0,     G.d0a, G.d0b, 0};
     int rc = SPP_OK;
 
-    auto gsrc = [&](int i, int level) {
-        conv::ConvArgs g;
-        g.B = B;
-        g.W = W >> level;
-        g.H = H >> level;
-        const Layer l = layer(net, i);
-        if (!l.relu) {
-            g.src_mode = conv::kSrcPlanarF32;
-            g.srcf = gheads[i];
-            g.cf = l.cout;
-        } else {
-            g.src_mode = conv::kSrcNHWC;
-            g.src0 = gb(gpre[i]);
-            g.c0 = l.cout;
-        }
-        return g;
+    // the BF16 NHWC gradient of layer i's pre-activation output and its channels
+    auto gout = [&](int i) {
+        return gb(layer(net, i).relu ? gpre[i] : G.gh[i == H0 ? 0 : i == H1 ? 1 : 2]);
+    };
+    auto gchan = [&](int i) {
+        return layer(net, i).relu ? layer(net, i).cout : round16(layer(net, i).cout);
+    };
+    auto head_gradient = [&](int i) {
+        if (rc != SPP_OK || !present(net, i)) return;
+        const int level = level_of(i), cp = gchan(i);
+        const int64_t hw = static_cast<int64_t>(W >> level) * (H >> level), n = B * hw;
+        if (n == 0) return;
+        launch_dependent(planar_to_nhwc_kernel,
+                         dim3(static_cast<unsigned>((n + 255) / 256), cp / 16), dim3(256), 0, stream,
+                         gheads[i], layer(net, i).cout, cp, n, hw, gout(i));
+        count_launch();
+        rc = launch_status();
     };
     auto wgrad_layer = [&](int i) {
         if (rc != SPP_OK || !present(net, i)) return;
         const Layer l = layer(net, i);
+        const conv::ConvArgs x = layer_input(net, i, B, W, H, fws);
         conv::WgradArgs w;
-        w.x = layer_input(net, i, B, W, H, fws);
-        w.g = gsrc(i, level_of(i));
+        w.B = B;
+        w.W = x.W;
+        w.H = x.H;
+        w.x0 = x.src0;
+        w.c0 = x.c0;
+        if (x.src_mode == conv::kSrcConcatUp) {
+            const int64_t pieces = static_cast<int64_t>(B) * (x.W / 2) * (x.H / 2) * (x.c1 / 8);
+            if (pieces > 0) {
+                launch_dependent(upsample_kernel, dim3(static_cast<unsigned>((pieces + 255) / 256)),
+                                 dim3(256), 0, stream, x.src1, x.H / 2, x.W / 2, x.c1, pieces,
+                                 gb(G.up));
+                count_launch();
+            }
+            w.x1 = gb(G.up);
+            w.c1 = x.c1;
+        }
+        w.g = gout(i);
+        w.cg = gchan(i);
         w.cin = l.cin;
         w.cout = l.cout;
-        w.n = fwd_n(net, i);
         w.status = status;
         rc = conv::wgrad(w, grad_theta + P.theta_w[i], grad_theta + P.theta_b[i], bws + G.wg,
                          stream);
@@ -224,7 +297,13 @@ int backward(int net, const unsigned char *packed, int B, int W, int H, const un
         if (rc != SPP_OK || !present(net, i)) return;
         const Layer l = layer(net, i);
         const int level = level_of(i);
-        conv::ConvArgs a = gsrc(i, level);
+        conv::ConvArgs a;
+        a.B = B;
+        a.W = W >> level;
+        a.H = H >> level;
+        a.src_mode = conv::kSrcNHWC;
+        a.src0 = gout(i);
+        a.c0 = gchan(i);
         a.cin_pad = round16(l.cout);
         a.n = i == E0A ? input_channels_padded(net) : l.cin;
         a.cout = a.n;
@@ -244,6 +323,7 @@ int backward(int net, const unsigned char *packed, int B, int W, int H, const un
     };
 
     // decoder, level 0
+    head_gradient(H0);
     wgrad_layer(H0);
     dgrad_layer(H0, gb(G.d0b), act(A.t0));
     wgrad_layer(D0B);
@@ -251,6 +331,7 @@ int backward(int net, const unsigned char *packed, int B, int W, int H, const un
     wgrad_layer(D0A);
     dgrad_layer(D0A, gb(G.cat0), nullptr);
     // decoder, level 1
+    head_gradient(H1);
     wgrad_layer(H1);
     dgrad_layer(H1, gb(G.t1h), nullptr);
     junction(1, 64, act(A.t1), has_h1 ? gb(G.t1h) : nullptr, 64, 0, gb(G.cat0), 96, 32, nullptr,
@@ -260,6 +341,7 @@ int backward(int net, const unsigned char *packed, int B, int W, int H, const un
     wgrad_layer(D1A);
     dgrad_layer(D1A, gb(G.cat1), nullptr);
     // bottleneck, level 2
+    head_gradient(H2);
     wgrad_layer(H2);
     dgrad_layer(H2, gb(G.bth), nullptr);
     junction(2, 128, act(A.bt), has_h2 ? gb(G.bth) : nullptr, 128, 0, gb(G.cat1), 192, 64,
@@ -365,12 +447,10 @@ extern "C" int spp_adamw_step(float *theta, const float *grad, float *m, float *
                             grad_scale, stream);
 }
 
-static int wgrad_n(int cout) { return cout <= 32 ? 32 : cout <= 64 ? 64 : 128; }
-
 extern "C" size_t spp_conv3x3_backward_weights_workspace_bytes(int B, int W, int H, int cin,
                                                                int cout) {
     if (B < 0 || W < 0 || H < 0 || cin <= 0 || cout <= 0 || cout > 128) return 0;
-    return spp::conv::wgrad_workspace_bytes(B, W, H, spp::unet::round16(cin), wgrad_n(cout));
+    return spp::conv::wgrad_workspace_bytes(B, W, H, cin, cout);
 }
 
 extern "C" int spp_conv3x3_backward_weights(const uint16_t *x, const uint16_t *g, int B, int W,
@@ -381,22 +461,18 @@ extern "C" int spp_conv3x3_backward_weights(const uint16_t *x, const uint16_t *g
         return SPP_ERR_ARG;
     if (cin % 8 || cout % 8) return SPP_ERR_ARG;
     if (!aligned16(x) || !aligned16(g) || !aligned16(ws)) return SPP_ERR_ALIGN;
-    if (ws_bytes < spp::conv::wgrad_workspace_bytes(B, W, H, spp::unet::round16(cin), wgrad_n(cout)))
+    if (ws_bytes < spp::conv::wgrad_workspace_bytes(B, W, H, cin, cout))
         return SPP_ERR_WORKSPACE;
     spp::conv::WgradArgs a;
-    a.x.B = a.g.B = B;
-    a.x.W = a.g.W = W;
-    a.x.H = a.g.H = H;
-    a.x.cin_pad = spp::unet::round16(cin);
-    a.x.src_mode = spp::conv::kSrcNHWC;
-    a.x.src0 = reinterpret_cast<const __nv_bfloat16 *>(x);
-    a.x.c0 = cin;
-    a.g.src_mode = spp::conv::kSrcNHWC;
-    a.g.src0 = reinterpret_cast<const __nv_bfloat16 *>(g);
-    a.g.c0 = cout;
+    a.B = B;
+    a.W = W;
+    a.H = H;
+    a.x0 = reinterpret_cast<const __nv_bfloat16 *>(x);
+    a.c0 = cin;
+    a.g = reinterpret_cast<const __nv_bfloat16 *>(g);
+    a.cg = cout;
     a.cin = cin;
     a.cout = cout;
-    a.n = wgrad_n(cout);
     a.status = status;
     return spp::conv::wgrad(a, gw, gb, ws, stream);
 }

@@ -3,97 +3,149 @@
 //   gb[co]             = sum over pixels p of g[p][co]
 // BF16 operands, FP32 accumulation.
 //
-// GEMM view: M = 9 * cin_pad rows (tap-major, then input channel), N = the
-// output channels (padded to 16), K = the pixels.  Grid (M tiles of 128
-// rows) x (pixel splits); each CTA accumulates its rows over its share of
-// the pixels in TMEM and writes an FP32 partial sum; a second kernel adds
-// the partials in a fixed order (the result is deterministic) and writes gw
-// and gb in the natural layout.
+// GEMM view: K = the pixels, so that both operands are stored with K as the
+// slow axis (NHWC: a pixel's channels are contiguous).  tcgen05 reads such
+// "MN-major" operands directly, so TMA boxes of the tensors are the operands
+// and nothing is transposed: a box row is one pixel of 32 channels (64 bytes,
+// 64-byte swizzle), a core matrix is 8 consecutive pixels.
+//   A (M = 128): 4 atoms of 32 input channels, each atom one pixel (64 bytes)
+//     after the one before it: the taps dx = 0, 1, 2 of an input row are the
+//     same bytes at row shifts 0, 1, 2 (the fourth atom is a spare shift whose
+//     32 accumulator rows are not read).
+//   B (N = cout padded to 32): the row of g, one atom per 32 output channels.
+// A CTA owns one block of 32 input channels, one dy and one share ("split") of
+// the pixel chunks of 64 pixels of a row; its 128 x N accumulator stays in TMEM
+// for the whole kernel and is written once as a partial sum.  A second kernel
+// adds the partials in a fixed order (the result is deterministic) and writes
+// gw and gb in the natural layout.
 //
-// K chunk: 64 consecutive pixels of one image row.  Both operands must be
-// K-major (pixels contiguous inside a core matrix) while the tensors are
-// stored pixel-major (NHWC), so each producer thread loads the 8 x 16-byte
-// rows of one 8-pixel x 8-channel block (the im2col gather of its tap, with
-// the fused pooling / upsample / concatenation of the layer's input), turns
-// the 8x8 BF16 block over with byte permutes and stores it as one core
-// matrix.  Warp roles, stage recycling and the bounded waits are those of
-// conv_tc.cu.
+// The accumulation in TMEM truncates, so a sum's error grows with the length
+// of its chain of MMAs, and where the chains are cut shows in the 5th digit of
+// a gradient.  The cut is part of the result: split s of S takes the chunks s,
+// s + S, ... in order, S = (SM count) / ceil(9 cin / 128), and the partials are
+// added in the order of s.
+//
+// Bound: the TMA feed (8.3 KB per chunk for 32 output channels, 4 MMAs of
+// about 40 cycles), with up to 150 to 190 CTAs resident.  Pixels as the fast
+// axis, the form before this one, made four warps transpose every operand
+// through registers for each of the 9 taps (1.21 ms instead of 0.16 ms for
+// the three gradients of a 64 -> 64 layer on 2 x 500 x 281 pixels) and left the
+// tensor cores idle.
+//
+// Warp roles (192 threads): warps 0-3 sum g over the pixels of each stage
+// (the bias gradient, on CTAs of the first input block and dy) and read TMEM at
+// the end; warp 4 issues the TMA boxes; warp 5 issues the MMAs.  Every wait is
+// bounded as in conv_tc.cu: on expiry the CTA records SPP_ERR_TIMEOUT, the
+// other roles leave at their next wait, the issuing threads wait for their
+// copies and MMAs in flight, and TMEM is freed before the kernel returns.
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cstring>
 
 #include "conv_src.cuh"
 #include "conv_tc.cuh"
 #include "spp_internal.cuh"
 #include "tc_common.cuh"
+#include "tma_host.cuh"
 
 namespace spp {
 namespace conv {
 namespace {
 
-constexpr int kKP = 64;  // pixels per K chunk
-constexpr int kThreads = 288;
-constexpr int kHeader = 256;
-constexpr int kNS = 4;
-
-template <int N>
-struct WCfg {
-    static constexpr int kA = 128 * kKP * 2;  // 16 KB
-    static constexpr int kB = N * kKP * 2;
-    static constexpr int kStage = kA + kB;
-    static constexpr int kSmem = kHeader + kNS * kStage + 128;
-    static constexpr int kCols = tc::pow2_cols(N);
-};
+constexpr int kThreads = 192;
+constexpr int kPX = 64;                 // pixels per K chunk (of one row)
+constexpr int kHX = kPX + 2;            // input pixels under a chunk's three dx taps
+constexpr int kBlk = 32;                // channels of a block (64 bytes)
+constexpr int kLanes = 3 * kBlk;        // accumulator rows that are read: dx 0, 1, 2
+constexpr int kXBytes = kHX * 64;                    // one x box
+constexpr int kXSlot = (kXBytes + 511) / 512 * 512;  // its slot (swizzle period)
+constexpr int kGBytes = kPX * 64;                    // one g box
+constexpr int kHeader = 512;
+constexpr int kMaxStages = 3;
+constexpr int kBiasGroups = 8;          // pixel groups of a chunk in the bias sums
+// shared memory per CTA: two CTAs fit an SM where the grid exceeds the SMs
+constexpr int kSmemLimit = 110 * 1024;
+// the spare fourth shift of the last pixel stays inside the x slot
+static_assert(kXSlot - kXBytes >= 64, "no room for the spare tap");
 
 struct WBars {
-    uint64_t full[kNS];
-    uint64_t empty[kNS];
+    uint64_t full[kMaxStages];
+    uint64_t empty[kMaxStages];
     uint64_t accf;
     uint64_t drain;
     uint32_t tmem_base;
     int abort;
 };
+static_assert(sizeof(WBars) <= kHeader, "header");
 
-// 8x8 transpose of 16-bit values: in[p] holds channels 0..7 of pixel p,
-// out[c] receives pixels 0..7 of channel c.
-__device__ __forceinline__ void transpose8x8(const uint4 (&in)[8], uint4 (&out)[8]) {
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        uint32_t o[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t *w0 = &in[2 * q].x, *w1 = &in[2 * q + 1].x;
-            o[q] = __byte_perm(w0[c >> 1], w1[c >> 1], (c & 1) ? 0x7632 : 0x5410);
-        }
-        out[c] = make_uint4(o[0], o[1], o[2], o[3]);
-    }
+struct WKernelArgs {
+    int H, W;
+    int64_t nchunks;
+    int nci, nco;    // 32-channel blocks of x and of g
+    int n0;          // blocks of x that come from the first source
+    int ns, nch;     // stages, chunks per stage
+    float *partial;  // [split][nci][dy][nco * 32][96 rows]
+    float *pbias;    // [split][8][nco * 32]
+    int32_t *status;
+};
+
+// MN-major operand in the 64-byte swizzle (layout type 4): atoms of 32
+// channels x 8 pixels; atoms along M / N are lbo bytes apart, groups of 8
+// pixels 512 bytes.  The swizzle follows the absolute address (boxes start on
+// its 512-byte period), so any pixel may be the first.
+__device__ __forceinline__ uint64_t desc_mn64(uint32_t saddr, uint32_t lbo) {
+    return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) |
+           (static_cast<uint64_t>(lbo >> 4) << 16) | (static_cast<uint64_t>(512 >> 4) << 32) |
+           (1ull << 46) | (4ull << 61);
+}
+// both operands MN-major (bits 15 and 16)
+__host__ __device__ constexpr uint32_t idesc_mn(int N) {
+    return tc::idesc_bf16_f32(128, N) | (1u << 15) | (1u << 16);
 }
 
-template <int N>
-__global__ void __launch_bounds__(kThreads, 1) wgrad_kernel(const WgradArgs a) {
-    using C = WCfg<N>;
+__device__ __forceinline__ void tma_box(const CUtensorMap *map, uint32_t dst, uint64_t *bar, int c,
+                                        int x, int y, int b) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(tc::smem_u32(bar)), "r"(c), "r"(x), "r"(y),
+        "r"(b)
+        : "memory");
+}
+
+__global__ void __launch_bounds__(kThreads)
+wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
+             const __grid_constant__ CUtensorMap xmap1, const __grid_constant__ CUtensorMap gmap) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    unsigned char *base = smem_raw + ((128u - (tc::smem_u32(smem_raw) & 127u)) & 127u);
+    unsigned char *base = smem_raw + ((512u - (tc::smem_u32(smem_raw) & 511u)) & 511u);
     WBars &bars = *reinterpret_cast<WBars *>(base);
     unsigned char *stages = base + kHeader;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int mt = blockIdx.x, split = blockIdx.y, splits = gridDim.y;
-    const int B = a.x.B, H = a.x.H, W = a.x.W;
-    const int cw = (W + kKP - 1) / kKP;
-    const int64_t nchunks = static_cast<int64_t>(B) * H * cw;
-    const int mpad = gridDim.x * 128;
+    const int split = blockIdx.x, splits = gridDim.x;
+    const int ci = blockIdx.y / 3, dy = blockIdx.y % 3;
+    const int N = a.nco * kBlk;
+    const int cw = (a.W + kPX - 1) / kPX;
+    // chunks of this split, and the stages they fill
+    const int mine = static_cast<int>((a.nchunks - split + splits - 1) / splits);
+    const int nstages = (mine + a.nch - 1) / a.nch;
+    const int chunk_bytes = kXSlot + a.nco * kGBytes, stage_bytes = a.nch * chunk_bytes;
+    const bool has_bias = blockIdx.y == 0;
+    const uint32_t cols = N <= 32 ? 32 : N <= 64 ? 64 : 128;
 
     if (tid == 0) {
-        for (int s = 0; s < kNS; ++s) {
-            tc::mbar_init(&bars.full[s], 128);
-            tc::mbar_init(&bars.empty[s], 1);
+        for (int s = 0; s < a.ns; ++s) {
+            tc::mbar_init(&bars.full[s], 1);
+            tc::mbar_init(&bars.empty[s], has_bias ? 5 : 1);
         }
         tc::mbar_init(&bars.accf, 1);
         tc::mbar_init(&bars.drain, 1);
         bars.abort = 0;
         tc::fence_mbar_init();
     }
-    if (warp == 8) tc::tmem_alloc(&bars.tmem_base, C::kCols);
+    if (warp == 5) tc::tmem_alloc(&bars.tmem_base, cols);
+    pdl_wait();
+    pdl_trigger();
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
@@ -104,225 +156,307 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_kernel(const WgradArgs a) {
         set_status(a.status, SPP_ERR_TIMEOUT);
     };
 
-    if (warp >= 4 && warp < 8) {
-        // ---------------------------------------------------------- producers
-        const int ptid = tid - 128;
-        const int ga = ptid >> 3, ja = ptid & 7;  // A block: row group, pixel group
-        const int m0 = mt * 128 + ga * 8;
-        const int tap = m0 / a.x.cin_pad, ci0 = m0 - tap * a.x.cin_pad;
-        const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-        const bool has_b = ptid < N;
-        const int gb_ = ptid >> 3, jb = ptid & 7;  // B block: channel group, pixel group
-        float bsum[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) bsum[e] = 0.f;
-        uint32_t it = 0;
-        for (int64_t q = split; q < nchunks; q += splits, ++it) {
-            const int s = static_cast<int>(it % kNS);
-            const uint32_t ph = (it / kNS) & 1u;
-            if (!tc::mbar_wait(&bars.empty[s], ph ^ 1u, abort_flag)) {
-                fail();
-                break;
-            }
-            const int b = static_cast<int>(q / (static_cast<int64_t>(H) * cw));
-            const int r = static_cast<int>(q - static_cast<int64_t>(b) * H * cw);
-            const int y = r / cw, x0 = (r % cw) * kKP;
-            unsigned char *As = stages + s * C::kStage;
-            unsigned char *Bs = As + C::kA;
-            {
-                uint4 v[8], t[8];
-#pragma unroll
-                for (int p = 0; p < 8; ++p) {
-                    const int x = x0 + 8 * ja + p;
-                    v[p] = (tap < 9 && x < W) ? load_chunk(a.x, b, y + dy, x + dx, ci0)
-                                              : make_uint4(0, 0, 0, 0);
+    if (warp == 4) {
+        // --------------------------------------------------------- TMA boxes
+        if (lane == 0) {
+            const CUtensorMap *xmap = ci < a.n0 ? &xmap0 : &xmap1;
+            const int cx = (ci < a.n0 ? ci : ci - a.n0) * kBlk;
+            int s = 0, issued = 0;
+            uint32_t ph = 0;
+            for (; issued < nstages; ++issued) {
+                if (!tc::mbar_wait(&bars.empty[s], ph ^ 1u, abort_flag)) {
+                    fail();
+                    break;
                 }
-                transpose8x8(v, t);
-                uint4 *dst = reinterpret_cast<uint4 *>(As + ja * 2048 + ga * 128);
-#pragma unroll
-                for (int c = 0; c < 8; ++c) dst[c] = t[c];
-            }
-            if (has_b) {
-                uint4 v[8], t[8];
-#pragma unroll
-                for (int p = 0; p < 8; ++p) {
-                    const int x = x0 + 8 * jb + p;
-                    v[p] = x < W ? load_chunk(a.g, b, y, x, 8 * gb_) : make_uint4(0, 0, 0, 0);
-                    const uint32_t *u = &v[p].x;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const float2 f = unpack_bf16x2(u[k]);
-                        bsum[2 * k] += f.x;
-                        bsum[2 * k + 1] += f.y;
-                    }
+                const int k0 = issued * a.nch, kn = min(a.nch, mine - k0);
+                uint32_t at = tc::smem_u32(stages + s * stage_bytes);
+                tc::mbar_arrive_expect_tx(&bars.full[s],
+                                          static_cast<uint32_t>(kn * (kXBytes + a.nco * kGBytes)));
+                for (int k = 0; k < kn; ++k, at += chunk_bytes) {
+                    const int64_t q = split + static_cast<int64_t>(k0 + k) * splits;
+                    const int64_t by = q / cw;  // b H + y
+                    const int x0 = static_cast<int>(q - by * cw) * kPX;
+                    const int b = static_cast<int>(by / a.H);
+                    const int y = static_cast<int>(by - static_cast<int64_t>(b) * a.H);
+                    tma_box(xmap, at, &bars.full[s], cx, x0 - 1, y + dy - 1, b);
+                    for (int j = 0; j < a.nco; ++j)
+                        tma_box(&gmap, at + kXSlot + j * kGBytes, &bars.full[s], j * kBlk, x0, y, b);
                 }
-                transpose8x8(v, t);
-                uint4 *dst = reinterpret_cast<uint4 *>(Bs + jb * (N * 16) + gb_ * 128);
-#pragma unroll
-                for (int c = 0; c < 8; ++c) dst[c] = t[c];
+                if (++s == a.ns) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
-            tc::fence_proxy_async();
-            tc::mbar_arrive(&bars.full[s]);
+            // after a wait gave up: the copies of the last stages issued have to
+            // land before the CTA exits
+            if (issued < nstages)
+                for (int k = max(issued - a.ns, 0); k < issued; ++k)
+                    (void)tc::mbar_wait(&bars.full[k % a.ns], (k / a.ns) & 1u, nullptr);
         }
-        if (has_b && mt == 0) {
-            float *pb = a.pbias + (static_cast<int64_t>(split) * 8 + jb) * N + 8 * gb_;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) pb[e] = bsum[e];
-        }
-    } else if (warp == 8) {
+        __syncwarp();
+    } else if (warp == 5) {
         // -------------------------------------------------------- MMA issuer
         if (lane == 0) {
-            constexpr uint32_t idesc = tc::idesc_bf16_f32(128, N);
-            uint32_t it = 0;
+            const uint32_t idesc = idesc_mn(N);
             bool ok = true;
-            for (int64_t q = split; q < nchunks; q += splits, ++it) {
-                const int s = static_cast<int>(it % kNS);
-                if (!tc::mbar_wait(&bars.full[s], (it / kNS) & 1u, abort_flag)) {
+            int s = 0;
+            uint32_t ph = 0, acc = 0;
+            for (int g = 0; g < nstages; ++g) {
+                if (!tc::mbar_wait(&bars.full[s], ph, abort_flag)) {
                     fail();
                     ok = false;
                     break;
                 }
                 tc::tc_fence_after();
-                const uint32_t a_base = tc::smem_u32(stages + s * C::kStage);
-                const uint32_t b_base = a_base + C::kA;
+                const int kn = min(a.nch, mine - g * a.nch);
+                uint32_t at = tc::smem_u32(stages + s * stage_bytes);
+                for (int k = 0; k < kn; ++k, at += chunk_bytes) {
+                    const uint64_t ad = desc_mn64(at, 64), bd = desc_mn64(at + kXSlot, kGBytes);
 #pragma unroll
-                for (int ks = 0; ks < kKP / 16; ++ks) {
-                    tc::mma_bf16(tmem, tc::smem_desc(a_base + ks * 2 * 2048, 2048, 128),
-                                 tc::smem_desc(b_base + ks * 2 * N * 16, N * 16, 128), idesc,
-                                 (it | ks) != 0);
+                    for (int ks = 0; ks < kPX / 16; ++ks) {
+                        tc::mma_bf16(tmem, ad + ((ks * 16 * 64) >> 4), bd + ((ks * 16 * 64) >> 4),
+                                     idesc, acc);
+                        acc = 1;
+                    }
                 }
                 tc::mma_commit(&bars.empty[s]);
+                if (++s == a.ns) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
             if (ok) {
                 tc::mma_commit(&bars.accf);
-            } else if (it > 0) {
+            } else if (acc) {
                 tc::mma_commit(&bars.drain);
                 (void)tc::mbar_wait(&bars.drain, 0, nullptr);
             }
         }
         __syncwarp();
     } else {
-        // ----------------------------------------------------------- epilogue
-        const bool any = split < nchunks;
+        // ----------------------------- bias gradient, then the accumulator
         bool ok = true;
-        if (any && !tc::mbar_wait(&bars.accf, 0, abort_flag)) {
+        if (has_bias) {
+            // thread: 8 channels (16-byte piece c4 of block j) of the pixels 8 pg
+            // .. 8 pg + 7 of every chunk, added one after the other
+            const int c4 = lane & 3, pg = lane >> 2, j = warp;
+            float bs[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) bs[e] = 0.f;
+            int s = 0;
+            uint32_t ph = 0;
+            for (int g = 0; g < nstages; ++g) {
+                if (!tc::mbar_wait(&bars.full[s], ph, abort_flag)) {
+                    fail();
+                    ok = false;
+                    break;
+                }
+                if (j < a.nco) {
+                    const int kn = min(a.nch, mine - g * a.nch);
+                    const unsigned char *gs =
+                        stages + s * stage_bytes + kXSlot + j * kGBytes + 8 * pg * 64;
+                    for (int k = 0; k < kn; ++k, gs += chunk_bytes) {
+                        uint4 v[8];
+#pragma unroll
+                        for (int p = 0; p < 8; ++p)
+                            v[p] = *reinterpret_cast<const uint4 *>(gs + p * 64 +
+                                                                    16 * (c4 ^ ((p >> 1) & 3)));
+#pragma unroll
+                        for (int p = 0; p < 8; ++p) {
+                            const uint32_t *u = &v[p].x;
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) {
+                                const float2 f = unpack_bf16x2(u[h]);
+                                bs[2 * h] += f.x;
+                                bs[2 * h + 1] += f.y;
+                            }
+                        }
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&bars.empty[s]);
+                if (++s == a.ns) {
+                    s = 0;
+                    ph ^= 1u;
+                }
+            }
+            if (j < a.nco) {
+                float *pb = a.pbias + (static_cast<int64_t>(split) * kBiasGroups + pg) * N +
+                            j * kBlk + 8 * c4;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) pb[e] = bs[e];
+            }
+        }
+        if (ok && !tc::mbar_wait(&bars.accf, 0, abort_flag)) {
             fail();
             ok = false;
         }
-        if (ok) {
+        if (ok && warp < 3) {  // TMEM lanes 32 dx + channel
             tc::tc_fence_after();
-            const int m = mt * 128 + warp * 32 + lane;
+            const uint32_t lbase = tmem + (static_cast<uint32_t>(warp * 32) << 16);
+            float *o = a.partial +
+                       ((static_cast<int64_t>(split) * a.nci + ci) * 3 + dy) * N * kLanes + tid;
 #pragma unroll 1
-            for (int j0 = 0; j0 < N; j0 += 16) {
-                uint32_t v[16];
-                tc::tmem_ld16(tmem + (static_cast<uint32_t>(warp * 32) << 16) + j0, v);
+            for (int c = 0; c < N; c += 32) {
+                uint32_t v[32];
+                tc::tmem_ld16(lbase + c, *reinterpret_cast<uint32_t(*)[16]>(v));
+                tc::tmem_ld16(lbase + c + 16, *reinterpret_cast<uint32_t(*)[16]>(v + 16));
                 tc::tmem_wait_ld();
 #pragma unroll
-                for (int e = 0; e < 16; ++e)
-                    a.partial[(static_cast<int64_t>(split) * N + j0 + e) * mpad + m] =
-                        any ? __uint_as_float(v[e]) : 0.f;
+                for (int e = 0; e < 32; ++e) o[(c + e) * kLanes] = __uint_as_float(v[e]);
             }
         }
     }
 
     tc::tc_fence_before();
     __syncthreads();
-    if (warp == 8) {
+    if (warp == 5) {
         tc::tc_fence_after();
-        tc::tmem_dealloc(tmem, C::kCols);
+        tc::tmem_dealloc(tmem, cols);
     }
 }
 
-// gw[co][ci][ky][kx] = sum_s partial[s][co][tap * cin_pad + ci]; gb[co] =
-// sum_s sum_j pbias[s][j][co].  Fixed summation order.
-__global__ void wgrad_reduce_kernel(const float *__restrict__ partial,
-                                    const float *__restrict__ pbias, int splits, int n, int mpad,
-                                    int cin, int cin_pad, int cout, float *__restrict__ gw,
-                                    float *__restrict__ gb) {
-    const int64_t total = static_cast<int64_t>(cout) * cin * 9;
-    for (int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-         idx < total + cout; idx += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        if (idx < total) {
-            const int tap = static_cast<int>(idx % 9);
-            const int ci = static_cast<int>((idx / 9) % cin);
-            const int co = static_cast<int>(idx / (9 * static_cast<int64_t>(cin)));
-            const int m = tap * cin_pad + ci;
-            float acc = 0.f;
-            for (int s = 0; s < splits; ++s)
-                acc += partial[(static_cast<int64_t>(s) * n + co) * mpad + m];
-            gw[idx] = acc;
-        } else {
-            const int co = static_cast<int>(idx - total);
-            float acc = 0.f;
-            for (int s = 0; s < splits; ++s)
-                for (int j = 0; j < 8; ++j) acc += pbias[(static_cast<int64_t>(s) * 8 + j) * n + co];
-            if (gb) gb[co] = acc;
-        }
+// gw[co][ci][dy][dx] = sum over the splits of their partial sums, gb[co] =
+// sum over the splits and their eight pixel groups, one thread per value, in
+// order (the loads of 16 splits are in flight together).  Blocks of 64 threads
+// spread a small layer's 9216 values over the SMs.
+constexpr int kRedThreads = 64;
+
+__global__ void __launch_bounds__(kRedThreads)
+wgrad_reduce_kernel(const float *__restrict__ partial, const float *__restrict__ pbias, int splits,
+                    int nci, int nco, int cin, int cout, float *__restrict__ gw,
+                    float *__restrict__ gb) {
+    pdl_wait();
+    pdl_trigger();
+    const int N = nco * kBlk;
+    const int64_t nw = static_cast<int64_t>(nci) * 3 * N * kLanes;
+    const int64_t at = static_cast<int64_t>(blockIdx.x) * kRedThreads + threadIdx.x;
+    const bool weight = at < nw;
+    const int co_b = static_cast<int>(at - nw);
+    if (!weight && co_b >= N) return;
+    const float *p = weight ? partial + at : pbias + co_b;
+    const int64_t stride = weight ? nw : N;
+    const int terms = weight ? splits : kBiasGroups * splits;
+    float acc = 0.f;
+    constexpr int kU = 16;
+    int s = 0;
+    for (; s + kU <= terms; s += kU) {
+        float v[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) v[u] = p[(s + u) * stride];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) acc += v[u];
+    }
+    for (; s < terms; ++s) acc += p[s * stride];
+    if (weight) {
+        const int row = static_cast<int>(at % kLanes);
+        const int64_t r = at / kLanes;
+        const int co = static_cast<int>(r % N), cd = static_cast<int>(r / N);  // ci 3 + dy
+        const int ci = (cd / 3) * kBlk + row % kBlk;
+        if (ci < cin && co < cout)
+            gw[(static_cast<int64_t>(co) * cin + ci) * 9 + (cd % 3) * 3 + row / kBlk] = acc;
+    } else if (co_b < cout && gb) {
+        gb[co_b] = acc;
     }
 }
 
-template <int N>
-int launch_wgrad(const WgradArgs &a, int mtiles, int splits, cudaStream_t stream) {
-    using C = WCfg<N>;
-    static int configured_dev = -1;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (configured_dev != dev) {
-        if (cudaFuncSetAttribute(wgrad_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 C::kSmem) != cudaSuccess)
-            return SPP_ERR_CUDA;
-        configured_dev = dev;
-    }
-    wgrad_kernel<N><<<dim3(mtiles, splits), kThreads, C::kSmem, stream>>>(a);
-    count_launch();
-    return launch_status();
+// NHWC BF16 [B][H][W][C] as a 4-D tensor (channel, x, y, image), box 32
+// channels x bx pixels of one row; channels beyond C and pixels outside the image
+// arrive as zeros.
+bool nhwc_map(CUtensorMap *map, const __nv_bfloat16 *p, int B, int H, int W, int C, int bx) {
+    auto enc = tensor_map_encoder();
+    if (!enc) return false;
+    cuuint64_t dims[4] = {static_cast<cuuint64_t>(C), static_cast<cuuint64_t>(W),
+                          static_cast<cuuint64_t>(H), static_cast<cuuint64_t>(B)};
+    cuuint64_t strides[3] = {static_cast<cuuint64_t>(C) * 2, static_cast<cuuint64_t>(W) * C * 2,
+                             static_cast<cuuint64_t>(H) * W * C * 2};
+    cuuint32_t box[4] = {kBlk, static_cast<cuuint32_t>(bx), 1, 1};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16 *>(p), dims,
+               strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+struct Plan {
+    int nci, nco, splits, nch, ns;
+    int64_t nchunks;
+};
+
+Plan plan(int B, int W, int H, int cin, int cout) {
+    Plan p;
+    p.nci = (cin + kBlk - 1) / kBlk;
+    p.nco = (cout + kBlk - 1) / kBlk;
+    p.nchunks = static_cast<int64_t>(B) * H * ((W + kPX - 1) / kPX);
+    // the cut of the sums (see the top of this file)
+    const int want = std::max(1, sm_count() / ((9 * ((cin + 15) / 16 * 16) + 127) / 128));
+    p.splits = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(p.nchunks, want)));
+    // four chunks per stage (one barrier round trip for 16 MMAs), two where g
+    // is wide
+    p.nch = p.nco <= 2 ? 4 : 2;
+    const int stage = p.nch * (kXSlot + p.nco * kGBytes);
+    p.ns = std::min(kMaxStages, (kSmemLimit - kHeader - 512) / stage);  // 512: alignment slack
+    return p;
 }
 
 }  // namespace
 
-int wgrad_splits(int B, int W, int H, int cin_pad) {
-    const int mtiles = (9 * cin_pad + 127) / 128;
-    const int64_t nchunks = static_cast<int64_t>(B) * H * ((W + kKP - 1) / kKP);
-    const int want = std::max(1, sm_count() / mtiles);
-    return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(nchunks, want)));
+size_t wgrad_workspace_bytes(int B, int W, int H, int cin, int cout) {
+    const Plan p = plan(B, W, H, cin, cout);
+    return sizeof(float) * static_cast<size_t>(p.splits) * p.nco * kBlk *
+               (static_cast<size_t>(p.nci) * 3 * kLanes + kBiasGroups) +
+           256;
 }
 
-size_t wgrad_workspace_bytes(int B, int W, int H, int cin_pad, int n) {
-    const int mtiles = (9 * cin_pad + 127) / 128;
-    const int splits = wgrad_splits(B, W, H, cin_pad);
-    return sizeof(float) * (static_cast<size_t>(splits) * n * mtiles * 128 +
-                            static_cast<size_t>(splits) * 8 * n) + 256;
-}
-
-int wgrad(const WgradArgs &a0, float *gw, float *gb, void *ws, cudaStream_t stream) {
-    WgradArgs a = a0;
-    const int B = a.x.B, W = a.x.W, H = a.x.H;
-    if (a.n != 32 && a.n != 64 && a.n != 128) return SPP_ERR_ARG;
-    if (a.x.cin_pad <= 0 || a.x.cin_pad % 16) return SPP_ERR_ARG;
-    const int64_t npix = static_cast<int64_t>(B) * W * H;
-    const int mtiles = (9 * a.x.cin_pad + 127) / 128;
-    const int splits = wgrad_splits(B, W, H, a.x.cin_pad);
-    const int mpad = mtiles * 128;
-    a.partial = static_cast<float *>(ws);
-    a.pbias = a.partial + static_cast<size_t>(splits) * a.n * mpad;
-    if (npix > 0) {
-        int rc;
-        switch (a.n) {
-            case 32: rc = launch_wgrad<32>(a, mtiles, splits, stream); break;
-            case 64: rc = launch_wgrad<64>(a, mtiles, splits, stream); break;
-            default: rc = launch_wgrad<128>(a, mtiles, splits, stream); break;
-        }
-        if (rc != SPP_OK) return rc;
-    } else {
-        if (cudaMemsetAsync(ws, 0, wgrad_workspace_bytes(B, W, H, a.x.cin_pad, a.n), stream) !=
-            cudaSuccess)
+int wgrad(const WgradArgs &a, float *gw, float *gb, void *ws, cudaStream_t stream) {
+    if (a.cin <= 0 || a.cout <= 0 || a.c0 % 8 || a.c1 % 8 || a.cg % 8 ||
+        (a.c1 && a.c0 % kBlk) || (a.cout + kBlk - 1) / kBlk > 4)
+        return SPP_ERR_ARG;
+    if (static_cast<int64_t>(a.B) * a.W * a.H == 0) {
+        if (cudaMemsetAsync(gw, 0, sizeof(float) * 9 * static_cast<size_t>(a.cin) * a.cout,
+                            stream) != cudaSuccess)
             return SPP_ERR_CUDA;
+        if (gb && cudaMemsetAsync(gb, 0, sizeof(float) * a.cout, stream) != cudaSuccess)
+            return SPP_ERR_CUDA;
+        return SPP_OK;
     }
-    const int64_t total = static_cast<int64_t>(a.cout) * a.cin * 9 + a.cout;
-    const int grid = static_cast<int>(std::min<int64_t>((total + 255) / 256, 4 * sm_count()));
-    wgrad_reduce_kernel<<<grid, 256, 0, stream>>>(a.partial, a.pbias, splits, a.n, mpad, a.cin,
-                                                  a.x.cin_pad, a.cout, gw, gb);
-    count_launch();
+    const Plan p = plan(a.B, a.W, a.H, a.cin, a.cout);
+    CUtensorMap xm0, xm1, gm;
+    if (!nhwc_map(&xm0, a.x0, a.B, a.H, a.W, a.c0, kHX) ||
+        !nhwc_map(&gm, a.g, a.B, a.H, a.W, a.cg, kPX))
+        return SPP_ERR_CUDA;
+    xm1 = xm0;
+    if (a.c1 && !nhwc_map(&xm1, a.x1, a.B, a.H, a.W, a.c1, kHX)) return SPP_ERR_CUDA;
+    WKernelArgs k;
+    k.H = a.H;
+    k.W = a.W;
+    k.nchunks = p.nchunks;
+    k.nci = p.nci;
+    k.nco = p.nco;
+    k.n0 = a.c1 ? a.c0 / kBlk : p.nci;
+    k.ns = p.ns;
+    k.nch = p.nch;
+    k.partial = static_cast<float *>(ws);
+    k.pbias = k.partial + static_cast<size_t>(p.splits) * p.nci * 3 * p.nco * kBlk * kLanes;
+    k.status = a.status;
+    const int smem = kHeader + 512 + p.ns * p.nch * (kXSlot + p.nco * kGBytes);
+    static int configured_dev = -1;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (configured_dev != dev) {
+        if (cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kSmemLimit) != cudaSuccess)
+            return SPP_ERR_CUDA;
+        configured_dev = dev;
+    }
+    launch_dependent(wgrad_kernel, dim3(p.splits, 3 * p.nci), dim3(kThreads), smem, stream, k, xm0,
+                     xm1, gm);
+    const int64_t vals = static_cast<int64_t>(p.nci) * 3 * p.nco * kBlk * kLanes + p.nco * kBlk;
+    launch_dependent(wgrad_reduce_kernel,
+                     dim3(static_cast<unsigned>((vals + kRedThreads - 1) / kRedThreads)),
+                     dim3(kRedThreads), 0, stream, k.partial, k.pbias, p.splits, p.nci, p.nco,
+                     a.cin, a.cout, gw, gb);
+    count_launch(2);
     return launch_status();
 }
 

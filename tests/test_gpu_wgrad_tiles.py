@@ -1,0 +1,48 @@
+"""Weight gradient at the edges of its chunks: 64 pixels of a row, 32-channel
+blocks of the input and of the gradient.
+
+Against the FP64 oracle; the tolerance is the FP32 accumulation bound
+(pixels/16 + 64) 2^-24 sum |x g| with a factor 4, as for the other shapes.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle.unet as U
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def spp():
+    from conftest import build_spp_lib
+    build_spp_lib()
+    import paper_2602_08642_gb300 as spp
+    torch.cuda.set_device(0)
+    return spp
+
+
+@pytest.mark.parametrize("B,H,W", [(1, 1, 1), (1, 4, 64), (2, 3, 63), (1, 5, 65), (3, 9, 130)])
+@pytest.mark.parametrize("cin,cout", [(8, 8), (32, 32), (40, 24), (64, 72), (96, 32), (96, 96),
+                                      (192, 128)])
+def test_weight_gradient_tile_edges(spp, B, H, W, cin, cout):
+    g = torch.Generator().manual_seed(1000 * cin + 10 * cout + W)
+    x = torch.randn(B, H, W, cin, generator=g).to(torch.bfloat16)
+    gy = torch.randn(B, H, W, cout, generator=g).to(torch.bfloat16)
+    n = spp.binding.spp_conv3x3_backward_weights_workspace_bytes(B, W, H, cin, cout)
+    ws = torch.full((n,), 0xFF, dtype=torch.uint8, device="cuda")  # NaN where unwritten
+    gw = torch.full((cout, cin, 3, 3), float("nan"), device="cuda")
+    gb = torch.full((cout,), float("nan"), device="cuda")
+    st = torch.zeros(4, dtype=torch.int32, device="cuda")[:1]
+    spp.check(spp.binding.spp_conv3x3_backward_weights(x.cuda(), gy.cuda(), B, W, H, cin, cout, gw,
+                                                       gb, ws, st))
+    assert spp.binding.spp_get_status(st) == 0
+    nchw = lambda t: t.float().numpy().astype(np.float64).transpose(0, 3, 1, 2)
+    xb, gyb = nchw(x), nchw(gy)
+    w0 = np.zeros((cout, cin, 3, 3))
+    ref_w = sum(U.conv3x3_backward(xb[b], w0, gyb[b])[1] for b in range(B))
+    abs_w = sum(U.conv3x3_backward(np.abs(xb[b]), w0, np.abs(gyb[b]))[1] for b in range(B))
+    tol = 4 * (B * H * W / 16 + 64) * 2.0 ** -24
+    assert np.all(np.abs(gw.cpu().numpy() - ref_w) <= tol * abs_w)
+    assert np.all(np.abs(gb.cpu().numpy() - gyb.sum(axis=(0, 2, 3)))
+                  <= tol * np.abs(gyb).sum(axis=(0, 2, 3)))
