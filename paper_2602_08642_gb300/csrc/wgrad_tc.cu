@@ -28,7 +28,7 @@
 // Bound: the TMA feed (8.3 KB per chunk for 32 output channels, 4 MMAs of
 // about 40 cycles), with up to 150 to 190 CTAs resident.  Pixels as the fast
 // axis, the form before this one, made four warps transpose every operand
-// through registers for each of the 9 taps (1.21 ms instead of 0.16 ms for
+// through registers for each of the 9 taps (1.21 ms instead of 0.14 ms for
 // the three gradients of a 64 -> 64 layer on 2 x 500 x 281 pixels) and left the
 // tensor cores idle.
 //
@@ -81,7 +81,7 @@ static_assert(sizeof(WBars) <= kHeader, "header");
 
 struct WKernelArgs {
     int H, W;
-    int64_t nchunks;
+    int nchunks;     // B H ceil(W / 64)
     int nci, nco;    // 32-channel blocks of x and of g
     int n0;          // blocks of x that come from the first source
     int ns, nch;     // stages, chunks per stage
@@ -127,7 +127,7 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
     const int N = a.nco * kBlk;
     const int cw = (a.W + kPX - 1) / kPX;
     // chunks of this split, and the stages they fill
-    const int mine = static_cast<int>((a.nchunks - split + splits - 1) / splits);
+    const int mine = (a.nchunks - split + splits - 1) / splits;
     const int nstages = (mine + a.nch - 1) / a.nch;
     const int chunk_bytes = kXSlot + a.nco * kGBytes, stage_bytes = a.nch * chunk_bytes;
     const bool has_bias = blockIdx.y == 0;
@@ -161,6 +161,10 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
         if (lane == 0) {
             const CUtensorMap *xmap = ci < a.n0 ? &xmap0 : &xmap1;
             const int cx = (ci < a.n0 ? ci : ci - a.n0) * kBlk;
+            // the chunk's place, advanced by `splits` chunks with carries (a
+            // division per chunk made this thread the kernel's bound)
+            const int dxc = splits % cw, dby = splits / cw, dyy = dby % a.H, db = dby / a.H;
+            int xc = split % cw, y = (split / cw) % a.H, b = split / cw / a.H;
             int s = 0, issued = 0;
             uint32_t ph = 0;
             for (; issued < nstages; ++issued) {
@@ -173,14 +177,21 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
                 tc::mbar_arrive_expect_tx(&bars.full[s],
                                           static_cast<uint32_t>(kn * (kXBytes + a.nco * kGBytes)));
                 for (int k = 0; k < kn; ++k, at += chunk_bytes) {
-                    const int64_t q = split + static_cast<int64_t>(k0 + k) * splits;
-                    const int64_t by = q / cw;  // b H + y
-                    const int x0 = static_cast<int>(q - by * cw) * kPX;
-                    const int b = static_cast<int>(by / a.H);
-                    const int y = static_cast<int>(by - static_cast<int64_t>(b) * a.H);
+                    const int x0 = xc * kPX;
                     tma_box(xmap, at, &bars.full[s], cx, x0 - 1, y + dy - 1, b);
                     for (int j = 0; j < a.nco; ++j)
                         tma_box(&gmap, at + kXSlot + j * kGBytes, &bars.full[s], j * kBlk, x0, y, b);
+                    xc += dxc;
+                    y += dyy;
+                    b += db;
+                    if (xc >= cw) {
+                        xc -= cw;
+                        ++y;
+                    }
+                    if (y >= a.H) {
+                        y -= a.H;
+                        ++b;
+                    }
                 }
                 if (++s == a.ns) {
                     s = 0;
@@ -237,12 +248,14 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
         // ----------------------------- bias gradient, then the accumulator
         bool ok = true;
         if (has_bias) {
-            // thread: 8 channels (16-byte piece c4 of block j) of the pixels 8 pg
-            // .. 8 pg + 7 of every chunk, added one after the other
-            const int c4 = lane & 3, pg = lane >> 2, j = warp;
-            float bs[8];
+            // thread: channel pair `pair` of every block, of the pixels 8 pg .. 8
+            // pg + 7 of every chunk, added one after the other (all four warps
+            // share the sums: with 8 channels per thread one warp had them all
+            // for 32 output channels and held the stages back)
+            const int pair = lane & 15, pg = 2 * warp + (lane >> 4);
+            float bs[4][2];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) bs[e] = 0.f;
+            for (int j = 0; j < 4; ++j) bs[j][0] = bs[j][1] = 0.f;
             int s = 0;
             uint32_t ph = 0;
             for (int g = 0; g < nstages; ++g) {
@@ -251,25 +264,23 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
                     ok = false;
                     break;
                 }
-                if (j < a.nco) {
-                    const int kn = min(a.nch, mine - g * a.nch);
-                    const unsigned char *gs =
-                        stages + s * stage_bytes + kXSlot + j * kGBytes + 8 * pg * 64;
-                    for (int k = 0; k < kn; ++k, gs += chunk_bytes) {
-                        uint4 v[8];
+                const int kn = min(a.nch, mine - g * a.nch);
+                const unsigned char *gs = stages + s * stage_bytes + kXSlot + 8 * pg * 64;
+                for (int k = 0; k < kn; ++k, gs += chunk_bytes) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if (j >= a.nco) break;
+                        uint32_t v[8];
 #pragma unroll
                         for (int p = 0; p < 8; ++p)
-                            v[p] = *reinterpret_cast<const uint4 *>(gs + p * 64 +
-                                                                    16 * (c4 ^ ((p >> 1) & 3)));
+                            v[p] = *reinterpret_cast<const uint32_t *>(
+                                gs + j * kGBytes + p * 64 +
+                                16 * ((pair >> 2) ^ ((p >> 1) & 3)) + 4 * (pair & 3));
 #pragma unroll
                         for (int p = 0; p < 8; ++p) {
-                            const uint32_t *u = &v[p].x;
-#pragma unroll
-                            for (int h = 0; h < 4; ++h) {
-                                const float2 f = unpack_bf16x2(u[h]);
-                                bs[2 * h] += f.x;
-                                bs[2 * h + 1] += f.y;
-                            }
+                            const float2 f = unpack_bf16x2(v[p]);
+                            bs[j][0] += f.x;
+                            bs[j][1] += f.y;
                         }
                     }
                 }
@@ -280,12 +291,11 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
                     ph ^= 1u;
                 }
             }
-            if (j < a.nco) {
-                float *pb = a.pbias + (static_cast<int64_t>(split) * kBiasGroups + pg) * N +
-                            j * kBlk + 8 * c4;
+            float *pb = a.pbias + (static_cast<int64_t>(split) * kBiasGroups + pg) * N + 2 * pair;
 #pragma unroll
-                for (int e = 0; e < 8; ++e) pb[e] = bs[e];
-            }
+            for (int j = 0; j < 4; ++j)
+                if (j < a.nco)
+                    *reinterpret_cast<float2 *>(pb + j * kBlk) = make_float2(bs[j][0], bs[j][1]);
         }
         if (ok && !tc::mbar_wait(&bars.accf, 0, abort_flag)) {
             fail();
@@ -317,47 +327,69 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
 }
 
 // gw[co][ci][dy][dx] = sum over the splits of their partial sums, gb[co] =
-// sum over the splits and their eight pixel groups, one thread per value, in
-// order (the loads of 16 splits are in flight together).  Blocks of 64 threads
-// spread a small layer's 9216 values over the SMs.
+// sum over the splits and their eight pixel groups, each added one after the
+// other in order.  A weight has one thread (the loads of 32 splits are in flight
+// together; blocks of 64 threads spread a small layer's 9216 values over the
+// SMs).  A bias is a chain of 8 x splits terms, up to 608: a block of its own
+// brings 8 channels' terms into shared memory, then 8 threads add (as a
+// thread's loop over global memory this chain took 26 to 39 us of a layer).
 constexpr int kRedThreads = 64;
+constexpr int kBiasChannels = 8, kBiasTerms = 320;
 
 __global__ void __launch_bounds__(kRedThreads)
 wgrad_reduce_kernel(const float *__restrict__ partial, const float *__restrict__ pbias, int splits,
                     int nci, int nco, int cin, int cout, float *__restrict__ gw,
                     float *__restrict__ gb) {
+    __shared__ float s_terms[kBiasTerms][kBiasChannels];
     pdl_wait();
     pdl_trigger();
-    const int N = nco * kBlk;
+    const int N = nco * kBlk, tid = threadIdx.x;
+    const int bias_blocks = N / kBiasChannels;
+    if (static_cast<int>(blockIdx.x) < bias_blocks) {
+        const int co0 = blockIdx.x * kBiasChannels, terms = kBiasGroups * splits;
+        float acc = 0.f;
+        for (int t0 = 0; t0 < terms; t0 += kBiasTerms) {
+            constexpr int kPer = kBiasTerms * kBiasChannels / kRedThreads;
+            float v[kPer];
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                const int e = k * kRedThreads + tid, t = t0 + e / kBiasChannels;
+                v[k] = t < terms ? pbias[static_cast<int64_t>(t) * N + co0 + e % kBiasChannels] : 0.f;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                const int e = k * kRedThreads + tid;
+                s_terms[e / kBiasChannels][e % kBiasChannels] = v[k];
+            }
+            __syncthreads();
+            if (tid < kBiasChannels) {
+#pragma unroll 16
+                for (int t = 0; t < kBiasTerms; ++t) acc += s_terms[t][tid];  // zeros past the end
+            }
+        }
+        if (tid < kBiasChannels && co0 + tid < cout && gb) gb[co0 + tid] = acc;
+        return;
+    }
     const int64_t nw = static_cast<int64_t>(nci) * 3 * N * kLanes;
-    const int64_t at = static_cast<int64_t>(blockIdx.x) * kRedThreads + threadIdx.x;
-    const bool weight = at < nw;
-    const int co_b = static_cast<int>(at - nw);
-    if (!weight && co_b >= N) return;
-    const float *p = weight ? partial + at : pbias + co_b;
-    const int64_t stride = weight ? nw : N;
-    const int terms = weight ? splits : kBiasGroups * splits;
+    const int64_t at = static_cast<int64_t>(blockIdx.x - bias_blocks) * kRedThreads + tid;
+    if (at >= nw) return;
+    const float *p = partial + at;
     float acc = 0.f;
-    constexpr int kU = 16;
-    int s = 0;
-    for (; s + kU <= terms; s += kU) {
+    constexpr int kU = 32;
+    for (int s = 0; s < splits; s += kU) {
         float v[kU];
 #pragma unroll
-        for (int u = 0; u < kU; ++u) v[u] = p[(s + u) * stride];
+        for (int u = 0; u < kU; ++u) v[u] = s + u < splits ? p[(s + u) * nw] : 0.f;
 #pragma unroll
         for (int u = 0; u < kU; ++u) acc += v[u];
     }
-    for (; s < terms; ++s) acc += p[s * stride];
-    if (weight) {
-        const int row = static_cast<int>(at % kLanes);
-        const int64_t r = at / kLanes;
-        const int co = static_cast<int>(r % N), cd = static_cast<int>(r / N);  // ci 3 + dy
-        const int ci = (cd / 3) * kBlk + row % kBlk;
-        if (ci < cin && co < cout)
-            gw[(static_cast<int64_t>(co) * cin + ci) * 9 + (cd % 3) * 3 + row / kBlk] = acc;
-    } else if (co_b < cout && gb) {
-        gb[co_b] = acc;
-    }
+    const int row = static_cast<int>(at % kLanes);
+    const int r = static_cast<int>(at / kLanes);
+    const int co = r % N, cd = r / N;  // cd = ci 3 + dy
+    const int ci = (cd / 3) * kBlk + row % kBlk;
+    if (ci < cin && co < cout)
+        gw[(static_cast<int64_t>(co) * cin + ci) * 9 + (cd % 3) * 3 + row / kBlk] = acc;
 }
 
 // NHWC BF16 [B][H][W][C] as a 4-D tensor (channel, x, y, image), box 32
@@ -421,6 +453,7 @@ int wgrad(const WgradArgs &a, float *gw, float *gb, void *ws, cudaStream_t strea
         return SPP_OK;
     }
     const Plan p = plan(a.B, a.W, a.H, a.cin, a.cout);
+    if (p.nchunks > 0x7fffffff) return SPP_ERR_ARG;
     CUtensorMap xm0, xm1, gm;
     if (!nhwc_map(&xm0, a.x0, a.B, a.H, a.W, a.c0, kHX) ||
         !nhwc_map(&gm, a.g, a.B, a.H, a.W, a.cg, kPX))
@@ -430,7 +463,7 @@ int wgrad(const WgradArgs &a, float *gw, float *gb, void *ws, cudaStream_t strea
     WKernelArgs k;
     k.H = a.H;
     k.W = a.W;
-    k.nchunks = p.nchunks;
+    k.nchunks = static_cast<int>(p.nchunks);
     k.nci = p.nci;
     k.nco = p.nco;
     k.n0 = a.c1 ? a.c0 / kBlk : p.nci;
@@ -451,10 +484,8 @@ int wgrad(const WgradArgs &a, float *gw, float *gb, void *ws, cudaStream_t strea
     }
     launch_dependent(wgrad_kernel, dim3(p.splits, 3 * p.nci), dim3(kThreads), smem, stream, k, xm0,
                      xm1, gm);
-    const int64_t vals = static_cast<int64_t>(p.nci) * 3 * p.nco * kBlk * kLanes + p.nco * kBlk;
-    launch_dependent(wgrad_reduce_kernel,
-                     dim3(static_cast<unsigned>((vals + kRedThreads - 1) / kRedThreads)),
-                     dim3(kRedThreads), 0, stream, k.partial, k.pbias, p.splits, p.nci, p.nco,
+    const int blocks = p.nci * 3 * p.nco * kBlk * kLanes / kRedThreads + p.nco * kBlk / kBiasChannels;
+    launch_dependent(wgrad_reduce_kernel, dim3(blocks), dim3(kRedThreads), 0, stream, k.partial, k.pbias, p.splits, p.nci, p.nco,
                      a.cin, a.cout, gw, gb);
     count_launch(2);
     return launch_status();
