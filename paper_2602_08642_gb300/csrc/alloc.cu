@@ -50,6 +50,11 @@ struct AllocHeader {
     double S, a, c, lam, h;
     float a_hi, a_lo, c_hi, c_lo, lam_f, h_f;
     int fast_ok;
+    // fixed-point form of the systematic map (FixCoef)
+    unsigned long long c64, a52;
+    float lh_hi, lh_lo;
+    int r0;
+    int fix_ok;
 };
 constexpr size_t kHeaderBytes = 256;
 static_assert(sizeof(AllocHeader) <= kHeaderBytes, "alloc header too large");
@@ -205,6 +210,14 @@ __device__ void finalize_budget(AllocHeader *hdr, const unsigned long long *limb
     const bool c_ok = c >= 0x1p-60 && c <= 0x1p60;
     const bool a_ok = a == 0.0 || (a >= 0x1p-60 && a <= 0x1p60);
     hdr->fast_ok = (c_ok && a_ok && !args.force_exact) ? 1 : 0;
+    const unsigned long long cb = static_cast<unsigned long long>(__double_as_longlong(c));
+    hdr->c64 = ((cb & ((1ull << 52) - 1ull)) | (1ull << 52)) << 11;
+    hdr->r0 = 85 - (static_cast<int>(cb >> 52) - 1075);
+    hdr->a52 = __double2ull_rz(__dmul_rn(a, 0x1p52));
+    const double lh = __dmul_rn(args.lambda, h);
+    hdr->lh_hi = __double2float_rn(lh);
+    hdr->lh_lo = __double2float_rn(__dsub_rn(lh, static_cast<double>(hdr->lh_hi)));
+    hdr->fix_ok = (c_ok && a < 1024.0 && lh < 0x1p60 && !args.force_exact) ? 1 : 0;
     __threadfence();
     hdr->valid = 1;
 }
@@ -866,9 +879,108 @@ offsets_kernel(const int32_t *__restrict__ counts, long long N, const int *__res
 //   p_i = q_i mod 2^32; the holdout ramp of Sec. 4.3 at u = a_i 2^-32.
 // Reduce-then-scan with no waits between blocks: tile sums of q, one block
 // scans them, then every tile scans its own pixels from its prefix.
-__device__ __forceinline__ long long fixed_q(float d, double a, double c) {
+//
+// q_i and s_i are those of FP64 round-to-nearest arithmetic.  In FP64 the two
+// passes kept the FP64 pipe (2 results per clock and SM) busy for most of the
+// map's 264 us at 2560 x 1440; integers decide all but about 1e-5 of the pixels
+// (71 us).  With c = C
+// 2^ec (C of 53 bits) and d = m 2^(E - 150) (m of 24 bits)
+//   X = floor(a 2^52) + (floor(C m 2^-13) >> r),  r = 85 - ec - E,
+// is s 2^52 short of the exact value by less than 3, and the two FP64
+// roundings of a + c d move s by at most 2^-52 s.  So the FP64 result lies
+// within `margin` of X, and where both ends of that interval round to the
+// same q (or to the same FP32 s) that is the FP64 result's; else, and where
+// the shift leaves its range, the FP64 sequence runs.
+struct FixCoef {
+    unsigned long long c64, a52;
+    int r0, ok;
+    double a, c;
+};
+
+__device__ __forceinline__ FixCoef fix_coef(const AllocHeader *hdr) {
+    FixCoef k;
+    k.c64 = hdr->c64;
+    k.a52 = hdr->a52;
+    k.r0 = hdr->r0;
+    k.ok = hdr->fix_ok;
+    k.a = hdr->a;
+    k.c = hdr->c;
+    return k;
+}
+
+struct SysPixel {
+    long long q;
+    float s;
+};
+
+__device__ __noinline__ SysPixel sys_exact(float d, double a, double c) {
     const double sd = __dadd_rn(a, __dmul_rn(c, static_cast<double>(d)));
-    return __double2ll_rn(__dmul_rn(sd, 4294967296.0));
+    SysPixel r;
+    r.q = __double2ll_rn(__dmul_rn(sd, 4294967296.0));
+    r.s = __double2float_rn(sd);
+    return r;
+}
+
+// The pixel's q and, with WITH_S, its FP32 s.
+template <bool WITH_S>
+__device__ __forceinline__ SysPixel sys_pixel(float d, const FixCoef &k) {
+    const uint32_t bits = __float_as_uint(d);
+    const uint32_t e = bits >> 23;
+    const uint32_t m8 = ((bits & 0x7fffffu) | (e ? 0x800000u : 0u)) << 8;
+    const int r = k.r0 - static_cast<int>(e ? e : 1u);
+    const unsigned long long Z =
+        (k.c64 >> 32) * m8 + (((k.c64 & 0xffffffffull) * m8) >> 32);
+    const unsigned long long X = k.a52 + (r < 64 ? Z >> (r & 63) : 0ull);
+    const unsigned long long margin = 6ull + (X >> 52);
+    const unsigned long long lo = X - margin, hi = X + margin;
+    SysPixel o;
+    o.q = static_cast<long long>((lo + (1ull << 19)) >> 20);
+    bool ok = k.ok && r >= 0 && X >= margin && X < (1ull << 62) &&
+              o.q == static_cast<long long>((hi + (1ull << 19)) >> 20);
+    o.s = 0.0f;
+    if (WITH_S) {
+        o.s = __ull2float_rn(lo);
+        ok = ok && o.s == __ull2float_rn(hi);
+        o.s *= 0x1p-52f;
+    }
+    if (!ok) o = sys_exact(d, k.a, k.c);
+    return o;
+}
+
+// The holdout weight h clip((lambda / p)(u + p - 1), 0, 1) of an extra sample,
+// u = a32 2^-32 and p = p32 2^-32, rounded once from its FP64 sequence.
+__device__ __noinline__ float sys_weight_exact(uint32_t a32, uint32_t p32, double lam, double h) {
+    const double u = __dmul_rn(static_cast<double>(a32), 0x1p-32);
+    const double p = __dmul_rn(static_cast<double>(p32), 0x1p-32);
+    const double r0 = __dmul_rn(__ddiv_rn(lam, p), __dsub_rn(__dadd_rn(u, p), 1.0));
+    return __double2float_rn(__dmul_rn(h, r0 < 0.0 ? 0.0 : (r0 > 1.0 ? 1.0 : r0)));
+}
+
+// The same in float-float: lambda h v / p with v = a32 + p32 - 2^32 (relative
+// error below 2^-42), used where it is clear of the clip and of a rounding
+// boundary (all but about 1e-5 of the extra samples).
+__device__ __forceinline__ float sys_weight(uint32_t a32, uint32_t p32, const AllocHeader *hdr,
+                                            float lh_hi, float lh_lo, float h_f, int fix_ok) {
+    const uint32_t v32 = a32 + p32;  // mod 2^32: exact, 0 <= v < p
+    // leading 24 bits and the (at most 8-bit) rest of each, exact
+    const float ph = __uint2float_rz(p32), vh = __uint2float_rz(v32);
+    const float pl = static_cast<float>(p32 - __float2uint_rz(ph));
+    const float vl = static_cast<float>(v32 - __float2uint_rz(vh));
+    const float rc = __frcp_rn(__fadd_rn(ph, pl));
+    const float q1 = __fmul_rn(__fadd_rn(vh, vl), rc);
+    const float rem = __fmaf_rn(-q1, pl, __fadd_rn(__fmaf_rn(-q1, ph, vh), vl));
+    const float q2 = __fmul_rn(rem, rc);
+    const float w1 = __fmul_rn(q1, lh_hi);
+    const float e = __fadd_rn(__fmaf_rn(q1, lh_hi, -w1),
+                              __fmaf_rn(q1, lh_lo, __fmul_rn(q2, lh_hi)));
+    const float wh = __fadd_rn(w1, e), wl = __fsub_rn(e, __fsub_rn(wh, w1));
+    if (fix_ok) {
+        if (wh > __fmul_rn(h_f, 1.0f + 0x1p-20f)) return h_f;
+        const float tol = __fmul_rn(wh, 0x1p-41f);
+        const float f1 = __fadd_rn(wh, __fsub_rn(wl, tol)), f2 = __fadd_rn(wh, __fadd_rn(wl, tol));
+        if (wh < __fmul_rn(h_f, 1.0f - 0x1p-20f) && f1 == f2) return f1;
+    }
+    return sys_weight_exact(a32, p32, hdr->lam, hdr->h);
 }
 
 __device__ __forceinline__ long long block_excl_scan_ll(long long v, long long &total) {
@@ -894,17 +1006,36 @@ __device__ __forceinline__ long long block_excl_scan_ll(long long v, long long &
     return before + incl - v;
 }
 
+// The densities of a thread's eight neighbouring pixels (zeros past the end).
+__device__ __forceinline__ void load_density(const float *__restrict__ d, long long base,
+                                             long long N, float (&dv)[kScanItems]) {
+    if (base + kScanItems <= N) {
+        const float4 v0 = __ldg(reinterpret_cast<const float4 *>(d + base));
+        const float4 v1 = __ldg(reinterpret_cast<const float4 *>(d + base) + 1);
+        dv[0] = v0.x; dv[1] = v0.y; dv[2] = v0.z; dv[3] = v0.w;
+        dv[4] = v1.x; dv[5] = v1.y; dv[6] = v1.z; dv[7] = v1.w;
+    } else {
+#pragma unroll
+        for (int q = 0; q < kScanItems; ++q) dv[q] = (base + q < N) ? d[base + q] : 0.0f;
+    }
+}
+
 __global__ void __launch_bounds__(kScanThreads)
 sys_tile_sum_kernel(const float *__restrict__ d, long long N, const AllocHeader *hdr,
                     long long *__restrict__ tile_sums) {
+    pdl_wait();
+    pdl_trigger();
     const long long base = static_cast<long long>(blockIdx.x) * kTile +
                            static_cast<long long>(threadIdx.x) * kScanItems;
-    const int valid = hdr->valid;
-    const double a = hdr->a, c = hdr->c;
+    float dv[kScanItems];
+    load_density(d, base, N, dv);
     long long sum = 0;
+    if (hdr->valid) {
+        const FixCoef k = fix_coef(hdr);
 #pragma unroll
-    for (int q = 0; q < kScanItems; ++q)
-        if (base + q < N && valid) sum += fixed_q(d[base + q], a, c);
+        for (int q = 0; q < kScanItems; ++q)
+            if (base + q < N) sum += sys_pixel<false>(dv[q], k).q;
+    }
     long long total;
     (void)block_excl_scan_ll(sum, total);
     if (threadIdx.x == 0) tile_sums[blockIdx.x] = total;
@@ -913,6 +1044,8 @@ sys_tile_sum_kernel(const float *__restrict__ d, long long N, const AllocHeader 
 // Exclusive scan of the tile sums in place, one block.
 __global__ void __launch_bounds__(kScanThreads)
 sys_scan_tiles_kernel(long long *__restrict__ tile_sums, int num_tiles) {
+    pdl_wait();
+    pdl_trigger();
     const int per = (num_tiles + kScanThreads - 1) / kScanThreads;
     const int t0 = static_cast<int>(threadIdx.x) * per;
     long long mine = 0;
@@ -933,53 +1066,81 @@ sys_assign_kernel(const float *__restrict__ d, long long N, const AllocHeader *h
                   int32_t *__restrict__ sample_pixel, long long capacity,
                   float *__restrict__ s_out, float *__restrict__ w_out, long long *total,
                   int32_t *status) {
+    pdl_wait();
+    pdl_trigger();
     const long long base = static_cast<long long>(blockIdx.x) * kTile +
                            static_cast<long long>(threadIdx.x) * kScanItems;
     const int valid = hdr->valid;
-    const double a = hdr->a, c = hdr->c, lam = hdr->lam, h = hdr->h;
+    const float lh_hi = hdr->lh_hi, lh_lo = hdr->lh_lo, h_f = hdr->h_f;
+    const int fix_ok = hdr->fix_ok;
+    const FixCoef k = fix_coef(hdr);
+    float dv[kScanItems], sv[kScanItems], wv[kScanItems];
+    load_density(d, base, N, dv);
     long long qv[kScanItems];
     long long sum = 0;
 #pragma unroll
     for (int q = 0; q < kScanItems; ++q) {
-        qv[q] = (base + q < N && valid) ? fixed_q(d[base + q], a, c) : 0;
+        qv[q] = 0;
+        sv[q] = 1.0f;
+        if (base + q < N && valid) {
+            const SysPixel r = sys_pixel<true>(dv[q], k);
+            qv[q] = r.q;
+            sv[q] = r.s;
+        }
         sum += qv[q];
     }
     long long tot;
     long long A = tile_prefix[blockIdx.x] + block_excl_scan_ll(sum, tot) +
                   static_cast<long long>(U);
+    int n[kScanItems], off[kScanItems];
 #pragma unroll
     for (int q = 0; q < kScanItems; ++q) {
-        const long long i = base + q;
-        if (i >= N) break;
-        const long long f = qv[q] >> 32;
-        const unsigned long long p32 = static_cast<unsigned long long>(qv[q]) & 0xFFFFFFFFull;
-        const unsigned long long a32 = static_cast<unsigned long long>(A) & 0xFFFFFFFFull;
-        const bool extra = a32 + p32 >= (1ull << 32);
-        const int n = static_cast<int>(f) + (extra ? 1 : 0);
-        const int off = static_cast<int>(A >> 32);
-        double wd = 1.0;
-        if (extra && !hard) {
-            const double u = __dmul_rn(static_cast<double>(a32), 0x1p-32);
-            const double p = __dmul_rn(static_cast<double>(p32), 0x1p-32);
-            const double r0 = __dmul_rn(__ddiv_rn(lam, p), __dsub_rn(__dadd_rn(u, p), 1.0));
-            wd = __dmul_rn(h, r0 < 0.0 ? 0.0 : (r0 > 1.0 ? 1.0 : r0));
-        }
-        offsets[i] = off;
-        if (counts) counts[i] = n;
-        s_out[i] = valid ? __double2float_rn(__dadd_rn(a, __dmul_rn(c, static_cast<double>(d[i]))))
-                         : 1.0f;
-        w_out[i] = __double2float_rn(wd);
-        for (int r = 0; r < n; ++r) {
-            const long long t = static_cast<long long>(off) + r;
-            if (t < capacity) sample_pixel[t] = static_cast<int32_t>(i);
-        }
+        const uint32_t p32 = static_cast<uint32_t>(qv[q]), a32 = static_cast<uint32_t>(A);
+        const bool extra = a32 + p32 < a32;  // carries out of 32 bits
+        n[q] = static_cast<int>(qv[q] >> 32) + (extra ? 1 : 0);
+        off[q] = static_cast<int>(A >> 32);
+        wv[q] = extra && !hard ? sys_weight(a32, p32, hdr, lh_hi, lh_lo, h_f, fix_ok) : 1.0f;
         A += qv[q];
-        if (i == N - 1) {
-            const long long T = A >> 32;
-            offsets[N] = static_cast<int32_t>(T);
-            *total = T;
-            if (T > capacity) set_status(status, SPP_ERR_CAPACITY);
+    }
+    if (base + kScanItems <= N) {
+        int4 *o4 = reinterpret_cast<int4 *>(offsets + base);
+        o4[0] = make_int4(off[0], off[1], off[2], off[3]);
+        o4[1] = make_int4(off[4], off[5], off[6], off[7]);
+        float4 *s4 = reinterpret_cast<float4 *>(s_out + base);
+        s4[0] = make_float4(sv[0], sv[1], sv[2], sv[3]);
+        s4[1] = make_float4(sv[4], sv[5], sv[6], sv[7]);
+        float4 *w4 = reinterpret_cast<float4 *>(w_out + base);
+        w4[0] = make_float4(wv[0], wv[1], wv[2], wv[3]);
+        w4[1] = make_float4(wv[4], wv[5], wv[6], wv[7]);
+        if (counts) {
+            int4 *c4 = reinterpret_cast<int4 *>(counts + base);
+            c4[0] = make_int4(n[0], n[1], n[2], n[3]);
+            c4[1] = make_int4(n[4], n[5], n[6], n[7]);
         }
+    } else {
+#pragma unroll
+        for (int q = 0; q < kScanItems; ++q) {
+            if (base + q < N) {
+                offsets[base + q] = off[q];
+                s_out[base + q] = sv[q];
+                w_out[base + q] = wv[q];
+                if (counts) counts[base + q] = n[q];
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kScanItems; ++q) {
+        for (int r = 0; r < n[q]; ++r) {
+            const long long t = static_cast<long long>(off[q]) + r;
+            if (t < capacity) sample_pixel[t] = static_cast<int32_t>(base + q);
+        }
+    }
+    // the owner of the last pixel closes the scan (pixels past the end have q = 0)
+    if (base <= N - 1 && N - 1 < base + kScanItems) {
+        const long long T = A >> 32;
+        offsets[N] = static_cast<int32_t>(T);
+        *total = T;
+        if (T > capacity) set_status(status, SPP_ERR_CAPACITY);
     }
 }
 
@@ -1079,11 +1240,13 @@ int alloc_impl(const float *d, int W, int H, const spp_params *p, const Dither &
         const unsigned long long U =
             stream_bits(stream_key(p->seed, p->frame), 1ull << 62) >> 32;
         auto *tile_sums = reinterpret_cast<long long *>(tiles);
-        sys_tile_sum_kernel<<<num_tiles, kScanThreads, 0, stream>>>(d, N, hdr, tile_sums);
-        sys_scan_tiles_kernel<<<1, kScanThreads, 0, stream>>>(tile_sums, num_tiles);
-        sys_assign_kernel<<<num_tiles, kScanThreads, 0, stream>>>(
-            d, N, hdr, tile_sums, U, args.hard, counts, offsets, sample_pixel, capacity, s_out,
-            holdout_w, reinterpret_cast<long long *>(total), status);
+        launch_dependent(sys_tile_sum_kernel, dim3(num_tiles), dim3(kScanThreads), 0, stream, d, N,
+                         hdr, tile_sums);
+        launch_dependent(sys_scan_tiles_kernel, dim3(1), dim3(kScanThreads), 0, stream, tile_sums,
+                         num_tiles);
+        launch_dependent(sys_assign_kernel, dim3(num_tiles), dim3(kScanThreads), 0, stream, d, N,
+                         hdr, tile_sums, U, args.hard, counts, offsets, sample_pixel, capacity,
+                         s_out, holdout_w, reinterpret_cast<long long *>(total), status);
         count_launch(4);
         return launch_status();
     }
