@@ -794,6 +794,77 @@ int spp_splat_backward_estimator(const int32_t *offsets, const int32_t *counts, 
 int spp_density_lowres(const float *d, int W, int H, int factor, float *out,
                        cudaStream_t stream);
 
+/* ------------------------------------------------------------- batches
+ * The steps of a training batch, B images of one size per call and launch.
+ * Each is the entry of the same name without _batch on every image (the same
+ * results, image by image), with this layout:
+ *   - contiguous arrays hold the images one after the other; offsets take
+ *     W*H + SPP_BATCH_OFFSETS_PAD values per image, total 2, status 4 (the
+ *     first of each is used), sample buffers `capacity` slots, losses 4 floats;
+ *   - inputs that a caller holds image by image (G-buffers, clean radiance,
+ *     motion, previous outputs) are HOST arrays of B device pointers;
+ *   - seeds and render_seeds are HOST arrays of B seeds (p->seed is not read);
+ *   - the mask is shared.
+ * With B > 1 every image's data starts on a 16-byte boundary: W*H, and for
+ * logits C * Wl * Hl, are multiples of 4 (SPP_ERR_ALIGN otherwise). */
+#define SPP_BATCH_OFFSETS_PAD 4
+int spp_assemble_features_batch(int B, const float *const *albedo, const float *const *normal,
+                                const float *const *depth, const float *const *mv,
+                                const float *prev_ldr, int W, int H, float *in12,
+                                cudaStream_t stream);
+size_t spp_alloc_batch_workspace_bytes(int B, int W, int H);
+/* counts are required, p->flags must be 0 */
+int spp_alloc_sample_map_batch(int B, const float *d, int W, int H, const spp_params *p,
+                               const uint64_t *seeds, int32_t *counts, int32_t *offsets,
+                               int32_t *sample_pixel, int64_t capacity, float *s_out,
+                               float *holdout_w, int64_t *total, int32_t *status, void *ws,
+                               size_t ws_bytes, cudaStream_t stream);
+int spp_render_synthetic_batch(int B, const float *const *clean, const int32_t *offsets,
+                               const int32_t *sample_pixel, const int64_t *total, int64_t capacity,
+                               int W, int H, const uint64_t *seeds, uint32_t frame, float *rgb,
+                               cudaStream_t stream);
+int spp_splat_samples_batch(int B, const int32_t *offsets, const float *rgb, const float *s,
+                            const float *holdout_w, int64_t capacity, int W, int H, int L,
+                            float *const *layers, cudaStream_t stream);
+/* logits [B][C][Hl][Wl] with C at least the planes that the level uses */
+int spp_reconstruct_level_batch(int B, const float *noisy, const float *logits, int C,
+                                const float *coarse, const float *warped_prev, const uint8_t *mask,
+                                int Wl, int Hl, const spp_tonemap *tm, float *out, float *out_ldr,
+                                int32_t *status, cudaStream_t stream);
+int spp_warp_previous_batch(int B, const float *const *prev_hdr, const float *const *mv, int W,
+                            int H, float *warped, cudaStream_t stream);
+int spp_tonemap_image_batch(int B, const float *const *hdr, int W, int H, const spp_tonemap *tm,
+                            float *ldr, cudaStream_t stream);
+int spp_l1_loss_batch(int B, const float *ldr, const float *ref, int64_t n, float *loss,
+                      float *grad_ldr, cudaStream_t stream);
+int spp_combined_loss_batch(int B, const float *ldr, const float *ref, const float *prev_warped,
+                            const float *ref_prev_warped, int64_t n, float temporal_weight,
+                            float spatial_weight, float *loss, float *grad_ldr,
+                            cudaStream_t stream);
+int spp_tonemap_backward_batch(int B, const float *hdr, int W, int H, const spp_tonemap *tm,
+                               const float *grad_ldr, float *grad_hdr, cudaStream_t stream);
+/* grad_logits has the layout of logits; its planes [0, Cg) are written */
+int spp_reconstruct_level_backward_batch(int B, const float *noisy, const float *logits, int C,
+                                         const float *coarse, const float *warped_prev,
+                                         const uint8_t *mask, int Wl, int Hl,
+                                         const float *grad_out, float *grad_logits, int Cg,
+                                         float *grad_noisy, float *grad_coarse,
+                                         float *grad_warped, cudaStream_t stream);
+int spp_pyramid_backward_batch(int B, const float *const *grad_layers, int W, int H, int L,
+                               float *grad_L0, cudaStream_t stream);
+int spp_splat_backward_batch(int B, const int32_t *offsets, const int32_t *counts, const float *rgb,
+                             const float *s, const float *layer0, const float *grad_layer0,
+                             const float *holdout_w, int64_t capacity, int W, int H,
+                             const spp_params *p, const uint64_t *seeds, int estimator,
+                             const float *const *clean, const uint64_t *render_seeds,
+                             float *grad_s, cudaStream_t stream);
+/* ws: B times spp_density_backward_workspace_bytes(); grad_z_stride floats
+ * between the images' grad_z */
+int spp_density_backward_batch(int B, const float *d, int64_t N, double budget,
+                               double uniform_fraction, const float *grad_s, float *grad_z,
+                               int64_t grad_z_stride, void *ws, size_t ws_bytes,
+                               cudaStream_t stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -155,6 +155,27 @@ _SIGS = {
     "spp_warp_channels": (_I, [_P, _I, _P, _I, _I, _P, _P]),
     "spp_splat_backward_estimator": (_I, [_P, _P, _P, _P, _P, _P, _P, _I64, _I, _I,
                                           ctypes.POINTER(spp_params), _I, _P, _U64, _P, _P]),
+    "spp_assemble_features_batch": (_I, [_I, _P, _P, _P, _P, _P, _I, _I, _P, _P]),
+    "spp_alloc_batch_workspace_bytes": (_SZ, [_I, _I, _I]),
+    "spp_alloc_sample_map_batch": (_I, [_I, _P, _I, _I, ctypes.POINTER(spp_params), _P, _P, _P, _P,
+                                        _I64, _P, _P, _P, _P, _P, _SZ, _P]),
+    "spp_render_synthetic_batch": (_I, [_I, _P, _P, _P, _P, _I64, _I, _I, _P, _U32, _P, _P]),
+    "spp_splat_samples_batch": (_I, [_I, _P, _P, _P, _P, _I64, _I, _I, _I, _P, _P]),
+    "spp_reconstruct_level_batch": (_I, [_I, _P, _P, _I, _P, _P, _P, _I, _I,
+                                         ctypes.POINTER(spp_tonemap), _P, _P, _P, _P]),
+    "spp_warp_previous_batch": (_I, [_I, _P, _P, _I, _I, _P, _P]),
+    "spp_tonemap_image_batch": (_I, [_I, _P, _I, _I, ctypes.POINTER(spp_tonemap), _P, _P]),
+    "spp_l1_loss_batch": (_I, [_I, _P, _P, _I64, _P, _P, _P]),
+    "spp_combined_loss_batch": (_I, [_I, _P, _P, _P, _P, _I64, ctypes.c_float, ctypes.c_float, _P,
+                                     _P, _P]),
+    "spp_tonemap_backward_batch": (_I, [_I, _P, _I, _I, ctypes.POINTER(spp_tonemap), _P, _P, _P]),
+    "spp_reconstruct_level_backward_batch": (_I, [_I, _P, _P, _I, _P, _P, _P, _I, _I, _P, _P, _I,
+                                                  _P, _P, _P, _P]),
+    "spp_pyramid_backward_batch": (_I, [_I, _P, _I, _I, _I, _P, _P]),
+    "spp_splat_backward_batch": (_I, [_I, _P, _P, _P, _P, _P, _P, _P, _I64, _I, _I,
+                                      ctypes.POINTER(spp_params), _P, _I, _P, _P, _P, _P]),
+    "spp_density_backward_batch": (_I, [_I, _P, _I64, ctypes.c_double, ctypes.c_double, _P, _P,
+                                        _I64, _P, _SZ, _P]),
 }
 for _name, (_res, _args) in _SIGS.items():
     _fn = getattr(lib, _name)
@@ -708,3 +729,132 @@ def spp_assemble_denoiser_input(L0, s, counts, albedo, normal, depth, mv, warped
         _dev(L0, f), _dev(s, f), _dev(counts, torch.int32), _dev(albedo, f), _dev(normal, f),
         _dev(depth, f), _dev(mv, f), _dev(warped_prev_hdr, f), _dev(warped_latent, f), W, H,
         _dev(x_nhwc32, torch.bfloat16), _stream(stream))
+
+
+# ---------------------------------------------------------------- batches
+# Arguments named *_list are lists of B tensors (one per image); the others
+# hold the images one after the other.
+SPP_BATCH_OFFSETS_PAD = 4
+
+
+def _seed_array(seeds):
+    return (ctypes.c_uint64 * len(seeds))(*[s & 0xFFFFFFFFFFFFFFFF for s in seeds])
+
+
+def _list(ts):
+    return ctypes.cast(_ptr_array(ts, torch.float32), _P)
+
+
+def spp_assemble_features_batch(albedo_list, normal_list, depth_list, mv_list, prev_ldr, W, H, in12,
+                                stream=None) -> int:
+    f = torch.float32
+    return lib.spp_assemble_features_batch(
+        len(mv_list), _list(albedo_list), _list(normal_list), _list(depth_list), _list(mv_list),
+        _dev(prev_ldr, f), W, H, _dev(in12, f), _stream(stream))
+
+
+def spp_alloc_batch_workspace_bytes(B: int, W: int, H: int) -> int:
+    return int(lib.spp_alloc_batch_workspace_bytes(B, W, H))
+
+
+def spp_alloc_sample_map_batch(B, d, W, H, params: spp_params, seeds, counts, offsets, sample_pixel,
+                               capacity, s_out, holdout_w, total, status, ws, stream=None) -> int:
+    return lib.spp_alloc_sample_map_batch(
+        B, _dev(d, torch.float32), W, H, ctypes.byref(params), ctypes.cast(_seed_array(seeds), _P),
+        _dev(counts, torch.int32), _dev(offsets, torch.int32), _dev(sample_pixel, torch.int32),
+        int(capacity), _dev(s_out, torch.float32), _dev(holdout_w, torch.float32),
+        _dev(total, torch.int64), _dev(status, torch.int32), _dev(ws), _nbytes(ws),
+        _stream(stream))
+
+
+def spp_render_synthetic_batch(clean_list, offsets, sample_pixel, total, capacity, W, H, seeds,
+                               frame, rgb, stream=None) -> int:
+    return lib.spp_render_synthetic_batch(
+        len(clean_list), _list(clean_list), _dev(offsets, torch.int32),
+        _dev(sample_pixel, torch.int32), _dev(total, torch.int64), int(capacity), W, H,
+        ctypes.cast(_seed_array(seeds), _P), frame, _dev(rgb, torch.float32), _stream(stream))
+
+
+def spp_splat_samples_batch(B, offsets, rgb, s, holdout_w, capacity, W, H, L, layers,
+                            stream=None) -> int:
+    f = torch.float32
+    return lib.spp_splat_samples_batch(
+        B, _dev(offsets, torch.int32), _dev(rgb, f), _dev(s, f), _dev(holdout_w, f), int(capacity),
+        W, H, L, _list(layers), _stream(stream))
+
+
+def spp_reconstruct_level_batch(B, noisy, logits, C, coarse, warped_prev, mask, Wl, Hl, tm, out,
+                                out_ldr, status=None, stream=None) -> int:
+    f = torch.float32
+    return lib.spp_reconstruct_level_batch(
+        B, _dev(noisy, f), _dev(logits, f), C, _dev(coarse, f), _dev(warped_prev, f),
+        _dev(mask, torch.uint8), Wl, Hl, ctypes.byref(tm) if tm is not None else None,
+        _dev(out, f), _dev(out_ldr, f), _dev(status, torch.int32), _stream(stream))
+
+
+def spp_warp_previous_batch(prev_list, mv_list, W, H, warped, stream=None) -> int:
+    return lib.spp_warp_previous_batch(len(mv_list), _list(prev_list), _list(mv_list), W, H,
+                                       _dev(warped, torch.float32), _stream(stream))
+
+
+def spp_tonemap_image_batch(hdr_list, W, H, tm, ldr, stream=None) -> int:
+    return lib.spp_tonemap_image_batch(len(hdr_list), _list(hdr_list), W, H, ctypes.byref(tm),
+                                       _dev(ldr, torch.float32), _stream(stream))
+
+
+def spp_l1_loss_batch(B, ldr, ref, n, loss, grad_ldr, stream=None) -> int:
+    f = torch.float32
+    return lib.spp_l1_loss_batch(B, _dev(ldr, f), _dev(ref, f), int(n), _dev(loss, f),
+                                 _dev(grad_ldr, f), _stream(stream))
+
+
+def spp_combined_loss_batch(B, ldr, ref, prev_warped, ref_prev_warped, n, temporal_weight,
+                            spatial_weight, loss, grad_ldr, stream=None) -> int:
+    f = torch.float32
+    return lib.spp_combined_loss_batch(
+        B, _dev(ldr, f), _dev(ref, f), _dev(prev_warped, f), _dev(ref_prev_warped, f), int(n),
+        float(temporal_weight), float(spatial_weight), _dev(loss, f), _dev(grad_ldr, f),
+        _stream(stream))
+
+
+def spp_tonemap_backward_batch(B, hdr, W, H, tm, grad_ldr, grad_hdr, stream=None) -> int:
+    f = torch.float32
+    return lib.spp_tonemap_backward_batch(B, _dev(hdr, f), W, H,
+                                          ctypes.byref(tm) if tm is not None else None,
+                                          _dev(grad_ldr, f), _dev(grad_hdr, f), _stream(stream))
+
+
+def spp_reconstruct_level_backward_batch(B, noisy, logits, C, coarse, warped_prev, mask, Wl, Hl,
+                                         grad_out, grad_logits, Cg, grad_noisy, grad_coarse,
+                                         grad_warped, stream=None) -> int:
+    f = torch.float32
+    return lib.spp_reconstruct_level_backward_batch(
+        B, _dev(noisy, f), _dev(logits, f), C, _dev(coarse, f), _dev(warped_prev, f),
+        _dev(mask, torch.uint8), Wl, Hl, _dev(grad_out, f), _dev(grad_logits, f), Cg,
+        _dev(grad_noisy, f), _dev(grad_coarse, f), _dev(grad_warped, f), _stream(stream))
+
+
+def spp_pyramid_backward_batch(B, grad_layers, W, H, L, grad_L0, stream=None) -> int:
+    return lib.spp_pyramid_backward_batch(B, _list(grad_layers), W, H, L,
+                                          _dev(grad_L0, torch.float32), _stream(stream))
+
+
+def spp_splat_backward_batch(B, offsets, counts, rgb, s, layer0, grad_layer0, holdout_w, capacity,
+                             W, H, params: spp_params, seeds, estimator: int, clean_list,
+                             render_seeds, grad_s, stream=None) -> int:
+    f = torch.float32
+    return lib.spp_splat_backward_batch(
+        B, _dev(offsets, torch.int32), _dev(counts, torch.int32), _dev(rgb, f), _dev(s, f),
+        _dev(layer0, f), _dev(grad_layer0, f), _dev(holdout_w, f), int(capacity), W, H,
+        ctypes.byref(params), ctypes.cast(_seed_array(seeds), _P), int(estimator),
+        _list(clean_list), ctypes.cast(_seed_array(render_seeds), _P), _dev(grad_s, f),
+        _stream(stream))
+
+
+def spp_density_backward_batch(B, d, N, budget, uniform_fraction, grad_s, grad_z, grad_z_stride, ws,
+                               stream=None) -> int:
+    f = torch.float32
+    return lib.spp_density_backward_batch(B, _dev(d, f), int(N), float(budget),
+                                          float(uniform_fraction), _dev(grad_s, f),
+                                          _dev(grad_z, f), int(grad_z_stride), _dev(ws),
+                                          _nbytes(ws), _stream(stream))

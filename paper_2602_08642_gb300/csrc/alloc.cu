@@ -37,6 +37,10 @@ constexpr int kTile = kScanThreads * kScanItems;
 // larger ones the two-pass form without waits between blocks
 constexpr int kSinglePassMaxTiles = 64;
 
+// per-image strides of a batched map (spp_alloc_sample_map_batch)
+constexpr int kOffsetsPad = SPP_BATCH_OFFSETS_PAD;
+constexpr int kTotalStride = 2, kStatusStride = 4;
+
 constexpr unsigned long long kFlagAgg = 1ull << 62;
 constexpr unsigned long long kFlagInc = 2ull << 62;
 constexpr int kSpinLimit = 1 << 20;
@@ -225,9 +229,13 @@ __device__ void finalize_budget(AllocHeader *hdr, const unsigned long long *limb
 template <int U>
 __global__ void __launch_bounds__(kSumThreads)
 budget_sum_kernel(const float *__restrict__ d, long long N, AllocHeader *hdr, BudgetArgs args,
-                  int32_t *status) {
+                  int32_t *status, size_t ws_stride) {
     pdl_wait();
     pdl_trigger();
+    // image blockIdx.y of a batch
+    d += blockIdx.y * N;
+    hdr = reinterpret_cast<AllocHeader *>(reinterpret_cast<char *>(hdr) + blockIdx.y * ws_stride);
+    status += blockIdx.y * kStatusStride;
     unsigned long long lim[kLimbs];
 #pragma unroll
     for (int j = 0; j < kLimbs; ++j) lim[j] = 0ull;
@@ -690,11 +698,22 @@ assign_scan_kernel(const float *__restrict__ d, long long N, const AllocHeader *
 // second pass re-reads them from L2); small frames keep the single pass.
 __global__ void __launch_bounds__(kScanThreads, 4)
 assign_tile_kernel(const float *__restrict__ d, long long N, const AllocHeader *hdr_c,
-                   uint64_t key, Dither dither, int hard, int32_t *__restrict__ counts,
+                   const __grid_constant__ StreamKeys keys, Dither dither, int hard,
+                   int32_t *__restrict__ counts,
                    float *__restrict__ s_out, float *__restrict__ w_out,
-                   int *__restrict__ tile_sums) {
+                   int *__restrict__ tile_sums, size_t ws_stride) {
     pdl_wait();
     pdl_trigger();
+    // image blockIdx.y of a batch
+    const uint64_t key = keys.k[blockIdx.y];
+    d += blockIdx.y * N;
+    counts += blockIdx.y * N;
+    s_out += blockIdx.y * N;
+    w_out += blockIdx.y * N;
+    hdr_c = reinterpret_cast<const AllocHeader *>(reinterpret_cast<const char *>(hdr_c) +
+                                                  blockIdx.y * ws_stride);
+    tile_sums = reinterpret_cast<int *>(reinterpret_cast<char *>(tile_sums) +
+                                        blockIdx.y * ws_stride);
     const int tile = blockIdx.x;
     const long long base = static_cast<long long>(tile) * kTile +
                            static_cast<long long>(threadIdx.x) * kScanItems;
@@ -788,9 +807,17 @@ assign_tile_kernel(const float *__restrict__ d, long long N, const AllocHeader *
 __global__ void __launch_bounds__(kScanThreads)
 offsets_kernel(const int32_t *__restrict__ counts, long long N, const int *__restrict__ tile_sums,
                int num_tiles, int32_t *__restrict__ offsets, int32_t *__restrict__ sample_pixel,
-               long long capacity, long long *total, int32_t *status) {
+               long long capacity, long long *total, int32_t *status, size_t ws_stride) {
     pdl_wait();
     pdl_trigger();
+    // image blockIdx.y of a batch
+    counts += blockIdx.y * N;
+    offsets += blockIdx.y * (N + kOffsetsPad);
+    sample_pixel += blockIdx.y * capacity;
+    total += blockIdx.y * kTotalStride;
+    status += blockIdx.y * kStatusStride;
+    tile_sums = reinterpret_cast<const int *>(reinterpret_cast<const char *>(tile_sums) +
+                                              blockIdx.y * ws_stride);
     const int tile = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __shared__ int s_w[kScanThreads / 32];
@@ -1165,9 +1192,12 @@ namespace {
 int alloc_impl(const float *d, int W, int H, const spp_params *p, const Dither &dither,
                int32_t *counts, int32_t *offsets, int32_t *sample_pixel, int64_t capacity,
                float *s_out, float *holdout_w, int64_t *total, int32_t *status, void *ws,
-               size_t ws_bytes, cudaStream_t stream, bool systematic = false) {
+               size_t ws_bytes, cudaStream_t stream, bool systematic = false, int B = 1,
+               const uint64_t *seeds = nullptr) {
+    // B > 1 or seeds: a batch of B images (two-kernel form), `seeds` in place of p->seed
     if (!p || W < 0 || H < 0 || capacity < 0) return SPP_ERR_ARG;
-    if (static_cast<long long>(W) * H == 0) {  // empty frame: T = 0, offsets[0] = 0
+    const bool batch = seeds != nullptr;
+    if (static_cast<long long>(W) * H == 0 && !batch) {  // empty frame: T = 0, offsets[0] = 0
         if (!offsets || !total) return SPP_ERR_ARG;
         if (!aligned16(offsets) || !aligned16(total)) return SPP_ERR_ALIGN;
         if (cudaMemsetAsync(offsets, 0, sizeof(int32_t), stream) != cudaSuccess) return SPP_ERR_CUDA;
@@ -1197,9 +1227,11 @@ int alloc_impl(const float *d, int W, int H, const spp_params *p, const Dither &
         (counts && !aligned16(counts)) || !aligned16(ws) || !aligned16(total))
         return SPP_ERR_ALIGN;
     const size_t need = spp_alloc_workspace_bytes(W, H);
-    if (ws_bytes < need) return SPP_ERR_WORKSPACE;
+    const size_t ws_stride = batch ? (need + 255) / 256 * 256 : 0;
+    if (ws_bytes < need + (B - 1) * ws_stride) return SPP_ERR_WORKSPACE;
 
-    if (cudaMemsetAsync(ws, 0, need, stream) != cudaSuccess) return SPP_ERR_CUDA;
+    if (cudaMemsetAsync(ws, 0, need + (B - 1) * ws_stride, stream) != cudaSuccess)
+        return SPP_ERR_CUDA;
     auto *hdr = static_cast<AllocHeader *>(ws);
     auto *tiles = reinterpret_cast<unsigned long long *>(static_cast<char *>(ws) + kHeaderBytes);
 
@@ -1232,8 +1264,8 @@ int alloc_impl(const float *d, int W, int H, const spp_params *p, const Dither &
     const long long max_grid = static_cast<long long>(sm_count()) * 8;
     if (grid > max_grid) grid = max_grid;
     if (grid < 1) grid = 1;
-    launch_dependent(budget_sum_kernel<kSumU>, dim3(static_cast<unsigned>(grid)),
-                     dim3(kSumThreads), 0, stream, d, N, hdr, args, status);
+    launch_dependent(budget_sum_kernel<kSumU>, dim3(static_cast<unsigned>(grid), B),
+                     dim3(kSumThreads), 0, stream, d, N, hdr, args, status, ws_stride);
     const int num_tiles = static_cast<int>(alloc_tiles(N));
     if (systematic) {
         // the frame offset U: the top 32 bits of element 2^62 of the stream
@@ -1253,14 +1285,16 @@ int alloc_impl(const float *d, int W, int H, const spp_params *p, const Dither &
     Dither dt = dither;
     dt.W = W;
     const bool stall = (p->flags & SPP_FLAG_TEST_STALL_TILE1) != 0;
-    if (num_tiles > kSinglePassMaxTiles && counts && !stall) {
+    if ((num_tiles > kSinglePassMaxTiles && counts && !stall) || batch) {
         auto *tile_sums = reinterpret_cast<int *>(tiles);
-        launch_dependent(assign_tile_kernel, dim3(num_tiles), dim3(kScanThreads), 0, stream, d,
-                         N, hdr, stream_key(p->seed, p->frame), dt, args.hard, counts, s_out,
-                         holdout_w, tile_sums);
-        launch_dependent(offsets_kernel, dim3(num_tiles), dim3(kScanThreads), 0, stream, counts,
+        StreamKeys keys{};
+        for (int b = 0; b < B; ++b) keys.k[b] = stream_key(batch ? seeds[b] : p->seed, p->frame);
+        launch_dependent(assign_tile_kernel, dim3(num_tiles, B), dim3(kScanThreads), 0, stream, d,
+                         N, hdr, keys, dt, args.hard, counts, s_out, holdout_w, tile_sums,
+                         ws_stride);
+        launch_dependent(offsets_kernel, dim3(num_tiles, B), dim3(kScanThreads), 0, stream, counts,
                          N, tile_sums, num_tiles, offsets, sample_pixel, capacity,
-                         reinterpret_cast<long long *>(total), status);
+                         reinterpret_cast<long long *>(total), status, ws_stride);
         count_launch(3);
         return launch_status();
     }
@@ -1272,10 +1306,50 @@ int alloc_impl(const float *d, int W, int H, const spp_params *p, const Dither &
     count_launch(2);
     return launch_status();
 }
+
+Dither make_dither(const uint16_t *mask, int T, uint32_t frame, uint64_t seed) {
+    Dither dt;
+    dt.mask = mask;
+    dt.log2T = 0;
+    while ((1 << dt.log2T) < T) ++dt.log2T;
+    dt.off48 = (static_cast<uint64_t>(frame) * (kGamma >> 16) + (mix64(seed) >> 16)) &
+               0xFFFFFFFFFFFFull;
+    return dt;
+}
 }  // namespace
 }  // namespace spp
 
 extern "C" {
+
+size_t spp_alloc_batch_workspace_bytes(int B, int W, int H) {
+    if (B < 0 || W < 0 || H < 0) return 0;
+    return static_cast<size_t>(B) * ((spp_alloc_workspace_bytes(W, H) + 255) / 256 * 256);
+}
+
+int spp_alloc_sample_map_batch(int B, const float *d, int W, int H, const spp_params *p,
+                               const uint64_t *seeds, int32_t *counts, int32_t *offsets,
+                               int32_t *sample_pixel, int64_t capacity, float *s_out,
+                               float *holdout_w, int64_t *total, int32_t *status, void *ws,
+                               size_t ws_bytes, cudaStream_t stream) {
+    using namespace spp;
+    if (B < 0 || W <= 0 || H <= 0 || !seeds || !counts || (p && p->flags)) return SPP_ERR_ARG;
+    const size_t n = static_cast<size_t>(W) * H;
+    if (B > 1 && n % 4) return SPP_ERR_ALIGN;
+    const size_t stride = (spp_alloc_workspace_bytes(W, H) + 255) / 256 * 256;
+    if (ws_bytes < B * stride) return SPP_ERR_WORKSPACE;
+    for (int b = 0; b < B; b += kMaxBatch) {
+        const int k = B - b < kMaxBatch ? B - b : kMaxBatch;
+        const int rc = alloc_impl(d + b * n, W, H, p, Dither{}, counts + b * n,
+                                  offsets + b * (n + kOffsetsPad),
+                                  sample_pixel ? sample_pixel + b * capacity : nullptr, capacity,
+                                  s_out + b * n, holdout_w + b * n, total + b * kTotalStride,
+                                  status + b * kStatusStride,
+                                  static_cast<char *>(ws) + b * stride, k * stride, stream, false,
+                                  k, seeds + b);
+        if (rc != SPP_OK) return rc;
+    }
+    return SPP_OK;
+}
 
 int spp_alloc_sample_map(const float *d, int W, int H, const spp_params *p, int32_t *counts,
                          int32_t *offsets, int32_t *sample_pixel, int64_t capacity, float *s_out,
@@ -1304,12 +1378,7 @@ int spp_alloc_sample_map_dithered(const float *d, int W, int H, const spp_params
     if (!mask || !p) return SPP_ERR_ARG;
     if (T < 4 || T > 256 || (T & (T - 1))) return SPP_ERR_ARG;
     if (!aligned16(mask)) return SPP_ERR_ALIGN;
-    Dither dt;
-    dt.mask = mask;
-    dt.log2T = 0;
-    while ((1 << dt.log2T) < T) ++dt.log2T;
-    dt.off48 = (static_cast<uint64_t>(p->frame) * (kGamma >> 16) + (mix64(p->seed) >> 16)) &
-               0xFFFFFFFFFFFFull;
+    const Dither dt = make_dither(mask, T, p->frame, p->seed);
     return alloc_impl(d, W, H, p, dt, counts, offsets, sample_pixel, capacity, s_out, holdout_w,
                       total, status, ws, ws_bytes, stream);
 }

@@ -72,7 +72,7 @@ recon_backward_kernel(const float *__restrict__ noisy, const float *__restrict__
                       const uint8_t *__restrict__ mask, int Wl, int Hl,
                       const float *__restrict__ g, float *__restrict__ grad_logits,
                       float *__restrict__ grad_noisy, float *__restrict__ grad_coarse,
-                      float *__restrict__ grad_warped) {
+                      float *__restrict__ grad_warped, int Cg, long long gl_stride) {
     constexpr int kSpatial = 25 + (UP ? 4 : 0);
     constexpr int kNK = kSpatial + (TEMP ? 25 : 0);
     extern __shared__ __align__(16) unsigned char bwd_smem_raw[];
@@ -84,6 +84,17 @@ recon_backward_kernel(const float *__restrict__ noisy, const float *__restrict__
     const int Wc = Wl >> 1, Hc = Hl >> 1;
     const long long Nc = static_cast<long long>(Wc) * Hc;
     const int cbx = bx0 >> 1, cby = by0 >> 1;  // first coarse cell under the tile
+    // image blockIdx.z of a batch (which shares the mask); gl_stride: floats
+    // between the images' logit gradients
+    noisy += blockIdx.z * 3 * Nl;
+    logits += blockIdx.z * C * Nl;
+    g += blockIdx.z * 3 * Nl;
+    grad_logits += blockIdx.z * gl_stride;
+    if (grad_noisy) grad_noisy += blockIdx.z * 3 * Nl;
+    if (UP) coarse += blockIdx.z * 3 * Nc;
+    if (UP && grad_coarse) grad_coarse += blockIdx.z * 3 * Nc;
+    if (TEMP) warped += blockIdx.z * 3 * Nl;
+    if (TEMP && grad_warped) grad_warped += blockIdx.z * 3 * Nl;
 
     // tap values of the region (clamp-to-edge)
     for (int idx = tid; idx < kRN; idx += kBX * kBY) {
@@ -205,7 +216,7 @@ recon_backward_kernel(const float *__restrict__ noisy, const float *__restrict__
                     grad_logits[(29 + k) * Nl + pix] =
                         use_t ? w[kSpatial + k] * (q[kSpatial + k] - qbar) : 0.0f;
             }
-            for (int k = TEMP ? 54 : kSpatial; k < C; ++k) grad_logits[k * Nl + pix] = 0.0f;
+            for (int k = TEMP ? 54 : kSpatial; k < Cg; ++k) grad_logits[k * Nl + pix] = 0.0f;
         }
     }
     // the halo's consumers (rows 0-1 and 10-11, then columns 0-1 and 34-35)
@@ -368,6 +379,10 @@ tonemap_backward_kernel(const float *__restrict__ hdr, long long N, ToneArgs tm,
                         const float *__restrict__ gl, float *__restrict__ gh) {
     const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= N) return;
+    // image blockIdx.y of a batch
+    hdr += blockIdx.y * 3 * N;
+    gl += blockIdx.y * 3 * N;
+    gh += blockIdx.y * 3 * N;
     float v[3], l[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -389,11 +404,19 @@ tonemap_backward_kernel(const float *__restrict__ hdr, long long N, ToneArgs tm,
     }
 }
 
+// floats between the losses of a batch's images
+constexpr int kScalarStride = 4;
+
 // Mean absolute error and its gradient sign(ldr - ref) / n.
 __global__ void __launch_bounds__(256)
 l1_loss_kernel(const float *__restrict__ a, const float *__restrict__ b, long long n,
                float *__restrict__ loss, float *__restrict__ grad) {
     const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+    // image blockIdx.y of a batch
+    a += blockIdx.y * n;
+    b += blockIdx.y * n;
+    if (grad) grad += blockIdx.y * n;
+    loss += blockIdx.y * kScalarStride;
     float v = 0.0f;
     if (i < n) {
         const float d = a[i] - b[i];
@@ -420,6 +443,13 @@ __global__ void combined_loss_kernel(const float *__restrict__ I, const float *_
                                      long long n, float w, float ws,
                                      float *__restrict__ loss, float *__restrict__ grad) {
     const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+    // image blockIdx.y of a batch
+    I += blockIdx.y * n;
+    R += blockIdx.y * n;
+    P += blockIdx.y * n;
+    Q += blockIdx.y * n;
+    if (grad) grad += blockIdx.y * n;
+    loss += blockIdx.y * kScalarStride;
     float v = 0.0f;
     if (i < n) {
         const float ds = I[i] - R[i];
@@ -478,13 +508,14 @@ pyramid_backward_kernel(GradLayers gl, int W, int H, int L, float *__restrict__ 
     if (x >= W || y >= H) return;
     const long long N = static_cast<long long>(W) * H;
     const long long i = static_cast<long long>(y) * W + x;
+    g0 += blockIdx.z * 3 * N;  // image blockIdx.z of a batch
     float a[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int l = 1; l < 5; ++l) {
         if (l >= L) break;
         const int Wl = W >> l, Hl = H >> l;
         const long long Nl = static_cast<long long>(Wl) * Hl;
-        const long long q = static_cast<long long>(y >> l) * Wl + (x >> l);
+        const long long q = blockIdx.z * 3 * Nl + static_cast<long long>(y >> l) * Wl + (x >> l);
         const float sc = 1.0f / static_cast<float>(1 << (2 * l));
 #pragma unroll
         for (int c = 0; c < 3; ++c) a[c] = fmaf(sc, __ldg(gl.p[l] + c * Nl + q), a[c]);
@@ -500,10 +531,20 @@ __global__ void __launch_bounds__(256)
 splat_backward_kernel(const int32_t *__restrict__ offsets, const int32_t *__restrict__ counts,
                       const float4 *__restrict__ rgb, const float *__restrict__ s,
                       const float *__restrict__ L0, const float *__restrict__ gL0, long long N,
-                      long long capacity, uint64_t key, float lam, float h, int hard,
+                      long long capacity, const __grid_constant__ StreamKeys keys, float lam,
+                      float h, int hard,
                       float *__restrict__ grad_s) {
     const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= N) return;
+    // image blockIdx.y of a batch
+    const uint64_t key = keys.k[blockIdx.y];
+    offsets += blockIdx.y * (N + SPP_BATCH_OFFSETS_PAD);
+    counts += blockIdx.y * N;
+    rgb += blockIdx.y * capacity;
+    s += blockIdx.y * N;
+    L0 += blockIdx.y * 3 * N;
+    gL0 += blockIdx.y * 3 * N;
+    grad_s += blockIdx.y * N;
     const float si = s[i];
     float acc = 0.0f;
 #pragma unroll
@@ -535,10 +576,23 @@ splat_backward_est_kernel(const int32_t *__restrict__ offsets, const int32_t *__
                           const float4 *__restrict__ rgb, const float *__restrict__ s,
                           const float *__restrict__ L0, const float *__restrict__ gL0,
                           const float *__restrict__ hw, long long N, long long capacity,
-                          int estimator, float lam, const float *__restrict__ clean,
-                          uint64_t render_key, float *__restrict__ grad_s) {
+                          int estimator, float lam,
+                          const __grid_constant__ BatchImages images,
+                          const __grid_constant__ StreamKeys render_keys,
+                          float *__restrict__ grad_s) {
     const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= N) return;
+    // image blockIdx.y of a batch
+    const float *__restrict__ clean = images.p[blockIdx.y];
+    const uint64_t render_key = render_keys.k[blockIdx.y];
+    offsets += blockIdx.y * (N + SPP_BATCH_OFFSETS_PAD);
+    counts += blockIdx.y * N;
+    rgb += blockIdx.y * capacity;
+    s += blockIdx.y * N;
+    L0 += blockIdx.y * 3 * N;
+    gL0 += blockIdx.y * 3 * N;
+    hw += blockIdx.y * N;
+    grad_s += blockIdx.y * N;
     const float si = s[i];
     float acc = 0.0f;
 #pragma unroll
@@ -578,10 +632,17 @@ splat_backward_est_kernel(const int32_t *__restrict__ offsets, const int32_t *__
 // where it has none.
 __global__ void __launch_bounds__(256)
 splat_backward_dasr_kernel(const int32_t *__restrict__ counts, const float *__restrict__ L0,
-                           const float *__restrict__ gL0, const float *__restrict__ ref,
-                           long long N, float *__restrict__ grad_s) {
+                           const float *__restrict__ gL0,
+                           const __grid_constant__ BatchImages refs, long long N,
+                           float *__restrict__ grad_s) {
     const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= N) return;
+    // image blockIdx.y of a batch
+    const float *__restrict__ ref = refs.p[blockIdx.y];
+    counts += blockIdx.y * N;
+    L0 += blockIdx.y * 3 * N;
+    gL0 += blockIdx.y * 3 * N;
+    grad_s += blockIdx.y * N;
     const int n = counts[i];
     float acc = 0.0f;
     if (n >= 1) {
@@ -599,10 +660,16 @@ splat_backward_dasr_kernel(const int32_t *__restrict__ counts, const float *__re
 // the block's own slot; pass 1b adds the slots in index order.  No atomics:
 // the sums, and the gradient, are the same from run to run.
 constexpr int kDensityMaxBlocks = 2048;
+// workspace of an image: the two sums, then the blocks' slots
+constexpr int kDensityWsDoubles = 32 + 2 * kDensityMaxBlocks;
 
 __global__ void __launch_bounds__(256)
 density_reduce_kernel(const float *__restrict__ d, const float *__restrict__ g, long long N,
                       double *__restrict__ partial) {
+    // image blockIdx.y of a batch
+    d += blockIdx.y * N;
+    g += blockIdx.y * N;
+    partial += blockIdx.y * kDensityWsDoubles;
     double a = 0.0, b = 0.0;
     for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < N;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -634,6 +701,8 @@ density_reduce_kernel(const float *__restrict__ d, const float *__restrict__ g, 
 
 __global__ void __launch_bounds__(256)
 density_sum_kernel(const double *__restrict__ partial, int blocks, double *__restrict__ sums) {
+    partial += blockIdx.y * kDensityWsDoubles;
+    sums += blockIdx.y * kDensityWsDoubles;
     double a = 0.0, b = 0.0;
     for (int k = threadIdx.x; k < blocks; k += blockDim.x) {
         a += partial[2 * k];
@@ -664,9 +733,15 @@ density_sum_kernel(const double *__restrict__ partial, int blocks, double *__res
 // Pass 2 (Sec. 3): dLoss/dz_j = (1 - phi) B N pi_j (g_j - sum_i pi_i g_i).
 __global__ void __launch_bounds__(256)
 density_grad_kernel(const float *__restrict__ d, const float *__restrict__ g, long long N,
-                    const double *__restrict__ sums, double K, float *__restrict__ gz) {
+                    const double *__restrict__ sums, double K, float *__restrict__ gz,
+                    long long gz_stride) {
     const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= N) return;
+    // image blockIdx.y of a batch
+    d += blockIdx.y * N;
+    g += blockIdx.y * N;
+    sums += blockIdx.y * kDensityWsDoubles;
+    gz += blockIdx.y * gz_stride;
     const double S = sums[0];
     const double dot = sums[1] / S;
     const double pi = static_cast<double>(d[i]) / S;
@@ -691,7 +766,8 @@ template <bool UP, bool TEMP>
 int launch_recon_backward(dim3 grid, dim3 block, cudaStream_t stream, const float *noisy,
                           const float *logits, int C, const float *coarse, const float *warped,
                           const uint8_t *mask, int Wl, int Hl, const float *g, float *grad_logits,
-                          float *grad_noisy, float *grad_coarse, float *grad_warped) {
+                          float *grad_noisy, float *grad_coarse, float *grad_warped, int Cg,
+                          long long gl_stride) {
     constexpr int kSmem = static_cast<int>(sizeof(BwdSmem<UP, TEMP>));
     static int configured_dev = -1;
     int dev = 0;
@@ -704,7 +780,7 @@ int launch_recon_backward(dim3 grid, dim3 block, cudaStream_t stream, const floa
     }
     recon_backward_kernel<UP, TEMP><<<grid, block, kSmem, stream>>>(
         noisy, logits, C, coarse, warped, mask, Wl, Hl, g, grad_logits, grad_noisy, grad_coarse,
-        grad_warped);
+        grad_warped, Cg, gl_stride);
     return SPP_OK;
 }
 
@@ -718,11 +794,23 @@ int spp_reconstruct_level_backward(const float *noisy, const float *logits, int 
                                    const uint8_t *mask, int Wl, int Hl, const float *grad_out,
                                    float *grad_logits, float *grad_noisy, float *grad_coarse,
                                    float *grad_warped, cudaStream_t stream) {
+    return spp_reconstruct_level_backward_batch(1, noisy, logits, C, coarse, warped_prev, mask, Wl,
+                                                Hl, grad_out, grad_logits, C, grad_noisy,
+                                                grad_coarse, grad_warped, stream);
+}
+
+int spp_reconstruct_level_backward_batch(int B, const float *noisy, const float *logits, int C,
+                                         const float *coarse, const float *warped_prev,
+                                         const uint8_t *mask, int Wl, int Hl,
+                                         const float *grad_out, float *grad_logits, int Cg,
+                                         float *grad_noisy, float *grad_coarse,
+                                         float *grad_warped, cudaStream_t stream) {
     using namespace spp;
-    if (Wl < 0 || Hl < 0 || !noisy || !logits || !grad_out || !grad_logits) return SPP_ERR_ARG;
+    if (B < 0 || B > 65535 || Wl < 0 || Hl < 0 || !noisy || !logits || !grad_out || !grad_logits)
+        return SPP_ERR_ARG;
     if (warped_prev && !coarse) return SPP_ERR_ARG;
-    const int need = 25 + (coarse ? 4 : 0);
-    if (C < need || (warped_prev && C < 54)) return SPP_ERR_ARG;
+    const int need = warped_prev ? 54 : 25 + (coarse ? 4 : 0);
+    if (C < need || Cg < need || Cg > C) return SPP_ERR_ARG;
     if (coarse && ((Wl & 1) || (Hl & 1))) return SPP_ERR_SHAPE;
     if (!aligned16(noisy) || !aligned16(logits) || !aligned16(grad_out) ||
         !aligned16(grad_logits) || (coarse && !aligned16(coarse)) ||
@@ -730,22 +818,24 @@ int spp_reconstruct_level_backward(const float *noisy, const float *logits, int 
         (grad_noisy && !aligned16(grad_noisy)) || (grad_coarse && !aligned16(grad_coarse)) ||
         (grad_warped && !aligned16(grad_warped)))
         return SPP_ERR_ALIGN;
-    if (static_cast<long long>(Wl) * Hl == 0) return SPP_OK;
+    const long long n = static_cast<long long>(Wl) * Hl;
+    if (B == 0 || n == 0) return SPP_OK;
+    if (B > 1 && (C * n) % 4) return SPP_ERR_ALIGN;
     dim3 block(kBX, kBY);
-    dim3 grid((Wl + kBX - 1) / kBX, (Hl + kBY - 1) / kBY);
+    dim3 grid((Wl + kBX - 1) / kBX, (Hl + kBY - 1) / kBY, B);
     int rc;
     if (!coarse)
         rc = launch_recon_backward<false, false>(grid, block, stream, noisy, logits, C, coarse,
                                                  warped_prev, mask, Wl, Hl, grad_out, grad_logits,
-                                                 grad_noisy, grad_coarse, grad_warped);
+                                                 grad_noisy, grad_coarse, grad_warped, Cg, C * n);
     else if (!warped_prev)
         rc = launch_recon_backward<true, false>(grid, block, stream, noisy, logits, C, coarse,
                                                 warped_prev, mask, Wl, Hl, grad_out, grad_logits,
-                                                grad_noisy, grad_coarse, grad_warped);
+                                                grad_noisy, grad_coarse, grad_warped, Cg, C * n);
     else
         rc = launch_recon_backward<true, true>(grid, block, stream, noisy, logits, C, coarse,
                                                warped_prev, mask, Wl, Hl, grad_out, grad_logits,
-                                               grad_noisy, grad_coarse, grad_warped);
+                                               grad_noisy, grad_coarse, grad_warped, Cg, C * n);
     count_launch();
     return rc != SPP_OK ? rc : launch_status();
 }
@@ -764,14 +854,19 @@ int spp_warp_previous_backward(const float *mv, int W, int H, const float *grad_
 
 int spp_tonemap_backward(const float *hdr, int W, int H, const spp_tonemap *tm,
                          const float *grad_ldr, float *grad_hdr, cudaStream_t stream) {
+    return spp_tonemap_backward_batch(1, hdr, W, H, tm, grad_ldr, grad_hdr, stream);
+}
+
+int spp_tonemap_backward_batch(int B, const float *hdr, int W, int H, const spp_tonemap *tm,
+                               const float *grad_ldr, float *grad_hdr, cudaStream_t stream) {
     using namespace spp;
-    if (W < 0 || H < 0 || !hdr || !grad_ldr || !grad_hdr) return SPP_ERR_ARG;
+    if (B < 0 || B > 65535 || W < 0 || H < 0 || !hdr || !grad_ldr || !grad_hdr) return SPP_ERR_ARG;
     if (!aligned16(hdr) || !aligned16(grad_ldr) || !aligned16(grad_hdr)) return SPP_ERR_ALIGN;
     const ToneArgs ta = tone_args_bwd(tm);
     if (!(ta.s > 0.0f && ta.s < 1.0f && ta.h > 0.0f && ta.h < 1.0f)) return SPP_ERR_ARG;
     const long long N = static_cast<long long>(W) * H;
-    if (N == 0) return SPP_OK;
-    tonemap_backward_kernel<<<static_cast<unsigned>((N + 255) / 256), 256, 0, stream>>>(
+    if (B == 0 || N == 0) return SPP_OK;
+    tonemap_backward_kernel<<<dim3(static_cast<unsigned>((N + 255) / 256), B), 256, 0, stream>>>(
         hdr, N, ta, grad_ldr, grad_hdr);
     count_launch();
     return launch_status();
@@ -786,6 +881,22 @@ int spp_l1_loss(const float *ldr, const float *ref, int64_t n, float *loss, floa
     if (cudaMemsetAsync(loss, 0, sizeof(float), stream) != cudaSuccess) return SPP_ERR_CUDA;
     if (n == 0) return SPP_OK;
     l1_loss_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(
+        ldr, ref, static_cast<long long>(n), loss, grad_ldr);
+    count_launch();
+    return launch_status();
+}
+
+int spp_l1_loss_batch(int B, const float *ldr, const float *ref, int64_t n, float *loss,
+                      float *grad_ldr, cudaStream_t stream) {
+    using namespace spp;
+    if (B < 0 || B > 65535 || n < 0 || !ldr || !ref || !loss) return SPP_ERR_ARG;
+    if (!aligned16(ldr) || !aligned16(ref) || (grad_ldr && !aligned16(grad_ldr)) || !aligned16(loss))
+        return SPP_ERR_ALIGN;
+    if (B == 0) return SPP_OK;
+    if (cudaMemsetAsync(loss, 0, sizeof(float) * kScalarStride * B, stream) != cudaSuccess)
+        return SPP_ERR_CUDA;
+    if (n == 0) return SPP_OK;
+    l1_loss_kernel<<<dim3(static_cast<unsigned>((n + 255) / 256), B), 256, 0, stream>>>(
         ldr, ref, static_cast<long long>(n), loss, grad_ldr);
     count_launch();
     return launch_status();
@@ -808,6 +919,27 @@ int spp_combined_loss(const float *ldr, const float *ref, const float *prev_warp
     return launch_status();
 }
 
+int spp_combined_loss_batch(int B, const float *ldr, const float *ref, const float *prev_warped,
+                            const float *ref_prev_warped, int64_t n, float temporal_weight,
+                            float spatial_weight, float *loss, float *grad_ldr,
+                            cudaStream_t stream) {
+    using namespace spp;
+    if (B < 0 || B > 65535 || n < 0 || !ldr || !ref || !prev_warped || !ref_prev_warped || !loss)
+        return SPP_ERR_ARG;
+    if (!aligned16(ldr) || !aligned16(ref) || !aligned16(prev_warped) ||
+        !aligned16(ref_prev_warped) || !aligned16(loss) || (grad_ldr && !aligned16(grad_ldr)))
+        return SPP_ERR_ALIGN;
+    if (B == 0) return SPP_OK;
+    if (cudaMemsetAsync(loss, 0, sizeof(float) * kScalarStride * B, stream) != cudaSuccess)
+        return SPP_ERR_CUDA;
+    if (n == 0) return SPP_OK;
+    combined_loss_kernel<<<dim3(static_cast<unsigned>((n + 255) / 256), B), 256, 0, stream>>>(
+        ldr, ref, prev_warped, ref_prev_warped, static_cast<long long>(n), temporal_weight,
+        spatial_weight, loss, grad_ldr);
+    count_launch();
+    return launch_status();
+}
+
 int spp_mse(const float *a, const float *b, int64_t n, double *mse, cudaStream_t stream) {
     using namespace spp;
     if (n < 0 || !a || !b || !mse) return SPP_ERR_ARG;
@@ -822,8 +954,13 @@ int spp_mse(const float *a, const float *b, int64_t n, double *mse, cudaStream_t
 
 int spp_pyramid_backward(const float *const *grad_layers, int W, int H, int L, float *grad_L0,
                          cudaStream_t stream) {
+    return spp_pyramid_backward_batch(1, grad_layers, W, H, L, grad_L0, stream);
+}
+
+int spp_pyramid_backward_batch(int B, const float *const *grad_layers, int W, int H, int L,
+                               float *grad_L0, cudaStream_t stream) {
     using namespace spp;
-    if (W < 0 || H < 0 || !grad_layers || !grad_L0) return SPP_ERR_ARG;
+    if (B < 0 || B > 65535 || W < 0 || H < 0 || !grad_layers || !grad_L0) return SPP_ERR_ARG;
     if (L < 1 || L > 5) return SPP_ERR_SHAPE;
     if ((W % (1 << (L - 1))) != 0 || (H % (1 << (L - 1))) != 0) return SPP_ERR_SHAPE;
     GradLayers gl{};
@@ -833,56 +970,71 @@ int spp_pyramid_backward(const float *const *grad_layers, int W, int H, int L, f
         gl.p[l] = grad_layers[l];
     }
     if (!aligned16(grad_L0)) return SPP_ERR_ALIGN;
-    if (static_cast<long long>(W) * H == 0 || L == 1) return SPP_OK;
-    dim3 grid((W + 63) / 64, (H + 3) / 4);
+    if (B == 0 || static_cast<long long>(W) * H == 0 || L == 1) return SPP_OK;
+    dim3 grid((W + 63) / 64, (H + 3) / 4, B);
     pyramid_backward_kernel<<<grid, 256, 0, stream>>>(gl, W, H, L, grad_L0);
     count_launch();
     return launch_status();
 }
 
-int spp_splat_backward(const int32_t *offsets, const int32_t *counts, const float *rgb,
-                       const float *s, const float *layer0, const float *grad_layer0,
-                       int64_t capacity, int W, int H, const spp_params *p, float *grad_s,
-                       cudaStream_t stream) {
-    using namespace spp;
-    if (W < 0 || H < 0 || capacity < 0 || !p || !offsets || !counts || !s || !layer0 ||
+}  // extern "C"
+
+namespace spp {
+namespace {
+
+// The splat's gradient for at most kMaxBatch images; offsets, counts, rgb, s,
+// layer0 and the gradients hold the images one after the other.
+int splat_backward(int B, const int32_t *offsets, const int32_t *counts, const float *rgb,
+                   const float *s, const float *layer0, const float *grad_layer0, int64_t capacity,
+                   int W, int H, const spp_params *p, const uint64_t *seeds, float *grad_s,
+                   cudaStream_t stream) {
+    if (W < 0 || H < 0 || capacity < 0 || !p || !seeds || !offsets || !counts || !s || !layer0 ||
         !grad_layer0 || !grad_s || (capacity > 0 && !rgb))
         return SPP_ERR_ARG;
     if (!aligned16(offsets) || !aligned16(counts) || (rgb && !aligned16(rgb)) || !aligned16(s) ||
         !aligned16(layer0) || !aligned16(grad_layer0) || !aligned16(grad_s))
         return SPP_ERR_ALIGN;
     const long long N = static_cast<long long>(W) * H;
-    if (N == 0) return SPP_OK;
+    if (B == 0 || N == 0) return SPP_OK;
     const bool hard = p->holdout_mode == SPP_HOLDOUT_HARD;
     const double lam = hard ? 1.0 : p->lambda;
     const double h = 2.0 * lam / (2.0 * lam - 1.0);
-    splat_backward_kernel<<<static_cast<unsigned>((N + 255) / 256), 256, 0, stream>>>(
+    StreamKeys keys{};
+    for (int b = 0; b < B; ++b) keys.k[b] = stream_key(seeds[b], p->frame);
+    splat_backward_kernel<<<dim3(static_cast<unsigned>((N + 255) / 256), B), 256, 0, stream>>>(
         offsets, counts, reinterpret_cast<const float4 *>(rgb), s, layer0, grad_layer0, N, capacity,
-        stream_key(p->seed, p->frame), static_cast<float>(lam), static_cast<float>(h), hard ? 1 : 0,
-        grad_s);
+        keys, static_cast<float>(lam), static_cast<float>(h), hard ? 1 : 0, grad_s);
     count_launch();
     return launch_status();
 }
 
-int spp_splat_backward_estimator(const int32_t *offsets, const int32_t *counts, const float *rgb,
-                                 const float *s, const float *layer0, const float *grad_layer0,
-                                 const float *holdout_w, int64_t capacity, int W, int H,
-                                 const spp_params *p, int estimator, const float *clean,
-                                 uint64_t render_seed, float *grad_s, cudaStream_t stream) {
-    using namespace spp;
+int splat_backward_estimator(int B, const int32_t *offsets, const int32_t *counts, const float *rgb,
+                             const float *s, const float *layer0, const float *grad_layer0,
+                             const float *holdout_w, int64_t capacity, int W, int H,
+                             const spp_params *p, const uint64_t *seeds, int estimator,
+                             const float *const *clean, const uint64_t *render_seeds, float *grad_s,
+                             cudaStream_t stream) {
     if (estimator == SPP_ESTIMATOR_RELAXED)
-        return spp_splat_backward(offsets, counts, rgb, s, layer0, grad_layer0, capacity, W, H, p,
-                                  grad_s, stream);
+        return splat_backward(B, offsets, counts, rgb, s, layer0, grad_layer0, capacity, W, H, p,
+                              seeds, grad_s, stream);
+    BatchImages images{};
+    bool all_clean = clean != nullptr, clean_aligned = true;
+    for (int b = 0; all_clean && b < B; ++b) {
+        images.p[b] = clean[b];
+        clean_aligned = clean_aligned && aligned16(clean[b]);
+        all_clean = clean[b] != nullptr;
+    }
+    const long long N = static_cast<long long>(W) * H;
+    const dim3 grid(static_cast<unsigned>((N + 255) / 256), B);
     if (estimator == SPP_ESTIMATOR_DASR) {
-        if (W < 0 || H < 0 || !counts || !layer0 || !grad_layer0 || !clean || !grad_s)
+        if (W < 0 || H < 0 || !counts || !layer0 || !grad_layer0 || !all_clean || !grad_s)
             return SPP_ERR_ARG;
         if (!aligned16(counts) || !aligned16(layer0) || !aligned16(grad_layer0) ||
-            !aligned16(clean) || !aligned16(grad_s))
+            !clean_aligned || !aligned16(grad_s))
             return SPP_ERR_ALIGN;
-        const long long N = static_cast<long long>(W) * H;
-        if (N == 0) return SPP_OK;
-        splat_backward_dasr_kernel<<<static_cast<unsigned>((N + 255) / 256), 256, 0, stream>>>(
-            counts, layer0, grad_layer0, clean, N, grad_s);
+        if (B == 0 || N == 0) return SPP_OK;
+        splat_backward_dasr_kernel<<<grid, 256, 0, stream>>>(counts, layer0, grad_layer0, images, N,
+                                                             grad_s);
         count_launch();
         return launch_status();
     }
@@ -893,46 +1045,100 @@ int spp_splat_backward_estimator(const int32_t *offsets, const int32_t *counts, 
         return SPP_ERR_ARG;
     if (estimator == SPP_ESTIMATOR_GUMBEL && (!holdout_w || !(p->lambda > 0.0)))
         return SPP_ERR_ARG;
-    if (estimator == SPP_ESTIMATOR_STRAIGHT_THROUGH && !clean) return SPP_ERR_ARG;
+    if (estimator == SPP_ESTIMATOR_STRAIGHT_THROUGH && !all_clean) return SPP_ERR_ARG;
     if (!aligned16(offsets) || !aligned16(counts) || !aligned16(s) || !aligned16(layer0) ||
         !aligned16(grad_layer0) || !aligned16(grad_s) || (rgb && !aligned16(rgb)) ||
-        (holdout_w && !aligned16(holdout_w)) || (clean && !aligned16(clean)))
+        (holdout_w && !aligned16(holdout_w)) || !clean_aligned)
         return SPP_ERR_ALIGN;
-    const long long N = static_cast<long long>(W) * H;
-    if (N == 0) return SPP_OK;
-    splat_backward_est_kernel<<<static_cast<unsigned>((N + 255) / 256), 256, 0, stream>>>(
+    if (B == 0 || N == 0) return SPP_OK;
+    StreamKeys keys{};
+    for (int b = 0; b < B; ++b) keys.k[b] = stream_key(render_seeds[b], p->frame);
+    splat_backward_est_kernel<<<grid, 256, 0, stream>>>(
         offsets, counts, reinterpret_cast<const float4 *>(rgb), s, layer0, grad_layer0, holdout_w,
-        N, capacity, estimator, static_cast<float>(p->lambda), clean,
-        stream_key(render_seed, p->frame), grad_s);
+        N, capacity, estimator, static_cast<float>(p->lambda), images, keys, grad_s);
     count_launch();
     return launch_status();
 }
 
+}  // namespace
+}  // namespace spp
+
+extern "C" {
+
+int spp_splat_backward(const int32_t *offsets, const int32_t *counts, const float *rgb,
+                       const float *s, const float *layer0, const float *grad_layer0,
+                       int64_t capacity, int W, int H, const spp_params *p, float *grad_s,
+                       cudaStream_t stream) {
+    return spp::splat_backward(1, offsets, counts, rgb, s, layer0, grad_layer0, capacity, W, H, p,
+                               p ? &p->seed : nullptr, grad_s, stream);
+}
+
+int spp_splat_backward_estimator(const int32_t *offsets, const int32_t *counts, const float *rgb,
+                                 const float *s, const float *layer0, const float *grad_layer0,
+                                 const float *holdout_w, int64_t capacity, int W, int H,
+                                 const spp_params *p, int estimator, const float *clean,
+                                 uint64_t render_seed, float *grad_s, cudaStream_t stream) {
+    return spp::splat_backward_estimator(1, offsets, counts, rgb, s, layer0, grad_layer0, holdout_w,
+                                         capacity, W, H, p, p ? &p->seed : nullptr, estimator,
+                                         &clean, &render_seed, grad_s, stream);
+}
+
+int spp_splat_backward_batch(int B, const int32_t *offsets, const int32_t *counts, const float *rgb,
+                             const float *s, const float *layer0, const float *grad_layer0,
+                             const float *holdout_w, int64_t capacity, int W, int H,
+                             const spp_params *p, const uint64_t *seeds, int estimator,
+                             const float *const *clean, const uint64_t *render_seeds,
+                             float *grad_s, cudaStream_t stream) {
+    using namespace spp;
+    if (B < 0 || W < 0 || H < 0 || capacity < 0 || !p || !seeds || !render_seeds || !offsets ||
+        !counts || !rgb || !s || !layer0 || !grad_layer0 || !holdout_w || !clean || !grad_s)
+        return SPP_ERR_ARG;
+    const int64_t n = static_cast<int64_t>(W) * H;
+    if (B > 1 && n % 4) return SPP_ERR_ALIGN;
+    for (int b = 0; b < B; b += kMaxBatch) {
+        const int k = B - b < kMaxBatch ? B - b : kMaxBatch;
+        const int rc = splat_backward_estimator(
+            k, offsets + b * (n + SPP_BATCH_OFFSETS_PAD), counts + b * n, rgb + 4 * b * capacity,
+            s + b * n, layer0 + b * 3 * n, grad_layer0 + b * 3 * n, holdout_w + b * n, capacity, W,
+            H, p, seeds + b, estimator, clean + b, render_seeds + b, grad_s + b * n, stream);
+        if (rc != SPP_OK) return rc;
+    }
+    return SPP_OK;
+}
+
 size_t spp_density_backward_workspace_bytes(void) {
-    return 256 + static_cast<size_t>(spp::kDensityMaxBlocks) * 2 * sizeof(double);
+    return spp::kDensityWsDoubles * sizeof(double);
 }
 
 int spp_density_backward(const float *d, int64_t N, double budget, double uniform_fraction,
                          const float *grad_s, float *grad_z, void *ws, size_t ws_bytes,
                          cudaStream_t stream) {
+    return spp_density_backward_batch(1, d, N, budget, uniform_fraction, grad_s, grad_z, N, ws,
+                                      ws_bytes, stream);
+}
+
+int spp_density_backward_batch(int B, const float *d, int64_t N, double budget,
+                               double uniform_fraction, const float *grad_s, float *grad_z,
+                               int64_t grad_z_stride, void *ws, size_t ws_bytes,
+                               cudaStream_t stream) {
     using namespace spp;
-    if (N < 0 || !d || !grad_s || !grad_z || !ws) return SPP_ERR_ARG;
-    if (ws_bytes < spp_density_backward_workspace_bytes()) return SPP_ERR_WORKSPACE;
+    if (B < 0 || B > 65535 || N < 0 || !d || !grad_s || !grad_z || !ws) return SPP_ERR_ARG;
+    if (ws_bytes < B * spp_density_backward_workspace_bytes()) return SPP_ERR_WORKSPACE;
     if (!aligned16(d) || !aligned16(grad_s) || !aligned16(grad_z) || !aligned16(ws))
         return SPP_ERR_ALIGN;
-    if (N == 0) return SPP_OK;
+    if (B == 0 || N == 0) return SPP_OK;
     double *sums = static_cast<double *>(ws);
-    double *partial = reinterpret_cast<double *>(static_cast<unsigned char *>(ws) + 256);
+    double *partial = sums + 32;
     long long blocks = (N + 255) / 256;
     long long rblocks = static_cast<long long>(sm_count()) * 8;
     if (rblocks > blocks) rblocks = blocks;
     if (rblocks > kDensityMaxBlocks) rblocks = kDensityMaxBlocks;
-    density_reduce_kernel<<<static_cast<unsigned>(rblocks), 256, 0, stream>>>(d, grad_s, N,
-                                                                           partial);
-    density_sum_kernel<<<1, 256, 0, stream>>>(partial, static_cast<int>(rblocks), sums);
+    density_reduce_kernel<<<dim3(static_cast<unsigned>(rblocks), B), 256, 0, stream>>>(d, grad_s, N,
+                                                                                    partial);
+    density_sum_kernel<<<dim3(1, B), 256, 0, stream>>>(partial, static_cast<int>(rblocks), sums);
     const double K = (1.0 - uniform_fraction) * budget * static_cast<double>(N);
-    density_grad_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(d, grad_s, N, sums, K,
-                                                                           grad_z);
+    density_grad_kernel<<<dim3(static_cast<unsigned>(blocks), B), 256, 0, stream>>>(
+        d, grad_s, N, sums, K, grad_z, grad_z_stride);
     count_launch(3);
     return launch_status();
 }

@@ -68,14 +68,17 @@ __device__ __forceinline__ void tone_map(float o0, float o1, float o2, const Ton
 // Launches the TMA-pipelined reconstruction of one level when the level's
 // shape allows it (row pitch a multiple of 16 bytes).  Returns false, with
 // nothing launched, when it does not; *rc then stays SPP_OK.  warped is
-// W_t L_{t-1} at full resolution, or NULL for no temporal term.
-bool launch_recon_tma(const float *noisy, const float *logits, int C_total, int C_used,
+// W_t L_{t-1} at full resolution, or NULL for no temporal term.  B images,
+// each array holding them one after the other ([B][C_total][Hl][Wl] logits);
+// they share the mask.
+bool launch_recon_tma(int B, const float *noisy, const float *logits, int C_total, int C_used,
                       const float *coarse, const float *warped, const uint8_t *mask, int Wl,
                       int Hl, float *out, float *out_ldr, const ToneArgs &tm, int32_t *status,
                       cudaStream_t stream, int *rc);
 
-// Launches the bilinear reprojection W_t L_{t-1} of the previous HDR output.
-void launch_warp_prev(const float *prev, const float *mv, int Wl, int Hl, float *warped,
-                      cudaStream_t stream);
+// Launches the bilinear reprojection W_t L_{t-1} of the previous HDR outputs of
+// B images (at most kMaxBatch).
+void launch_warp_prev(int B, const BatchImages &prev, const BatchImages &mv, int Wl, int Hl,
+                      float *warped, cudaStream_t stream);
 
 }  // namespace spp

@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(kTX *kTY, 2)
 recon_kernel(const float *__restrict__ noisy, const float *__restrict__ logits,
              const float *__restrict__ coarse, const float *__restrict__ warped,
              const uint8_t *__restrict__ mask, int Wl, int Hl, float *__restrict__ out,
-             float *__restrict__ out_ldr, ToneArgs tm) {
+             float *__restrict__ out_ldr, ToneArgs tm, int C) {
     static_assert(!TEMP || UP, "the temporal term lives at full resolution, below a coarser level");
     constexpr int kSpatial = 25 + (UP ? 4 : 0);
     constexpr int kNK = kSpatial + (TEMP ? 25 : 0);
@@ -45,6 +45,13 @@ recon_kernel(const float *__restrict__ noisy, const float *__restrict__ logits,
     const int yc = y < Hl ? y : Hl - 1;
     const long long Nl = static_cast<long long>(Wl) * Hl;
     const long long pix = static_cast<long long>(yc) * Wl + xc;
+    // image blockIdx.z of a batch (which shares the mask)
+    noisy += blockIdx.z * 3 * Nl;
+    logits += blockIdx.z * C * Nl;
+    out += blockIdx.z * 3 * Nl;
+    if (TONE) out_ldr += blockIdx.z * 3 * Nl;
+    if (TEMP) warped += blockIdx.z * 3 * Nl;
+    if (UP) coarse += blockIdx.z * 3 * (static_cast<long long>(Wl >> 1) * (Hl >> 1));
 
     // logits first: the longest-latency, largest stream
     float lg[kNK];
@@ -151,19 +158,22 @@ template <bool UP, bool TEMP>
 void launch_level(bool tone, dim3 grid, dim3 block, cudaStream_t st, const float *noisy,
                   const float *logits, const float *coarse, const float *warped,
                   const uint8_t *mask, int Wl, int Hl, float *out, float *out_ldr,
-                  const ToneArgs &tm) {
+                  const ToneArgs &tm, int C) {
     if (tone)
         recon_kernel<UP, TEMP, true><<<grid, block, 0, st>>>(noisy, logits, coarse, warped, mask,
-                                                             Wl, Hl, out, out_ldr, tm);
+                                                             Wl, Hl, out, out_ldr, tm, C);
     else
         recon_kernel<UP, TEMP, false><<<grid, block, 0, st>>>(noisy, logits, coarse, warped, mask,
-                                                              Wl, Hl, out, out_ldr, tm);
+                                                              Wl, Hl, out, out_ldr, tm, C);
 }
 
 // Tone map of a whole HDR image (Sec. 5), for reference images and the
 // recurrent network input.
-__global__ void tonemap_image_kernel(const float *__restrict__ hdr, int64_t n,
-                                     float *__restrict__ ldr, ToneArgs tm) {
+__global__ void tonemap_image_kernel(const __grid_constant__ BatchImages hdrs, int64_t n,
+                                     float *__restrict__ ldr,
+                                     ToneArgs tm) {
+    const float *__restrict__ hdr = hdrs.p[blockIdx.y];
+    ldr += blockIdx.y * 3 * n;
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         float r, g, b;
@@ -205,27 +215,59 @@ extern "C" {
 
 int spp_tonemap_image(const float *hdr, int W, int H, const spp_tonemap *tm, float *ldr,
                       cudaStream_t stream) {
+    return spp_tonemap_image_batch(1, &hdr, W, H, tm, ldr, stream);
+}
+
+int spp_tonemap_image_batch(int B, const float *const *hdr, int W, int H, const spp_tonemap *tm,
+                            float *ldr, cudaStream_t stream) {
     using namespace spp;
-    if (W < 0 || H < 0 || !hdr || !ldr) return SPP_ERR_ARG;
-    if (!aligned16(hdr) || !aligned16(ldr)) return SPP_ERR_ALIGN;
+    if (B < 0 || W < 0 || H < 0 || !hdr || !ldr) return SPP_ERR_ARG;
+    const int64_t n = static_cast<int64_t>(W) * H;
+    for (int b = 0; b < B; ++b) {
+        if (!hdr[b]) return SPP_ERR_ARG;
+        if (!aligned16(hdr[b])) return SPP_ERR_ALIGN;
+    }
+    if (!aligned16(ldr)) return SPP_ERR_ALIGN;
     const ToneArgs t = tone_args(tm);
     if (!tone_ok(t)) return SPP_ERR_ARG;
-    const int64_t n = static_cast<int64_t>(W) * H;
     if (n == 0) return SPP_OK;
     const int grid = static_cast<int>(std::min<int64_t>((n + 255) / 256, 8 * sm_count()));
-    tonemap_image_kernel<<<grid, 256, 0, stream>>>(hdr, n, ldr, t);
-    count_launch();
+    for (int b = 0; b < B; b += kMaxBatch) {
+        const int k = std::min(B - b, kMaxBatch);
+        BatchImages im{};
+        for (int i = 0; i < k; ++i) im.p[i] = hdr[b + i];
+        tonemap_image_kernel<<<dim3(grid, k), 256, 0, stream>>>(im, n, ldr + b * 3 * n, t);
+        count_launch();
+    }
     return launch_status();
 }
 
 int spp_warp_previous(const float *prev_hdr, const float *mv, int W, int H, float *warped,
                       cudaStream_t stream) {
+    return spp_warp_previous_batch(1, &prev_hdr, &mv, W, H, warped, stream);
+}
+
+int spp_warp_previous_batch(int B, const float *const *prev_hdr, const float *const *mv, int W,
+                            int H, float *warped, cudaStream_t stream) {
     using namespace spp;
-    if (W < 0 || H < 0 || !prev_hdr || !mv || !warped) return SPP_ERR_ARG;
-    if (!aligned16(prev_hdr) || !aligned16(mv) || !aligned16(warped)) return SPP_ERR_ALIGN;
-    if (static_cast<long long>(W) * H == 0) return SPP_OK;
-    launch_warp_prev(prev_hdr, mv, W, H, warped, stream);
-    count_launch();
+    if (B < 0 || W < 0 || H < 0 || !prev_hdr || !mv || !warped) return SPP_ERR_ARG;
+    for (int b = 0; b < B; ++b) {
+        if (!prev_hdr[b] || !mv[b]) return SPP_ERR_ARG;
+        if (!aligned16(prev_hdr[b]) || !aligned16(mv[b])) return SPP_ERR_ALIGN;
+    }
+    if (!aligned16(warped)) return SPP_ERR_ALIGN;
+    const int64_t n = static_cast<int64_t>(W) * H;
+    if (n == 0) return SPP_OK;
+    for (int b = 0; b < B; b += kMaxBatch) {
+        const int k = std::min(B - b, kMaxBatch);
+        BatchImages pr{}, m{};
+        for (int i = 0; i < k; ++i) {
+            pr.p[i] = prev_hdr[b + i];
+            m.p[i] = mv[b + i];
+        }
+        launch_warp_prev(k, pr, m, W, H, warped + b * 3 * n, stream);
+        count_launch();
+    }
     return launch_status();
 }
 
@@ -233,8 +275,16 @@ int spp_reconstruct_level(const float *noisy, const float *logits, int C, const 
                           const float *warped_prev, const uint8_t *mask, int Wl, int Hl,
                           const spp_tonemap *tm, float *out, float *out_ldr, int32_t *status,
                           cudaStream_t stream) {
+    return spp_reconstruct_level_batch(1, noisy, logits, C, coarse, warped_prev, mask, Wl, Hl, tm,
+                                       out, out_ldr, status, stream);
+}
+
+int spp_reconstruct_level_batch(int B, const float *noisy, const float *logits, int C,
+                                const float *coarse, const float *warped_prev, const uint8_t *mask,
+                                int Wl, int Hl, const spp_tonemap *tm, float *out, float *out_ldr,
+                                int32_t *status, cudaStream_t stream) {
     using namespace spp;
-    if (Wl < 0 || Hl < 0 || !noisy || !logits || !out) return SPP_ERR_ARG;
+    if (B < 0 || Wl < 0 || Hl < 0 || !noisy || !logits || !out) return SPP_ERR_ARG;
     if (warped_prev && !coarse) return SPP_ERR_ARG;
     const int need = 25 + (coarse ? 4 : 0);
     if (C < need || (warped_prev && C < 54)) return SPP_ERR_ARG;
@@ -246,24 +296,28 @@ int spp_reconstruct_level(const float *noisy, const float *logits, int C, const 
         return SPP_ERR_ALIGN;
     const ToneArgs ta = tone_args(tm);
     if (out_ldr && !tone_ok(ta)) return SPP_ERR_ARG;
-    if (static_cast<long long>(Wl) * Hl == 0) return SPP_OK;
+    const int64_t n = static_cast<int64_t>(Wl) * Hl;
+    if (B == 0 || n == 0) return SPP_OK;
+    // every image's logits start on a 16-byte boundary
+    if (B > 1 && (C * n) % 4) return SPP_ERR_ALIGN;
     const int C_used = warped_prev ? 54 : (coarse ? 29 : 25);
     int rc = SPP_OK;
-    if (launch_recon_tma(noisy, logits, C, C_used, coarse, warped_prev, mask, Wl, Hl, out, out_ldr,
-                         ta, status, stream, &rc))
+    if (launch_recon_tma(B, noisy, logits, C, C_used, coarse, warped_prev, mask, Wl, Hl, out,
+                         out_ldr, ta, status, stream, &rc))
         return rc;
+    if (B > 65535) return SPP_ERR_ARG;
     dim3 block(kTX, kTY);
-    dim3 grid((Wl + kTX - 1) / kTX, (Hl + kTY - 1) / kTY);
+    dim3 grid((Wl + kTX - 1) / kTX, (Hl + kTY - 1) / kTY, B);
     const bool tone = out_ldr != nullptr;
     if (!coarse)
         launch_level<false, false>(tone, grid, block, stream, noisy, logits, coarse, warped_prev,
-                                   mask, Wl, Hl, out, out_ldr, ta);
+                                   mask, Wl, Hl, out, out_ldr, ta, C);
     else if (!warped_prev)
         launch_level<true, false>(tone, grid, block, stream, noisy, logits, coarse, warped_prev,
-                                  mask, Wl, Hl, out, out_ldr, ta);
+                                  mask, Wl, Hl, out, out_ldr, ta, C);
     else
         launch_level<true, true>(tone, grid, block, stream, noisy, logits, coarse, warped_prev,
-                                 mask, Wl, Hl, out, out_ldr, ta);
+                                 mask, Wl, Hl, out, out_ldr, ta, C);
     count_launch();
     return launch_status();
 }

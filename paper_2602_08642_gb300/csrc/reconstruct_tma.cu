@@ -132,13 +132,16 @@ __device__ __forceinline__ void tma_load_3d(float *dst, const CUtensorMap *map, 
 // ------------------------------------------------------------ the kernel
 struct TileGeom {
     int tiles_x, num_tiles;
+    int per_image, C_total;  // batches: tiles and logit planes of an image
 };
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-template <int C, bool UP, bool TEMP, bool TONE, int NS>
+// BATCH: the tiles of several images, one image after the other (a template
+// parameter so that single frames pay nothing for it).
+template <int C, bool UP, bool TEMP, bool TONE, int NS, bool BATCH>
 __global__ void __launch_bounds__(kThreads, 1)
 recon_tma_kernel(const __grid_constant__ CUtensorMap map_logits,
                  const __grid_constant__ CUtensorMap map_noisy,
@@ -182,8 +185,10 @@ recon_tma_kernel(const __grid_constant__ CUtensorMap map_logits,
     pdl_trigger();
     if (my_tiles == 0) return;
 
+    auto image_of = [&](int k) { return BATCH ? (blockIdx.x + k * G) / geom.per_image : 0; };
     auto tile_xy = [&](int k, int &x0, int &y0) {
-        const int t = blockIdx.x + k * G;
+        int t = blockIdx.x + k * G;
+        if (BATCH) t %= geom.per_image;
         x0 = (t % geom.tiles_x) * kPX;
         y0 = (t / geom.tiles_x) * kPY;
     };
@@ -204,10 +209,11 @@ recon_tma_kernel(const __grid_constant__ CUtensorMap map_logits,
         uses[s] = k / NS + 1;
         fence_proxy_async();
         mbar_expect_tx(&full[s], S::kBytes);
-        tma_load_3d(logits_of(s), &map_logits, &full[s], x0, y0, 0);
-        tma_load_3d(noisy_of(s), &map_noisy, &full[s], x0 - 4, y0 - 2, 0);
-        if (TEMP) tma_load_3d(warped_of(s), &map_warped, &full[s], x0 - 4, y0 - 2, 0);
-        if (UP) tma_load_3d(coarse_of(s), &map_coarse, &full[s], x0 / 2 - 4, y0 / 2, 0);
+        const int b = image_of(k);
+        tma_load_3d(logits_of(s), &map_logits, &full[s], x0, y0, b * geom.C_total);
+        tma_load_3d(noisy_of(s), &map_noisy, &full[s], x0 - 4, y0 - 2, 3 * b);
+        if (TEMP) tma_load_3d(warped_of(s), &map_warped, &full[s], x0 - 4, y0 - 2, 3 * b);
+        if (UP) tma_load_3d(coarse_of(s), &map_coarse, &full[s], x0 / 2 - 4, y0 / 2, 3 * b);
     };
     if (tid == 0)
         for (int k = 0; k < NS && k < my_tiles; ++k) issue(k);
@@ -413,7 +419,8 @@ recon_tma_kernel(const __grid_constant__ CUtensorMap map_logits,
             const float o0 = (a0 * s0 + pk[2 * kPixels + p] * s1) * inv;
             const float o1 = (a1 * s0 + pk[3 * kPixels + p] * s1) * inv;
             const float o2 = (a2 * s0 + pk[4 * kPixels + p] * s1) * inv;
-            const long long op = static_cast<long long>(y) * Wl + x;
+            long long op = static_cast<long long>(y) * Wl + x;
+            if (BATCH) op += 3 * Nl * image_of(k);
             __stcs(out + op, o0);
             __stcs(out + Nl + op, o1);
             __stcs(out + 2 * Nl + op, o2);
@@ -432,8 +439,12 @@ recon_tma_kernel(const __grid_constant__ CUtensorMap map_logits,
 // y + mv_y), pixel centres at integers, the position clamped to the frame.
 // The fraction is taken from the motion vector itself so that it is exact.
 __global__ void __launch_bounds__(256)
-warp_prev_kernel(const float *__restrict__ prev, const float *__restrict__ mv, int Wl, int Hl,
+warp_prev_kernel(const __grid_constant__ BatchImages prevs,
+                 const __grid_constant__ BatchImages mvs, int Wl, int Hl,
                  float *__restrict__ warped) {
+    const float *__restrict__ prev = prevs.p[blockIdx.z];
+    const float *__restrict__ mv = mvs.p[blockIdx.z];
+    warped += blockIdx.z * 3 * static_cast<long long>(Wl) * Hl;
     const int gx = blockIdx.x * 64 + (threadIdx.x & 63);
     const int gy = blockIdx.y * 4 + (threadIdx.x >> 6);
     if (gx >= Wl || gy >= Hl) return;
@@ -482,22 +493,25 @@ bool make_map(CUtensorMap *map, const float *base, int W, int H, int planes, int
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int C, bool UP, bool TEMP, bool TONE, int NS>
-int launch_variant(const CUtensorMap &ml, const CUtensorMap &mn, const CUtensorMap &mw,
-                   const CUtensorMap &mc, const uint8_t *mask, int Wl, int Hl, float *out,
-                   float *out_ldr, const ToneArgs &tm, int32_t *status, int stall_tile,
-                   cudaStream_t stream) {
+template <int C, bool UP, bool TEMP, bool TONE, int NS, bool BATCH>
+int launch_kernel(int B, int C_total, const CUtensorMap &ml, const CUtensorMap &mn,
+                  const CUtensorMap &mw, const CUtensorMap &mc, const uint8_t *mask, int Wl, int Hl,
+                  float *out, float *out_ldr, const ToneArgs &tm, int32_t *status, int stall_tile,
+                  cudaStream_t stream) {
     using S = Stage<C, UP, TEMP>;
     const size_t smem =
         128 + 256 + static_cast<size_t>(NS) * S::kFloats * 4u + 2u * 5u * kPixels * sizeof(float);
-    auto kern = recon_tma_kernel<C, UP, TEMP, TONE, NS>;
+    auto kern = recon_tma_kernel<C, UP, TEMP, TONE, NS, BATCH>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem)) != cudaSuccess)
         return SPP_ERR_CUDA;
     TileGeom g;
     g.tiles_x = (Wl + kPX - 1) / kPX;
     const int tiles_y = (Hl + kPY - 1) / kPY;
-    g.num_tiles = g.tiles_x * tiles_y;
+    g.per_image = g.tiles_x * tiles_y;
+    g.C_total = C_total;
+    if (static_cast<int64_t>(B) * g.per_image > 0x7fffffff) return SPP_ERR_ARG;
+    g.num_tiles = B * g.per_image;
     int grid = sm_count();
     if (grid > g.num_tiles) grid = g.num_tiles;
     launch_dependent(kern, dim3(grid), dim3(kThreads), smem, stream, ml, mn, mw, mc, mask, Wl, Hl,
@@ -506,15 +520,21 @@ int launch_variant(const CUtensorMap &ml, const CUtensorMap &mn, const CUtensorM
     return launch_status();
 }
 
+template <int C, bool UP, bool TEMP, bool TONE, int NS, typename... Args>
+int launch_variant(int B, Args &&...args) {
+    return B == 1 ? launch_kernel<C, UP, TEMP, TONE, NS, false>(B, args...)
+                  : launch_kernel<C, UP, TEMP, TONE, NS, true>(B, args...);
+}
+
 }  // namespace
 
-void launch_warp_prev(const float *prev, const float *mv, int Wl, int Hl, float *warped,
-                      cudaStream_t stream) {
-    dim3 grid((Wl + 63) / 64, (Hl + 3) / 4);
+void launch_warp_prev(int B, const BatchImages &prev, const BatchImages &mv, int Wl, int Hl,
+                      float *warped, cudaStream_t stream) {
+    dim3 grid((Wl + 63) / 64, (Hl + 3) / 4, B);
     warp_prev_kernel<<<grid, 256, 0, stream>>>(prev, mv, Wl, Hl, warped);
 }
 
-bool launch_recon_tma(const float *noisy, const float *logits, int C_total, int C_used,
+bool launch_recon_tma(int B, const float *noisy, const float *logits, int C_total, int C_used,
                       const float *coarse, const float *warped, const uint8_t *mask, int Wl,
                       int Hl, float *out, float *out_ldr, const ToneArgs &tm, int32_t *status,
                       cudaStream_t stream, int *rc) {
@@ -529,34 +549,34 @@ bool launch_recon_tma(const float *noisy, const float *logits, int C_total, int 
     // the coarse level's map needs 16-byte row strides
     if (up && (((Wl >> 1) % 4) != 0 || !aligned16(coarse))) return false;
     CUtensorMap ml, mn, mw, mc;
-    if (!make_map(&ml, logits, Wl, Hl, C_total, kPX, kPY, C_used)) return false;
-    if (!make_map(&mn, noisy, Wl, Hl, 3, kBoxX, kBoxY, 3)) return false;
+    if (!make_map(&ml, logits, Wl, Hl, B * C_total, kPX, kPY, C_used)) return false;
+    if (!make_map(&mn, noisy, Wl, Hl, 3 * B, kBoxX, kBoxY, 3)) return false;
     if (temp) {
-        if (!make_map(&mw, warped, Wl, Hl, 3, kBoxX, kBoxY, 3)) return false;
+        if (!make_map(&mw, warped, Wl, Hl, 3 * B, kBoxX, kBoxY, 3)) return false;
     } else {
         mw = mn;  // unused
     }
     if (up) {
-        if (!make_map(&mc, coarse, Wl >> 1, Hl >> 1, 3, kCoarseX, kCoarseY, 3)) return false;
+        if (!make_map(&mc, coarse, Wl >> 1, Hl >> 1, 3 * B, kCoarseX, kCoarseY, 3)) return false;
     } else {
         mc = mn;  // unused
     }
     const bool tone = out_ldr != nullptr;
     const int stall = g_recon_stall_tile.exchange(-1);
     if (temp) {
-        *rc = tone ? launch_variant<54, true, true, true, 3>(ml, mn, mw, mc, mask, Wl, Hl, out,
+        *rc = tone ? launch_variant<54, true, true, true, 3>(B, C_total, ml, mn, mw, mc, mask, Wl, Hl, out,
                                                              out_ldr, tm, status, stall, stream)
-                   : launch_variant<54, true, true, false, 3>(ml, mn, mw, mc, mask, Wl, Hl, out,
+                   : launch_variant<54, true, true, false, 3>(B, C_total, ml, mn, mw, mc, mask, Wl, Hl, out,
                                                               out_ldr, tm, status, stall, stream);
     } else if (up) {
-        *rc = tone ? launch_variant<29, true, false, true, 5>(ml, mn, mw, mc, mask, Wl, Hl, out,
+        *rc = tone ? launch_variant<29, true, false, true, 5>(B, C_total, ml, mn, mw, mc, mask, Wl, Hl, out,
                                                               out_ldr, tm, status, stall, stream)
-                   : launch_variant<29, true, false, false, 5>(ml, mn, mw, mc, mask, Wl, Hl,
+                   : launch_variant<29, true, false, false, 5>(B, C_total, ml, mn, mw, mc, mask, Wl, Hl,
                                                                out, out_ldr, tm, status, stall, stream);
     } else {
-        *rc = tone ? launch_variant<25, false, false, true, 5>(ml, mn, mw, mc, mask, Wl, Hl,
+        *rc = tone ? launch_variant<25, false, false, true, 5>(B, C_total, ml, mn, mw, mc, mask, Wl, Hl,
                                                                out, out_ldr, tm, status, stall, stream)
-                   : launch_variant<25, false, false, false, 5>(ml, mn, mw, mc, mask, Wl, Hl,
+                   : launch_variant<25, false, false, false, 5>(B, C_total, ml, mn, mw, mc, mask, Wl, Hl,
                                                                 out, out_ldr, tm, status, stall, stream);
     }
     return true;

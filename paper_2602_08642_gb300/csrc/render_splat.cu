@@ -11,11 +11,19 @@ constexpr int kRenderThreads = 256;
 // Sample t of the list: pixel i = sample_pixel[t], slot k = t - offsets[i];
 // value clean_i * render_factor(key, i, k).
 __global__ void __launch_bounds__(kRenderThreads)
-render_kernel(const float *__restrict__ clean, const int32_t *__restrict__ offsets,
+render_kernel(const __grid_constant__ BatchImages images, const int32_t *__restrict__ offsets,
               const int32_t *__restrict__ sample_pixel, const long long *__restrict__ total,
-              long long capacity, long long N, uint64_t key, float4 *__restrict__ rgb) {
+              long long capacity, long long N, const __grid_constant__ StreamKeys keys,
+              float4 *__restrict__ rgb) {
     pdl_wait();
     pdl_trigger();
+    // image blockIdx.y of a batch
+    const float *__restrict__ clean = images.p[blockIdx.y];
+    const uint64_t key = keys.k[blockIdx.y];
+    offsets += blockIdx.y * (N + SPP_BATCH_OFFSETS_PAD);
+    sample_pixel += blockIdx.y * capacity;
+    total += blockIdx.y * 2;
+    rgb += blockIdx.y * capacity;
     long long T = *total;
     if (T > capacity) T = capacity;
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
@@ -52,6 +60,14 @@ splat_kernel(const int32_t *__restrict__ offsets, const float4 *__restrict__ rgb
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int x0 = blockIdx.x * kSplatTX, y0 = blockIdx.y * kSplatH;
     const long long N = static_cast<long long>(W) * H;
+    // image blockIdx.z of a batch
+    offsets += blockIdx.z * (N + SPP_BATCH_OFFSETS_PAD);
+    rgb += blockIdx.z * capacity;
+    s += blockIdx.z * N;
+    hw += blockIdx.z * N;
+#pragma unroll
+    for (int l = 0; l < kMaxLevels; ++l)
+        layers.p[l] += blockIdx.z * 3 * (static_cast<long long>(W >> l) * (H >> l));
     // all independent per-pixel loads of both rows first, then the samples
     long long beg[kSplatRows], end[kSplatRows];
     float wl[kSplatRows], si[kSplatRows];
@@ -144,36 +160,42 @@ splat_kernel(const int32_t *__restrict__ offsets, const float4 *__restrict__ rgb
 }  // namespace
 }  // namespace spp
 
-extern "C" {
+namespace spp {
+namespace {
 
-int spp_render_synthetic(const float *clean, const int32_t *offsets, const int32_t *sample_pixel,
-                         const int64_t *total, int64_t capacity, int W, int H, uint64_t seed,
-                         uint32_t frame, float *rgb, cudaStream_t stream) {
-    using namespace spp;
-    if (W < 0 || H < 0 || capacity < 0) return SPP_ERR_ARG;
-    if (!clean || !offsets || !total) return SPP_ERR_ARG;
+int render(int B, const float *const *clean, const int32_t *offsets, const int32_t *sample_pixel,
+           const int64_t *total, int64_t capacity, int W, int H, const uint64_t *seeds,
+           uint32_t frame, float *rgb, cudaStream_t stream) {
+    if (B < 0 || B > kMaxBatch || W < 0 || H < 0 || capacity < 0) return SPP_ERR_ARG;
+    if (!clean || !offsets || !total || !seeds) return SPP_ERR_ARG;
     if (capacity > 0 && (!sample_pixel || !rgb)) return SPP_ERR_ARG;
-    if (!aligned16(clean) || !aligned16(offsets) || !aligned16(total) ||
-        (rgb && !aligned16(rgb)) || (sample_pixel && !aligned16(sample_pixel)))
+    BatchImages images{};
+    StreamKeys keys{};
+    for (int b = 0; b < B; ++b) {
+        if (!clean[b]) return SPP_ERR_ARG;
+        if (!aligned16(clean[b])) return SPP_ERR_ALIGN;
+        images.p[b] = clean[b];
+        keys.k[b] = stream_key(seeds[b], frame);
+    }
+    if (!aligned16(offsets) || !aligned16(total) || (rgb && !aligned16(rgb)) ||
+        (sample_pixel && !aligned16(sample_pixel)))
         return SPP_ERR_ALIGN;
     const long long N = static_cast<long long>(W) * H;
-    if (N == 0 || capacity == 0) return SPP_OK;
+    if (B == 0 || N == 0 || capacity == 0) return SPP_OK;
     long long grid = (capacity + kRenderThreads - 1) / kRenderThreads;
     const long long max_grid = static_cast<long long>(sm_count()) * 8;
     if (grid > max_grid) grid = max_grid;
-    launch_dependent(render_kernel, dim3(static_cast<unsigned>(grid)), dim3(kRenderThreads), 0,
-                     stream, clean, offsets, sample_pixel,
-                     reinterpret_cast<const long long *>(total), capacity, N,
-                     stream_key(seed, frame), reinterpret_cast<float4 *>(rgb));
+    launch_dependent(render_kernel, dim3(static_cast<unsigned>(grid), B), dim3(kRenderThreads), 0,
+                     stream, images, offsets, sample_pixel,
+                     reinterpret_cast<const long long *>(total), capacity, N, keys,
+                     reinterpret_cast<float4 *>(rgb));
     count_launch();
     return launch_status();
 }
 
-int spp_splat_samples(const int32_t *offsets, const float *rgb, const float *s,
-                      const float *holdout_w, int64_t capacity, int W, int H, int L,
-                      float *const *layers, cudaStream_t stream) {
-    using namespace spp;
-    if (W < 0 || H < 0 || capacity < 0 || !layers) return SPP_ERR_ARG;
+int splat(int B, const int32_t *offsets, const float *rgb, const float *s, const float *holdout_w,
+          int64_t capacity, int W, int H, int L, float *const *layers, cudaStream_t stream) {
+    if (B < 0 || W < 0 || H < 0 || capacity < 0 || !layers) return SPP_ERR_ARG;
     if (L < 1 || L > kMaxLevels) return SPP_ERR_SHAPE;
     if ((W % (1 << (L - 1))) != 0 || (H % (1 << (L - 1))) != 0) return SPP_ERR_SHAPE;
     if (!offsets || !s || !holdout_w || (capacity > 0 && !rgb)) return SPP_ERR_ARG;
@@ -185,13 +207,57 @@ int spp_splat_samples(const int32_t *offsets, const float *rgb, const float *s,
     }
     if (!aligned16(offsets) || !aligned16(s) || !aligned16(holdout_w) || (rgb && !aligned16(rgb)))
         return SPP_ERR_ALIGN;
-    if (static_cast<long long>(W) * H == 0) return SPP_OK;
+    if (B == 0 || static_cast<long long>(W) * H == 0) return SPP_OK;
     dim3 block(kSplatTX, kSplatTY);
-    dim3 grid((W + kSplatTX - 1) / kSplatTX, (H + kSplatH - 1) / kSplatH);
+    dim3 grid((W + kSplatTX - 1) / kSplatTX, (H + kSplatH - 1) / kSplatH, B);
     launch_dependent(splat_kernel, grid, block, 0, stream, offsets,
                      reinterpret_cast<const float4 *>(rgb), s, holdout_w, capacity, W, H, L, lp);
     count_launch();
     return launch_status();
+}
+
+}  // namespace
+}  // namespace spp
+
+extern "C" {
+
+int spp_render_synthetic(const float *clean, const int32_t *offsets, const int32_t *sample_pixel,
+                         const int64_t *total, int64_t capacity, int W, int H, uint64_t seed,
+                         uint32_t frame, float *rgb, cudaStream_t stream) {
+    return spp::render(1, &clean, offsets, sample_pixel, total, capacity, W, H, &seed, frame, rgb,
+                       stream);
+}
+
+int spp_render_synthetic_batch(int B, const float *const *clean, const int32_t *offsets,
+                               const int32_t *sample_pixel, const int64_t *total, int64_t capacity,
+                               int W, int H, const uint64_t *seeds, uint32_t frame, float *rgb,
+                               cudaStream_t stream) {
+    using namespace spp;
+    if (B < 0 || W < 0 || H < 0 || capacity < 0 || !clean || !offsets || !sample_pixel || !total ||
+        !seeds || !rgb)
+        return SPP_ERR_ARG;
+    const int64_t n = static_cast<int64_t>(W) * H;
+    if (B > 1 && n % 4) return SPP_ERR_ALIGN;
+    for (int b = 0; b < B; b += kMaxBatch) {
+        const int k = B - b < kMaxBatch ? B - b : kMaxBatch;
+        const int rc = render(k, clean + b, offsets + b * (n + SPP_BATCH_OFFSETS_PAD),
+                              sample_pixel + b * capacity, total + 2 * b, capacity, W, H, seeds + b,
+                              frame, rgb + 4 * b * capacity, stream);
+        if (rc != SPP_OK) return rc;
+    }
+    return SPP_OK;
+}
+
+int spp_splat_samples(const int32_t *offsets, const float *rgb, const float *s,
+                      const float *holdout_w, int64_t capacity, int W, int H, int L,
+                      float *const *layers, cudaStream_t stream) {
+    return spp::splat(1, offsets, rgb, s, holdout_w, capacity, W, H, L, layers, stream);
+}
+
+int spp_splat_samples_batch(int B, const int32_t *offsets, const float *rgb, const float *s,
+                            const float *holdout_w, int64_t capacity, int W, int H, int L,
+                            float *const *layers, cudaStream_t stream) {
+    return spp::splat(B, offsets, rgb, s, holdout_w, capacity, W, H, L, layers, stream);
 }
 
 }  // extern "C"

@@ -69,6 +69,19 @@ inline void launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
     (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Batched launches: one grid dimension runs over the images of a batch, whose
+// per-image stream keys and input images travel in the kernel's parameters.
+// Larger batches are launched in parts of kMaxBatch images.
+constexpr int kMaxBatch = 16;
+// (kernels take them as __grid_constant__, so that indexing by the image reads
+// constant memory; a plain parameter would be copied to local memory first)
+struct StreamKeys {
+    uint64_t k[kMaxBatch];
+};
+struct BatchImages {
+    const float *p[kMaxBatch];
+};
+
 // Records a device-side error: the first one wins.
 __device__ __forceinline__ void set_status(int32_t *status, int code) {
     if (status) atomicCAS(reinterpret_cast<int *>(status), 0, code);

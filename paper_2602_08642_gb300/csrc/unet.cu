@@ -119,10 +119,20 @@ ActLayout act_layout(int net, int B, int W, int H) {
 
 namespace {
 
-__global__ void assemble_kernel(const float *__restrict__ albedo, const float *__restrict__ normal,
-                                const float *__restrict__ depth, const float *__restrict__ mv,
-                                const float *__restrict__ prev, int64_t n, float *__restrict__ out) {
+// Input images of a batch's G-buffers; prev is [B][3][H][W] or null.
+struct FeatureImages {
+    BatchImages albedo, normal, depth, mv;
+};
+
+__global__ void assemble_kernel(const __grid_constant__ FeatureImages im,
+                                const float *__restrict__ prev, int64_t n,
+                                float *__restrict__ out) {
     const float inv_ln100 = 1.0f / 4.605170185988091f;
+    const int b = blockIdx.y;
+    const float *__restrict__ albedo = im.albedo.p[b], *__restrict__ normal = im.normal.p[b];
+    const float *__restrict__ depth = im.depth.p[b], *__restrict__ mv = im.mv.p[b];
+    if (prev) prev += b * 3 * n;
+    out += b * 12 * n;
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         out[i] = albedo[i];
@@ -357,13 +367,25 @@ int pack(int net, const float *theta, int with_backward, unsigned char *packed,
     return launch_status();
 }
 
-int assemble(const float *albedo, const float *normal, const float *depth, const float *mv,
-             const float *prev, int W, int H, float *in12, cudaStream_t stream) {
+int assemble(int B, const float *const *albedo, const float *const *normal,
+             const float *const *depth, const float *const *mv, const float *prev, int W, int H,
+             float *in12, cudaStream_t stream) {
     const int64_t n = static_cast<int64_t>(W) * H;
     if (n == 0) return SPP_OK;
     const int grid = static_cast<int>(std::min<int64_t>((n + 255) / 256, 4 * sm_count()));
-    assemble_kernel<<<grid, 256, 0, stream>>>(albedo, normal, depth, mv, prev, n, in12);
-    count_launch();
+    for (int b = 0; b < B; b += kMaxBatch) {
+        const int k = std::min(B - b, kMaxBatch);
+        FeatureImages im{};
+        for (int i = 0; i < k; ++i) {
+            im.albedo.p[i] = albedo[b + i];
+            im.normal.p[i] = normal[b + i];
+            im.depth.p[i] = depth[b + i];
+            im.mv.p[i] = mv[b + i];
+        }
+        assemble_kernel<<<dim3(grid, k), 256, 0, stream>>>(im, prev ? prev + b * 3 * n : nullptr, n,
+                                                           in12 + b * 12 * n);
+        count_launch();
+    }
     return launch_status();
 }
 
@@ -500,11 +522,23 @@ extern "C" int spp_unet_pack(const float *theta, int with_backward, void *packed
 extern "C" int spp_assemble_features(const float *albedo, const float *normal, const float *depth,
                                      const float *mv, const float *prev_ldr, int W, int H,
                                      float *in12, cudaStream_t stream) {
-    if (W < 0 || H < 0 || !albedo || !normal || !depth || !mv || !in12) return SPP_ERR_ARG;
-    if (!aligned16(albedo) || !aligned16(normal) || !aligned16(depth) || !aligned16(mv) ||
-        !aligned16(in12) || (prev_ldr && !aligned16(prev_ldr)))
-        return SPP_ERR_ALIGN;
-    return spp::unet::assemble(albedo, normal, depth, mv, prev_ldr, W, H, in12, stream);
+    return spp_assemble_features_batch(1, &albedo, &normal, &depth, &mv, prev_ldr, W, H, in12,
+                                       stream);
+}
+
+extern "C" int spp_assemble_features_batch(int B, const float *const *albedo,
+                                           const float *const *normal, const float *const *depth,
+                                           const float *const *mv, const float *prev_ldr, int W,
+                                           int H, float *in12, cudaStream_t stream) {
+    if (B < 0 || W < 0 || H < 0 || !albedo || !normal || !depth || !mv || !in12) return SPP_ERR_ARG;
+    for (int b = 0; b < B; ++b) {
+        if (!albedo[b] || !normal[b] || !depth[b] || !mv[b]) return SPP_ERR_ARG;
+        if (!aligned16(albedo[b]) || !aligned16(normal[b]) || !aligned16(depth[b]) ||
+            !aligned16(mv[b]))
+            return SPP_ERR_ALIGN;
+    }
+    if (!aligned16(in12) || (prev_ldr && !aligned16(prev_ldr))) return SPP_ERR_ALIGN;
+    return spp::unet::assemble(B, albedo, normal, depth, mv, prev_ldr, W, H, in12, stream);
 }
 
 extern "C" size_t spp_predict_workspace_bytes(int B, int W, int H) {

@@ -85,8 +85,9 @@ int adamw(float *theta, const float *grad, float *m, float *v, int64_t n, int st
           float b1, float b2, float eps, float wd, float grad_scale, cudaStream_t stream);
 int pack(int net, const float *theta, int with_backward, unsigned char *packed,
          cudaStream_t stream);
-int assemble(const float *albedo, const float *normal, const float *depth, const float *mv,
-             const float *prev, int W, int H, float *in12, cudaStream_t stream);
+int assemble(int B, const float *const *albedo, const float *const *normal,
+             const float *const *depth, const float *const *mv, const float *prev, int W, int H,
+             float *in12, cudaStream_t stream);
 int density_softmax(const float *z, int B, int64_t hw, int64_t batch_stride, float *d,
                     uint32_t *zmax, cudaStream_t stream);
 

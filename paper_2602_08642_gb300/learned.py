@@ -25,7 +25,7 @@ import math
 import torch
 
 from . import _binding as B
-from .pipeline import Frame
+from .pipeline import Frame, FrameBatch
 
 LEVELS = 3
 PHI = 0.125
@@ -111,6 +111,13 @@ class Predictor:
     def features(self, b: int, albedo, normal, depth, mv, prev_ldr=None):
         B.check(B.spp_assemble_features(albedo, normal, depth, mv, prev_ldr, self.W, self.H,
                                         self.x[b]), "spp_assemble_features")
+
+    def features_batch(self, gbufs: list, mvs: list, prev_ldr=None):
+        """features for every image of the batch; prev_ldr [B][3][H][W]."""
+        B.check(B.spp_assemble_features_batch([g["albedo"] for g in gbufs],
+                                              [g["normal"] for g in gbufs],
+                                              [g["depth"] for g in gbufs], mvs, prev_ldr, self.W,
+                                              self.H, self.x), "spp_assemble_features_batch")
 
     def forward(self):
         if self.net == B.SPP_NET_JOINT:
@@ -245,33 +252,64 @@ class Renderer:
         # to the nearest integer adds at most half a sample per pixel
         cap_budget = (budget + 1.0 if (estimator == "gumbel" and train)
                       else budget + 0.5 if estimator == "dasr" else budget)
-        self.frames = [Frame(W, H, LEVELS, max_budget=cap_budget) for _ in range(B_)]
+        # the images of a batch lie one after the other where every image then
+        # starts on a 16-byte boundary; the *_all methods work on all of them
+        self.batched = B_ == 1 or FrameBatch.fits(W, H, LEVELS)
+        if self.batched:
+            self.batch = FrameBatch(B_, W, H, LEVELS, max_budget=cap_budget)
+            self.frames = self.batch.frames
+        else:
+            self.frames = [Frame(W, H, LEVELS, max_budget=cap_budget) for _ in range(B_)]
         self.cur_clean = [None] * B_
         self.cur_seed = [0] * B_
         self.tm = B.make_tonemap()
-        self.hdr_prev = [_zeros(3, H, W) for _ in range(B_)]
-        self.warped = [_zeros(3, H, W) for _ in range(B_)]
-        self.prev_ldr = [_zeros(3, H, W) for _ in range(B_)]
-        self.ref = [_zeros(3, H, W) for _ in range(B_)]
         self.mask = _zeros(H, W, dtype=torch.uint8)
-        self.hats = [[_zeros(3, H >> l, W >> l) for l in range(LEVELS)] for _ in range(B_)]
-        self.hdr = [_zeros(3, H, W) for _ in range(B_)]
-        self.ldr = [_zeros(3, H, W) for _ in range(B_)]
-        self.loss = [_zeros(4)[:1] for _ in range(B_)]
-        self.g_ldr = _zeros(3, H, W)
-        self.g_hdr = [_zeros(3, H >> l, W >> l) for l in range(LEVELS)]
-        self.g_noisy = [_zeros(3, H >> l, W >> l) for l in range(LEVELS)]
-        self.g_warped = _zeros(3, H, W)
-        self.g_s = _zeros(W * H)
+        self.all = {}
+        for name in ("hdr_prev", "warped", "prev_ldr", "ref", "hdr", "ldr",
+                     # temporal term of the objective: previous tone-mapped output and
+                     # reference, warped to the current frame
+                     "ldr_prev", "wldr_prev", "wref_prev"):
+            setattr(self, name, self._images(name, B_, 3, H, W))
+        per_level = [self._images(f"hats{l}", B_, 3, H >> l, W >> l) for l in range(LEVELS)]
+        self.hats = [[per_level[l][b] for l in range(LEVELS)] for b in range(B_)]
+        self.all["loss"] = _zeros(B_, 4)
+        self.loss = [self.all["loss"][b, :1] for b in range(B_)]
+        self.tmp = _zeros(B_ if self.batched else 1, 3, H, W)
+        # gradient images; those that the backward adds to lie in one buffer, so
+        # that one fill clears them
+        nb = B_ if self.batched else 1
+        shapes = [(nb, 3, H >> l, W >> l) for l in range(LEVELS)]
+        sizes = [-(-math.prod(s) // 64) * 64 for s in shapes]
+        self.g_sum = _zeros(2 * sum(sizes) + sizes[0])
+        at = 0
+
+        def part(s):
+            nonlocal at
+            v = self.g_sum[at:at + math.prod(s)].view(s)
+            at += -(-math.prod(s) // 64) * 64
+            return v
+
+        self.all["g_hdr"] = [part(s) for s in shapes]
+        self.all["g_noisy"] = [part(s) for s in shapes]
+        self.all["g_warped"] = part(shapes[0])
+        self.all["g_ldr"] = _zeros(nb, 3, H, W)
+        self.all["g_s"] = _zeros(nb, W * H)
+        # the images that the methods for one sample work on
+        self.g_hdr = [x[0] for x in self.all["g_hdr"]]
+        self.g_noisy = [x[0] for x in self.all["g_noisy"]]
+        self.g_warped, self.g_ldr = self.all["g_warped"][0], self.all["g_ldr"][0]
+        self.g_s = self.all["g_s"][0]
         self.mse = torch.zeros(2, dtype=torch.float64, device="cuda")[:1]
-        self.dws = Predictor._aligned(B.spp_density_backward_workspace_bytes())
+        self.dws = Predictor._aligned(nb * B.spp_density_backward_workspace_bytes())
         self.cur_params = [None] * B_
-        # temporal term of the objective: previous tone-mapped output and
-        # reference, warped to the current frame
-        self.ldr_prev = [_zeros(3, H, W) for _ in range(B_)]
-        self.wldr_prev = [_zeros(3, H, W) for _ in range(B_)]
-        self.wref_prev = [_zeros(3, H, W) for _ in range(B_)]
-        self.tmp = _zeros(3, H, W)
+
+    def _images(self, name: str, *shape):
+        """A list of one zeroed image per sample, parts of self.all[name] where
+        the batch is held together."""
+        if not self.batched:
+            return [_zeros(*shape[1:]) for _ in range(shape[0])]
+        self.all[name] = _zeros(*shape)
+        return list(self.all[name].unbind(0))
 
     def _alloc(self, fr, d, params):
         if self.dither is not None:
@@ -329,8 +367,8 @@ class Renderer:
         tone-mapped output and reference warped to frame t."""
         B.check(B.spp_warp_previous(self.ldr_prev[b], mv, self.W, self.H, self.wldr_prev[b]),
                 "warp")
-        B.check(B.spp_tonemap_image(hdr_ref_prev, self.W, self.H, self.tm, self.tmp), "tonemap")
-        B.check(B.spp_warp_previous(self.tmp, mv, self.W, self.H, self.wref_prev[b]), "warp")
+        B.check(B.spp_tonemap_image(hdr_ref_prev, self.W, self.H, self.tm, self.tmp[0]), "tonemap")
+        B.check(B.spp_warp_previous(self.tmp[0], mv, self.W, self.H, self.wref_prev[b]), "warp")
 
     def backward(self, b: int, d, logits, g_logits, objective: str = "l1"):
         """Loss of sample b and its gradient into g_logits (level 0 planes
@@ -370,6 +408,101 @@ class Renderer:
             self.cur_clean[b], self.cur_seed[b], self.g_s), "splat backward")
         B.check(B.spp_density_backward(d, self.W * self.H, self.budget, PHI, self.g_s,
                                        g_logits[3], self.dws), "density backward")
+
+    # ---- the same steps for all samples of a batch held together: one launch
+    # per step instead of one per sample
+    def _render_all(self, d, cleans, seed: int, frame: int):
+        """Sample maps, samples and pyramids of all samples (seed + b each)."""
+        fb, W, H, n = self.batch, self.W, self.H, self.B
+        params = self.params(frame, seed)
+        seeds = [seed + b for b in range(n)]
+        if self.dither is not None:
+            for b, fr in enumerate(self.frames):
+                fr.alloc_dithered(d[b], self.params(frame, seed + b), self.dither)
+        else:
+            B.check(B.spp_alloc_sample_map_batch(n, d, W, H, params, seeds, fb.counts, fb.offsets,
+                                                 fb.sample_pixel, fb.capacity, fb.s, fb.holdout_w,
+                                                 fb.total, fb.status, fb.alloc_ws),
+                    "spp_alloc_sample_map_batch")
+        B.check(B.spp_render_synthetic_batch(cleans, fb.offsets, fb.sample_pixel, fb.total,
+                                             fb.capacity, W, H, [s ^ 0xC0FFEE for s in seeds],
+                                             frame, fb.rgb), "spp_render_synthetic_batch")
+        B.check(B.spp_splat_samples_batch(n, fb.offsets, fb.rgb, fb.s, fb.holdout_w, fb.capacity,
+                                          W, H, LEVELS, fb.layers), "spp_splat_samples_batch")
+
+    def _reconstruct_all(self, logits, hdr, ldr, warped=None):
+        for l in range(LEVELS - 1, -1, -1):
+            B.check(B.spp_reconstruct_level_batch(
+                self.B, self.batch.layers[l], logits[l], logits[l].shape[1],
+                self.all[f"hats{l + 1}"] if l + 1 < LEVELS else None, warped if l == 0 else None,
+                self.mask if l == 0 and warped is not None else None, self.W >> l, self.H >> l,
+                self.tm if l == 0 else None, self.all[f"hats{l}"] if l else hdr,
+                None if l else ldr), "level")
+
+    def previous_frame_all(self, d, logits, cleans, seed: int, frame: int):
+        """previous_frame and warp_previous's source for all samples: d
+        [B][H][W], logits the network's heads [B][C][H>>l][W>>l]."""
+        self._render_all(d, cleans, seed, frame)
+        self._reconstruct_all(logits, self.all["hdr_prev"], self.all["ldr_prev"])
+
+    def warp_previous_all(self, mvs):
+        a = self.all
+        B.check(B.spp_warp_previous_batch(self.hdr_prev, mvs, self.W, self.H, a["warped"]), "warp")
+        B.check(B.spp_tonemap_image_batch(self.warped, self.W, self.H, self.tm, a["prev_ldr"]),
+                "tonemap")
+
+    def current_frame_all(self, d, logits, cleans, seed: int, frame: int):
+        for b in range(self.B):
+            self.cur_params[b] = self.params(frame, seed + b)
+            self.cur_clean[b], self.cur_seed[b] = cleans[b], (seed + b) ^ 0xC0FFEE
+        self._render_all(d, cleans, seed, frame)
+        self._reconstruct_all(logits, self.all["hdr"], self.all["ldr"], self.all["warped"])
+
+    def reference_all(self, hdr_refs):
+        B.check(B.spp_tonemap_image_batch(hdr_refs, self.W, self.H, self.tm, self.all["ref"]),
+                "tonemap")
+
+    def temporal_references_all(self, hdr_refs_prev, mvs):
+        W, H, a = self.W, self.H, self.all
+        B.check(B.spp_warp_previous_batch(self.ldr_prev, mvs, W, H, a["wldr_prev"]), "warp")
+        B.check(B.spp_tonemap_image_batch(hdr_refs_prev, W, H, self.tm, self.tmp), "tonemap")
+        B.check(B.spp_warp_previous_batch(list(self.tmp.unbind(0)), mvs, W, H, a["wref_prev"]),
+                "warp")
+
+    def backward_all(self, d, logits, g_heads, objective: str = "l1"):
+        """backward for all samples; g_heads are the heads' gradients (the
+        density plane follows the 54 logit planes of level 0)."""
+        W, H, nb, a, fb = self.W, self.H, self.B, self.all, self.batch
+        n = 3 * W * H
+        if objective == "combined":
+            B.check(B.spp_combined_loss_batch(nb, a["ldr"], a["ref"], a["wldr_prev"],
+                                              a["wref_prev"], n, 1.25, 1.0, a["loss"], a["g_ldr"]),
+                    "combined loss")
+        else:
+            B.check(B.spp_l1_loss_batch(nb, a["ldr"], a["ref"], n, a["loss"], a["g_ldr"]), "l1")
+        self.g_sum.zero_()
+        g = a["g_hdr"]
+        B.check(B.spp_tonemap_backward_batch(nb, a["hdr"], W, H, self.tm, a["g_ldr"], g[0]),
+                "tonemap backward")
+        for l in range(LEVELS):
+            top = l == 0
+            B.check(B.spp_reconstruct_level_backward_batch(
+                nb, fb.layers[l], logits[l], logits[l].shape[1],
+                a[f"hats{l + 1}"] if l + 1 < LEVELS else None, a["warped"] if top else None,
+                self.mask if top else None, W >> l, H >> l, g[l], g_heads[l],
+                54 if top else logits[l].shape[1], a["g_noisy"][l],
+                g[l + 1] if l + 1 < LEVELS else None, a["g_warped"] if top else None),
+                "level backward")
+        B.check(B.spp_pyramid_backward_batch(nb, a["g_noisy"], W, H, LEVELS, a["g_noisy"][0]),
+                "pyramid backward")
+        B.check(B.spp_splat_backward_batch(
+            nb, fb.offsets, fb.counts, fb.rgb, fb.s, fb.layers[0], a["g_noisy"][0], fb.holdout_w,
+            fb.capacity, W, H, self.cur_params[0], [p.seed for p in self.cur_params],
+            ESTIMATORS[self.estimator], self.cur_clean, self.cur_seed, a["g_s"]),
+            "splat backward")
+        B.check(B.spp_density_backward_batch(nb, d, W * H, self.budget, PHI, a["g_s"],
+                                             g_heads[0][0, 54], g_heads[0].stride(0), self.dws),
+                "density backward")
 
     def psnr(self, b: int) -> float:
         B.check(B.spp_mse(self.ldr[b], self.ref[b], 3 * self.W * self.H, self.mse), "mse")
@@ -427,6 +560,32 @@ class Trainer:
         f_prev, f_cur = 2 * self.step_index, 2 * self.step_index + 1
         if self.random_tmo:
             rnd.tm = random_tonemap(self.rng)
+        if rnd.batched and len(samples) == rnd.B:
+            mvs = [s.mv for s in samples]
+            net.features_batch([s.gprev for s in samples], mvs)
+            net.forward()
+            rnd.previous_frame_all(net.density, net.heads, [s.clean_prev for s in samples], seed,
+                                   f_prev)
+            rnd.warp_previous_all(mvs)
+            net.features_batch([s.g for s in samples], mvs, rnd.all["prev_ldr"])
+            net.forward()
+            rnd.current_frame_all(net.density, net.heads, [s.clean for s in samples], seed, f_cur)
+            rnd.reference_all([s.reference(self.reference) for s in samples])
+            if self.objective == "combined":
+                rnd.temporal_references_all([s.reference(self.reference, prev=True)
+                                             for s in samples], mvs)
+            rnd.backward_all(net.density, net.heads, net.g_heads, self.objective)
+        else:
+            self._forward_backward(samples, seed, f_prev, f_cur)
+        net.backward()
+        net.adamw(self.current_lr(), self.wd, grad_scale=1.0 / len(samples), betas=self.betas)
+        self.step_index += 1
+        return float(sum(rnd.all["loss"][:, 0].tolist())) / len(samples)
+
+    def _forward_backward(self, samples, seed: int, f_prev: int, f_cur: int):
+        """step's forward and renderer backward sample by sample (a part of a
+        batch, or images that do not all start on a 16-byte boundary)."""
+        net, rnd = self.net, self.rnd
         for b, s in enumerate(samples):
             net.features(b, s.gprev["albedo"], s.gprev["normal"], s.gprev["depth"], s.mv, None)
         net.forward()
@@ -445,10 +604,6 @@ class Trainer:
             gl = [net.g_logits[0][b, :54], net.g_logits[1][b], net.g_logits[2][b],
                   net.g_logits[0][b, 54]]
             rnd.backward(b, net.density[b], logits, gl, self.objective)
-        net.backward()
-        net.adamw(self.current_lr(), self.wd, grad_scale=1.0 / len(samples), betas=self.betas)
-        self.step_index += 1
-        return float(sum(l.item() for l in rnd.loss)) / len(samples)
 
 
 def evaluate(samples: list[FrameData], budget: float, theta: torch.Tensor | None,

@@ -35,24 +35,31 @@ class Frame:
     """Device buffers for W x H frames with an L-level pyramid."""
 
     def __init__(self, W: int, H: int, L: int, *, max_budget: float = 0.5,
-                 capacity: int | None = None, device: str | torch.device = "cuda"):
+                 capacity: int | None = None, device: str | torch.device = "cuda",
+                 storage: dict | None = None):
+        """storage: buffers to use instead of new ones, by attribute name (the
+        images of a FrameBatch share theirs)."""
         self.W, self.H, self.L = W, H, L
         self.N = N = W * H
         self.device = torch.device(device)
         dev = self.device
         self.capacity = capacity if capacity is not None else default_capacity(W, H, max_budget)
         i32, f32 = torch.int32, torch.float32
-        self.counts = torch.empty(N, dtype=i32, device=dev)
-        self.offsets = torch.empty(N + 1, dtype=i32, device=dev)
-        self.sample_pixel = torch.empty(max(self.capacity, 1), dtype=i32, device=dev)
-        self.s = torch.empty(N, dtype=f32, device=dev)
-        self.holdout_w = torch.empty(N, dtype=f32, device=dev)
-        self.total = torch.zeros(2, dtype=torch.int64, device=dev)[:1]
-        self.status = torch.zeros(4, dtype=i32, device=dev)[:1]
-        self.alloc_ws = torch.empty(max(B.spp_alloc_workspace_bytes(W, H), 16),
-                                    dtype=torch.uint8, device=dev)
-        self.rgb = torch.empty((max(self.capacity, 1), 4), dtype=f32, device=dev)
-        self.layers = [torch.empty((3, H >> l, W >> l), dtype=f32, device=dev) for l in range(L)]
+        st = storage or {}
+        new = lambda name, shape, dtype: (st[name] if name in st else
+                                          torch.empty(shape, dtype=dtype, device=dev))
+        self.counts = new("counts", N, i32)
+        self.offsets = new("offsets", N + 1, i32)
+        self.sample_pixel = new("sample_pixel", max(self.capacity, 1), i32)
+        self.s = new("s", N, f32)
+        self.holdout_w = new("holdout_w", N, f32)
+        self.total = st["total"] if "total" in st else torch.zeros(2, dtype=torch.int64,
+                                                                   device=dev)[:1]
+        self.status = st["status"] if "status" in st else torch.zeros(4, dtype=i32, device=dev)[:1]
+        self.alloc_ws = new("alloc_ws", max(B.spp_alloc_workspace_bytes(W, H), 16), torch.uint8)
+        self.rgb = new("rgb", (max(self.capacity, 1), 4), f32)
+        self.layers = st["layers"] if "layers" in st else [
+            torch.empty((3, H >> l, W >> l), dtype=f32, device=dev) for l in range(L)]
         self.recon_ws = torch.empty(max(B.spp_reconstruct_workspace_bytes(W, H, L), 16),
                                     dtype=torch.uint8, device=dev)
         self.hdr = [torch.zeros((3, H, W), dtype=f32, device=dev) for _ in range(2)]
@@ -122,3 +129,37 @@ class Frame:
 
     def sample_count(self) -> int:
         return int(self.total.item())
+
+
+class FrameBatch:
+    """Device buffers of a batch of n frames of one size, held image after
+    image as the batched entry points take them, and ``frames``, the n Frames
+    whose buffers are parts of them.  Every image has to start on a 16-byte
+    boundary on every level (``fits``)."""
+
+    @staticmethod
+    def fits(W: int, H: int, L: int) -> bool:
+        return all((W >> l) * (H >> l) % 4 == 0 for l in range(L))
+
+    def __init__(self, n: int, W: int, H: int, L: int, *, max_budget: float = 0.5,
+                 device: str | torch.device = "cuda"):
+        N = W * H
+        # whole 16-byte pieces, for the images' sample lists too
+        self.capacity = cap = -(-default_capacity(W, H, max_budget) // 4) * 4
+        i32, f32 = torch.int32, torch.float32
+        e = lambda *shape, dtype=f32: torch.empty(shape, dtype=dtype, device=device)
+        self.counts = e(n, N, dtype=i32)
+        self.offsets = e(n, N + B.SPP_BATCH_OFFSETS_PAD, dtype=i32)
+        self.sample_pixel = e(n, cap, dtype=i32)
+        self.s, self.holdout_w = e(n, N), e(n, N)
+        self.total = torch.zeros(n, 2, dtype=torch.int64, device=device)
+        self.status = torch.zeros(n, 4, dtype=i32, device=device)
+        self.alloc_ws = e(B.spp_alloc_batch_workspace_bytes(n, W, H), dtype=torch.uint8)
+        self.rgb = e(n, cap, 4)
+        self.layers = [e(n, 3, H >> l, W >> l) for l in range(L)]
+        ws = self.alloc_ws.view(n, -1)
+        self.frames = [Frame(W, H, L, capacity=cap, device=device, storage=dict(
+            counts=self.counts[b], offsets=self.offsets[b, :N + 1],
+            sample_pixel=self.sample_pixel[b], s=self.s[b], holdout_w=self.holdout_w[b],
+            total=self.total[b, :1], status=self.status[b, :1], alloc_ws=ws[b], rgb=self.rgb[b],
+            layers=[x[b] for x in self.layers])) for b in range(n)]
