@@ -898,41 +898,59 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
     }
 }
 
-__global__ void pack_weights_kernel(const float *__restrict__ w, int cin, int cout, int transpose,
-                                    int cin_pad, int n, __nv_bfloat16 *__restrict__ dst) {
-    const int64_t total = static_cast<int64_t>(cin_pad / 16) * 9 * 2 * n * 8;
-    for (int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; idx < total;
-         idx += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int e = static_cast<int>(idx % 8);
-        int o, kg, c, dy, dx;
-        if (n == 32 || n == 64) {
-            // stacked: [chunk][dx][kg][3 n = (dy = 2, 1, 0) x n][8]
-            const int64_t S = 3 * static_cast<int64_t>(n);
-            const int n3 = static_cast<int>((idx / 8) % S);
-            kg = static_cast<int>((idx / (8 * S)) % 2);
-            dx = static_cast<int>((idx / (16 * S)) % 3);
-            c = static_cast<int>(idx / (48 * S));
-            o = n3 % n;
-            dy = 2 - n3 / n;
-        } else {
-            // [chunk][tap][kg][n][8]
-            o = static_cast<int>((idx / 8) % n);
-            kg = static_cast<int>((idx / (8 * n)) % 2);
-            const int tap = static_cast<int>((idx / (16 * n)) % 9);
-            c = static_cast<int>(idx / (144 * static_cast<int64_t>(n)));
-            dy = tap / 3;
-            dx = tap % 3;
-        }
-        const int k = c * 16 + kg * 8 + e;  // input channel of this convolution
-        float v = 0.f;
-        if (!transpose) {
-            if (o < cout && k < cin) v = w[((static_cast<int64_t>(o) * cin + k) * 3 + dy) * 3 + dx];
-        } else {  // data gradient: input channel k is an output channel of w
-            if (o < cin && k < cout)
-                v = w[((static_cast<int64_t>(k) * cin + o) * 3 + (2 - dy)) * 3 + (2 - dx)];
-        }
-        dst[idx] = __float2bfloat16_rn(v);
+// Eight consecutive input channels of one operand row per thread (a 16-byte
+// store); a block works on one item of the table.
+constexpr int kPackThreads = 256;
+
+__global__ void __launch_bounds__(kPackThreads)
+pack_weights_kernel(const __grid_constant__ PackTable table) {
+    int i = 0;
+    while (i + 1 < table.count && static_cast<int>(blockIdx.x) >= table.it[i + 1].first_block) ++i;
+    const PackItem &it = table.it[i];
+    const int cin = it.cin, cout = it.cout, n = it.n;
+    const int block = blockIdx.x - it.first_block;
+    if (block == 0 && it.bias_dst)
+        for (int j = threadIdx.x; j < n; j += kPackThreads)
+            it.bias_dst[j] = j < cout ? it.bias[j] : 0.f;
+    const int idx = block * kPackThreads + threadIdx.x;
+    if (idx >= it.cin_pad / 16 * 18 * n) return;
+    int o, kg, c, dy, dx;
+    if (n == 32 || n == 64) {
+        // stacked: [chunk][dx][kg][3 n = (dy = 2, 1, 0) x n][8]
+        const int S = 3 * n, n3 = idx % S;
+        kg = (idx / S) % 2;
+        dx = (idx / (2 * S)) % 3;
+        c = idx / (6 * S);
+        o = n3 % n;
+        dy = 2 - n3 / n;
+    } else {
+        // [chunk][tap][kg][n][8]
+        o = idx % n;
+        kg = (idx / n) % 2;
+        const int tap = (idx / (2 * n)) % 9;
+        c = idx / (18 * n);
+        dy = tap / 3;
+        dx = tap % 3;
     }
+    uint32_t w[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        float v[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int k = c * 16 + kg * 8 + 2 * h + e;  // input channel of this convolution
+            v[e] = 0.f;
+            if (!it.transpose) {
+                if (o < cout && k < cin)
+                    v[e] = it.w[((static_cast<int64_t>(o) * cin + k) * 3 + dy) * 3 + dx];
+            } else {  // data gradient: input channel k is an output channel of w
+                if (o < cin && k < cout)
+                    v[e] = it.w[((static_cast<int64_t>(k) * cin + o) * 3 + (2 - dy)) * 3 + (2 - dx)];
+            }
+        }
+        w[h] = pack_bf16x2(v[0], v[1]);
+    }
+    reinterpret_cast<uint4 *>(it.dst)[idx] = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 // SPP_CONV_NO_TMA_IN=1 selects the cp.async halo producers instead of TMA
@@ -1048,14 +1066,25 @@ int launch(const ConvArgs &a, cudaStream_t stream) {
 
 }  // namespace
 
-int pack_weights(const float *w, int cin, int cout, int transpose, int cin_pad, int n,
-                 __nv_bfloat16 *dst, cudaStream_t stream) {
-    const int64_t total = static_cast<int64_t>(cin_pad / 16) * 9 * 2 * n * 8;
-    if (total == 0) return SPP_OK;
-    const int grid = static_cast<int>(std::min<int64_t>((total + 255) / 256, 4 * sm_count()));
-    pack_weights_kernel<<<grid, 256, 0, stream>>>(w, cin, cout, transpose, cin_pad, n, dst);
+int pack_weights(PackTable &table, cudaStream_t stream) {
+    int blocks = 0;
+    for (int i = 0; i < table.count; ++i) {
+        PackItem &it = table.it[i];
+        it.first_block = blocks;
+        blocks += std::max(1, (it.cin_pad / 16 * 18 * it.n + kPackThreads - 1) / kPackThreads);
+    }
+    if (blocks == 0) return SPP_OK;
+    pack_weights_kernel<<<blocks, kPackThreads, 0, stream>>>(table);
     count_launch();
     return launch_status();
+}
+
+int pack_weights(const float *w, int cin, int cout, int transpose, int cin_pad, int n,
+                 __nv_bfloat16 *dst, cudaStream_t stream) {
+    PackTable table;
+    table.count = 1;
+    table.it[0] = PackItem{w, dst, nullptr, nullptr, cin, cout, transpose, cin_pad, n, 0};
+    return pack_weights(table, stream);
 }
 
 int conv3x3(const ConvArgs &a, cudaStream_t stream) {

@@ -193,11 +193,6 @@ __global__ void features_nhwc32_kernel(const float *__restrict__ in, int C, int6
     }
 }
 
-__global__ void copy_bias_kernel(const float *__restrict__ b, int cout, int n, float *__restrict__ dst) {
-    const int i = threadIdx.x;
-    if (i < n) dst[i] = i < cout ? b[i] : 0.f;
-}
-
 // Order-preserving map of a float to an unsigned integer (for atomicMax).
 __device__ __forceinline__ uint32_t ordered(float f) {
     const uint32_t u = __float_as_uint(f);
@@ -347,24 +342,21 @@ int forward(int net, const unsigned char *packed, const float *in, int B, int W,
 int pack(int net, const float *theta, int with_backward, unsigned char *packed,
          cudaStream_t stream) {
     const PackedLayout P = packed_layout(net, with_backward);
+    auto operand = [&](size_t off) { return reinterpret_cast<__nv_bfloat16 *>(packed + off); };
+    conv::PackTable table;
     for (int i = 0; i < kNumLayers; ++i) {
         const Layer l = layer(net, i);
         if (l.cout == 0) continue;
-        int rc = conv::pack_weights(theta + P.theta_w[i], l.cin, l.cout, 0, round16(l.cin),
-                                    fwd_n(net, i),
-                                    reinterpret_cast<__nv_bfloat16 *>(packed + P.fwd[i]), stream);
-        if (rc != SPP_OK) return rc;
-        copy_bias_kernel<<<1, 256, 0, stream>>>(theta + P.theta_b[i], l.cout, fwd_n(net, i),
-                                                reinterpret_cast<float *>(packed + P.bias[i]));
-        count_launch();
-        if (with_backward) {
-            rc = conv::pack_weights(theta + P.theta_w[i], l.cin, l.cout, 1, round16(l.cout),
-                                    i == E0A ? round16(l.cin) : l.cin,
-                                    reinterpret_cast<__nv_bfloat16 *>(packed + P.bwd[i]), stream);
-            if (rc != SPP_OK) return rc;
-        }
+        table.it[table.count++] = conv::PackItem{
+            theta + P.theta_w[i], operand(P.fwd[i]), theta + P.theta_b[i],
+            reinterpret_cast<float *>(packed + P.bias[i]), l.cin, l.cout, 0, round16(l.cin),
+            fwd_n(net, i), 0};
+        if (with_backward)
+            table.it[table.count++] = conv::PackItem{
+                theta + P.theta_w[i], operand(P.bwd[i]), nullptr, nullptr, l.cin, l.cout, 1,
+                round16(l.cout), i == E0A ? round16(l.cin) : l.cin, 0};
     }
-    return launch_status();
+    return conv::pack_weights(table, stream);
 }
 
 int assemble(int B, const float *const *albedo, const float *const *normal,
