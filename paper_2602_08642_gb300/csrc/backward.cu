@@ -406,22 +406,34 @@ tonemap_backward_kernel(const float *__restrict__ hdr, long long N, ToneArgs tm,
 
 // floats between the losses of a batch's images
 constexpr int kScalarStride = 4;
+// elements of a loss per thread: a block sum and one atomic per 2048 elements
+// (per 256, the atomics on the one sum and the block reductions made the loss of
+// 8 x 256 x 256 pixels take 15 us)
+constexpr int kLossItems = 8;
+
+inline unsigned loss_blocks(int64_t n) {
+    return static_cast<unsigned>((n + 256 * kLossItems - 1) / (256 * kLossItems));
+}
 
 // Mean absolute error and its gradient sign(ldr - ref) / n.
 __global__ void __launch_bounds__(256)
 l1_loss_kernel(const float *__restrict__ a, const float *__restrict__ b, long long n,
                float *__restrict__ loss, float *__restrict__ grad) {
-    const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const long long i0 = static_cast<long long>(blockIdx.x) * (256 * kLossItems) + threadIdx.x;
     // image blockIdx.y of a batch
     a += blockIdx.y * n;
     b += blockIdx.y * n;
     if (grad) grad += blockIdx.y * n;
     loss += blockIdx.y * kScalarStride;
     float v = 0.0f;
-    if (i < n) {
+    const float unit = 1.0f / static_cast<float>(n);
+#pragma unroll
+    for (int k = 0; k < kLossItems; ++k) {
+        const long long i = i0 + 256 * k;
+        if (i >= n) continue;
         const float d = a[i] - b[i];
-        v = fabsf(d);
-        if (grad) grad[i] = (d > 0.0f ? 1.0f : (d < 0.0f ? -1.0f : 0.0f)) / static_cast<float>(n);
+        v += fabsf(d);
+        if (grad) grad[i] = d > 0.0f ? unit : (d < 0.0f ? -unit : 0.0f);
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
@@ -442,7 +454,7 @@ __global__ void combined_loss_kernel(const float *__restrict__ I, const float *_
                                      const float *__restrict__ P, const float *__restrict__ Q,
                                      long long n, float w, float ws,
                                      float *__restrict__ loss, float *__restrict__ grad) {
-    const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const long long i0 = static_cast<long long>(blockIdx.x) * (256 * kLossItems) + threadIdx.x;
     // image blockIdx.y of a batch
     I += blockIdx.y * n;
     R += blockIdx.y * n;
@@ -451,12 +463,15 @@ __global__ void combined_loss_kernel(const float *__restrict__ I, const float *_
     if (grad) grad += blockIdx.y * n;
     loss += blockIdx.y * kScalarStride;
     float v = 0.0f;
-    if (i < n) {
+#pragma unroll
+    for (int q = 0; q < kLossItems; ++q) {
+        const long long i = i0 + 256 * q;
+        if (i >= n) continue;
         const float ds = I[i] - R[i];
         const float dt = (I[i] - P[i]) - (R[i] - Q[i]);
         const float s = ws * fabsf(ds), t = w * fabsf(dt);
         const bool temporal = t > s;
-        v = temporal ? t : s;
+        v += temporal ? t : s;
         if (grad) {
             const float sg = temporal ? (dt > 0.0f ? w : (dt < 0.0f ? -w : 0.0f))
                                       : (ds > 0.0f ? ws : (ds < 0.0f ? -ws : 0.0f));
@@ -700,7 +715,8 @@ density_reduce_kernel(const float *__restrict__ d, const float *__restrict__ g, 
 }
 
 __global__ void __launch_bounds__(256)
-density_sum_kernel(const double *__restrict__ partial, int blocks, double *__restrict__ sums) {
+density_sum_kernel(const double *__restrict__ partial, int blocks, double K,
+                   double *__restrict__ sums) {
     partial += blockIdx.y * kDensityWsDoubles;
     sums += blockIdx.y * kDensityWsDoubles;
     double a = 0.0, b = 0.0;
@@ -725,15 +741,16 @@ density_sum_kernel(const double *__restrict__ partial, int blocks, double *__res
             ta += pa[w];
             tb += pb[w];
         }
-        sums[0] = ta;
-        sums[1] = tb;
+        sums[0] = K / ta;
+        sums[1] = tb / ta;
     }
 }
 
-// Pass 2 (Sec. 3): dLoss/dz_j = (1 - phi) B N pi_j (g_j - sum_i pi_i g_i).
+// Pass 2 (Sec. 3): dLoss/dz_j = (1 - phi) B N pi_j (g_j - sum_i pi_i g_i), the
+// divisions by the sum done once (per pixel they kept the FP64 pipe busy).
 __global__ void __launch_bounds__(256)
 density_grad_kernel(const float *__restrict__ d, const float *__restrict__ g, long long N,
-                    const double *__restrict__ sums, double K, float *__restrict__ gz,
+                    const double *__restrict__ sums, float *__restrict__ gz,
                     long long gz_stride) {
     const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= N) return;
@@ -742,10 +759,9 @@ density_grad_kernel(const float *__restrict__ d, const float *__restrict__ g, lo
     g += blockIdx.y * N;
     sums += blockIdx.y * kDensityWsDoubles;
     gz += blockIdx.y * gz_stride;
-    const double S = sums[0];
-    const double dot = sums[1] / S;
-    const double pi = static_cast<double>(d[i]) / S;
-    gz[i] = static_cast<float>(K * pi * (static_cast<double>(g[i]) - dot));
+    const double scale = sums[0], dot = sums[1];
+    gz[i] = static_cast<float>(scale * static_cast<double>(d[i]) *
+                               (static_cast<double>(g[i]) - dot));
 }
 
 ToneArgs tone_args_bwd(const spp_tonemap *tm) {
@@ -880,7 +896,7 @@ int spp_l1_loss(const float *ldr, const float *ref, int64_t n, float *loss, floa
         return SPP_ERR_ALIGN;
     if (cudaMemsetAsync(loss, 0, sizeof(float), stream) != cudaSuccess) return SPP_ERR_CUDA;
     if (n == 0) return SPP_OK;
-    l1_loss_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(
+    l1_loss_kernel<<<loss_blocks(n), 256, 0, stream>>>(
         ldr, ref, static_cast<long long>(n), loss, grad_ldr);
     count_launch();
     return launch_status();
@@ -896,7 +912,7 @@ int spp_l1_loss_batch(int B, const float *ldr, const float *ref, int64_t n, floa
     if (cudaMemsetAsync(loss, 0, sizeof(float) * kScalarStride * B, stream) != cudaSuccess)
         return SPP_ERR_CUDA;
     if (n == 0) return SPP_OK;
-    l1_loss_kernel<<<dim3(static_cast<unsigned>((n + 255) / 256), B), 256, 0, stream>>>(
+    l1_loss_kernel<<<dim3(loss_blocks(n), B), 256, 0, stream>>>(
         ldr, ref, static_cast<long long>(n), loss, grad_ldr);
     count_launch();
     return launch_status();
@@ -912,7 +928,7 @@ int spp_combined_loss(const float *ldr, const float *ref, const float *prev_warp
         return SPP_ERR_ALIGN;
     if (cudaMemsetAsync(loss, 0, sizeof(float), stream) != cudaSuccess) return SPP_ERR_CUDA;
     if (n == 0) return SPP_OK;
-    combined_loss_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(
+    combined_loss_kernel<<<loss_blocks(n), 256, 0, stream>>>(
         ldr, ref, prev_warped, ref_prev_warped, static_cast<long long>(n), temporal_weight,
         spatial_weight, loss, grad_ldr);
     count_launch();
@@ -933,7 +949,7 @@ int spp_combined_loss_batch(int B, const float *ldr, const float *ref, const flo
     if (cudaMemsetAsync(loss, 0, sizeof(float) * kScalarStride * B, stream) != cudaSuccess)
         return SPP_ERR_CUDA;
     if (n == 0) return SPP_OK;
-    combined_loss_kernel<<<dim3(static_cast<unsigned>((n + 255) / 256), B), 256, 0, stream>>>(
+    combined_loss_kernel<<<dim3(loss_blocks(n), B), 256, 0, stream>>>(
         ldr, ref, prev_warped, ref_prev_warped, static_cast<long long>(n), temporal_weight,
         spatial_weight, loss, grad_ldr);
     count_launch();
@@ -1130,15 +1146,16 @@ int spp_density_backward_batch(int B, const float *d, int64_t N, double budget,
     double *sums = static_cast<double *>(ws);
     double *partial = sums + 32;
     long long blocks = (N + 255) / 256;
-    long long rblocks = static_cast<long long>(sm_count()) * 8;
-    if (rblocks > blocks) rblocks = blocks;
+    // 16 pixels per thread: with fewer, the block reductions (FP64 adds) are
+    // most of the work
+    long long rblocks = (blocks + 15) / 16;
     if (rblocks > kDensityMaxBlocks) rblocks = kDensityMaxBlocks;
     density_reduce_kernel<<<dim3(static_cast<unsigned>(rblocks), B), 256, 0, stream>>>(d, grad_s, N,
                                                                                     partial);
-    density_sum_kernel<<<dim3(1, B), 256, 0, stream>>>(partial, static_cast<int>(rblocks), sums);
     const double K = (1.0 - uniform_fraction) * budget * static_cast<double>(N);
+    density_sum_kernel<<<dim3(1, B), 256, 0, stream>>>(partial, static_cast<int>(rblocks), K, sums);
     density_grad_kernel<<<dim3(static_cast<unsigned>(blocks), B), 256, 0, stream>>>(
-        d, grad_s, N, sums, K, grad_z, grad_z_stride);
+        d, grad_s, N, sums, grad_z, grad_z_stride);
     count_launch(3);
     return launch_status();
 }

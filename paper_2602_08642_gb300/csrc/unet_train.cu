@@ -77,24 +77,23 @@ GradLayout grad_layout(int net, int B, int W, int H) {
 
 // out[p][c] = (act[p][c] > 0) * (A[p][a_off + c] + sum over the 2x2 fine
 // pixels of F[.][f_off + c] + Cq[p/2][c] / 4), each term optional; 8
-// channels per thread.
-__global__ void junction_kernel(int B, int H, int W, int C, const __nv_bfloat16 *__restrict__ act,
-                                const __nv_bfloat16 *__restrict__ A, int a_c, int a_off,
-                                const __nv_bfloat16 *__restrict__ F, int f_c, int f_off,
-                                const __nv_bfloat16 *__restrict__ Cq, int c_c,
-                                __nv_bfloat16 *__restrict__ out) {
+// channels per thread, one image row per blockIdx.y (no divisions: with a flat
+// 64-bit index they took half of the kernel's time).
+__global__ void __launch_bounds__(256)
+junction_kernel(int rows, int W, int log2_c8, const __nv_bfloat16 *__restrict__ act,
+                const __nv_bfloat16 *__restrict__ A, int a_c, int a_off,
+                const __nv_bfloat16 *__restrict__ F, int f_c, int f_off,
+                const __nv_bfloat16 *__restrict__ Cq, int c_c, __nv_bfloat16 *__restrict__ out) {
     using conv::ldg16;
     using conv::pack_bf16x2;
     using conv::unpack_bf16x2;
-    const int c8 = C / 8;
-    const int64_t total = static_cast<int64_t>(B) * H * W * c8;
-    for (int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; idx < total;
-         idx += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int c = static_cast<int>(idx % c8) * 8;
-        const int64_t p = idx / c8;
-        const int x = static_cast<int>(p % W);
-        const int y = static_cast<int>((p / W) % H);
-        const int b = static_cast<int>(p / (static_cast<int64_t>(W) * H));
+    pdl_wait();
+    pdl_trigger();
+    const int idx = blockIdx.x * 256 + threadIdx.x;
+    const int x = idx >> log2_c8, c = (idx & ((1 << log2_c8) - 1)) * 8, C = 8 << log2_c8;
+    if (x >= W) return;
+    for (int row = blockIdx.y; row < rows; row += gridDim.y) {  // row = b H + y, H even
+        const int64_t p = static_cast<int64_t>(row) * W + x;
         float v[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] = 0.f;
@@ -110,14 +109,14 @@ __global__ void junction_kernel(int B, int H, int W, int C, const __nv_bfloat16 
         if (A) add(ldg16(A + p * a_c + a_off + c), 1.f);
         if (F) {
             const int Wf = 2 * W;
-            const int64_t f0 = (static_cast<int64_t>(b) * 2 * H + 2 * y) * Wf + 2 * x;
+            const int64_t f0 = static_cast<int64_t>(row) * 2 * Wf + 2 * x;
             add(ldg16(F + f0 * f_c + f_off + c), 1.f);
             add(ldg16(F + (f0 + 1) * f_c + f_off + c), 1.f);
             add(ldg16(F + (f0 + Wf) * f_c + f_off + c), 1.f);
             add(ldg16(F + (f0 + Wf + 1) * f_c + f_off + c), 1.f);
         }
         if (Cq) {
-            const int64_t q = (static_cast<int64_t>(b) * (H / 2) + y / 2) * (W / 2) + x / 2;
+            const int64_t q = static_cast<int64_t>(row / 2) * (W / 2) + x / 2;
             add(ldg16(Cq + q * c_c + c), 0.25f);
         }
         const uint4 m = ldg16(act + p * C + c);
@@ -211,11 +210,15 @@ upsample_kernel(const __nv_bfloat16 *__restrict__ src, int H, int W, int C, int6
 int launch_junction(int B, int H, int W, int C, const __nv_bfloat16 *act, const __nv_bfloat16 *A,
                     int a_c, int a_off, const __nv_bfloat16 *F, int f_c, int f_off,
                     const __nv_bfloat16 *Cq, int c_c, __nv_bfloat16 *out, cudaStream_t stream) {
-    const int64_t total = static_cast<int64_t>(B) * H * W * (C / 8);
-    if (total == 0) return SPP_OK;
-    const int grid = static_cast<int>(std::min<int64_t>((total + 255) / 256, 8 * sm_count()));
-    junction_kernel<<<grid, 256, 0, stream>>>(B, H, W, C, act, A, a_c, a_off, F, f_c, f_off, Cq,
-                                              c_c, out);
+    const int64_t rows = static_cast<int64_t>(B) * H;
+    if (rows * W == 0) return SPP_OK;
+    if (rows > 0x7fffffff) return SPP_ERR_ARG;
+    int log2_c8 = 0;  // C is 32, 64 or 128
+    while ((8 << log2_c8) < C) ++log2_c8;
+    const dim3 grid(static_cast<unsigned>((static_cast<int64_t>(W) * (C / 8) + 255) / 256),
+                    static_cast<unsigned>(std::min<int64_t>(rows, 65535)));
+    launch_dependent(junction_kernel, grid, dim3(256), 0, stream, static_cast<int>(rows), W,
+                     log2_c8, act, A, a_c, a_off, F, f_c, f_off, Cq, c_c, out);
     count_launch();
     return launch_status();
 }
