@@ -16,9 +16,9 @@
 //              producers: per K chunk of 16 input channels they stage the
 //              (TR+2) x 130 pixel halo of the tile in shared memory as K-major
 //              rows of 32 bytes per pixel in the 32-byte swizzle ([row][pixel]
-//              [16 ch], a_off), with zero padding, fused 2x2 pooling, fused
-//              upsample + concat or FP32 -> BF16 conversion on the way (a TMA
-//              box writes the plain NHWC case directly); one elected thread
+//              [16 ch], a_off), with zero padding and the fused upsample +
+//              concat on the way (a TMA box writes the plain NHWC case
+//              directly); one elected thread
 //              bulk-copies the pre-packed weights of the chunk;
 //   warp 8     lane 0 issues the MMAs: for each row r and tap (dy, dx) the A
 //              operand is the halo window starting at row r+dy, pixel dx
@@ -83,16 +83,16 @@ struct Cfg {
     static constexpr int kZeroBytes = kStack ? 2 * kZeroRows * 16 : 0;
     static constexpr int kWOff = kZeroOff + kZeroBytes;          // resident weights
     static constexpr int kStagesOff = (kWOff + kWRegion + 255) / 256 * 256;
-    // BF16 NHWC outputs leave through a per-warp staging row buffer, so that
-    // each warp store writes contiguous 512-byte runs ([32 px][kCBs ch] with
-    // a 16-byte pad per pixel: conflict-free 16-byte shared accesses)
+    // BF16 NHWC outputs leave through TMA tensor stores: a warp stages 32 pixels
+    // x kCBs channels in one of its two slots, in the swizzle of that row length
+    // (64 or 32 bytes; 16-byte shared stores without bank conflicts)
     static constexpr int kCBs = N < 32 ? N : 32;
-    static constexpr int kStageRow = 2 * kCBs + 16;
+    static constexpr int kSlot = 32 * 2 * kCBs;
     // eight epilogue warps (two per TMEM sub-partition, each taking half of
     // a tile's rows) when the layer's input comes by TMA and N <= 64, else four
     static constexpr int kEpiWarps = N <= 64 ? 8 : 4;
-    static constexpr int kStoreBytes = kEpiWarps * 32 * kStageRow;
-    // the FP32 planar staging buffers and the BF16 staging rows share one
+    static constexpr int kStoreBytes = kEpiWarps * 2 * kSlot;
+    // the FP32 planar staging buffers and the BF16 slots share one
     // region (a launch uses one of the two epilogues)
     static constexpr int kOutBytes = kEpiBytes > kStoreBytes ? kEpiBytes : kStoreBytes;
     static constexpr int kNS0 = (kSmemBudget - kStagesOff - kOutBytes) / kStage;
@@ -112,18 +112,19 @@ struct Cfg {
     static_assert(2 * kAccCols <= 512, "accumulators exceed TMEM");
     // FP32 planar outputs leave through two 8 KB staging buffers ([16 ch][128 px])
     // and TMA tensor stores (resident-weight variants; the heads are)
-    static constexpr int kEpiOff = (kStagesOff + kNS * kStage + 127) / 128 * 128;
+    static constexpr int kEpiOff = (kStagesOff + kNS * kStage + 511) / 512 * 512;
     static constexpr int kStoreOff = kEpiOff;
-    static constexpr int kSmem = kEpiOff + kOutBytes + 256;  // + alignment slack
+    static constexpr int kSmem = kEpiOff + kOutBytes + 512;  // + alignment slack
     // Upsampling layers (tma_in == 3): the coarse rows under a tile's halo,
     // one TMA box of 16 channels, in two buffers after the other areas (when
     // they fit): [buffer 2][kUpRows][kUpW][16 ch], not swizzled
     static constexpr int kUpRows = TR / 2 + 2;
     static constexpr int kUpBox = kUpRows * kUpW * 32;         // bytes of one box
     static constexpr int kUpG = (kUpBox + 127) / 128 * 128;     // its 128-byte aligned slot
-    static constexpr int kUpOff = (kStoreOff + kStoreBytes + 127) / 128 * 128;
-    // (upsampling layers have BF16 outputs: the buffers may overlap the FP32 area)
-    static constexpr int kSmemUp0 = kUpOff + 2 * kUpG + 256;
+    // (upsampling layers have BF16 outputs from four epilogue warps: the buffers
+    // may overlap the rest of the staging area)
+    static constexpr int kUpOff = (kStoreOff + 4 * 2 * kSlot + 127) / 128 * 128;
+    static constexpr int kSmemUp0 = kUpOff + 2 * kUpG + 512;
     static constexpr int kSmemUp = kSmemUp0 > kSmem ? kSmemUp0 : kSmem;
     static constexpr bool kUpFits = kSmemUp <= kSmemLimit;
     static_assert(kSmem <= kSmemLimit, "shared memory over the per-CTA limit");
@@ -177,6 +178,41 @@ __device__ __forceinline__ void tma_store_planes(const CUtensorMap *map, const v
         : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
+// TMA tensor store of 32 pixels x kCBs channels of BF16 NHWC from a warp's
+// staging slot at (c, x, y, b), clipped at the image's edges.
+__device__ __forceinline__ void tma_store_nhwc(const CUtensorMap *map, const void *src, int c, int x,
+                                               int y, int b) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(
+            reinterpret_cast<uint64_t>(map)),
+        "r"(tc::smem_u32(src)), "r"(c), "r"(x), "r"(y), "r"(b)
+        : "memory");
+}
+__device__ __forceinline__ void tma_store_commit() {
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+// Two FP32 additions in one instruction (each rounded to nearest even).
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 x, y, z;\n\t"
+        "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+        "add.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+// bf16x2 maximum with 0 of each half (NaN gives 0, as fmaxf(x, 0) does)
+__device__ __forceinline__ uint32_t relu_bf16x2(uint32_t u) {
+    uint32_t d;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(u), "r"(0u));
+    return d;
+}
+// the BF16 pair u where the halves of m are positive, else 0
+__device__ __forceinline__ uint32_t mask_bf16x2(uint32_t u, uint32_t m) {
+    uint32_t on;
+    asm("set.gt.u32.bf16x2 %0, %1, %2;" : "=r"(on) : "r"(m), "r"(0u));
+    return u & on;
+}
 // the stores committed before the last `pending` have finished reading shared memory
 template <int P>
 __device__ __forceinline__ void tma_store_wait_read() {
@@ -191,10 +227,12 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
                                                              const __grid_constant__ CUtensorMap omap,
                                                              const __grid_constant__ CUtensorMap imap,
                                                              const __grid_constant__ CUtensorMap umap) {
+    // omap: the output (FP32 planes or BF16 NHWC), imap: the NHWC input, umap: the
+    // coarse source of an upsampling layer
     using C = Cfg<N, RES>;
     constexpr int TR = C::TR, NS = C::kNS;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    unsigned char *base = smem_raw + ((256u - (tc::smem_u32(smem_raw) & 255u)) & 255u);
+    unsigned char *base = smem_raw + ((512u - (tc::smem_u32(smem_raw) & 511u)) & 511u);
     Bars &bars = *reinterpret_cast<Bars *>(base);
     unsigned char *wres = base + C::kWOff;              // resident weights (RES)
     unsigned char *stages = base + C::kStagesOff;
@@ -261,15 +299,6 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
         const int ptid = ep8 ? tid - 288 : warp == 9 ? tid - 160 : tid - 128;
         const int nprod = up5 ? 160 : 128;  // threads sharing the expansion tasks
         constexpr int kTasks = 2 * (TR + 2) * kPitch;  // 16-byte chunks per stage
-        constexpr int kPer = (kTasks + 127) / 128;
-        // this thread's tasks (the same in every stage): row << 10 | px << 1 | kg
-        int tinfo[kPer];
-#pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-            const int j = u * nprod + ptid;
-            tinfo[u] = j < kTasks ? (((j >> 1) / kPitch) << 10) | (((j >> 1) % kPitch) << 1) | (j & 1)
-                                  : -1;
-        }
         // upsampling layers: this thread's coarse pieces (the same in every
         // chunk): coarse row << 10 | coarse column << 1 | 8-channel half
         constexpr int kUpTasks = C::kUpRows * kUpW * 2;
@@ -284,12 +313,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
         uint32_t it = 0;
         uint32_t issued = 0;  // weight copies issued (by ptid 0)
         bool ok = true;
-        // Sources that need no arithmetic go through cp.async (zero-fill for
-        // the padding); a stage is published NS-1 stages later, so that up to
-        // NS-1 stages of copies are in flight per thread.  The other modes
-        // (FP32 planar gradients of the heads, pooling on load) stage through
-        // registers and publish at once.
-        const bool async_src = a.src_mode == kSrcNHWC || a.src_mode == kSrcConcatUp;
+        // Without TMA the halo goes through cp.async (zero-fill for the
+        // padding); a stage is published kLag stages later, so that up to kLag
+        // stages of copies are in flight per thread.
         constexpr uint32_t kLag = C::kLag;
         uint32_t published = 0;
         // arrival for a cp.async stage whose copies have landed (TMA stages of
@@ -438,12 +464,11 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
                         publish_lagged(published);
                         ++published;
                     }
-                } else if (async_src) {
+                } else {
                     const uint32_t sbase = tc::smem_u32(As);
-#pragma unroll
-                    for (int u = 0; u < kPer; ++u) {
-                        if (tinfo[u] < 0) continue;
-                        const int row = tinfo[u] >> 10, px = (tinfo[u] >> 1) & 511, kg = tinfo[u] & 1;
+#pragma unroll 4
+                    for (int j = ptid; j < kTasks; j += nprod) {
+                        const int row = (j >> 1) / kPitch, px = (j >> 1) % kPitch, kg = j & 1;
                         const __nv_bfloat16 *src = chunk_address(a, b, y0 - 1 + row, x0 - 1 + px,
                                                                  c * 16 + kg * 8);
                         cp_async16(sbase + a_off(row, px, kg),
@@ -456,34 +481,6 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
                         publish_lagged(published);
                         ++published;
                     }
-                } else {
-                    constexpr int kUnroll = 4;
-#pragma unroll 1
-                    for (int j0 = 0; j0 < kTasks; j0 += 128 * kUnroll) {
-                        uint4 v[kUnroll];
-#pragma unroll
-                        for (int u = 0; u < kUnroll; ++u) {
-                            const int j = j0 + u * 128 + ptid;
-                            v[u] = make_uint4(0, 0, 0, 0);
-                            if (j < kTasks) {
-                                const int kg = j & 1, px = (j >> 1) % kPitch, row = (j >> 1) / kPitch;
-                                v[u] = load_chunk(a, b, y0 - 1 + row, x0 - 1 + px,
-                                                  c * 16 + kg * 8);
-                            }
-                        }
-#pragma unroll
-                        for (int u = 0; u < kUnroll; ++u) {
-                            const int j = j0 + u * 128 + ptid;
-                            if (j < kTasks) {
-                                const int kg = j & 1, px = (j >> 1) % kPitch, row = (j >> 1) / kPitch;
-                                *reinterpret_cast<uint4 *>(As + a_off(row, px, kg)) = v[u];
-                            }
-                        }
-                    }
-                    tc::fence_proxy_async();
-                    tc::mbar_arrive(&bars.full[s]);
-                    ++it;
-                    ++published;
                 }
             }
         }
@@ -611,50 +608,83 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
         const int row_lo = ep8 ? (warp >> 2) * (TR / 2) : 0;
         const int row_hi = ep8 ? row_lo + TR / 2 : TR;
         uint32_t tl = 0;
-        uint32_t eblk = 0;  // TMA-stored blocks (planar outputs)
+        uint32_t eblk = 0;  // TMA-stored blocks
         const uint32_t lane_base = static_cast<uint32_t>(sub * 32) << 16;
+        // BF16 NHWC blocks: 32 pixels x kCB channels, kW packed pairs per pixel
+        constexpr int kCB = C::kCBs, kW = kCB / 2;
+        unsigned char *slots = base + C::kStoreOff + warp * 2 * C::kSlot;
+        // this lane's pixel row in a slot, and its swizzle (bits 7.. of the address)
+        const uint32_t swz = kCB == 32 ? (lane >> 1) & 3 : (lane >> 2) & 1;
+        auto store_block = [&](const uint32_t (&w)[kW], int c, int x0, int y, int b) {
+            unsigned char *slot = slots + (eblk & 1) * C::kSlot;
+            if (lane == 0) tma_store_wait_read<1>();  // the slot's previous store
+            __syncwarp();
+            uint4 *row = reinterpret_cast<uint4 *>(slot + lane * 2 * kCB);
+#pragma unroll
+            for (int q = 0; q < kW / 4; ++q)
+                row[q ^ swz] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+            tc::fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) {
+                if (y < a.H && x0 < a.W) tma_store_nhwc(&omap, slot, c, x0, y, b);
+                tma_store_commit();
+            }
+            ++eblk;
+        };
+        // accumulators + bias as BF16 pairs
+        auto pack_bias = [&](const uint32_t *v, int j0, bool relu, uint32_t (&w)[kW]) {
+#pragma unroll
+            for (int e = 0; e < kCB; e += 4) {
+                const float4 bb = *reinterpret_cast<const float4 *>(sbias + j0 + e);
+                const float2 f0 = add2(make_float2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])),
+                                       make_float2(bb.x, bb.y));
+                const float2 f1 =
+                    add2(make_float2(__uint_as_float(v[e + 2]), __uint_as_float(v[e + 3])),
+                         make_float2(bb.z, bb.w));
+                w[e / 2] = pack_bf16x2(f0.x, f0.y);
+                w[e / 2 + 1] = pack_bf16x2(f1.x, f1.y);
+                if (relu) {
+                    w[e / 2] = relu_bf16x2(w[e / 2]);
+                    w[e / 2 + 1] = relu_bf16x2(w[e / 2 + 1]);
+                }
+            }
+        };
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++tl) {
             const int acc = tl & 1;
+            const int b = t / per_img, rr = t - b * per_img;
+            const int y0 = (rr / tiles_x) * TR, x = (rr % tiles_x) * kTileX + sub * 32 + lane;
+            // the layer below's activations (mask) of block k of the tile; each
+            // block's are requested one block ahead, the first before the wait
+            constexpr int kRowBlocks = N / kCB;
+            constexpr int kBlocks = TR * kRowBlocks;
+            uint4 mask[2][kW / 4];
+            auto load_mask = [&](int k, uint4 (&m)[kW / 4]) {
+                const int y = y0 + k / kRowBlocks, j0 = (k % kRowBlocks) * kCB;
+                const bool inside = x < a.W && y < a.H;
+                const size_t pix = (static_cast<size_t>(b) * a.H + y) * a.W + x;
+                const uint4 *src = reinterpret_cast<const uint4 *>(a.act + pix * N + j0);
+#pragma unroll
+                for (int q = 0; q < kW / 4; ++q)
+                    m[q] = inside ? __ldg(src + q) : make_uint4(0, 0, 0, 0);
+            };
+            if (a.epi_mode == kEpiMaskBF16) load_mask(row_lo * kRowBlocks, mask[0]);
             if (!tc::mbar_wait(&bars.accf[acc], (tl >> 1) & 1u, abort_flag)) {
                 fail();
                 break;
             }
             tc::tc_fence_after();
-            const int b = t / per_img, rr = t - b * per_img;
-            const int y0 = (rr / tiles_x) * TR, x = (rr % tiles_x) * kTileX + sub * 32 + lane;
             const uint32_t abase = tmem + lane_base + acc * C::kAccCols + C::kRowOff * N;
             // hands the accumulator back to the MMA warp
             auto release_acc = [&]() {
                 tc::tc_fence_before();
                 tc::mbar_arrive(&bars.acce[acc]);
             };
+            const int xw = x - lane;  // the warp's first pixel
             if (TR % 2 == 0 && a.pool_out) {
                 // ReLU rows in pairs, plus the 2x2 average of their BF16 values
                 // (lanes x and x^1 hold horizontal neighbours), up to 32 columns
-                // of both rows per TMEM round trip; each of the two rows and the
-                // pooled row leaves through the warp's staging row buffer as
-                // contiguous runs
-                constexpr int kCB = N < 32 ? N : 32;
-                constexpr int kW = kCB / 2;  // packed BF16 pairs per pixel and block
-                unsigned char *srow = base + C::kStoreOff + (warp * 32) * C::kStageRow;
-                const int xw = x - lane;     // the warp's first pixel
-                // stages kW words per lane (or per listed pixel) and writes the
-                // pixels [0, npx) of the staging rows as 16-byte chunks to dst
-                auto flush = [&](int npx, auto valid, auto address) {
-                    __syncwarp();
-                    constexpr int kChunks = kCB / 8;
-#pragma unroll
-                    for (int i = 0; i < kChunks; ++i) {
-                        const int pp = i * (32 / kChunks) + lane / kChunks;
-                        const int ch = lane % kChunks;
-                        if (pp < npx && valid(pp)) {
-                            const uint4 val = *reinterpret_cast<const uint4 *>(
-                                srow + pp * C::kStageRow + 16 * ch);
-                            *reinterpret_cast<uint4 *>(address(pp) + 8 * ch) = val;
-                        }
-                    }
-                    __syncwarp();
-                };
+                // of both rows per TMEM round trip.  Each lane of a pair averages
+                // half of the channels and stores them as one 32-byte sector.
 #pragma unroll 1
                 for (int r = row_lo; r < row_hi; r += 2) {
                     const int y = y0 + r;
@@ -669,58 +699,40 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
                                           *reinterpret_cast<uint32_t(*)[16]>(v1 + 16 * q));
                         }
                         tc::tmem_wait_ld();
-                        uint32_t w1[kW], wp[kW];
+                        uint32_t w0[kW], w1[kW];
+                        pack_bias(v0, j0, true, w0);
+                        pack_bias(v1, j0, true, w1);
+                        store_block(w0, j0, xw, y, b);
+                        store_block(w1, j0, xw, y + 1, b);
+                        const bool odd = lane & 1;
+                        uint32_t wp[kW / 2];
+                        auto sum2 = [](uint32_t p, uint32_t q) {  // p + q, as FP32 pairs
+                            return add2(make_float2(__uint_as_float(p << 16),
+                                                    __uint_as_float(p & 0xffff0000u)),
+                                        make_float2(__uint_as_float(q << 16),
+                                                    __uint_as_float(q & 0xffff0000u)));
+                        };
 #pragma unroll
-                        for (int e = 0; e < kCB; e += 2) {
-                            float f0[2], f1[2], sm[2];
-#pragma unroll
-                            for (int t = 0; t < 2; ++t) {
-                                const float bb = sbias[j0 + e + t];
-                                f0[t] = __bfloat162float(__float2bfloat16_rn(
-                                    fmaxf(__uint_as_float(v0[e + t]) + bb, 0.f)));
-                                f1[t] = __bfloat162float(__float2bfloat16_rn(
-                                    fmaxf(__uint_as_float(v1[e + t]) + bb, 0.f)));
-                                sm[t] = f0[t] + f1[t];
-                                sm[t] += __shfl_xor_sync(0xffffffffu, sm[t], 1);
-                            }
-                            v0[e / 2] = pack_bf16x2(f0[0], f0[1]);  // row r, packed in place
-                            w1[e / 2] = pack_bf16x2(f1[0], f1[1]);
-                            wp[e / 2] = pack_bf16x2(0.25f * sm[0], 0.25f * sm[1]);
+                        for (int k = 0; k < kW / 2; ++k) {
+                            const uint32_t mine0 = odd ? w0[k + kW / 2] : w0[k];
+                            const uint32_t mine1 = odd ? w1[k + kW / 2] : w1[k];
+                            const uint32_t other0 = __shfl_xor_sync(
+                                0xffffffffu, odd ? w0[k] : w0[k + kW / 2], 1);
+                            const uint32_t other1 = __shfl_xor_sync(
+                                0xffffffffu, odd ? w1[k] : w1[k + kW / 2], 1);
+                            const float2 s = add2(sum2(mine0, mine1), sum2(other0, other1));
+                            wp[k] = pack_bf16x2(0.25f * s.x, 0.25f * s.y);
                         }
-                        // row r
+                        if (x - (lane & 1) < a.W && y + 1 < a.H) {
+                            uint4 *o = reinterpret_cast<uint4 *>(
+                                a.pool_out +
+                                ((static_cast<size_t>(b) * (a.H >> 1) + (y >> 1)) * (a.W >> 1) +
+                                 (x >> 1)) * N + j0 + (odd ? kCB / 2 : 0));
 #pragma unroll
-                        for (int q = 0; q < kW / 4; ++q)
-                            reinterpret_cast<uint4 *>(srow + lane * C::kStageRow)[q] =
-                                make_uint4(v0[4 * q], v0[4 * q + 1], v0[4 * q + 2], v0[4 * q + 3]);
-                        flush(32, [&](int pp) { return xw + pp < a.W && y < a.H; },
-                              [&](int pp) {
-                                  return a.out +
-                                         ((static_cast<size_t>(b) * a.H + y) * a.W + xw + pp) * N + j0;
-                              });
-                        // row r + 1
-#pragma unroll
-                        for (int q = 0; q < kW / 4; ++q)
-                            reinterpret_cast<uint4 *>(srow + lane * C::kStageRow)[q] =
-                                make_uint4(w1[4 * q], w1[4 * q + 1], w1[4 * q + 2], w1[4 * q + 3]);
-                        flush(32, [&](int pp) { return xw + pp < a.W && y + 1 < a.H; },
-                              [&](int pp) {
-                                  return a.out + ((static_cast<size_t>(b) * a.H + y + 1) * a.W +
-                                                  xw + pp) * N + j0;
-                              });
-                        // the pooled row: pixel pair k (lanes 2k, 2k+1) at staging row k
-                        if (!(lane & 1)) {
-#pragma unroll
-                            for (int q = 0; q < kW / 4; ++q)
-                                reinterpret_cast<uint4 *>(srow + (lane >> 1) * C::kStageRow)[q] =
-                                    make_uint4(wp[4 * q], wp[4 * q + 1], wp[4 * q + 2], wp[4 * q + 3]);
+                            for (int q = 0; q < kW / 8; ++q)
+                                o[q] = make_uint4(wp[4 * q], wp[4 * q + 1], wp[4 * q + 2],
+                                                  wp[4 * q + 3]);
                         }
-                        flush(16, [&](int pp) { return xw + 2 * pp + 1 < a.W + 1 &&
-                                                       xw + 2 * pp < a.W && y + 1 < a.H; },
-                              [&](int pp) {
-                                  return a.pool_out +
-                                         ((static_cast<size_t>(b) * (a.H >> 1) + (y >> 1)) *
-                                              (a.W >> 1) + (xw >> 1) + pp) * N + j0;
-                              });
                     }
                 }
                 release_acc();
@@ -786,9 +798,6 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
             // next block's TMEM read is in flight while this one is stored
             // (tcgen05.wait::ld waits for every outstanding read, so each
             // wait covers exactly the one issued before the stores)
-            constexpr int kCB = N < 32 ? N : 32;
-            constexpr int kRowBlocks = N / kCB;
-            constexpr int kBlocks = TR * kRowBlocks;
             auto tmem_read = [&](int k, uint32_t (&vv)[kCB]) {
                 const int r = k / kRowBlocks, j0 = (k % kRowBlocks) * kCB;
 #pragma unroll
@@ -806,14 +815,15 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
 #pragma unroll
                 for (int kk = 0; kk < kCount; ++kk) {
                     const int kb = kb_lo + kk;
-                    if (kk + 1 < kCount) tmem_read(kb + 1, vbuf[(kk + 1) & 1]);
+                    if (kk + 1 < kCount) {
+                        tmem_read(kb + 1, vbuf[(kk + 1) & 1]);
+                        if (a.epi_mode == kEpiMaskBF16) load_mask(kb + 1, mask[(kk + 1) & 1]);
+                    }
                     const uint32_t (&v)[kCB] = vbuf[kk & 1];
                     const int r = kb / kRowBlocks, j0 = (kb % kRowBlocks) * kCB;
                     const int y = y0 + r;
-                    const bool inside = (x < a.W) && (y < a.H);
-                    const size_t pix = (static_cast<size_t>(b) * a.H + y) * a.W + x;
                     if (a.epi_mode == kEpiF32Planar) {
-                        if (inside) {
+                        if (x < a.W && y < a.H) {
                             const size_t plane = static_cast<size_t>(a.H) * a.W;
                             float *o = a.outf + static_cast<size_t>(b) * a.cout * plane +
                                        static_cast<size_t>(y) * a.W + x;
@@ -824,59 +834,22 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
                             }
                         }
                     } else {
-                        // BF16 values of this pixel's kCB channels into the warp's
-                        // staging row
-                        unsigned char *srow = base + C::kStoreOff + (warp * 32) * C::kStageRow;
+                        uint32_t w[kW];
+                        if (a.epi_mode == kEpiMaskBF16) {
 #pragma unroll
-                        for (int q = 0; q < kCB / 16; ++q) {
-                            const int j = j0 + 16 * q;
-                            float f[16];
+                            for (int q = 0; q < kW / 4; ++q) {
+                                const uint32_t *mu = &mask[kk & 1][q].x;
 #pragma unroll
-                            for (int e = 0; e < 16; ++e) f[e] = __uint_as_float(v[16 * q + e]);
-                            if (a.epi_mode == kEpiReluBF16 || a.epi_mode == kEpiBF16) {
-#pragma unroll
-                                for (int e = 0; e < 16; ++e) f[e] += sbias[j + e];
-                                if (a.epi_mode == kEpiReluBF16) {
-#pragma unroll
-                                    for (int e = 0; e < 16; ++e) f[e] = fmaxf(f[e], 0.f);
-                                }
-                            } else if (a.epi_mode == kEpiMaskBF16) {
-                                const uint4 *m = reinterpret_cast<const uint4 *>(a.act + pix * N + j);
-#pragma unroll
-                                for (int h = 0; h < 2; ++h) {
-                                    const uint4 qq = inside ? __ldg(m + h) : make_uint4(0, 0, 0, 0);
-                                    const uint32_t *u = &qq.x;
-#pragma unroll
-                                    for (int k = 0; k < 4; ++k) {
-                                        const float2 mv = unpack_bf16x2(u[k]);
-                                        f[8 * h + 2 * k] = mv.x > 0.f ? f[8 * h + 2 * k] : 0.f;
-                                        f[8 * h + 2 * k + 1] = mv.y > 0.f ? f[8 * h + 2 * k + 1] : 0.f;
-                                    }
-                                }
+                                for (int k = 0; k < 4; ++k)
+                                    w[4 * q + k] = mask_bf16x2(
+                                        pack_bf16x2(__uint_as_float(v[8 * q + 2 * k]),
+                                                    __uint_as_float(v[8 * q + 2 * k + 1])),
+                                        mu[k]);
                             }
-                            uint4 *d4 = reinterpret_cast<uint4 *>(srow + lane * C::kStageRow + 32 * q);
-                            d4[0] = make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]),
-                                               pack_bf16x2(f[4], f[5]), pack_bf16x2(f[6], f[7]));
-                            d4[1] = make_uint4(pack_bf16x2(f[8], f[9]), pack_bf16x2(f[10], f[11]),
-                                               pack_bf16x2(f[12], f[13]), pack_bf16x2(f[14], f[15]));
+                        } else {
+                            pack_bias(v, j0, a.epi_mode == kEpiReluBF16, w);
                         }
-                        __syncwarp();
-                        // the warp's 32 pixels x kCB channels as contiguous 16-byte
-                        // chunks: kCB / 8 chunks per pixel, one warp store per 32 chunks
-                        constexpr int kChunks = kCB / 8;
-                        const int xw = x - lane;  // the warp's first pixel
-#pragma unroll
-                        for (int i = 0; i < kChunks; ++i) {
-                            const int pp = i * (32 / kChunks) + lane / kChunks;
-                            const int ch = lane % kChunks;
-                            const uint4 val =
-                                *reinterpret_cast<const uint4 *>(srow + pp * C::kStageRow + 16 * ch);
-                            if (xw + pp < a.W && y < a.H) {
-                                const size_t q = (static_cast<size_t>(b) * a.H + y) * a.W + xw + pp;
-                                *reinterpret_cast<uint4 *>(a.out + q * N + j0 + 8 * ch) = val;
-                            }
-                        }
-                        __syncwarp();  // the staging row is rewritten by the next block
+                        store_block(w, j0, xw, y, b);
                     }
                     tc::tmem_wait_ld();
                 }
@@ -999,6 +972,23 @@ int launch_variant(const ConvArgs &a, cudaStream_t stream) {
                        CU_TENSOR_MAP_L2_PROMOTION_NONE,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
             b.tma_out = 1;
+    }
+    if (a.epi_mode != kEpiF32Planar) {
+        // BF16 NHWC [B][H][W][N] as (channel, x, y, image), box kCBs x 32 x 1 x 1
+        auto enc = tensor_map_encoder();
+        cuuint64_t dims[4] = {static_cast<cuuint64_t>(N), static_cast<cuuint64_t>(a.W),
+                              static_cast<cuuint64_t>(a.H), static_cast<cuuint64_t>(a.B)};
+        cuuint64_t strides[3] = {static_cast<cuuint64_t>(N) * 2,
+                                 static_cast<cuuint64_t>(a.W) * N * 2,
+                                 static_cast<cuuint64_t>(a.W) * a.H * N * 2};
+        cuuint32_t box[4] = {static_cast<cuuint32_t>(C::kCBs), 32, 1, 1};
+        cuuint32_t estr[4] = {1, 1, 1, 1};
+        if (!enc || enc(&omap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, a.out, dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        C::kCBs == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+                        CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return SPP_ERR_CUDA;
     }
     CUtensorMap imap;
     memset(&imap, 0, sizeof(imap));

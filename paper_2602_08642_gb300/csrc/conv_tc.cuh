@@ -12,10 +12,8 @@ namespace conv {
 // Where the K operand (the input channels of the convolution) comes from.
 enum SrcMode : int {
     kSrcNHWC = 0,       // src0: BF16 [B][H][W][c0]
-    kSrcPool = 1,       // src0: BF16 [B][2H][2W][c0], 2x2 average taken on load
-    kSrcConcatUp = 2,   // channels [0,c0) from src0 [B][H][W][c0], then [c0,c0+c1)
+    kSrcConcatUp = 1,   // channels [0,c0) from src0 [B][H][W][c0], then [c0,c0+c1)
                         // from src1 [B][H/2][W/2][c1] upsampled (nearest)
-    kSrcPlanarF32 = 3,  // srcf: FP32 [B][cf][H][W]
 };
 
 // What the epilogue does with the FP32 accumulator of output channel n.
@@ -36,8 +34,6 @@ struct ConvArgs {
     int c0 = 0;
     const __nv_bfloat16 *src1 = nullptr;
     int c1 = 0;
-    const float *srcf = nullptr;
-    int cf = 0;
     const __nv_bfloat16 *wpack = nullptr;  // pack_weights() layout for (cin_pad, n)
     const float *bias = nullptr;           // [cout] or null (zero)
     int epi_mode = kEpiReluBF16;
