@@ -355,6 +355,30 @@ int spp_reconstruct_level_backward(const float *noisy, const float *logits, int 
                                    float *grad_logits, float *grad_noisy, float *grad_coarse,
                                    float *grad_warped, cudaStream_t stream);
 
+/* All levels of the gather pyramid in one call, with the coarse levels' outputs
+ * kept for the backward: spp_reconstruct_level from level L - 1 (2 <= L <= 16) to
+ * level 0, whose temporal term reads warped_prev (W_t L_{t-1}, may be NULL).
+ *   channels [L]   planes of each logits[l]
+ *   hats [L]       hats[1..L-1] receive the coarse levels' outputs ([0] unused) */
+int spp_reconstruct_pyramid(const float *const *layers, const float *const *logits,
+                            const int *channels, const float *warped_prev, const uint8_t *mask,
+                            int W, int H, int L, const spp_tonemap *tm, float *const *hats,
+                            float *out_hdr, float *out_ldr, int32_t *status, cudaStream_t stream);
+
+/* Backward of spp_reconstruct_pyramid given dLoss/d out_hdr and dLoss/d out_ldr
+ * (each may be NULL: zero).  Every gradient output is OVERWRITTEN.
+ *   grad_out [3][H][W]  scratch: the gradient that reaches level 0
+ *   grad_hats [L]       grad_hats[1..L-1], scratch like hats ([0] unused)
+ *   grad_warped         NULL without a temporal term */
+int spp_reconstruct_pyramid_backward(const float *const *layers, const float *const *logits,
+                                     const int *channels, const float *const *hats,
+                                     const float *warped_prev, const uint8_t *mask,
+                                     const float *hdr, int W, int H, int L, const spp_tonemap *tm,
+                                     const float *grad_hdr, const float *grad_ldr, float *grad_out,
+                                     float *const *grad_layers, float *const *grad_logits,
+                                     float *const *grad_hats, float *grad_warped,
+                                     cudaStream_t stream);
+
 /* W_t backward: grad_prev [3][H][W] += the bilinear weights of every pixel
  * applied to grad_warped (the transpose of spp_warp_previous). */
 int spp_warp_previous_backward(const float *mv, int W, int H, const float *grad_warped,

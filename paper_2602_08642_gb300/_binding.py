@@ -171,6 +171,11 @@ _SIGS = {
     "spp_tonemap_backward_batch": (_I, [_I, _P, _I, _I, ctypes.POINTER(spp_tonemap), _P, _P, _P]),
     "spp_reconstruct_level_backward_batch": (_I, [_I, _P, _P, _I, _P, _P, _P, _I, _I, _P, _P, _I,
                                                   _P, _P, _P, _P]),
+    "spp_reconstruct_pyramid": (_I, [_P, _P, _P, _P, _P, _I, _I, _I, ctypes.POINTER(spp_tonemap),
+                                     _P, _P, _P, _P, _P]),
+    "spp_reconstruct_pyramid_backward": (_I, [_P, _P, _P, _P, _P, _P, _P, _I, _I, _I,
+                                              ctypes.POINTER(spp_tonemap), _P, _P, _P, _P, _P, _P,
+                                              _P, _P]),
     "spp_pyramid_backward_batch": (_I, [_I, _P, _I, _I, _I, _P, _P]),
     "spp_splat_backward_batch": (_I, [_I, _P, _P, _P, _P, _P, _P, _P, _I64, _I, _I,
                                       ctypes.POINTER(spp_params), _P, _I, _P, _P, _P, _P]),
@@ -347,6 +352,35 @@ def spp_reconstruct_level_backward(noisy, logits, C, coarse, warped_prev, mask, 
         _dev(noisy, f), _dev(logits, f), C, _dev(coarse, f), _dev(warped_prev, f),
         _dev(mask, torch.uint8), Wl, Hl, _dev(grad_out, f), _dev(grad_logits, f),
         _dev(grad_noisy, f), _dev(grad_coarse, f), _dev(grad_warped, f), _stream(stream))
+
+
+def _ptr_list(ts):
+    """Device pointers of FP32 tensors as a C array (None entries pass NULL)."""
+    f = torch.float32
+    ps = [_dev(t, f) for t in ts]
+    return (ctypes.c_void_p * len(ps))(*[0 if p is None else p.value for p in ps])
+
+
+def spp_reconstruct_pyramid(layers, logits, warped_prev, mask, W, H, tm, hats, out_hdr, out_ldr,
+                            status=None, stream=None) -> int:
+    f, L = torch.float32, len(layers)
+    return lib.spp_reconstruct_pyramid(
+        _ptr_list(layers), _ptr_list(logits), (_I * L)(*[t.shape[0] for t in logits]),
+        _dev(warped_prev, f), _dev(mask, torch.uint8), W, H, L,
+        ctypes.byref(tm) if tm is not None else None, _ptr_list(hats), _dev(out_hdr, f),
+        _dev(out_ldr, f), _dev(status, torch.int32), _stream(stream))
+
+
+def spp_reconstruct_pyramid_backward(layers, logits, hats, warped_prev, mask, hdr, W, H, tm,
+                                     grad_hdr, grad_ldr, grad_out, grad_layers, grad_logits,
+                                     grad_hats, grad_warped, stream=None) -> int:
+    f, L = torch.float32, len(layers)
+    return lib.spp_reconstruct_pyramid_backward(
+        _ptr_list(layers), _ptr_list(logits), (_I * L)(*[t.shape[0] for t in logits]),
+        _ptr_list(hats), _dev(warped_prev, f), _dev(mask, torch.uint8), _dev(hdr, f), W, H, L,
+        ctypes.byref(tm) if tm is not None else None, _dev(grad_hdr, f), _dev(grad_ldr, f),
+        _dev(grad_out, f), _ptr_list(grad_layers), _ptr_list(grad_logits), _ptr_list(grad_hats),
+        _dev(grad_warped, f), _stream(stream))
 
 
 def spp_warp_previous_backward(mv, W, H, grad_warped, grad_prev, stream=None) -> int:

@@ -19,10 +19,6 @@ import torch
 from . import _binding as B
 
 
-def _z(t: torch.Tensor) -> torch.Tensor:
-    return torch.zeros_like(t)
-
-
 class Reconstruct(torch.autograd.Function):
     """Coarse-to-fine gather pyramid (Appendix A) with the tone map of Sec. 5.
 
@@ -34,18 +30,15 @@ class Reconstruct(torch.autograd.Function):
     def forward(ctx, L, tm, warped, mask, *tensors):
         layers, logits = list(tensors[:L]), list(tensors[L:2 * L])
         _, H, W = layers[0].shape
-        hats = [None] * L
-        for l in range(L - 1, 0, -1):
-            hats[l] = torch.empty_like(layers[l])
-            B.check(B.spp_reconstruct_level(layers[l], logits[l], logits[l].shape[0],
-                                            hats[l + 1] if l + 1 < L else None, None, None,
-                                            W >> l, H >> l, None, hats[l], None), "level")
+        hats = [None] + [torch.empty_like(x) for x in layers[1:]]
         hdr = torch.empty_like(layers[0])
         ldr = torch.empty_like(layers[0])
-        B.check(B.spp_reconstruct_level(layers[0], logits[0], logits[0].shape[0], hats[1], warped,
-                                        mask if warped is not None else None, W, H, tm, hdr, ldr),
-                "level 0")
+        B.check(B.spp_reconstruct_pyramid(layers, logits, warped,
+                                          mask if warped is not None else None, W, H, tm, hats,
+                                          hdr, ldr), "reconstruct")
         ctx.L, ctx.tm = L, tm
+        # an output that the loss does not use needs no gradient of zeros
+        ctx.set_materialize_grads(False)
         ctx.save_for_backward(warped if warped is not None else torch.empty(0, device=hdr.device),
                               mask if mask is not None else torch.empty(0, device=hdr.device,
                                                                         dtype=torch.uint8),
@@ -65,21 +58,14 @@ class Reconstruct(torch.autograd.Function):
         logits = list(saved[3 + L:3 + 2 * L])
         hats = [None] + list(saved[3 + 2 * L:])
         _, H, W = hdr.shape
-        g = torch.zeros_like(hdr) if g_hdr is None else g_hdr.contiguous().clone()
-        if g_ldr is not None:
-            B.check(B.spp_tonemap_backward(hdr, W, H, ctx.tm, g_ldr.contiguous(), g),
-                    "tonemap backward")
-        g_layers = [_z(x) for x in layers]
-        g_logits = [torch.empty_like(x) for x in logits]
-        g_warped = _z(hdr) if warped is not None else None
-        for l in range(L):
-            g_coarse = _z(hats[l + 1]) if l + 1 < L else None
-            B.check(B.spp_reconstruct_level_backward(
-                layers[l], logits[l], logits[l].shape[0], hats[l + 1] if l + 1 < L else None,
-                warped if l == 0 else None, mask if l == 0 else None, W >> l, H >> l, g,
-                g_logits[l], g_layers[l], g_coarse, g_warped if l == 0 else None),
-                "level backward")
-            g = g_coarse
+        new = lambda ts: [torch.empty_like(x) for x in ts]
+        g_layers, g_logits, g_hats = new(layers), new(logits), [None] + new(hats[1:])
+        g_warped = torch.empty_like(hdr) if warped is not None else None
+        B.check(B.spp_reconstruct_pyramid_backward(
+            layers, logits, hats, warped, mask, hdr, W, H, ctx.tm,
+            None if g_hdr is None else g_hdr.contiguous(),
+            None if g_ldr is None else g_ldr.contiguous(), torch.empty_like(hdr), g_layers,
+            g_logits, g_hats, g_warped), "reconstruct backward")
         return (None, None, g_warped, None, *g_layers, *g_logits)
 
 
@@ -108,7 +94,7 @@ class L1Loss(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, ldr, ref):
-        loss = torch.zeros(4, device=ldr.device)[:1]
+        loss = torch.empty(4, device=ldr.device)[:1]
         grad = torch.empty_like(ldr)
         B.check(B.spp_l1_loss(ldr, ref, ldr.numel(), loss, grad), "l1")
         ctx.save_for_backward(grad)

@@ -21,7 +21,9 @@ namespace {
 constexpr int kBX = 32, kBY = 8, kBH = 2;
 constexpr int kRX = kBX + 2 * kBH, kRY = kBY + 2 * kBH;  // consumer region 36 x 12
 constexpr int kRN = kRX * kRY;                           // 432 consumers
-constexpr int kHalo = kRN - kBX * kBY;                   // 176 of them outside the tile
+// a thread per consumer (with 256 threads the halo's 176 consumers, 54 dependent
+// loads each, were a second round)
+constexpr int kBwdThreads = (kRN + 31) / 32 * 32;
 constexpr int kFX = kBX / 2 + 1, kFY = kBY / 2 + 1;      // coarse cells the tile's taps read
 
 // Shared memory of the backward of one 32 x 8 tile: per consumer pixel of
@@ -60,25 +62,32 @@ __device__ __forceinline__ void tap_range(int q, int p, int n, int &lo, int &hi)
 // Backward of one reconstruction level in gather form: every output
 // gradient element has exactly one writer, which adds its consumers'
 // contributions in a fixed order, so the result does not depend on
-// scheduling.  A block owns a 32 x 8 tile: it computes the softmax weights
-// of the tile's pixels and of the 2-pixel halo around it (the consumers of
-// the tile's sources), dLoss/d logits of the tile's pixels, then for each
-// source pixel of the tile (and for each coarse cell under it) the sum of
-// w_k g over the consumers and taps that read it.
+// scheduling.  A block owns a 32 x 8 tile; a thread owns one of the 36 x 12
+// consumers of the tile's sources: it computes that pixel's softmax weights
+// and, inside the tile, dLoss/d logits; then the tile's threads sum for their
+// source pixel (and for each coarse cell under the tile) w_k g over the
+// consumers and taps that read it.
+//
+// Bound by its shared-memory accesses (about 560 per consumer), not by its bytes.
+// Two CTAs of 448 threads per SM (the weights of one tile take 109 KB) leave 72
+// registers, so the products q_k are formed twice (once for their mean, once for
+// the gradients) instead of being kept.  960 x 540, cold caches: level 0 with the
+// temporal term 144 -> 141 us, level 1 27 -> 21.5 us, level 2 14 -> 10.7 us
+// against 256 threads per tile and two rounds of loads.
 template <bool UP, bool TEMP>
-__global__ void __launch_bounds__(kBX *kBY)
+__global__ void __launch_bounds__(kBwdThreads, 2)
 recon_backward_kernel(const float *__restrict__ noisy, const float *__restrict__ logits, int C,
                       const float *__restrict__ coarse, const float *__restrict__ warped,
                       const uint8_t *__restrict__ mask, int Wl, int Hl,
                       const float *__restrict__ g, float *__restrict__ grad_logits,
                       float *__restrict__ grad_noisy, float *__restrict__ grad_coarse,
-                      float *__restrict__ grad_warped, int Cg, long long gl_stride) {
+                      float *__restrict__ grad_warped, int Cg, long long gl_stride,
+                      bool accumulate) {
     constexpr int kSpatial = 25 + (UP ? 4 : 0);
-    constexpr int kNK = kSpatial + (TEMP ? 25 : 0);
     extern __shared__ __align__(16) unsigned char bwd_smem_raw[];
     BwdSmem<UP, TEMP> &sm = *reinterpret_cast<BwdSmem<UP, TEMP> *>(bwd_smem_raw);
 
-    const int tid = threadIdx.y * kBX + threadIdx.x;
+    const int tid = threadIdx.x;
     const int bx0 = blockIdx.x * kBX, by0 = blockIdx.y * kBY;
     const long long Nl = static_cast<long long>(Wl) * Hl;
     const int Wc = Wl >> 1, Hc = Hl >> 1;
@@ -96,148 +105,137 @@ recon_backward_kernel(const float *__restrict__ noisy, const float *__restrict__
     if (TEMP) warped += blockIdx.z * 3 * Nl;
     if (TEMP && grad_warped) grad_warped += blockIdx.z * 3 * Nl;
 
+    // this thread's consumer: cell (rx, ry) of the region, pixel (px, py)
+    const int cell = min(tid, kRN - 1);
+    const int rx = tid % kRX, ry = tid / kRX;
+    const int px = bx0 + rx - kBH, py = by0 + ry - kBH;
+    const bool tile = rx >= kBH && rx < kBH + kBX && ry >= kBH && ry < kBH + kBY;
+    const bool in = tid < kRN && px >= 0 && px < Wl && py >= 0 && py < Hl;
+    const long long pix = in ? static_cast<long long>(py) * Wl + px : 0;
+
+    // spatial logits into registers, temporal ones straight into this thread's
+    // cells of shared memory (all of them in registers would spill)
+    float w[kSpatial];
+    bool use_t = false;
+    if (in) {
+        use_t = TEMP && !(mask && mask[pix]);
+        if (TEMP && use_t) {
+#pragma unroll
+            for (int k = 0; k < 25; ++k) copy_async4(&sm.wt[k][cell], logits + (29 + k) * Nl + pix);
+        }
+#pragma unroll
+        for (int k = 0; k < kSpatial; ++k) w[k] = __ldg(logits + k * Nl + pix);
+    }
     // tap values of the region (clamp-to-edge)
-    for (int idx = tid; idx < kRN; idx += kBX * kBY) {
-        const int rx = idx % kRX, ry = idx / kRX;
-        const int gx = clampi(bx0 + rx - kBH, 0, Wl - 1), gy = clampi(by0 + ry - kBH, 0, Hl - 1);
-        const long long q = static_cast<long long>(gy) * Wl + gx;
+    if (tid < kRN) {
+        const long long q = static_cast<long long>(clampi(py, 0, Hl - 1)) * Wl +
+                            clampi(px, 0, Wl - 1);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            sm.nz[c][idx] = __ldg(noisy + c * Nl + q);
-            if (TEMP) sm.wp[c][idx] = __ldg(warped + c * Nl + q);
+            sm.nz[c][cell] = __ldg(noisy + c * Nl + q);
+            if (TEMP) sm.wp[c][cell] = __ldg(warped + c * Nl + q);
+            sm.g[c][cell] = in ? __ldg(g + c * Nl + pix) : 0.0f;
         }
     }
-    if (UP)
-        for (int idx = tid; idx < kFX * kFY; idx += kBX * kBY) {
-            const int cx = min(cbx + idx % kFX, Wc - 1), cy = min(cby + idx / kFX, Hc - 1);
-            const long long q = static_cast<long long>(cy) * Wc + cx;
+    if (UP && tid < kFX * kFY) {
+        const int cx = min(cbx + tid % kFX, Wc - 1), cy = min(cby + tid / kFX, Hc - 1);
+        const long long q = static_cast<long long>(cy) * Wc + cx;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) sm.cv[c][idx] = __ldg(coarse + c * Nc + q);
+        for (int c = 0; c < 3; ++c) sm.cv[c][tid] = __ldg(coarse + c * Nc + q);
+    }
+    // the normalised weights of the consumer; a cell that is no pixel reads
+    // nothing and contributes nothing
+    if (TEMP) copy_async_wait();
+    if (in) {
+        float m = w[0];
+#pragma unroll
+        for (int k = 1; k < kSpatial; ++k) m = fmaxf(m, w[k]);
+        if (use_t) {
+#pragma unroll
+            for (int k = 0; k < 25; ++k) m = fmaxf(m, sm.wt[k][cell]);
         }
-
-    // the normalised weights and dLoss/d out of consumer (qx, qy) into its
-    // region cell; w receives them for the caller
-    auto consumer = [&](int qx, int qy, int cell, float (&w)[kNK], float (&gq)[3], bool &use_t) {
-        const bool in = qx >= 0 && qx < Wl && qy >= 0 && qy < Hl;
-        use_t = false;
-        if (!in) {  // not a pixel: reads nothing, contributes nothing
+        float wsum = 0.0f;
 #pragma unroll
-            for (int k = 0; k < kNK; ++k) w[k] = 0.0f;
-            gq[0] = gq[1] = gq[2] = 0.0f;
-        } else {
-            const long long pix = static_cast<long long>(qy) * Wl + qx;
-            use_t = TEMP && !(mask && mask[pix]);
-#pragma unroll
-            for (int k = 0; k < kSpatial; ++k) w[k] = __ldg(logits + k * Nl + pix);
-            if (TEMP) {
-#pragma unroll
-                for (int k = 0; k < 25; ++k)
-                    w[kSpatial + k] = use_t ? __ldg(logits + (29 + k) * Nl + pix) : 0.0f;
-            }
-            float m = w[0];
-#pragma unroll
-            for (int k = 1; k < kSpatial; ++k) m = fmaxf(m, w[k]);
-            if (use_t) {
-#pragma unroll
-                for (int k = kSpatial; k < kNK; ++k) m = fmaxf(m, w[k]);
-            }
-            float wsum = 0.0f;
-#pragma unroll
-            for (int k = 0; k < kNK; ++k) {
-                const bool on = k < kSpatial || use_t;
-                w[k] = on ? __expf(w[k] - m) : 0.0f;
-                wsum += w[k];
-            }
-            const float inv = 1.0f / wsum;
-#pragma unroll
-            for (int k = 0; k < kNK; ++k) w[k] *= inv;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) gq[c] = __ldg(g + c * Nl + pix);
+        for (int k = 0; k < kSpatial; ++k) {
+            w[k] = __expf(w[k] - m);
+            wsum += w[k];
         }
+        if (use_t) {
+#pragma unroll
+            for (int k = 0; k < 25; ++k) {
+                const float e = __expf(sm.wt[k][cell] - m);
+                sm.wt[k][cell] = e;
+                wsum += e;
+            }
+        }
+        const float inv = 1.0f / wsum;
+#pragma unroll
+        for (int k = 0; k < kSpatial; ++k) w[k] *= inv;
+        if (use_t) {
+#pragma unroll
+            for (int k = 0; k < 25; ++k) sm.wt[k][cell] *= inv;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < kSpatial; ++k) w[k] = 0.0f;
+    }
+    if (tid < kRN) {
 #pragma unroll
         for (int k = 0; k < 25; ++k) sm.wd[k][cell] = w[k];
         if (UP) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) sm.wu[k][cell] = w[25 + k];
         }
-        if (TEMP) {
+        if (TEMP && !use_t) {
 #pragma unroll
-            for (int k = 0; k < 25; ++k) sm.wt[k][cell] = w[kSpatial + k];
+            for (int k = 0; k < 25; ++k) sm.wt[k][cell] = 0.0f;
         }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) sm.g[c][cell] = gq[c];
-    };
+    }
     __syncthreads();
 
-    // the tile's own pixel: its weights, then dLoss/d logits
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int px = bx0 + tx, py = by0 + ty;
-    const bool inside = px < Wl && py < Hl;
-    {
-        float w[kNK], gq[3];
-        bool use_t;
-        const int cell = (ty + kBH) * kRX + tx + kBH;
-        consumer(px, py, cell, w, gq, use_t);
-        if (inside) {
-            const long long pix = static_cast<long long>(py) * Wl + px;
-            float q[kNK];
+    // dLoss/d logits of the tile: dLoss/dz_k = w_k (q_k - qbar), q_k = g . v_k
+    const bool inside = in && tile;
+    const float g0 = sm.g[0][cell], g1 = sm.g[1][cell], g2 = sm.g[2][cell];
+    const int o0 = cell - kBH * kRX - kBH;
+    auto up_cell = [&](int j, int i) {
+        return (min((py + j) >> 1, Hc - 1) - cby) * kFX + min((px + i) >> 1, Wc - 1) - cbx;
+    };
+    auto dot = [&](const auto &v, int o) { return g0 * v[0][o] + g1 * v[1][o] + g2 * v[2][o]; };
+    float qbar = 0.0f;
+    if (inside) {
 #pragma unroll
-            for (int j = 0; j < 5; ++j)
+        for (int k = 0; k < 25; ++k) qbar = fmaf(w[k], dot(sm.nz, o0 + k / 5 * kRX + k % 5), qbar);
+        if (UP) {
 #pragma unroll
-                for (int i = 0; i < 5; ++i) {
-                    const int o = (ty + j) * kRX + tx + i;
-                    q[j * 5 + i] =
-                        gq[0] * sm.nz[0][o] + gq[1] * sm.nz[1][o] + gq[2] * sm.nz[2][o];
-                    if (TEMP)
-                        q[kSpatial + j * 5 + i] =
-                            gq[0] * sm.wp[0][o] + gq[1] * sm.wp[1][o] + gq[2] * sm.wp[2][o];
-                }
-            if (UP) {
+            for (int k = 0; k < 4; ++k)
+                qbar = fmaf(w[25 + k], dot(sm.cv, up_cell(k / 2, k % 2)), qbar);
+        }
+        if (TEMP) {
 #pragma unroll
-                for (int j = 0; j < 2; ++j)
-#pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-                        const int cx = min((px + i) >> 1, Wc - 1) - cbx;
-                        const int cy = min((py + j) >> 1, Hc - 1) - cby;
-                        const int o = cy * kFX + cx;
-                        q[25 + 2 * j + i] =
-                            gq[0] * sm.cv[0][o] + gq[1] * sm.cv[1][o] + gq[2] * sm.cv[2][o];
-                    }
-            }
-            float qbar = 0.0f;
-#pragma unroll
-            for (int k = 0; k < kNK; ++k) qbar = fmaf(w[k], q[k], qbar);
-            // dLoss/dz_k = w_k (q_k - qbar); channels without a kernel get 0
-#pragma unroll
-            for (int k = 0; k < kSpatial; ++k) grad_logits[k * Nl + pix] = w[k] * (q[k] - qbar);
-            if (TEMP) {
-#pragma unroll
-                for (int k = 0; k < 25; ++k)
-                    grad_logits[(29 + k) * Nl + pix] =
-                        use_t ? w[kSpatial + k] * (q[kSpatial + k] - qbar) : 0.0f;
-            }
-            for (int k = TEMP ? 54 : kSpatial; k < Cg; ++k) grad_logits[k * Nl + pix] = 0.0f;
+            for (int k = 0; k < 25; ++k)
+                qbar = fmaf(sm.wt[k][cell], dot(sm.wp, o0 + k / 5 * kRX + k % 5), qbar);
         }
     }
-    // the halo's consumers (rows 0-1 and 10-11, then columns 0-1 and 34-35)
-    if (tid < kHalo) {
-        int rx, ry;
-        if (tid < 2 * kRX) {
-            rx = tid % kRX;
-            ry = tid / kRX;
-        } else if (tid < 4 * kRX) {
-            rx = (tid - 2 * kRX) % kRX;
-            ry = kRY - 2 + (tid - 2 * kRX) / kRX;
-        } else {
-            const int h = tid - 4 * kRX;
-            ry = kBH + h / 4;
-            rx = (h % 4) < 2 ? (h % 4) : kBX + (h % 4);
+    __syncthreads();  // or the compiler would keep the products, in local memory
+    if (inside) {
+        float *gl = grad_logits + pix;
+#pragma unroll
+        for (int k = 0; k < 25; ++k)
+            gl[k * Nl] = w[k] * (dot(sm.nz, o0 + k / 5 * kRX + k % 5) - qbar);
+        if (UP) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                gl[(25 + k) * Nl] = w[25 + k] * (dot(sm.cv, up_cell(k / 2, k % 2)) - qbar);
         }
-        float w[kNK], gq[3];
-        bool use_t;
-        consumer(bx0 + rx - kBH, by0 + ry - kBH, ry * kRX + rx, w, gq, use_t);
+        if (TEMP) {
+#pragma unroll
+            for (int k = 0; k < 25; ++k)
+                gl[(29 + k) * Nl] =
+                    use_t ? sm.wt[k][cell] * (dot(sm.wp, o0 + k / 5 * kRX + k % 5) - qbar) : 0.0f;
+        }
+        // channels without a kernel get 0
+        for (int k = TEMP ? 54 : kSpatial; k < Cg; ++k) gl[k * Nl] = 0.0f;
     }
-    __syncthreads();
 
     // sources of the tile: the sum of w_k g over the taps that read them
     if (inside && (grad_noisy || (TEMP && grad_warped))) {
@@ -250,15 +248,15 @@ recon_backward_kernel(const float *__restrict__ noisy, const float *__restrict__
             for (int dy = -2; dy <= 2; ++dy)
 #pragma unroll
                 for (int dx = -2; dx <= 2; ++dx) {
-                    const int cell = (ty + kBH + dy) * kRX + tx + kBH + dx;
+                    const int from = cell + dy * kRX + dx;
                     const int k = (2 - dy) * 5 + (2 - dx);
-                    const float wk = sm.wd[k][cell];
+                    const float wk = sm.wd[k][from];
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) an[c] = fmaf(wk, sm.g[c][cell], an[c]);
+                    for (int c = 0; c < 3; ++c) an[c] = fmaf(wk, sm.g[c][from], an[c]);
                     if (TEMP) {
-                        const float wt = sm.wt[k][cell];
+                        const float wt = sm.wt[k][from];
 #pragma unroll
-                        for (int c = 0; c < 3; ++c) aw[c] = fmaf(wt, sm.g[c][cell], aw[c]);
+                        for (int c = 0; c < 3; ++c) aw[c] = fmaf(wt, sm.g[c][from], aw[c]);
                     }
                 }
         } else {
@@ -272,27 +270,32 @@ recon_backward_kernel(const float *__restrict__ noisy, const float *__restrict__
                     if (qx < 0 || qx >= Wl) continue;
                     int ilo, ihi;
                     tap_range(qx, px, Wl, ilo, ihi);
-                    const int cell = (ty + kBH + dy) * kRX + tx + kBH + dx;
+                    const int from = cell + dy * kRX + dx;
                     for (int j = jlo; j <= jhi; ++j)
                         for (int i = ilo; i <= ihi; ++i) {
-                            const float wk = sm.wd[j * 5 + i][cell];
+                            const float wk = sm.wd[j * 5 + i][from];
 #pragma unroll
-                            for (int c = 0; c < 3; ++c) an[c] = fmaf(wk, sm.g[c][cell], an[c]);
+                            for (int c = 0; c < 3; ++c) an[c] = fmaf(wk, sm.g[c][from], an[c]);
                             if (TEMP) {
-                                const float wt = sm.wt[j * 5 + i][cell];
+                                const float wt = sm.wt[j * 5 + i][from];
 #pragma unroll
                                 for (int c = 0; c < 3; ++c)
-                                    aw[c] = fmaf(wt, sm.g[c][cell], aw[c]);
+                                    aw[c] = fmaf(wt, sm.g[c][from], aw[c]);
                             }
                         }
                 }
             }
         }
-        const long long pix = static_cast<long long>(py) * Wl + px;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            if (grad_noisy) grad_noisy[c * Nl + pix] += an[c];
-            if (TEMP && grad_warped) grad_warped[c * Nl + pix] += aw[c];
+            if (grad_noisy) {
+                float *o = grad_noisy + c * Nl + pix;
+                *o = accumulate ? *o + an[c] : an[c];
+            }
+            if (TEMP && grad_warped) {
+                float *o = grad_warped + c * Nl + pix;
+                *o = accumulate ? *o + aw[c] : aw[c];
+            }
         }
     }
     // coarse cells under the tile: the upsampling taps of the full-resolution
@@ -305,22 +308,25 @@ recon_backward_kernel(const float *__restrict__ noisy, const float *__restrict__
                 if (qy < 0 || qy >= Hl) continue;
                 for (int qx = 2 * cx - 1; qx <= 2 * cx + 1; ++qx) {
                     if (qx < 0 || qx >= Wl) continue;
-                    const int cell = (qy - by0 + kBH) * kRX + qx - bx0 + kBH;
+                    const int from = (qy - by0 + kBH) * kRX + qx - bx0 + kBH;
 #pragma unroll
                     for (int j = 0; j < 2; ++j)
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {
                             if (min((qx + i) >> 1, Wc - 1) != cx || min((qy + j) >> 1, Hc - 1) != cy)
                                 continue;
-                            const float wk = sm.wu[2 * j + i][cell];
+                            const float wk = sm.wu[2 * j + i][from];
 #pragma unroll
-                            for (int c = 0; c < 3; ++c) ac[c] = fmaf(wk, sm.g[c][cell], ac[c]);
+                            for (int c = 0; c < 3; ++c) ac[c] = fmaf(wk, sm.g[c][from], ac[c]);
                         }
                 }
             }
             const long long q = static_cast<long long>(cy) * Wc + cx;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) grad_coarse[c * Nc + q] += ac[c];
+            for (int c = 0; c < 3; ++c) {
+                float *o = grad_coarse + c * Nc + q;
+                *o = accumulate ? *o + ac[c] : ac[c];
+            }
         }
     }
 }
@@ -373,15 +379,17 @@ __device__ __forceinline__ float srgb_prime(float v) {
     return v <= 0.0031308f ? 12.92f : (1.055f / 2.4f) * powf(v, 1.0f / 2.4f - 1.0f);
 }
 
-// Sec. 5 backward: grad_hdr += d sRGB(tau(x)) / d hdr applied to grad_ldr.
+// Sec. 5 backward: gh = base + d sRGB(tau(x)) / d hdr applied to grad_ldr; base
+// NULL is 0, and may be gh itself (accumulation).
 __global__ void __launch_bounds__(256)
 tonemap_backward_kernel(const float *__restrict__ hdr, long long N, ToneArgs tm,
-                        const float *__restrict__ gl, float *__restrict__ gh) {
+                        const float *__restrict__ gl, const float *base, float *gh) {
     const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= N) return;
     // image blockIdx.y of a batch
     hdr += blockIdx.y * 3 * N;
     gl += blockIdx.y * 3 * N;
+    if (base) base += blockIdx.y * 3 * N;
     gh += blockIdx.y * 3 * N;
     float v[3], l[3];
 #pragma unroll
@@ -400,7 +408,8 @@ tonemap_backward_kernel(const float *__restrict__ hdr, long long N, ToneArgs tm,
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
         const float glog = tm.alpha * (tm.beta * gx[j] + (1.0f - tm.beta) * (1.0f / 3.0f) * gs);
-        if (v[j] >= 0x1p-24f) gh[j * N + i] += glog / v[j];
+        const float b = base ? base[j * N + i] : 0.0f;
+        gh[j * N + i] = v[j] >= 0x1p-24f ? b + glog / v[j] : b;
     }
 }
 
@@ -779,11 +788,11 @@ ToneArgs tone_args_bwd(const spp_tonemap *tm) {
 }
 
 template <bool UP, bool TEMP>
-int launch_recon_backward(dim3 grid, dim3 block, cudaStream_t stream, const float *noisy,
+int launch_recon_backward(dim3 grid, cudaStream_t stream, const float *noisy,
                           const float *logits, int C, const float *coarse, const float *warped,
                           const uint8_t *mask, int Wl, int Hl, const float *g, float *grad_logits,
                           float *grad_noisy, float *grad_coarse, float *grad_warped, int Cg,
-                          long long gl_stride) {
+                          long long gl_stride, bool accumulate) {
     constexpr int kSmem = static_cast<int>(sizeof(BwdSmem<UP, TEMP>));
     static int configured_dev = -1;
     int dev = 0;
@@ -794,10 +803,49 @@ int launch_recon_backward(dim3 grid, dim3 block, cudaStream_t stream, const floa
             return SPP_ERR_CUDA;
         configured_dev = dev;
     }
-    recon_backward_kernel<UP, TEMP><<<grid, block, kSmem, stream>>>(
+    recon_backward_kernel<UP, TEMP><<<grid, kBwdThreads, kSmem, stream>>>(
         noisy, logits, C, coarse, warped, mask, Wl, Hl, g, grad_logits, grad_noisy, grad_coarse,
-        grad_warped, Cg, gl_stride);
+        grad_warped, Cg, gl_stride, accumulate);
     return SPP_OK;
+}
+
+// accumulate: whether the gradients of the tap sources are added to what their
+// buffers hold or stored
+int level_backward(int B, const float *noisy, const float *logits, int C, const float *coarse,
+                   const float *warped_prev, const uint8_t *mask, int Wl, int Hl,
+                   const float *grad_out, float *grad_logits, int Cg, float *grad_noisy,
+                   float *grad_coarse, float *grad_warped, bool accumulate, cudaStream_t stream) {
+    if (B < 0 || B > 65535 || Wl < 0 || Hl < 0 || !noisy || !logits || !grad_out || !grad_logits)
+        return SPP_ERR_ARG;
+    if (warped_prev && !coarse) return SPP_ERR_ARG;
+    const int need = warped_prev ? 54 : 25 + (coarse ? 4 : 0);
+    if (C < need || Cg < need || Cg > C) return SPP_ERR_ARG;
+    if (coarse && ((Wl & 1) || (Hl & 1))) return SPP_ERR_SHAPE;
+    if (!aligned16(noisy) || !aligned16(logits) || !aligned16(grad_out) ||
+        !aligned16(grad_logits) || (coarse && !aligned16(coarse)) ||
+        (warped_prev && !aligned16(warped_prev)) || (mask && !aligned16(mask)) ||
+        (grad_noisy && !aligned16(grad_noisy)) || (grad_coarse && !aligned16(grad_coarse)) ||
+        (grad_warped && !aligned16(grad_warped)))
+        return SPP_ERR_ALIGN;
+    const long long n = static_cast<long long>(Wl) * Hl;
+    if (B == 0 || n == 0) return SPP_OK;
+    if (B > 1 && (C * n) % 4) return SPP_ERR_ALIGN;
+    dim3 grid((Wl + kBX - 1) / kBX, (Hl + kBY - 1) / kBY, B);
+    int rc;
+    if (!coarse)
+        rc = launch_recon_backward<false, false>(grid, stream, noisy, logits, C, coarse,
+                                                 warped_prev, mask, Wl, Hl, grad_out, grad_logits,
+                                                 grad_noisy, grad_coarse, grad_warped, Cg, C * n, accumulate);
+    else if (!warped_prev)
+        rc = launch_recon_backward<true, false>(grid, stream, noisy, logits, C, coarse,
+                                                warped_prev, mask, Wl, Hl, grad_out, grad_logits,
+                                                grad_noisy, grad_coarse, grad_warped, Cg, C * n, accumulate);
+    else
+        rc = launch_recon_backward<true, true>(grid, stream, noisy, logits, C, coarse,
+                                               warped_prev, mask, Wl, Hl, grad_out, grad_logits,
+                                               grad_noisy, grad_coarse, grad_warped, Cg, C * n, accumulate);
+    count_launch();
+    return rc != SPP_OK ? rc : launch_status();
 }
 
 }  // namespace
@@ -821,39 +869,50 @@ int spp_reconstruct_level_backward_batch(int B, const float *noisy, const float 
                                          const float *grad_out, float *grad_logits, int Cg,
                                          float *grad_noisy, float *grad_coarse,
                                          float *grad_warped, cudaStream_t stream) {
+    return spp::level_backward(B, noisy, logits, C, coarse, warped_prev, mask, Wl, Hl, grad_out,
+                               grad_logits, Cg, grad_noisy, grad_coarse, grad_warped, true, stream);
+}
+
+int spp_reconstruct_pyramid_backward(const float *const *layers, const float *const *logits,
+                                     const int *channels, const float *const *hats,
+                                     const float *warped_prev, const uint8_t *mask,
+                                     const float *hdr, int W, int H, int L, const spp_tonemap *tm,
+                                     const float *grad_hdr, const float *grad_ldr, float *grad_out,
+                                     float *const *grad_layers, float *const *grad_logits,
+                                     float *const *grad_hats, float *grad_warped,
+                                     cudaStream_t stream) {
     using namespace spp;
-    if (B < 0 || B > 65535 || Wl < 0 || Hl < 0 || !noisy || !logits || !grad_out || !grad_logits)
+    if (!layers || !logits || !channels || !hats || !grad_layers || !grad_logits || !grad_hats ||
+        !hdr || !grad_out || W < 0 || H < 0)
         return SPP_ERR_ARG;
-    if (warped_prev && !coarse) return SPP_ERR_ARG;
-    const int need = warped_prev ? 54 : 25 + (coarse ? 4 : 0);
-    if (C < need || Cg < need || Cg > C) return SPP_ERR_ARG;
-    if (coarse && ((Wl & 1) || (Hl & 1))) return SPP_ERR_SHAPE;
-    if (!aligned16(noisy) || !aligned16(logits) || !aligned16(grad_out) ||
-        !aligned16(grad_logits) || (coarse && !aligned16(coarse)) ||
-        (warped_prev && !aligned16(warped_prev)) || (mask && !aligned16(mask)) ||
-        (grad_noisy && !aligned16(grad_noisy)) || (grad_coarse && !aligned16(grad_coarse)) ||
-        (grad_warped && !aligned16(grad_warped)))
+    if (L < 2 || L > 16) return SPP_ERR_SHAPE;
+    if (!aligned16(hdr) || !aligned16(grad_out) || (grad_hdr && !aligned16(grad_hdr)) ||
+        (grad_ldr && !aligned16(grad_ldr)))
         return SPP_ERR_ALIGN;
-    const long long n = static_cast<long long>(Wl) * Hl;
-    if (B == 0 || n == 0) return SPP_OK;
-    if (B > 1 && (C * n) % 4) return SPP_ERR_ALIGN;
-    dim3 block(kBX, kBY);
-    dim3 grid((Wl + kBX - 1) / kBX, (Hl + kBY - 1) / kBY, B);
-    int rc;
-    if (!coarse)
-        rc = launch_recon_backward<false, false>(grid, block, stream, noisy, logits, C, coarse,
-                                                 warped_prev, mask, Wl, Hl, grad_out, grad_logits,
-                                                 grad_noisy, grad_coarse, grad_warped, Cg, C * n);
-    else if (!warped_prev)
-        rc = launch_recon_backward<true, false>(grid, block, stream, noisy, logits, C, coarse,
-                                                warped_prev, mask, Wl, Hl, grad_out, grad_logits,
-                                                grad_noisy, grad_coarse, grad_warped, Cg, C * n);
-    else
-        rc = launch_recon_backward<true, true>(grid, block, stream, noisy, logits, C, coarse,
-                                               warped_prev, mask, Wl, Hl, grad_out, grad_logits,
-                                               grad_noisy, grad_coarse, grad_warped, Cg, C * n);
-    count_launch();
-    return rc != SPP_OK ? rc : launch_status();
+    const ToneArgs ta = tone_args_bwd(tm);
+    if (grad_ldr && !(ta.s > 0.0f && ta.s < 1.0f && ta.h > 0.0f && ta.h < 1.0f)) return SPP_ERR_ARG;
+    const long long N = static_cast<long long>(W) * H;
+    const float *g = grad_out;
+    if (N && grad_ldr) {
+        tonemap_backward_kernel<<<static_cast<unsigned>((N + 255) / 256), 256, 0, stream>>>(
+            hdr, N, ta, grad_ldr, grad_hdr, grad_out);
+        count_launch();
+    } else if (N && grad_hdr) {
+        g = grad_hdr;
+    } else if (N && cudaMemsetAsync(grad_out, 0, 3 * N * sizeof(float), stream) != cudaSuccess) {
+        return SPP_ERR_CUDA;
+    }
+    for (int l = 0; l < L; ++l) {
+        const bool up = l + 1 < L;
+        const int rc = level_backward(1, layers[l], logits[l], channels[l], up ? hats[l + 1] : nullptr,
+                                      l == 0 ? warped_prev : nullptr, l == 0 ? mask : nullptr, W >> l,
+                                      H >> l, g, grad_logits[l], channels[l], grad_layers[l],
+                                      up ? grad_hats[l + 1] : nullptr,
+                                      l == 0 ? grad_warped : nullptr, false, stream);
+        if (rc != SPP_OK) return rc;
+        if (up) g = grad_hats[l + 1];
+    }
+    return launch_status();
 }
 
 int spp_warp_previous_backward(const float *mv, int W, int H, const float *grad_warped,
@@ -883,7 +942,7 @@ int spp_tonemap_backward_batch(int B, const float *hdr, int W, int H, const spp_
     const long long N = static_cast<long long>(W) * H;
     if (B == 0 || N == 0) return SPP_OK;
     tonemap_backward_kernel<<<dim3(static_cast<unsigned>((N + 255) / 256), B), 256, 0, stream>>>(
-        hdr, N, ta, grad_ldr, grad_hdr);
+        hdr, N, ta, grad_ldr, grad_hdr, grad_hdr);
     count_launch();
     return launch_status();
 }

@@ -14,6 +14,18 @@ constexpr float kLog2e = 1.4426950408889634f;
 
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
+// 4-byte asynchronous copy from global to shared memory.
+__device__ __forceinline__ void copy_async4(float *dst, const float *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                 "l"(src)
+                 : "memory");
+}
+// this thread's copies have landed
+__device__ __forceinline__ void copy_async_wait() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // 2^x on the SFU (relative error about 2^-22; results below 2^-126 flush to
 // 0, which only drops softmax weights smaller than 1e-38 of the largest).
 __device__ __forceinline__ float ex2_approx(float x) {

@@ -322,6 +322,23 @@ int spp_reconstruct_level_batch(int B, const float *noisy, const float *logits, 
     return launch_status();
 }
 
+int spp_reconstruct_pyramid(const float *const *layers, const float *const *logits,
+                            const int *channels, const float *warped_prev, const uint8_t *mask,
+                            int W, int H, int L, const spp_tonemap *tm, float *const *hats,
+                            float *out_hdr, float *out_ldr, int32_t *status, cudaStream_t stream) {
+    if (!layers || !logits || !channels || !hats) return SPP_ERR_ARG;
+    if (L < 2 || L > 16) return SPP_ERR_SHAPE;
+    for (int l = L - 1; l >= 0; --l) {
+        const int rc = spp_reconstruct_level(
+            layers[l], logits[l], channels[l], l + 1 < L ? hats[l + 1] : nullptr,
+            l == 0 ? warped_prev : nullptr, l == 0 && warped_prev ? mask : nullptr, W >> l, H >> l,
+            l == 0 ? tm : nullptr, l == 0 ? out_hdr : hats[l], l == 0 ? out_ldr : nullptr, status,
+            stream);
+        if (rc != SPP_OK) return rc;
+    }
+    return SPP_OK;
+}
+
 size_t spp_reconstruct_workspace_bytes(int W, int H, int L) {
     if (W < 0 || H < 0 || L < 2 || L > 5) return 0;
     size_t total = spp::align256(3 * sizeof(float) * static_cast<size_t>(W) *
