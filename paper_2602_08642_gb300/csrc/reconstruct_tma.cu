@@ -442,6 +442,8 @@ __global__ void __launch_bounds__(256)
 warp_prev_kernel(const __grid_constant__ BatchImages prevs,
                  const __grid_constant__ BatchImages mvs, int Wl, int Hl,
                  float *__restrict__ warped) {
+    pdl_wait();
+    pdl_trigger();
     const float *__restrict__ prev = prevs.p[blockIdx.z];
     const float *__restrict__ mv = mvs.p[blockIdx.z];
     warped += blockIdx.z * 3 * static_cast<long long>(Wl) * Hl;
@@ -531,7 +533,7 @@ int launch_variant(int B, Args &&...args) {
 void launch_warp_prev(int B, const BatchImages &prev, const BatchImages &mv, int Wl, int Hl,
                       float *warped, cudaStream_t stream) {
     dim3 grid((Wl + 63) / 64, (Hl + 3) / 4, B);
-    warp_prev_kernel<<<grid, 256, 0, stream>>>(prev, mv, Wl, Hl, warped);
+    launch_dependent(warp_prev_kernel, grid, dim3(256), 0, stream, prev, mv, Wl, Hl, warped);
 }
 
 bool launch_recon_tma(int B, const float *noisy, const float *logits, int C_total, int C_used,
