@@ -936,9 +936,387 @@ bool getenv_disable_tma_in() {
     return off;
 }
 
+// Upsampling layers (kSrcConcatUp: a skip tensor concatenated with the 2x
+// nearest upsampling of a coarse one) without expanding anything in shared
+// memory: the columns of the output are split into their even and odd ones.
+// Row m of an MMA is the pixel pair at coarse column xc = xc0 + m; output phase
+// a (pixel 2 xc + a) has its own accumulators, and tap dx of it reads
+//   the upsampled tensor at coarse column (2 xc + a + dx - 1) >> 1, one of
+//     xc - 1, xc, xc + 1;
+//   the skip tensor at pixel 2 xc + a + dx - 1, a column of its even or its odd
+//     plane, which TMA boxes with a doubled x stride bring.
+// Every operand is then a window of a staged row, as in conv3x3_kernel: the same
+// MMAs and weights, and every sum in the same order (dx by dx within a K chunk, so
+// both planes of a skip chunk are staged together): the same bits.
+// The rows of an upsampled chunk are shared too: halo row h reads coarse row
+// (h + 1) >> 1 of the box.
+//
+// The expansion (a thread per coarse piece, up to four 16-byte stores) bounded
+// these layers, the largest of the network: 96 -> 32 channels at 3840 x 2160
+// 550 -> 418 us, 192 -> 64 at 1920 x 1080 335 -> 317 us (of the same 4K forward).
+//
+// A tile is TR x 256 pixels.  Accumulators take 2 TR N columns: double-buffered
+// for N = 32, one set for N = 64 (half-height tiles with two sets would fetch the
+// streamed weights twice as often, and L2 is what they are close to).
+// Warps 0-3 and 4-7 are the epilogues of phase 0 and 1, warp 8 issues the MMAs,
+// warp 9 the copies.
+template <int N, bool RES>
+__global__ void __launch_bounds__(kThreads, 1)
+conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
+                  const __grid_constant__ CUtensorMap omap1,
+                  const __grid_constant__ CUtensorMap emap,
+                  const __grid_constant__ CUtensorMap dmap,
+                  const __grid_constant__ CUtensorMap umap) {
+    // omap0, omap1: the output's even and odd columns; emap, dmap: the skip
+    // tensor's; umap: the coarse tensor
+    using C = Cfg<N, RES>;
+    constexpr int TR = C::TR, NS = C::kNS;
+    static_assert(C::kStack && TR % 2 == 0 && C::kEpiWarps == 8, "stacked layers of even tiles");
+    constexpr int kPhase = C::kAccCols;  // accumulator columns of a phase
+    constexpr int kSets = 2 * 2 * kPhase <= 512 ? 2 : 1;
+    constexpr int kCols = 512;
+    constexpr int kUpBytes = (TR / 2 + 2) * kPitch * 32;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    unsigned char *base = smem_raw + ((512u - (tc::smem_u32(smem_raw) & 511u)) & 511u);
+    Bars &bars = *reinterpret_cast<Bars *>(base);
+    unsigned char *wres = base + C::kWOff;
+    unsigned char *stages = base + C::kStagesOff;
+    float *sbias = reinterpret_cast<float *>(base + C::kBiasOff);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    const int tiles_x = (a.W + 2 * kTileX - 1) / (2 * kTileX);
+    const int tiles_y = (a.H + TR - 1) / TR;
+    const int per_img = tiles_x * tiles_y;
+    const int ntiles = a.B * per_img;
+    const int kc0 = a.c0 / 16, kchunks = a.cin_pad / 16;
+    const int nst = kchunks + kc0;  // stages per tile: two planes of a skip chunk, an upsampled one
+
+    if (tid == 0) {
+        for (int s = 0; s < NS; ++s) {
+            tc::mbar_init(&bars.full[s], 1);
+            tc::mbar_init(&bars.wfull[s], 1);
+            tc::mbar_init(&bars.empty[s], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            tc::mbar_init(&bars.accf[i], 1);
+            tc::mbar_init(&bars.acce[i], 256);
+        }
+        tc::mbar_init(&bars.drain, 1);
+        bars.abort = 0;
+        tc::fence_mbar_init();
+    }
+    for (int i = tid; i < C::kZeroBytes / 16; i += kThreads)
+        reinterpret_cast<uint4 *>(base + C::kZeroOff)[i] = make_uint4(0, 0, 0, 0);
+    tc::fence_proxy_async();
+    if (warp == 8) tc::tmem_alloc(&bars.tmem_base, kCols);
+    pdl_wait();
+    pdl_trigger();
+    for (int i = tid; i < N; i += kThreads) sbias[i] = (a.bias && i < a.cout) ? a.bias[i] : 0.f;
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tmem = bars.tmem_base;
+    volatile int *abort_flag = &bars.abort;
+    auto fail = [&]() {
+        *abort_flag = 1;
+        set_status(a.status, SPP_ERR_TIMEOUT);
+    };
+
+    if (warp == 9) {
+        // ------------------------------------------------------------- copies
+        if (lane == 0) {
+            uint32_t it = 0;
+            bool ok = true;
+            if (RES && static_cast<int>(blockIdx.x) < ntiles) {
+                tc::mbar_arrive_expect_tx(&bars.wfull[0], static_cast<uint32_t>(kchunks * C::kB));
+                for (int c = 0; c < kchunks; ++c)
+                    tc::bulk_g2s(wres + c * C::kB,
+                                 reinterpret_cast<const unsigned char *>(a.wpack) +
+                                     static_cast<size_t>(c) * C::kB,
+                                 C::kB, &bars.wfull[0]);
+            }
+            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+                const int b = t / per_img, r = t - b * per_img;
+                const int y0 = (r / tiles_x) * TR, xc0 = (r % tiles_x) * kTileX;
+                for (int st = 0; st < nst; ++st, ++it) {
+                    const int s = static_cast<int>(it % NS);
+                    if (!tc::mbar_wait(&bars.empty[s], ((it / NS) & 1u) ^ 1u, abort_flag)) {
+                        fail();
+                        ok = false;
+                        break;
+                    }
+                    unsigned char *As = stages + s * C::kStage;
+                    const bool skip = st < 2 * kc0;
+                    const int c = skip ? st >> 1 : st - kc0;
+                    if (!RES && skip && (st & 1)) {
+                        tc::mbar_arrive(&bars.wfull[s]);  // its chunk's weights are there
+                    } else if (!RES) {
+                        tc::mbar_arrive_expect_tx(&bars.wfull[s], C::kB);
+                        tc::bulk_g2s(As + C::kA,
+                                     reinterpret_cast<const unsigned char *>(a.wpack) +
+                                         static_cast<size_t>(c) * C::kB,
+                                     C::kB, &bars.wfull[s]);
+                    }
+                    if (skip) {
+                        tc::mbar_arrive_expect_tx(&bars.full[s], kPitch * (TR + 2) * 32);
+                        tma_load_halo(st & 1 ? &dmap : &emap, As, &bars.full[s], xc0 - 1, y0 - 1, c, b);
+                    } else {
+                        tc::mbar_arrive_expect_tx(&bars.full[s], kUpBytes);
+                        tma_load_halo(&umap, As, &bars.full[s], xc0 - 1, y0 / 2 - 1, c - kc0, b);
+                    }
+                }
+            }
+            if (!ok) {
+                // wait (bounded, ignoring the abort flag) for the copies in flight
+                for (uint32_t k = it > NS ? it - NS : 0; k < it; ++k) {
+                    (void)tc::mbar_wait(&bars.full[k % NS], (k / NS) & 1u, nullptr);
+                    if (!RES) (void)tc::mbar_wait(&bars.wfull[k % NS], (k / NS) & 1u, nullptr);
+                }
+                if (RES) (void)tc::mbar_wait(&bars.wfull[0], 0, nullptr);
+            }
+        }
+        __syncwarp();
+    } else if (warp == 8) {
+        // -------------------------------------------------------- MMA issuer
+        if (lane == 0) {
+            uint32_t it = 0, tl = 0;
+            bool ok = true, pending = false;
+            if (RES && static_cast<int>(blockIdx.x) < ntiles &&
+                !tc::mbar_wait(&bars.wfull[0], 0, abort_flag)) {
+                fail();
+                ok = false;
+            }
+            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tl) {
+                const int acc = kSets == 2 ? tl & 1 : 0;
+                if (!tc::mbar_wait(&bars.acce[acc], ((tl / kSets) & 1u) ^ 1u, abort_flag)) {
+                    fail();
+                    ok = false;
+                    break;
+                }
+                tc::tc_fence_after();
+                const uint32_t d0 = tmem + acc * 2 * kPhase;
+                // reset the accumulators of both phases
+                const uint64_t zd =
+                    tc::smem_desc(tc::smem_u32(base + C::kZeroOff), C::kZeroRows * 16, 128);
+                tc::mma_bf16(d0, zd, zd, tc::idesc_bf16_f32(128, kPhase), 0u);
+                tc::mma_bf16(d0 + kPhase, zd, zd, tc::idesc_bf16_f32(128, kPhase), 0u);
+                for (int c = 0; c < kchunks; ++c) {
+                    // the two stages of a skip chunk (its even and odd columns; the
+                    // first brings the weights) or the one of an upsampled chunk
+                    const bool skip = c < kc0;
+                    const int s = static_cast<int>(it % NS);
+                    const uint32_t ph = (it / NS) & 1u;
+                    const int s1 = static_cast<int>((it + 1) % NS);
+                    if (!tc::mbar_wait(&bars.full[s], ph, abort_flag) ||
+                        (!RES && !tc::mbar_wait(&bars.wfull[s], ph, abort_flag)) ||
+                        (skip &&
+                         !tc::mbar_wait(&bars.full[s1], ((it + 1) / NS) & 1u, abort_flag))) {
+                        fail();
+                        ok = false;
+                        break;
+                    }
+                    tc::tc_fence_after();
+                    const uint32_t even = tc::smem_u32(stages + s * C::kStage);
+                    const uint32_t odd = tc::smem_u32(stages + s1 * C::kStage);
+                    const uint32_t b_base = RES ? tc::smem_u32(wres + c * C::kB) : even + C::kA;
+                    // tap dx of a phase from the staged columns starting at `col`
+                    // (0: xc0 - 1); rows as in conv3x3_kernel
+                    auto taps = [&](int phase, int dx, uint32_t rows, int col, bool up) {
+                        const uint32_t bdx = b_base + dx * 2 * 3 * N * 16;
+#pragma unroll
+                        for (int h = 0; h < TR + 2; ++h) {
+                            const int rlo = h - 2 < 0 ? 0 : h - 2;
+                            const int rhi = h < TR - 1 ? h : TR - 1;
+                            const int k0 = rlo - (h - 2);
+                            const int row = up ? (h + 1) >> 1 : h;
+                            tc::mma_bf16(d0 + phase * kPhase + rlo * N,
+                                         tc::smem_desc_sw32(rows + (row * kPitch + col) * 32),
+                                         tc::smem_desc(bdx + k0 * N * 16, 3 * N * 16, 128),
+                                         tc::idesc_bf16_f32(128, (rhi - rlo + 1) * N), 1u);
+                        }
+                    };
+                    // dx = 0, 1, 2 for each phase, as in conv3x3_kernel: the same sums
+                    if (skip) {
+                        taps(0, 0, odd, 0, false);
+                        taps(0, 1, even, 1, false);
+                        taps(0, 2, odd, 1, false);
+                        taps(1, 0, even, 1, false);
+                        taps(1, 1, odd, 1, false);
+                        taps(1, 2, even, 2, false);
+                    } else {
+                        taps(0, 0, even, 0, true);
+                        taps(0, 1, even, 1, true);
+                        taps(0, 2, even, 1, true);
+                        taps(1, 0, even, 1, true);
+                        taps(1, 1, even, 1, true);
+                        taps(1, 2, even, 2, true);
+                    }
+                    pending = true;
+                    tc::mma_commit(&bars.empty[s]);
+                    if (skip) tc::mma_commit(&bars.empty[s1]);
+                    it += skip ? 2 : 1;
+                }
+                if (!ok) break;
+                tc::mma_commit(&bars.accf[acc]);
+            }
+            if (!ok && pending) {
+                tc::mma_commit(&bars.drain);
+                (void)tc::mbar_wait(&bars.drain, 0, nullptr);
+            }
+        }
+        __syncwarp();
+    } else {
+        // ----------------------------------------------------------- epilogue
+        const int sub = warp & 3, phase = warp >> 2;
+        const CUtensorMap *omap = phase ? &omap1 : &omap0;
+        constexpr int kCB = C::kCBs, kW = kCB / 2;
+        static_assert(kCB == 32, "64-byte slots");
+        constexpr int kRowBlocks = N / kCB, kBlocks = TR * kRowBlocks;
+        unsigned char *slots = base + C::kStoreOff + warp * 2 * C::kSlot;
+        const uint32_t swz = (lane >> 1) & 3;
+        const uint32_t lane_base = static_cast<uint32_t>(sub * 32) << 16;
+        const int Wc = a.W >> 1;
+        uint32_t tl = 0, eblk = 0;
+        for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++tl) {
+            const int acc = kSets == 2 ? tl & 1 : 0;
+            const int b = t / per_img, r = t - b * per_img;
+            const int y0 = (r / tiles_x) * TR, xw = (r % tiles_x) * kTileX + sub * 32;
+            if (!tc::mbar_wait(&bars.accf[acc], (tl / kSets) & 1u, abort_flag)) {
+                fail();
+                break;
+            }
+            tc::tc_fence_after();
+            const uint32_t abase = tmem + lane_base + (acc * 2 + phase) * kPhase;
+            auto tmem_read = [&](int k, uint32_t (&v)[kCB]) {
+#pragma unroll
+                for (int q = 0; q < kCB / 16; ++q)
+                    tc::tmem_ld16(abase + (k / kRowBlocks) * N + (k % kRowBlocks) * kCB + 16 * q,
+                                  *reinterpret_cast<uint32_t(*)[16]>(v + 16 * q));
+            };
+            uint32_t vbuf[2][kCB];
+            tmem_read(0, vbuf[0]);
+            tc::tmem_wait_ld();
+#pragma unroll
+            for (int k = 0; k < kBlocks; ++k) {
+                if (k + 1 < kBlocks) tmem_read(k + 1, vbuf[(k + 1) & 1]);
+                const uint32_t (&v)[kCB] = vbuf[k & 1];
+                const int y = y0 + k / kRowBlocks, j0 = (k % kRowBlocks) * kCB;
+                uint32_t w[kW];
+#pragma unroll
+                for (int e = 0; e < kCB; e += 2) {
+                    const float2 bb = *reinterpret_cast<const float2 *>(sbias + j0 + e);
+                    const float2 f =
+                        add2(make_float2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])), bb);
+                    w[e / 2] = pack_bf16x2(f.x, f.y);
+                    if (a.epi_mode == kEpiReluBF16) w[e / 2] = relu_bf16x2(w[e / 2]);
+                }
+                unsigned char *slot = slots + (eblk & 1) * C::kSlot;
+                if (lane == 0) tma_store_wait_read<1>();  // the slot's previous store
+                __syncwarp();
+                uint4 *row = reinterpret_cast<uint4 *>(slot + lane * 2 * kCB);
+#pragma unroll
+                for (int q = 0; q < kW / 4; ++q)
+                    row[q ^ swz] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+                tc::fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) {
+                    if (y < a.H && xw < Wc) tma_store_nhwc(omap, slot, j0, xw, y, b);
+                    tma_store_commit();
+                }
+                ++eblk;
+                tc::tmem_wait_ld();
+            }
+            tc::tc_fence_before();
+            tc::mbar_arrive(&bars.acce[acc]);
+        }
+        if (lane == 0 && eblk) tma_store_wait_all();
+    }
+
+    tc::tc_fence_before();
+    __syncthreads();
+    if (warp == 8) {
+        tc::tc_fence_after();
+        tc::tmem_dealloc(tmem, kCols);
+    }
+}
+
+// Launches conv3x3_up_kernel where it applies and pays; false: not launched.
+template <int N, bool RES>
+bool launch_up(const ConvArgs &a, cudaStream_t stream, int *rc) {
+    using C = Cfg<N, RES>;
+    // A tile of 256 columns takes 1.5 (N = 32) or 1.77 (N = 64) times as long as one
+    // of 128 columns of the expanding kernel (the times above over their tiles), so
+    // the rounds of tiles per SM decide: padding columns and a last round that is
+    // nearly empty can cost more than the expansion.
+    const int64_t rows = static_cast<int64_t>(a.B) * ((a.H + C::TR - 1) / C::TR), sms = sm_count();
+    const int64_t ntiles = rows * ((a.W + 2 * kTileX - 1) / (2 * kTileX));
+    const int64_t rounds = (ntiles + sms - 1) / sms;
+    const int64_t rounds128 = (rows * ((a.W + kTileX - 1) / kTileX) + sms - 1) / sms;
+    if (a.src_mode != kSrcConcatUp || a.pool_out ||
+        (a.epi_mode != kEpiReluBF16 && a.epi_mode != kEpiBF16) || a.W % 2 || a.H % 2 ||
+        a.c0 % 16 || a.c1 % 16 || a.c0 <= 0 || a.c1 <= 0 || a.cin_pad != a.c0 + a.c1 ||
+        ntiles <= 0 || ntiles > 0x7fffffff || getenv_disable_tma_in() ||
+        (N == 32 ? 3 * rounds > 2 * rounds128 : 16 * rounds > 9 * rounds128))
+        return false;
+    auto enc = tensor_map_encoder();
+    if (!enc) return false;
+    const cuuint64_t Wc = a.W / 2, H = a.H, B = a.B, c0 = a.c0, c1 = a.c1;
+    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    CUtensorMap omap[2], smap[2], umap;
+    for (int p = 0; p < 2; ++p) {
+        // output columns 2 x + p, a block of 32 of them and 32 channels
+        cuuint64_t dims[4] = {static_cast<cuuint64_t>(N), Wc, H, B};
+        cuuint64_t strides[3] = {4ull * N, 4ull * N * Wc, 4ull * N * Wc * H};
+        cuuint32_t box[4] = {32, 32, 1, 1};
+        if (enc(&omap[p], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, a.out + p * N, dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return false;
+        // skip columns 2 x + p: (channel in chunk, x, y, 16-channel chunk, image)
+        cuuint64_t sdims[5] = {16, Wc, H, c0 / 16, B};
+        cuuint64_t sstr[4] = {4 * c0, 4 * c0 * Wc, 32, 4 * c0 * Wc * H};
+        cuuint32_t sbox[5] = {16, kPitch, C::TR + 2, 1, 1};
+        if (enc(&smap[p], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5,
+                const_cast<__nv_bfloat16 *>(a.src0 + p * c0), sdims, sstr, sbox, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
+                CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return false;
+    }
+    cuuint64_t udims[5] = {16, Wc, H / 2, c1 / 16, B};
+    cuuint64_t ustr[4] = {2 * c1, 2 * c1 * Wc, 32, 2 * c1 * Wc * (H / 2)};
+    cuuint32_t ubox[5] = {16, kPitch, C::TR / 2 + 2, 1, 1};
+    if (enc(&umap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<__nv_bfloat16 *>(a.src1), udims,
+            ustr, ubox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return false;
+    static int configured_dev = -1;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (configured_dev != dev) {
+        if (cudaFuncSetAttribute(conv3x3_up_kernel<N, RES>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 C::kSmem) != cudaSuccess) {
+            *rc = SPP_ERR_CUDA;
+            return true;
+        }
+        configured_dev = dev;
+    }
+    const int grid = static_cast<int>(std::min(ntiles, sms));
+    launch_dependent(conv3x3_up_kernel<N, RES>, dim3(grid), dim3(kThreads), C::kSmem, stream, a,
+                     omap[0], omap[1], smap[0], smap[1], umap);
+    count_launch();
+    *rc = launch_status();
+    return true;
+}
+
 template <int N, bool RES>
 int launch_variant(const ConvArgs &a, cudaStream_t stream) {
     using C = Cfg<N, RES>;
+    if constexpr (C::kStack) {
+        int rc;
+        if (launch_up<N, RES>(a, stream, &rc)) return rc;
+    }
     static int configured_dev = -1;
     int dev = 0;
     cudaGetDevice(&dev);
