@@ -12,7 +12,7 @@
 //              lanes 32w..32w+31 = pixels), bias / ReLU / mask, stores;
 //   warps 4-7  a second set of epilogue warps (the second half of each
 //              tile's rows, TMEM lanes 32 (w - 4)..) when the input arrives by
-//              TMA and N <= 64, with warp 9 issuing the copies; otherwise
+//              TMA and N <= 64 or N = 128, with warp 9 issuing the copies; otherwise
 //              producers: per K chunk of 16 input channels they stage the
 //              (TR+2) x 130 pixel halo of the tile in shared memory as K-major
 //              rows of 32 bytes per pixel in the 32-byte swizzle ([row][pixel]
@@ -89,8 +89,12 @@ struct Cfg {
     static constexpr int kCBs = N < 32 ? N : 32;
     static constexpr int kSlot = 32 * 2 * kCBs;
     // eight epilogue warps (two per TMEM sub-partition, each taking half of
-    // a tile's rows) when the layer's input comes by TMA and N <= 64, else four
-    static constexpr int kEpiWarps = N <= 64 ? 8 : 4;
+    // a tile's rows) when the layer's input comes by TMA and N <= 64 or N = 128, else four
+    // (N = 96 would spill).
+    // A block of 32 pixels x 32 channels takes a warp about 1300 cycles, mostly
+    // latency: with eight warps 64 -> 128 channels at 960 x 540 takes 64 us, with four
+    // 92 us, 128 -> 128 103 and 113 us.
+    static constexpr int kEpiWarps = N <= 64 || N == 128 ? 8 : 4;
     static constexpr int kStoreBytes = kEpiWarps * 2 * kSlot;
     // the FP32 planar staging buffers and the BF16 slots share one
     // region (a launch uses one of the two epilogues)
@@ -248,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
     // the second set of epilogue warps: for a plain NHWC input (TMA halo, one
     // issuing thread) the producer warps 4-7 take half of each tile's output
     // rows and warp 9 issues the copies
-    const bool ep8 = C::kEpiWarps == 8 && a.tma_in == 1;
+    const bool ep8 = C::kEpiWarps == 8 && a.tma_in == 1 && !(TR < 4 && a.pool_out);
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) {
             tc::mbar_init(&bars.full[s], a.tma_in == 1 ? 1 : a.tma_in == 3 ? 160 : 128);
