@@ -157,6 +157,148 @@ splat_kernel(const int32_t *__restrict__ offsets, const float4 *__restrict__ rgb
     }
 }
 
+constexpr int kQuadTX = 128;  // 32 lanes x 4 pixels
+constexpr int kQuadTY = 16;   // 8 warps x 2 rows: covers one level-4 block
+
+// The same for widths that are a multiple of 4: a thread owns 4 x 2 pixels, reads
+// offsets, weights and s in 16-byte pieces and forms its two level-1 pixels in
+// registers, so that only the levels below pass through shared memory.  Same sums
+// in the same order.
+//
+// Bound by latency (offsets, then samples, then divisions), with 32 bytes per pixel
+// to move: eight pixels per thread keep four times the loads in flight that two
+// did, in a quarter of the instructions.  1920 x 1080: 23.0 -> 17.9 us, the 4K frame
+// 739 -> 715 us.  (The same over arrays of a templated length took 90 registers for
+// 78, and the frame 738 us.)
+__global__ void __launch_bounds__(256)
+splat_quad_kernel(const int32_t *__restrict__ offsets, const float4 *__restrict__ rgb,
+                  const float *__restrict__ s, const float *__restrict__ hw, long long capacity,
+                  int W, int H, int L, LayerPtrs layers) {
+    __shared__ float lvl1[3][kQuadTY / 2][kQuadTX / 2 + 1];
+    __shared__ float lvl2[3][kQuadTY / 4][kQuadTX / 4 + 1];
+    pdl_wait();
+    pdl_trigger();
+    const int tid = threadIdx.x, lane = tid & 31, pair = tid >> 5;
+    const int x0 = blockIdx.x * kQuadTX, y0 = blockIdx.y * kQuadTY;
+    const int x = x0 + 4 * lane;
+    const long long N = static_cast<long long>(W) * H;
+    // image blockIdx.z of a batch
+    offsets += blockIdx.z * (N + SPP_BATCH_OFFSETS_PAD);
+    rgb += blockIdx.z * capacity;
+    s += blockIdx.z * N;
+    hw += blockIdx.z * N;
+    float *L0 = layers.p[0] + blockIdx.z * 3 * N;
+
+    // the loads of both rows first; W is a multiple of 4, so four pixels are inside
+    // or none
+    int o[2][5];
+    float4 w[2], sv[2];
+    bool in[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int y = y0 + 2 * pair + r;
+        in[r] = x < W && y < H;
+        int4 q = make_int4(0, 0, 0, 0);
+        o[r][4] = 0;
+        w[r] = sv[r] = make_float4(1.0f, 1.0f, 1.0f, 1.0f);
+        if (in[r]) {
+            const long long i = static_cast<long long>(y) * W + x;
+            q = __ldg(reinterpret_cast<const int4 *>(offsets + i));
+            o[r][4] = __ldg(offsets + i + 4);
+            w[r] = __ldg(reinterpret_cast<const float4 *>(hw + i));
+            sv[r] = __ldg(reinterpret_cast<const float4 *>(s + i));
+        }
+        o[r][0] = q.x;
+        o[r][1] = q.y;
+        o[r][2] = q.z;
+        o[r][3] = q.w;
+    }
+    float a[2][3][4];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const float wq[4] = {w[r].x, w[r].y, w[r].z, w[r].w};
+        const float sq[4] = {sv[r].x, sv[r].y, sv[r].z, sv[r].w};
+        float4 first[4], last[4];
+        int beg[4], end[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            beg[q] = max(o[r][q], 0);
+            end[q] = o[r][q + 1] > capacity ? static_cast<int>(capacity) : o[r][q + 1];
+            first[q] = last[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (end[q] > beg[q]) {
+                last[q] = __ldcs(rgb + end[q] - 1);                         // the holdout slot
+                if (end[q] - beg[q] >= 2) first[q] = __ldcs(rgb + beg[q]);  // the first regular one
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f;
+            if (end[q] > beg[q]) {
+                a0 = first[q].x;
+                a1 = first[q].y;
+                a2 = first[q].z;
+                for (int t = beg[q] + 1; t < end[q] - 1; ++t) {  // slots beyond two
+                    const float4 v = __ldcs(rgb + t);
+                    a0 += v.x;
+                    a1 += v.y;
+                    a2 += v.z;
+                }
+                a0 = __fdiv_rn(__fmaf_rn(wq[q], last[q].x, a0), sq[q]);
+                a1 = __fdiv_rn(__fmaf_rn(wq[q], last[q].y, a1), sq[q]);
+                a2 = __fdiv_rn(__fmaf_rn(wq[q], last[q].z, a2), sq[q]);
+            }
+            a[r][0][q] = a0;
+            a[r][1][q] = a1;
+            a[r][2][q] = a2;
+        }
+        if (in[r]) {
+            const long long i = static_cast<long long>(y0 + 2 * pair + r) * W + x;
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                __stcs(reinterpret_cast<float4 *>(L0 + c * N + i),
+                       make_float4(a[r][c][0], a[r][c][1], a[r][c][2], a[r][c][3]));
+        }
+    }
+    if (L < 2) return;
+    {
+        const int W1 = W >> 1, H1 = H >> 1;
+        const long long N1 = static_cast<long long>(W1) * H1;
+        const int gx = x >> 1, gy = (y0 >> 1) + pair;
+        float *L1 = layers.p[1] + blockIdx.z * 3 * N1 + static_cast<long long>(gy) * W1 + gx;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            float2 v;
+            v.x = 0.25f * ((a[0][c][0] + a[0][c][1]) + (a[1][c][0] + a[1][c][1]));
+            v.y = 0.25f * ((a[0][c][2] + a[0][c][3]) + (a[1][c][2] + a[1][c][3]));
+            lvl1[c][pair][2 * lane] = v.x;
+            lvl1[c][pair][2 * lane + 1] = v.y;
+            if (gx < W1 && gy < H1) *reinterpret_cast<float2 *>(L1 + c * N1) = v;
+        }
+    }
+    // levels 2 to 4: from lvl1 into lvl2, back, and once more
+    auto reduce = [&](int l, auto &src, auto &dst) {
+        const int bw = kQuadTX >> l, bh = kQuadTY >> l;
+        const int Wl = W >> l, Hl = H >> l;
+        const long long Nl = static_cast<long long>(Wl) * Hl;
+        __syncthreads();
+        if (tid < bw * bh) {
+            const int cx = tid % bw, cy = tid / bw;
+            const int gx = (x0 >> l) + cx, gy = (y0 >> l) + cy;
+            float *out = layers.p[l] + blockIdx.z * 3 * Nl;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float v = 0.25f * ((src[c][2 * cy][2 * cx] + src[c][2 * cy][2 * cx + 1]) +
+                                         (src[c][2 * cy + 1][2 * cx] + src[c][2 * cy + 1][2 * cx + 1]));
+                dst[c][cy][cx] = v;
+                if (gx < Wl && gy < Hl) out[c * Nl + static_cast<long long>(gy) * Wl + gx] = v;
+            }
+        }
+    };
+    if (L > 2) reduce(2, lvl1, lvl2);
+    if (L > 3) reduce(3, lvl2, lvl1);
+    if (L > 4) reduce(4, lvl1, lvl2);
+}
+
 }  // namespace
 }  // namespace spp
 
@@ -208,6 +350,13 @@ int splat(int B, const int32_t *offsets, const float *rgb, const float *s, const
     if (!aligned16(offsets) || !aligned16(s) || !aligned16(holdout_w) || (rgb && !aligned16(rgb)))
         return SPP_ERR_ALIGN;
     if (B == 0 || static_cast<long long>(W) * H == 0) return SPP_OK;
+    if (W % 4 == 0) {  // 16-byte pieces of a row
+        dim3 grid((W + kQuadTX - 1) / kQuadTX, (H + kQuadTY - 1) / kQuadTY, B);
+        launch_dependent(splat_quad_kernel, grid, dim3(256), 0, stream, offsets,
+                         reinterpret_cast<const float4 *>(rgb), s, holdout_w, capacity, W, H, L, lp);
+        count_launch();
+        return launch_status();
+    }
     dim3 block(kSplatTX, kSplatTY);
     dim3 grid((W + kSplatTX - 1) / kSplatTX, (H + kSplatH - 1) / kSplatH, B);
     launch_dependent(splat_kernel, grid, block, 0, stream, offsets,
