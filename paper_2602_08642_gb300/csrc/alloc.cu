@@ -317,9 +317,13 @@ budget_sum_kernel(const float *__restrict__ d, long long N, AllocHeader *hdr, Bu
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int j = 0; j < kLimbs; ++j) {
+        // values within a few binades of one another fill three or four of the
+        // limbs; reducing all eleven was most of this kernel's instructions
         unsigned long long v = lim[j];
+        if (__any_sync(0xffffffffu, v != 0ull)) {
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+            for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+        }
         if (lane == 0) s_part[warp][j] = v;
     }
     const int any_bad = __syncthreads_or(bad ? 1 : 0);

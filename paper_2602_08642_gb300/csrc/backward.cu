@@ -68,11 +68,12 @@ __device__ __forceinline__ void tap_range(int q, int p, int n, int &lo, int &hi)
 // source pixel (and for each coarse cell under the tile) w_k g over the
 // consumers and taps that read it.
 //
-// Bound by its shared-memory accesses (about 560 per consumer), not by its bytes.
+// Bound by its shared-memory and L1 accesses (about 560 and 110 per consumer of
+// the tile), not by its bytes, so a warp takes whole rows of the tile.
 // Two CTAs of 448 threads per SM (the weights of one tile take 109 KB) leave 72
 // registers, so the products q_k are formed twice (once for their mean, once for
 // the gradients) instead of being kept.  960 x 540, cold caches: level 0 with the
-// temporal term 144 -> 141 us, level 1 27 -> 21.5 us, level 2 14 -> 10.7 us
+// temporal term 144 -> 137 us, level 1 27 -> 20.6 us, level 2 14 -> 10.1 us
 // against 256 threads per tile and two rounds of loads.
 template <bool UP, bool TEMP>
 __global__ void __launch_bounds__(kBwdThreads, 2)
@@ -105,11 +106,25 @@ recon_backward_kernel(const float *__restrict__ noisy, const float *__restrict__
     if (TEMP) warped += blockIdx.z * 3 * Nl;
     if (TEMP && grad_warped) grad_warped += blockIdx.z * 3 * Nl;
 
-    // this thread's consumer: cell (rx, ry) of the region, pixel (px, py)
-    const int cell = min(tid, kRN - 1);
-    const int rx = tid % kRX, ry = tid / kRX;
+    // this thread's consumer: cell (rx, ry) of the region, pixel (px, py).  Warps
+    // 0-7 have the tile's rows (whole 128-byte lines of every plane), the others the
+    // halo: rows 0-1 and 10-11, then columns 0-1 and 34-35.
+    const bool tile = tid < kBX * kBY;
+    int rx, ry;
+    if (tile) {
+        rx = kBH + tid % kBX;
+        ry = kBH + tid / kBX;
+    } else if (tid < kBX * kBY + 4 * kRX) {
+        const int h = tid - kBX * kBY;
+        rx = h % kRX;
+        ry = h / kRX < 2 ? h / kRX : kRY - 4 + h / kRX;
+    } else {
+        const int h = min(tid, kRN - 1) - kBX * kBY - 4 * kRX;
+        ry = kBH + h / 4;
+        rx = (h % 4) < 2 ? (h % 4) : kBX + (h % 4);
+    }
+    const int cell = ry * kRX + rx;
     const int px = bx0 + rx - kBH, py = by0 + ry - kBH;
-    const bool tile = rx >= kBH && rx < kBH + kBX && ry >= kBH && ry < kBH + kBY;
     const bool in = tid < kRN && px >= 0 && px < Wl && py >= 0 && py < Hl;
     const long long pix = in ? static_cast<long long>(py) * Wl + px : 0;
 
