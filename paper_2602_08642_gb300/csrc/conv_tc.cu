@@ -20,7 +20,7 @@
 //              concat on the way (a TMA box writes the plain NHWC case
 //              directly); one elected thread
 //              bulk-copies the pre-packed weights of the chunk;
-//   warp 8     lane 0 issues the MMAs: for each row r and tap (dy, dx) the A
+//   warp 8     issues the MMAs (one lane): for each row r and tap (dy, dx) the A
 //              operand is the halo window starting at row r+dy, pixel dx
 //              (a start address moved by whole 32-byte pixel rows, which the
 //              swizzled descriptor allows because the swizzle follows the
@@ -90,11 +90,11 @@ struct Cfg {
     static constexpr int kSlot = 32 * 2 * kCBs;
     // eight epilogue warps (two per TMEM sub-partition, each taking half of
     // a tile's rows) when the layer's input comes by TMA and N <= 64 or N = 128, else four
-    // (N = 96 would spill).
+    // (N = 96 and the resident N = 128 would spill).
     // A block of 32 pixels x 32 channels takes a warp about 1300 cycles, mostly
     // latency: with eight warps 64 -> 128 channels at 960 x 540 takes 64 us, with four
     // 92 us, 128 -> 128 103 and 113 us.
-    static constexpr int kEpiWarps = N <= 64 || N == 128 ? 8 : 4;
+    static constexpr int kEpiWarps = N <= 64 || (N == 128 && !RES) ? 8 : 4;
     static constexpr int kStoreBytes = kEpiWarps * 2 * kSlot;
     // the FP32 planar staging buffers and the BF16 slots share one
     // region (a launch uses one of the two epilogues)
@@ -172,7 +172,7 @@ __device__ __forceinline__ void tma_load_halo(const CUtensorMap *map, void *dst,
         : "memory");
 }
 
-// TMA tensor store of a [16][1][128] FP32 box from shared memory at (x, y, c, b).
+// TMA tensor store of an FP32 box of 32 pixels x 32 (16) planes at (x, y, c, b).
 __device__ __forceinline__ void tma_store_planes(const CUtensorMap *map, const void *src, int x,
                                                  int y, int c, int b) {
     asm volatile(
@@ -180,7 +180,6 @@ __device__ __forceinline__ void tma_store_planes(const CUtensorMap *map, const v
             reinterpret_cast<uint64_t>(map)),
         "r"(tc::smem_u32(src)), "r"(x), "r"(y), "r"(c), "r"(b)
         : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 // TMA tensor store of 32 pixels x kCBs channels of BF16 NHWC from a warp's
 // staging slot at (c, x, y, b), clipped at the image's edges.
@@ -241,7 +240,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
     unsigned char *wres = base + C::kWOff;              // resident weights (RES)
     unsigned char *stages = base + C::kStagesOff;
     float *sbias = reinterpret_cast<float *>(base + C::kBiasOff);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // known to be the warp's
 
     const int tiles_x = (a.W + kTileX - 1) / kTileX;
     const int tiles_y = (a.H + TR - 1) / TR;
@@ -519,19 +519,28 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
         }
     } else if (warp == 8) {
         // -------------------------------------------------------- MMA issuer
-        if (lane == 0) {
+        {
+            // One lane issues, but the code is the whole warp's, so that descriptors,
+            // each one addition from a stage's first, can stay in uniform registers.
+            // The issue rate bounds the layers of N <= 64: 4K forward 2.48 ms with a
+            // descriptor built for every MMA in one lane's branch, 2.42 with
+            // additions, 2.38 with warp-uniform code.  All lanes take part in every
+            // wait: the warp stays converged, which uniform registers rely on.
+            const uint32_t lead = tc::elect_one();
+            auto wait = [&](uint64_t *bar, uint32_t parity) {
+                return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort_flag));
+            };
             constexpr uint32_t idesc = tc::idesc_bf16_f32(128, N);
             constexpr uint32_t kLboB = N * 16;
             uint32_t it = 0, tl = 0;
             bool ok = true, pending = false;
-            if (RES && ntiles > static_cast<int>(blockIdx.x) &&
-                !tc::mbar_wait(&bars.wfull[0], 0, abort_flag)) {
+            if (RES && ntiles > static_cast<int>(blockIdx.x) && !wait(&bars.wfull[0], 0)) {
                 fail();
                 ok = false;
             }
             for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tl) {
                 const int acc = tl & 1;
-                if (!tc::mbar_wait(&bars.acce[acc], ((tl >> 1) & 1u) ^ 1u, abort_flag)) {
+                if (!wait(&bars.acce[acc], ((tl >> 1) & 1u) ^ 1u)) {
                     fail();
                     ok = false;
                     break;
@@ -542,21 +551,22 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
                     // reset the TR accumulator rows
                     const uint64_t zd = tc::smem_desc(tc::smem_u32(base + C::kZeroOff),
                                                       C::kZeroRows * 16, 128);
-                    tc::mma_bf16(d0, zd, zd, tc::idesc_bf16_f32(128, TR * N), 0u);
+                    tc::mma_bf16(d0, zd, zd, tc::idesc_bf16_f32(128, TR * N), 0u, lead);
                 }
                 for (int c = 0; c < kchunks; ++c, ++it) {
                     const int s = static_cast<int>(it % NS);
                     const uint32_t ph = (it / NS) & 1u;
-                    if (!tc::mbar_wait(&bars.full[s], ph, abort_flag) ||
-                        (!RES && !tc::mbar_wait(&bars.wfull[s], ph, abort_flag))) {
+                    if (!wait(&bars.full[s], ph) || (!RES && !wait(&bars.wfull[s], ph))) {
                         fail();
                         ok = false;
                         break;
                     }
                     tc::tc_fence_after();
                     const uint32_t a_base = tc::smem_u32(stages + s * C::kStage);
-                    const uint32_t b_base =
-                        RES ? tc::smem_u32(wres + c * C::kB) : a_base + C::kA;
+                    const uint64_t a_desc = tc::smem_desc_sw32(a_base);
+                    const uint64_t b_desc =
+                        tc::smem_desc(RES ? tc::smem_u32(wres + c * C::kB) : a_base + C::kA,
+                                      C::kStack ? 3 * N * 16 : kLboB, 128);
                     if (C::kStack) {
                         // halo row h feeds output rows h-2, h-1, h through the
                         // stacked weights [dy = 2; dy = 1; dy = 0] of its dx tap;
@@ -564,42 +574,41 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
                         // the stacked weights, fewer MMA columns)
 #pragma unroll
                         for (int dx = 0; dx < 3; ++dx) {
-                            const uint32_t bdx = b_base + dx * 2 * 3 * N * 16;
 #pragma unroll
                             for (int h = 0; h < TR + 2; ++h) {
                                 const int rlo = h - 2 < 0 ? 0 : h - 2;   // first row fed
                                 const int rhi = h < TR - 1 ? h : TR - 1;  // last row fed
                                 const int k0 = rlo - (h - 2);             // its dy block
                                 const uint64_t bd =
-                                    tc::smem_desc(bdx + k0 * N * 16, 3 * N * 16, 128);
+                                    b_desc + tc::desc_offset((dx * 6 + k0) * N * 16);
                                 const uint64_t ad =
-                                    tc::smem_desc_sw32(a_base + (h * kPitch + dx) * 32);
+                                    a_desc + tc::desc_offset((h * kPitch + dx) * 32);
                                 tc::mma_bf16(d0 + rlo * N, ad, bd,
-                                             tc::idesc_bf16_f32(128, (rhi - rlo + 1) * N), 1u);
+                                             tc::idesc_bf16_f32(128, (rhi - rlo + 1) * N), 1u,
+                                             lead);
                             }
                         }
                     } else {
 #pragma unroll
                         for (int tap = 0; tap < 9; ++tap) {
                             const int dy = tap / 3, dx = tap % 3;
-                            const uint64_t bd =
-                                tc::smem_desc(b_base + tap * 2 * N * 16, kLboB, 128);
+                            const uint64_t bd = b_desc + tc::desc_offset(tap * 2 * N * 16);
 #pragma unroll
                             for (int r = 0; r < TR; ++r) {
                                 const uint64_t ad =
-                                    tc::smem_desc_sw32(a_base + ((r + dy) * kPitch + dx) * 32);
-                                tc::mma_bf16(d0 + r * N, ad, bd, idesc, (c | tap) != 0);
+                                    a_desc + tc::desc_offset(((r + dy) * kPitch + dx) * 32);
+                                tc::mma_bf16(d0 + r * N, ad, bd, idesc, (c | tap) != 0, lead);
                             }
                         }
                     }
                     pending = true;
-                    tc::mma_commit(&bars.empty[s]);
+                    tc::mma_commit(&bars.empty[s], lead);
                 }
                 if (!ok) break;
-                tc::mma_commit(&bars.accf[acc]);
+                tc::mma_commit(&bars.accf[acc], lead);
             }
             if (!ok && pending) {
-                tc::mma_commit(&bars.drain);
+                tc::mma_commit(&bars.drain, lead);
                 (void)tc::mbar_wait(&bars.drain, 0, nullptr);
             }
         }
@@ -784,8 +793,13 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
                                 buf[e * 32 + lane] = __uint_as_float(v[e]) + sbias[j0 + e];
                             tc::fence_proxy_async();
                             __syncwarp();
-                            if (lane == 0 && y < a.H && x0 + sub * 32 < a.W)
-                                tma_store_planes(&omap, buf, x0 + sub * 32, y, j0, b);
+                            if (lane == 0) {
+                                if (y < a.H && x0 + sub * 32 < a.W)
+                                    tma_store_planes(&omap, buf, x0 + sub * 32, y, j0, b);
+                                // a group per block, or a block outside the image would
+                                // shift the count of stores still to wait for
+                                tma_store_commit();
+                            }
                             ++eblk;
                         }
                         tc::tmem_wait_ld();
@@ -957,11 +971,13 @@ bool getenv_disable_tma_in() {
 //
 // The expansion (a thread per coarse piece, up to four 16-byte stores) bounded
 // these layers, the largest of the network: 96 -> 32 channels at 3840 x 2160
-// 550 -> 418 us, 192 -> 64 at 1920 x 1080 335 -> 317 us (of the same 4K forward).
+// 550 -> 418 us, 192 -> 64 at 1920 x 1080 335 -> 308 us (of the same 4K forward; 317 us with both
+// phases handed over together).
 //
 // A tile is TR x 256 pixels.  Accumulators take 2 TR N columns: double-buffered
 // for N = 32, one set for N = 64 (half-height tiles with two sets would fetch the
-// streamed weights twice as often, and L2 is what they are close to).
+// streamed weights twice as often, and L2 is what they are close to), whose phases
+// are handed over one by one: phase 0 is read while phase 1 of the last chunk runs.
 // Warps 0-3 and 4-7 are the epilogues of phase 0 and 1, warp 8 issues the MMAs,
 // warp 9 the copies.
 template <int N, bool RES>
@@ -986,7 +1002,8 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
     unsigned char *wres = base + C::kWOff;
     unsigned char *stages = base + C::kStagesOff;
     float *sbias = reinterpret_cast<float *>(base + C::kBiasOff);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // known to be the warp's
 
     const int tiles_x = (a.W + 2 * kTileX - 1) / (2 * kTileX);
     const int tiles_y = (a.H + TR - 1) / TR;
@@ -1003,7 +1020,7 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
         }
         for (int i = 0; i < 2; ++i) {
             tc::mbar_init(&bars.accf[i], 1);
-            tc::mbar_init(&bars.acce[i], 256);
+            tc::mbar_init(&bars.acce[i], kSets == 2 ? 256 : 128);
         }
         tc::mbar_init(&bars.drain, 1);
         bars.abort = 0;
@@ -1082,28 +1099,40 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
         __syncwarp();
     } else if (warp == 8) {
         // -------------------------------------------------------- MMA issuer
-        if (lane == 0) {
+        {
+            // warp-uniform, as in conv3x3_kernel
+            const uint32_t lead = tc::elect_one();
+            auto wait = [&](uint64_t *bar, uint32_t parity) {
+                return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort_flag));
+            };
             uint32_t it = 0, tl = 0;
             bool ok = true, pending = false;
-            if (RES && static_cast<int>(blockIdx.x) < ntiles &&
-                !tc::mbar_wait(&bars.wfull[0], 0, abort_flag)) {
+            if (RES && static_cast<int>(blockIdx.x) < ntiles && !wait(&bars.wfull[0], 0)) {
                 fail();
                 ok = false;
             }
             for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tl) {
                 const int acc = kSets == 2 ? tl & 1 : 0;
-                if (!tc::mbar_wait(&bars.acce[acc], ((tl / kSets) & 1u) ^ 1u, abort_flag)) {
+                const uint32_t free_parity = ((tl / kSets) & 1u) ^ 1u;
+                const uint32_t d0 = tmem + acc * 2 * kPhase;
+                // resets the accumulators of a phase, once the epilogue that reads them
+                // (of both phases with two sets) is through with them
+                auto begin = [&](int phase) {
+                    if (!wait(&bars.acce[kSets == 2 ? acc : phase], free_parity))
+                        return false;
+                    tc::tc_fence_after();
+                    pending = true;
+                    const uint64_t zd =
+                        tc::smem_desc(tc::smem_u32(base + C::kZeroOff), C::kZeroRows * 16, 128);
+                    tc::mma_bf16(d0 + phase * kPhase, zd, zd, tc::idesc_bf16_f32(128, kPhase), 0u,
+                                 lead);
+                    return true;
+                };
+                if (!begin(0) || (kSets == 2 && !begin(1))) {
                     fail();
                     ok = false;
                     break;
                 }
-                tc::tc_fence_after();
-                const uint32_t d0 = tmem + acc * 2 * kPhase;
-                // reset the accumulators of both phases
-                const uint64_t zd =
-                    tc::smem_desc(tc::smem_u32(base + C::kZeroOff), C::kZeroRows * 16, 128);
-                tc::mma_bf16(d0, zd, zd, tc::idesc_bf16_f32(128, kPhase), 0u);
-                tc::mma_bf16(d0 + kPhase, zd, zd, tc::idesc_bf16_f32(128, kPhase), 0u);
                 for (int c = 0; c < kchunks; ++c) {
                     // the two stages of a skip chunk (its even and odd columns; the
                     // first brings the weights) or the one of an upsampled chunk
@@ -1111,22 +1140,22 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
                     const int s = static_cast<int>(it % NS);
                     const uint32_t ph = (it / NS) & 1u;
                     const int s1 = static_cast<int>((it + 1) % NS);
-                    if (!tc::mbar_wait(&bars.full[s], ph, abort_flag) ||
-                        (!RES && !tc::mbar_wait(&bars.wfull[s], ph, abort_flag)) ||
-                        (skip &&
-                         !tc::mbar_wait(&bars.full[s1], ((it + 1) / NS) & 1u, abort_flag))) {
+                    if (!wait(&bars.full[s], ph) || (!RES && !wait(&bars.wfull[s], ph)) ||
+                        (skip && !wait(&bars.full[s1], ((it + 1) / NS) & 1u))) {
                         fail();
                         ok = false;
                         break;
                     }
                     tc::tc_fence_after();
-                    const uint32_t even = tc::smem_u32(stages + s * C::kStage);
-                    const uint32_t odd = tc::smem_u32(stages + s1 * C::kStage);
-                    const uint32_t b_base = RES ? tc::smem_u32(wres + c * C::kB) : even + C::kA;
+                    const uint32_t a_base = tc::smem_u32(stages + s * C::kStage);
+                    const uint64_t even = tc::smem_desc_sw32(a_base);
+                    const uint64_t odd = tc::smem_desc_sw32(tc::smem_u32(stages + s1 * C::kStage));
+                    const uint64_t b_desc =
+                        tc::smem_desc(RES ? tc::smem_u32(wres + c * C::kB) : a_base + C::kA,
+                                      3 * N * 16, 128);
                     // tap dx of a phase from the staged columns starting at `col`
                     // (0: xc0 - 1); rows as in conv3x3_kernel
-                    auto taps = [&](int phase, int dx, uint32_t rows, int col, bool up) {
-                        const uint32_t bdx = b_base + dx * 2 * 3 * N * 16;
+                    auto taps = [&](int phase, int dx, uint64_t rows, int col, bool up) {
 #pragma unroll
                         for (int h = 0; h < TR + 2; ++h) {
                             const int rlo = h - 2 < 0 ? 0 : h - 2;
@@ -1134,9 +1163,9 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
                             const int k0 = rlo - (h - 2);
                             const int row = up ? (h + 1) >> 1 : h;
                             tc::mma_bf16(d0 + phase * kPhase + rlo * N,
-                                         tc::smem_desc_sw32(rows + (row * kPitch + col) * 32),
-                                         tc::smem_desc(bdx + k0 * N * 16, 3 * N * 16, 128),
-                                         tc::idesc_bf16_f32(128, (rhi - rlo + 1) * N), 1u);
+                                         rows + tc::desc_offset((row * kPitch + col) * 32),
+                                         b_desc + tc::desc_offset((dx * 6 + k0) * N * 16),
+                                         tc::idesc_bf16_f32(128, (rhi - rlo + 1) * N), 1u, lead);
                         }
                     };
                     // dx = 0, 1, 2 for each phase, as in conv3x3_kernel: the same sums
@@ -1144,27 +1173,35 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
                         taps(0, 0, odd, 0, false);
                         taps(0, 1, even, 1, false);
                         taps(0, 2, odd, 1, false);
-                        taps(1, 0, even, 1, false);
-                        taps(1, 1, odd, 1, false);
-                        taps(1, 2, even, 2, false);
                     } else {
                         taps(0, 0, even, 0, true);
                         taps(0, 1, even, 1, true);
                         taps(0, 2, even, 1, true);
+                    }
+                    if (kSets == 1 && c == kchunks - 1) tc::mma_commit(&bars.accf[0], lead);
+                    if (kSets == 1 && c == 0 && !begin(1)) {
+                        fail();
+                        ok = false;
+                        break;
+                    }
+                    if (skip) {
+                        taps(1, 0, even, 1, false);
+                        taps(1, 1, odd, 1, false);
+                        taps(1, 2, even, 2, false);
+                    } else {
                         taps(1, 0, even, 1, true);
                         taps(1, 1, even, 1, true);
                         taps(1, 2, even, 2, true);
                     }
-                    pending = true;
-                    tc::mma_commit(&bars.empty[s]);
-                    if (skip) tc::mma_commit(&bars.empty[s1]);
+                    tc::mma_commit(&bars.empty[s], lead);
+                    if (skip) tc::mma_commit(&bars.empty[s1], lead);
                     it += skip ? 2 : 1;
                 }
                 if (!ok) break;
-                tc::mma_commit(&bars.accf[acc]);
+                tc::mma_commit(&bars.accf[kSets == 2 ? acc : 1], lead);
             }
             if (!ok && pending) {
-                tc::mma_commit(&bars.drain);
+                tc::mma_commit(&bars.drain, lead);
                 (void)tc::mbar_wait(&bars.drain, 0, nullptr);
             }
         }
@@ -1185,7 +1222,8 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
             const int acc = kSets == 2 ? tl & 1 : 0;
             const int b = t / per_img, r = t - b * per_img;
             const int y0 = (r / tiles_x) * TR, xw = (r % tiles_x) * kTileX + sub * 32;
-            if (!tc::mbar_wait(&bars.accf[acc], (tl / kSets) & 1u, abort_flag)) {
+            const int bar = kSets == 2 ? acc : phase;
+            if (!tc::mbar_wait(&bars.accf[bar], (tl / kSets) & 1u, abort_flag)) {
                 fail();
                 break;
             }
@@ -1231,7 +1269,7 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
                 tc::tmem_wait_ld();
             }
             tc::tc_fence_before();
-            tc::mbar_arrive(&bars.acce[acc]);
+            tc::mbar_arrive(&bars.acce[bar]);
         }
         if (lane == 0 && eblk) tma_store_wait_all();
     }

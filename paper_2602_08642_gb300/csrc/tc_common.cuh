@@ -158,6 +158,13 @@ __device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t saddr) {
            (static_cast<uint64_t>(256 >> 4) << 32) | (1ull << 46) | (6ull << 61);
 }
 
+// What moving the start address of a descriptor by `bytes` (a multiple of 16) adds
+// to it: the address field has 14 bits of 16 bytes, more than shared memory, so an
+// operand's descriptors are one addition from the first one's.
+__host__ __device__ constexpr uint64_t desc_offset(int bytes) {
+    return static_cast<uint64_t>(bytes >> 4);
+}
+
 // Instruction descriptor of kind::f16: D in FP32, A and B in BF16, both
 // K-major, M = 128, N (multiple of 16, <= 256).
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
@@ -165,21 +172,31 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
            (static_cast<uint32_t>(M >> 4) << 24);
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, issued by one thread.
+// One lane of the calling warp (all lanes call it): 1 for that lane, else 0.
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t lead;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(lead));
+    return lead;
+}
+// D[tmem] (+)= A[smem] * B[smem]^T, in warp-uniform code: issued by the lane with
+// `lead` set.
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate) {
+                                         uint32_t idesc, uint32_t accumulate, uint32_t lead) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead)
         : "memory");
 }
-// Arrives once on `bar` when every tcgen05 operation issued so far by this
-// thread has completed.
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
+// Arrives once on `bar` when every tcgen05 operation issued so far by the lane with
+// `lead` set has completed.
+__device__ __forceinline__ void mma_commit(uint64_t *bar, uint32_t lead) {
     asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            smem_u32(bar))
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
+            smem_u32(bar)),
+        "r"(lead)
         : "memory");
 }
 

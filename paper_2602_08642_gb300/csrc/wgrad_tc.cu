@@ -121,7 +121,8 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
     unsigned char *base = smem_raw + ((512u - (tc::smem_u32(smem_raw) & 511u)) & 511u);
     WBars &bars = *reinterpret_cast<WBars *>(base);
     unsigned char *stages = base + kHeader;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // known to be the warp's
     const int split = blockIdx.x, splits = gridDim.x;
     const int ci = blockIdx.y / 3, dy = blockIdx.y % 3;
     const int N = a.nco * kBlk;
@@ -207,13 +208,15 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
         __syncwarp();
     } else if (warp == 5) {
         // -------------------------------------------------------- MMA issuer
-        if (lane == 0) {
+        {
+            // warp-uniform code, one lane issues: descriptors in uniform registers
+            const uint32_t lead = tc::elect_one();
             const uint32_t idesc = idesc_mn(N);
             bool ok = true;
             int s = 0;
             uint32_t ph = 0, acc = 0;
             for (int g = 0; g < nstages; ++g) {
-                if (!tc::mbar_wait(&bars.full[s], ph, abort_flag)) {
+                if (!__all_sync(0xffffffffu, tc::mbar_wait(&bars.full[s], ph, abort_flag))) {
                     fail();
                     ok = false;
                     break;
@@ -225,21 +228,21 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
                     const uint64_t ad = desc_mn64(at, 64), bd = desc_mn64(at + kXSlot, kGBytes);
 #pragma unroll
                     for (int ks = 0; ks < kPX / 16; ++ks) {
-                        tc::mma_bf16(tmem, ad + ((ks * 16 * 64) >> 4), bd + ((ks * 16 * 64) >> 4),
-                                     idesc, acc);
+                        tc::mma_bf16(tmem, ad + tc::desc_offset(ks * 16 * 64),
+                                     bd + tc::desc_offset(ks * 16 * 64), idesc, acc, lead);
                         acc = 1;
                     }
                 }
-                tc::mma_commit(&bars.empty[s]);
+                tc::mma_commit(&bars.empty[s], lead);
                 if (++s == a.ns) {
                     s = 0;
                     ph ^= 1u;
                 }
             }
             if (ok) {
-                tc::mma_commit(&bars.accf);
+                tc::mma_commit(&bars.accf, lead);
             } else if (acc) {
-                tc::mma_commit(&bars.drain);
+                tc::mma_commit(&bars.drain, lead);
                 (void)tc::mbar_wait(&bars.drain, 0, nullptr);
             }
         }
