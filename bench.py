@@ -45,11 +45,11 @@ UNIT = "Mpix/s"
 # which the hash checks.
 LEVEL0_TRAFFIC = {
     "workload": "1080p",
-    "bytes_per_launch": 546_309_888,  # median of three captured launches
+    "bytes_per_launch": 546_430_208,  # median of three captured launches
     "sources": ("paper_2602_08642_gb300/csrc/reconstruct_tma.cu",
                 "paper_2602_08642_gb300/csrc/recon_common.cuh",
                 "paper_2602_08642_gb300/csrc/spp_internal.cuh"),
-    "sha256": "77c46e86595ef9af08362c1c849d2c0d56db33ed2a3145daae4acaee3ca1e294",
+    "sha256": "7908ab7fb66e67405833488d86037394361901286f3d54a0064cc454f0c44b3f",
 }
 
 

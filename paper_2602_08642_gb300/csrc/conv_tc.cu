@@ -982,8 +982,9 @@ bool getenv_disable_tma_in() {
 //
 // The expansion (a thread per coarse piece, up to four 16-byte stores) bounded
 // these layers, the largest of the network: 96 -> 32 channels at 3840 x 2160
-// 550 -> 418 us, 192 -> 64 at 1920 x 1080 335 -> 308 us (of the same 4K forward; 317 us with both
-// phases handed over together).
+// 550 -> 418 us, 192 -> 64 at 1920 x 1080 335 -> 308 us (of the same 4K forward; 317 us
+// with both phases handed over together), and 362 and 293 us with the issue from
+// warp-uniform code.
 //
 // A tile is TR x 256 pixels.  Accumulators take 2 TR N columns: double-buffered
 // for N = 32, one set for N = 64 (half-height tiles with two sets would fetch the
@@ -1297,10 +1298,11 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
 template <int N, bool RES>
 bool launch_up(const ConvArgs &a, cudaStream_t stream, int *rc) {
     using C = Cfg<N, RES>;
-    // A tile of 256 columns takes 1.5 (N = 32) or 1.77 (N = 64) times as long as one
-    // of 128 columns of the expanding kernel (the times above over their tiles), so
-    // the rounds of tiles per SM decide: padding columns and a last round that is
-    // nearly empty can cost more than the expansion.
+    // A tile of 256 columns took 1.5 (N = 32) or 1.77 (N = 64) times as long as one
+    // of 128 columns of the expanding kernel when this line was drawn (418 and 308 us
+    // against 550 and 335 us, over their tiles; with warp-uniform issue 362 and 293
+    // us), so the rounds of tiles per SM decide: padding columns and a last round that
+    // is nearly empty can cost more than the expansion.
     const int64_t rows = static_cast<int64_t>(a.B) * ((a.H + C::TR - 1) / C::TR), sms = sm_count();
     const int64_t ntiles = rows * ((a.W + 2 * kTileX - 1) / (2 * kTileX));
     const int64_t rounds = (ntiles + sms - 1) / sms;
