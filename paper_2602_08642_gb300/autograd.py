@@ -61,9 +61,12 @@ class Reconstruct(torch.autograd.Function):
         new = lambda ts: [torch.empty_like(x) for x in ts]
         g_layers, g_logits, g_hats = new(layers), new(logits), [None] + new(hats[1:])
         g_warped = torch.empty_like(hdr) if warped is not None else None
+        if g_hdr is not None:
+            g_hdr = g_hdr.contiguous()
+            if g_hdr.data_ptr() % 16:  # a view into a larger tensor
+                g_hdr = g_hdr.clone()
         B.check(B.spp_reconstruct_pyramid_backward(
-            layers, logits, hats, warped, mask, hdr, W, H, ctx.tm,
-            None if g_hdr is None else g_hdr.contiguous(),
+            layers, logits, hats, warped, mask, hdr, W, H, ctx.tm, g_hdr,
             None if g_ldr is None else g_ldr.contiguous(), torch.empty_like(hdr), g_layers,
             g_logits, g_hats, g_warped), "reconstruct backward")
         return (None, None, g_warped, None, *g_layers, *g_logits)

@@ -68,3 +68,25 @@ def test_pyramid_calls_equal_level_calls(spp, W, H, L, temporal, use_hdr, use_ld
             out = gc
     if temporal:
         assert torch.equal(gw, gw1)
+
+
+def test_gradient_views_of_any_alignment(spp):
+    """The gradient of the HDR output may be a view that starts between 16-byte
+    boundaries, or an expanded one."""
+    from paper_2602_08642_gb300 import autograd
+    W, H, L = 36, 12, 2
+    g = torch.Generator(device="cuda").manual_seed(5)
+    leaf = lambda *s: torch.randn(*s, generator=g, device="cuda").requires_grad_(True)
+    layers = [leaf(3, H >> l, W >> l) for l in range(L)]
+    logits = [leaf(29, H, W), leaf(25, H // 2, W // 2)]
+    hdr, _ = autograd.Reconstruct.apply(L, spp.binding.make_tonemap(), None, None, *layers, *logits)
+    inputs = layers + logits
+    grads = lambda go: torch.autograd.grad(hdr, inputs, go, retain_graph=True)
+    buf = torch.randn(3 * H * W + 1, generator=g, device="cuda")
+    view = buf[1:].view(3, H, W)
+    assert view.data_ptr() % 16
+    for a, b in zip(grads(view), grads(view.clone())):
+        assert torch.equal(a, b)
+    one = torch.ones(1, device="cuda")
+    for a, b in zip(grads(one.expand(3, H, W)), grads(torch.ones_like(hdr))):
+        assert torch.equal(a, b)
