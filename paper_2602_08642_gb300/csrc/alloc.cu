@@ -921,7 +921,9 @@ offsets_kernel(const int32_t *__restrict__ counts, long long N, const int *__res
 // roundings of a + c d move s by at most 2^-52 s.  So the FP64 result lies
 // within `margin` of X, and where both ends of that interval round to the
 // same q (or to the same FP32 s) that is the FP64 result's; else, and where
-// the shift leaves its range, the FP64 sequence runs.
+// the shift leaves its range or the sum its 64 bits (at r = 0 the product term is
+// 2^62 to 2^64, a pixel of up to 4096 samples before its uniform share), the FP64
+// sequence runs.
 struct FixCoef {
     unsigned long long c64, a52;
     int r0, ok;
@@ -966,7 +968,7 @@ __device__ __forceinline__ SysPixel sys_pixel(float d, const FixCoef &k) {
     const unsigned long long lo = X - margin, hi = X + margin;
     SysPixel o;
     o.q = static_cast<long long>((lo + (1ull << 19)) >> 20);
-    bool ok = k.ok && r >= 0 && X >= margin && X < (1ull << 62) &&
+    bool ok = k.ok && r >= 0 && X >= k.a52 && X >= margin && X < (1ull << 62) &&
               o.q == static_cast<long long>((hi + (1ull << 19)) >> 20);
     o.s = 0.0f;
     if (WITH_S) {

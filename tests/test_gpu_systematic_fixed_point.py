@@ -55,3 +55,31 @@ def test_integer_path_matches_fp64_path(spp, W, H, kind, budget, phi, lam, hard)
     for a, b in zip(*got):
         assert np.array_equal(a.view(np.uint32 if a.dtype == np.float32 else a.dtype),
                               b.view(np.uint32 if b.dtype == np.float32 else b.dtype))
+
+
+@pytest.mark.parametrize("N,budget,phi,base,spikes", [
+    (1000, 600.0, 0.5, 297.78, [4020.0]),
+    (1000, 600.0, 0.5, 297.0, [3000.0, 3790.0, 3800.0, 3900.0, 4000.0, 4050.0]),
+    (64, 1500.0, 0.6, 600.0, [3900.0, 4000.0, 4090.0]),
+    (5000, 900.0, 0.9, 90.0, [3100.0, 3300.0, 4000.0, 4095.0]),
+    (333, 1023.0, 0.9, 66.6, [4000.0, 4060.0, 4095.0])])
+def test_pixels_around_4096_samples(spp, N, budget, phi, base, spikes):
+    """A uniform share on top of a product just under 4096 passes 2^64 in units of
+    2^-52: those pixels, and their neighbours below and above, are the FP64
+    sequence's, and the frame keeps its exact total."""
+    d = torch.full((1, N), base, device="cuda")
+    for k, v in enumerate(spikes):
+        d[0, (k + 1) * N // (len(spikes) + 1)] = v
+    got = []
+    for exact in (False, True):
+        fr = spp.Frame(N, 1, 1, max_budget=budget + 1.0, capacity=int((budget + 2) * N) + 64)
+        fr.sample_pixel.fill_(-1)
+        fr.alloc_systematic(d, spp.binding.make_params(budget, uniform_fraction=phi, seed=11,
+                                                       frame=2, exact_fp64=exact))
+        assert fr.check_status() == 0
+        got.append([t.cpu().numpy().copy() for t in (fr.counts, fr.offsets, fr.sample_pixel, fr.s,
+                                                     fr.holdout_w, fr.total)])
+    assert got[1][3].max() > 3000 and abs(int(got[0][5][0]) - round(budget * N)) <= 1
+    for a, b in zip(*got):
+        assert np.array_equal(a.view(np.uint32 if a.dtype == np.float32 else a.dtype),
+                              b.view(np.uint32 if b.dtype == np.float32 else b.dtype))
