@@ -850,7 +850,8 @@ int spp_render_synthetic_batch(int B, const float *const *clean, const int32_t *
 int spp_splat_samples_batch(int B, const int32_t *offsets, const float *rgb, const float *s,
                             const float *holdout_w, int64_t capacity, int W, int H, int L,
                             float *const *layers, cudaStream_t stream);
-/* logits [B][C][Hl][Wl] with C at least the planes that the level uses */
+/* logits [B][C][Hl][Wl] with C at least the planes that the level uses; an expired
+ * wait is recorded with every image that has pixels left unwritten for it */
 int spp_reconstruct_level_batch(int B, const float *noisy, const float *logits, int C,
                                 const float *coarse, const float *warped_prev, const uint8_t *mask,
                                 int Wl, int Hl, const spp_tonemap *tm, float *out, float *out_ldr,

@@ -39,7 +39,7 @@ constexpr int kSinglePassMaxTiles = 64;
 
 // per-image strides of a batched map (spp_alloc_sample_map_batch)
 constexpr int kOffsetsPad = SPP_BATCH_OFFSETS_PAD;
-constexpr int kTotalStride = 2, kStatusStride = 4;
+constexpr int kTotalStride = 2;
 
 constexpr unsigned long long kFlagAgg = 1ull << 62;
 constexpr unsigned long long kFlagInc = 2ull << 62;

@@ -219,11 +219,17 @@ recon_tma_kernel(const __grid_constant__ CUtensorMap map_logits,
         for (int k = 0; k < NS && k < my_tiles; ++k) issue(k);
     __syncthreads();
 
-    // After a wait gave up: record it, wait (bounded) for the copies this CTA
-    // issued on every stage, and let the caller return.  Every wait in this
-    // kernel is bounded, so the other warps reach the same point.
-    auto abort = [&]() {
-        set_status(status, SPP_ERR_TIMEOUT);
+    // After a wait for tile k gave up: record it with every image that has a tile
+    // this CTA leaves out, wait (bounded) for the copies this CTA issued on every
+    // stage, and let the caller return.  Every wait in this kernel is bounded, so
+    // the other warps reach the same point.
+    auto abort = [&](int k) {
+        if (BATCH && status) {
+            for (; k < my_tiles; ++k)
+                set_status(status + image_of(k) * kStatusStride, SPP_ERR_TIMEOUT);
+        } else {
+            set_status(status, SPP_ERR_TIMEOUT);
+        }
         if (lane == 0)
             for (int s = 0; s < NS; ++s) {
                 const int u = *reinterpret_cast<volatile int *>(&uses[s]);
@@ -296,7 +302,7 @@ recon_tma_kernel(const __grid_constant__ CUtensorMap map_logits,
         int x0, y0;
         tile_xy(k, x0, y0);
         if (!mbar_wait_bounded(&full[s], static_cast<uint32_t>((k / NS) & 1))) {
-            abort();
+            abort(k);
             return;
         }
         bool use_tn = false;
@@ -407,7 +413,7 @@ recon_tma_kernel(const __grid_constant__ CUtensorMap map_logits,
         // rendezvous of the pixel row's two warps (bounded)
         mbar_arrive(&pair[wr]);
         if (!mbar_wait_bounded(&pair[wr], static_cast<uint32_t>(k & 1))) {
-            abort();
+            abort(k);
             return;
         }
         const int x = x0 + tx, y = y0 + ty;

@@ -73,6 +73,8 @@ inline void launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
 // per-image stream keys and input images travel in the kernel's parameters.
 // Larger batches are launched in parts of kMaxBatch images.
 constexpr int kMaxBatch = 16;
+// int32 words between the status words of a batch's images
+constexpr int kStatusStride = 4;
 // (kernels take them as __grid_constant__, so that indexing by the image reads
 // constant memory; a plain parameter would be copied to local memory first)
 struct StreamKeys {

@@ -437,7 +437,7 @@ class Renderer:
                 self.all[f"hats{l + 1}"] if l + 1 < LEVELS else None, warped if l == 0 else None,
                 self.mask if l == 0 and warped is not None else None, self.W >> l, self.H >> l,
                 self.tm if l == 0 else None, self.all[f"hats{l}"] if l else hdr,
-                None if l else ldr), "level")
+                None if l else ldr, self.batch.status), "level")
 
     def previous_frame_all(self, d, logits, cleans, seed: int, frame: int):
         """previous_frame and warp_previous's source for all samples: d

@@ -63,3 +63,37 @@ def test_part_of_a_batch_and_unaligned_sizes(Lm):
     assert np.isfinite(Lm.Trainer(theta, 1, 20, 0.4).step(odd[:1], 1))
     with pytest.raises(Lm.B.SppError):
         Lm.Trainer(theta, 2, 20, 0.4).step(odd, 1)
+
+
+def test_expired_waits_reach_the_status_of_their_images(Lm):
+    """A reconstruction tile whose copies never arrive: the status of every image
+    with a tile that its block then leaves out says so, and no other's."""
+    B, n, W, H = Lm.B, 3, 128, 128  # 64 tiles of 64 x 4 pixels per image
+    tiles = (W // 64) * (H // 4)
+    G = min(torch.cuda.get_device_properties(0).multi_processor_count, n * tiles)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    noisy, logits = (torch.randn(n, c, H, W, generator=g, device="cuda") for c in (3, 25))
+    out, st = torch.empty_like(noisy), torch.zeros(n, 4, dtype=torch.int32, device="cuda")
+    for stalled in (30, tiles + 1, n * tiles - 1):
+        st.zero_()
+        assert B.spp_test_stall_reconstruction(stalled) == 0
+        B.check(B.spp_reconstruct_level_batch(n, noisy, logits, 25, None, None, None, W, H, None,
+                                              out, None, st))
+        left_out = {t // tiles for t in range(stalled, n * tiles, G)}
+        assert [c != 0 for c in st[:, 0].tolist()] == [b in left_out for b in range(n)]
+        assert not st[:, 1:].any()
+
+    # the previous frames of a training step report to their frames
+    rnd = Lm.Renderer(2, 64, 64, 0.25)
+    heads = [torch.zeros(2, c, 64 >> l, 64 >> l, device="cuda") for l, c in enumerate((55, 29, 25))]
+    args = (torch.ones(2, 64, 64, device="cuda"), heads, [torch.ones(3, 64, 64, device="cuda")] * 2,
+            5, 0)
+    assert B.spp_test_stall_reconstruction(5) == 0  # level 2: tiles 4 to 7 are image 1's
+    rnd.previous_frame_all(*args)
+    assert rnd.frames[0].check_status() == 0
+    with pytest.raises(B.SppError) as e:
+        rnd.frames[1].check_status()
+    assert e.value.code == B.SPP_ERR_TIMEOUT
+    rnd.frames[1].clear_status()
+    rnd.previous_frame_all(*args)
+    assert all(fr.check_status() == 0 for fr in rnd.frames)
