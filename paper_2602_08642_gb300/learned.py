@@ -554,8 +554,8 @@ class Trainer:
         return 0.5 * self.lr * (1.0 + math.cos(math.pi * k / self.total_steps))
 
     def step(self, samples: list[FrameData], seed: int) -> float:
-        """One optimisation step on len(samples) == batch samples; returns
-        the mean loss (reading it synchronises)."""
+        """One optimisation step on `samples`, at most as many as the batch holds;
+        returns their mean loss (reading it synchronises)."""
         net, rnd = self.net, self.rnd
         f_prev, f_cur = 2 * self.step_index, 2 * self.step_index + 1
         if self.random_tmo:
@@ -580,12 +580,16 @@ class Trainer:
         net.backward()
         net.adamw(self.current_lr(), self.wd, grad_scale=1.0 / len(samples), betas=self.betas)
         self.step_index += 1
-        return float(sum(rnd.all["loss"][:, 0].tolist())) / len(samples)
+        return float(sum(rnd.all["loss"][:len(samples), 0].tolist())) / len(samples)
 
     def _forward_backward(self, samples, seed: int, f_prev: int, f_cur: int):
-        """step's forward and renderer backward sample by sample (a part of a
-        batch, or images that do not all start on a 16-byte boundary)."""
+        """step's forward and renderer backward sample by sample, for fewer samples
+        than the batch holds: the other images get no gradient.  (Of a size whose
+        heads' images do not all start on a 16-byte boundary, 4 modulo 8, only the
+        first image can be worked on.)"""
         net, rnd = self.net, self.rnd
+        for g in net.g_heads:
+            g[len(samples):].zero_()
         for b, s in enumerate(samples):
             net.features(b, s.gprev["albedo"], s.gprev["normal"], s.gprev["depth"], s.mv, None)
         net.forward()

@@ -97,3 +97,25 @@ def test_expired_waits_reach_the_status_of_their_images(Lm):
     rnd.frames[1].clear_status()
     rnd.previous_frame_all(*args)
     assert all(fr.check_status() == 0 for fr in rnd.frames)
+
+
+@pytest.mark.parametrize("objective", ["l1", "combined"])
+def test_part_of_a_batch_is_that_part_only(Lm, objective):
+    """A step of 2 samples on a trainer of 3, after a step of 3, against the same
+    step on a trainer of 2 in the same state: the third image's gradients and loss
+    of the step before take no part.  The two cut the weight gradients' sums
+    differently, which shows in the 5th digit: 1e-3 of the gradient's norm; an
+    image of the step before is of the norm's own size."""
+    theta = torch.from_numpy(inp.unet_params(Lm.layer_table(), seed=5, head_scale=0.3,
+                                             head_bias=inp.fixed_head_bias()))
+    samples = [Lm.FrameData(inp.training_pair(64, seed=50 + k), seed=k) for k in range(3)]
+    a = Lm.Trainer(theta, 3, 64, 0.4, objective=objective)
+    a.step(samples, 900)
+    b = Lm.Trainer(theta, 2, 64, 0.4, objective=objective)
+    for name in ("theta", "m", "v"):
+        getattr(b.net, name).copy_(getattr(a.net, name))
+    b.net.step_count, b.step_index = a.net.step_count, a.step_index
+    b.net.pack()
+    la, lb = a.step(samples[:2], 940), b.step(samples[:2], 940)
+    assert abs(la - lb) <= 1e-5 * lb
+    assert torch.linalg.norm(a.net.grad - b.net.grad) <= 1e-3 * torch.linalg.norm(b.net.grad)
