@@ -528,7 +528,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
             // wait: the warp stays converged, which uniform registers rely on.
             const uint32_t lead = tc::elect_one();
             auto wait = [&](uint64_t *bar, uint32_t parity) {
-                return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort_flag));
+                return tc::mbar_wait_warp(bar, parity, abort_flag);
             };
             constexpr uint32_t idesc = tc::idesc_bf16_f32(128, N);
             constexpr uint32_t kLboB = N * 16;
@@ -681,7 +681,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
                     m[q] = inside ? __ldg(src + q) : make_uint4(0, 0, 0, 0);
             };
             if (a.epi_mode == kEpiMaskBF16) load_mask(row_lo * kRowBlocks, mask[0]);
-            if (!tc::mbar_wait(&bars.accf[acc], (tl >> 1) & 1u, abort_flag)) {
+            if (!tc::mbar_wait_warp(&bars.accf[acc], (tl >> 1) & 1u, abort_flag)) {
                 fail();
                 break;
             }
@@ -1115,7 +1115,7 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
             // warp-uniform, as in conv3x3_kernel
             const uint32_t lead = tc::elect_one();
             auto wait = [&](uint64_t *bar, uint32_t parity) {
-                return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort_flag));
+                return tc::mbar_wait_warp(bar, parity, abort_flag);
             };
             uint32_t it = 0, tl = 0;
             bool ok = true, pending = false;
@@ -1235,7 +1235,7 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
             const int b = t / per_img, r = t - b * per_img;
             const int y0 = (r / tiles_x) * TR, xw = (r % tiles_x) * kTileX + sub * 32;
             const int bar = kSets == 2 ? acc : phase;
-            if (!tc::mbar_wait(&bars.accf[bar], (tl / kSets) & 1u, abort_flag)) {
+            if (!tc::mbar_wait_warp(&bars.accf[bar], (tl / kSets) & 1u, abort_flag)) {
                 fail();
                 break;
             }

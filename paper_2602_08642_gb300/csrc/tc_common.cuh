@@ -77,6 +77,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, const 
     }
 }
 
+// The same for a converged warp whose lanes go on together (warp-wide loads, votes
+// and synchronisation follow): one answer for all lanes, which by themselves may
+// expire, or see *abort, at different times, and would part.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity,
+                                               const volatile int *abort) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
+}
+
 // ------------------------------------------------------------ bulk copy
 // 1-D global -> shared copy completing on `bar` (16-byte aligned, size a
 // multiple of 16).

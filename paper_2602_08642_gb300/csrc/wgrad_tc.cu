@@ -216,7 +216,7 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
             int s = 0;
             uint32_t ph = 0, acc = 0;
             for (int g = 0; g < nstages; ++g) {
-                if (!__all_sync(0xffffffffu, tc::mbar_wait(&bars.full[s], ph, abort_flag))) {
+                if (!tc::mbar_wait_warp(&bars.full[s], ph, abort_flag)) {
                     fail();
                     ok = false;
                     break;
@@ -262,7 +262,7 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
             int s = 0;
             uint32_t ph = 0;
             for (int g = 0; g < nstages; ++g) {
-                if (!tc::mbar_wait(&bars.full[s], ph, abort_flag)) {
+                if (!tc::mbar_wait_warp(&bars.full[s], ph, abort_flag)) {
                     fail();
                     ok = false;
                     break;
@@ -300,7 +300,7 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
                 if (j < a.nco)
                     *reinterpret_cast<float2 *>(pb + j * kBlk) = make_float2(bs[j][0], bs[j][1]);
         }
-        if (ok && !tc::mbar_wait(&bars.accf, 0, abort_flag)) {
+        if (ok && !tc::mbar_wait_warp(&bars.accf, 0, abort_flag)) {
             fail();
             ok = false;
         }
