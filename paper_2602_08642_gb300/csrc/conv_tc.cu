@@ -31,8 +31,9 @@
 // arrival counts and transaction bytes, MMA -> producers via
 // tcgen05.commit).  Every wait is bounded: on expiry the CTA records
 // SPP_ERR_TIMEOUT in the status word, the other roles leave at their next
-// wait, the MMA thread waits for its issued MMAs, the copy thread for its
-// copies in flight, and TMEM is freed before the kernel returns.
+// wait, and TMEM is freed before the kernel returns.  On every path the MMA warp
+// waits for its issued MMAs and the copy thread for its last copies before they
+// leave: another role may have given up on them.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -492,8 +493,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
         // copies must land before the CTA exits)
         cp_async_wait<0>();
         for (; published < it; ++published) publish_lagged(published);
-        if (!ok && ptid == 0) {
-            // wait (bounded, ignoring the abort flag) for the copies still in flight
+        if (ptid == 0) {
+            // wait (bounded, ignoring the abort flag) for the copies still in flight:
+            // those of the last stages, of which the MMA warp may have given up
             if (a.tma_in == 1) {
                 const uint32_t first = it > NS ? it - NS : 0;
                 for (uint32_t k = first; k < it; ++k)
@@ -547,6 +549,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
                 }
                 tc::tc_fence_after();
                 const uint32_t d0 = tmem + acc * C::kAccCols;
+                pending = true;
                 if (C::kStack) {
                     // reset the TR accumulator rows
                     const uint64_t zd = tc::smem_desc(tc::smem_u32(base + C::kZeroOff),
@@ -601,13 +604,12 @@ __global__ void __launch_bounds__(kThreads, 1) conv3x3_kernel(const ConvArgs a,
                             }
                         }
                     }
-                    pending = true;
                     tc::mma_commit(&bars.empty[s], lead);
                 }
                 if (!ok) break;
                 tc::mma_commit(&bars.accf[acc], lead);
             }
-            if (!ok && pending) {
+            if (pending) {
                 tc::mma_commit(&bars.drain, lead);
                 (void)tc::mbar_wait(&bars.drain, 0, nullptr);
             }
@@ -1099,14 +1101,14 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
                     }
                 }
             }
-            if (!ok) {
-                // wait (bounded, ignoring the abort flag) for the copies in flight
-                for (uint32_t k = it > NS ? it - NS : 0; k < it; ++k) {
-                    (void)tc::mbar_wait(&bars.full[k % NS], (k / NS) & 1u, nullptr);
-                    if (!RES) (void)tc::mbar_wait(&bars.wfull[k % NS], (k / NS) & 1u, nullptr);
-                }
-                if (RES) (void)tc::mbar_wait(&bars.wfull[0], 0, nullptr);
+            // wait (bounded, ignoring the abort flag) for the copies in flight, as in
+            // conv3x3_kernel
+            for (uint32_t k = it > NS ? it - NS : 0; k < it; ++k) {
+                (void)tc::mbar_wait(&bars.full[k % NS], (k / NS) & 1u, nullptr);
+                if (!RES) (void)tc::mbar_wait(&bars.wfull[k % NS], (k / NS) & 1u, nullptr);
             }
+            if (RES && static_cast<int>(blockIdx.x) < ntiles)
+                (void)tc::mbar_wait(&bars.wfull[0], 0, nullptr);
         }
         __syncwarp();
     } else if (warp == 8) {
@@ -1212,7 +1214,7 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
                 if (!ok) break;
                 tc::mma_commit(&bars.accf[kSets == 2 ? acc : 1], lead);
             }
-            if (!ok && pending) {
+            if (pending) {
                 tc::mma_commit(&bars.drain, lead);
                 (void)tc::mbar_wait(&bars.drain, 0, nullptr);
             }

@@ -199,11 +199,10 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
                     ph ^= 1u;
                 }
             }
-            // after a wait gave up: the copies of the last stages issued have to
-            // land before the CTA exits
-            if (issued < nstages)
-                for (int k = max(issued - a.ns, 0); k < issued; ++k)
-                    (void)tc::mbar_wait(&bars.full[k % a.ns], (k / a.ns) & 1u, nullptr);
+            // the copies of the last stages issued have to land before the CTA exits,
+            // also where another role gave up on them
+            for (int k = max(issued - a.ns, 0); k < issued; ++k)
+                (void)tc::mbar_wait(&bars.full[k % a.ns], (k / a.ns) & 1u, nullptr);
         }
         __syncwarp();
     } else if (warp == 5) {
@@ -239,9 +238,8 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
                     ph ^= 1u;
                 }
             }
-            if (ok) {
-                tc::mma_commit(&bars.accf, lead);
-            } else if (acc) {
+            if (ok) tc::mma_commit(&bars.accf, lead);
+            if (acc) {
                 tc::mma_commit(&bars.drain, lead);
                 (void)tc::mbar_wait(&bars.drain, 0, nullptr);
             }

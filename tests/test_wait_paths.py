@@ -29,3 +29,16 @@ def test_waits_before_warp_wide_code_have_one_answer_per_warp(name):
     assert alone and alone <= {"bars.empty", "bars.updone", "bars.upfull"}
     together = [bar for fn, bar, _ in waits if fn == "mbar_wait_warp"]
     assert "bars.accf" in together and len(together) >= 3
+
+
+@pytest.mark.parametrize("name", KERNELS)
+def test_copies_and_mmas_are_waited_for_on_every_path(name):
+    """A role that never gave up itself may still have copies or MMAs in flight when
+    another one did; so the waits before it leaves hang on what it issued (`pending`,
+    `acc`, the counts in the loops), not on its own success."""
+    src = _source(name)
+    assert set(re.findall(r"if \(!ok\b[^{;]*[{;]", src)) <= {"if (!ok) break;"}
+    assert not re.search(r"if \(issued\b[^)]*<", src)
+    assert not re.search(r"\belse if \(acc\)", src)
+    drains = re.findall(r"if \((\w+)\) \{\s*tc::mma_commit\(&bars\.drain", src)
+    assert len(drains) == src.count("mma_commit(&bars.drain") and set(drains) <= {"pending", "acc"}
