@@ -197,6 +197,21 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead)
         : "memory");
 }
+// The same with the TMEM lanes 32 i .. 32 i + 31 of every i whose `off` bit is set left
+// as they are (the operand that disables output lanes).
+template <uint32_t OFF>
+__device__ __forceinline__ void mma_bf16_lanes(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
+                                               uint32_t idesc, uint32_t accumulate, uint32_t lead) {
+    constexpr uint32_t m[4] = {OFF & 1 ? ~0u : 0u, OFF & 2 ? ~0u : 0u, OFF & 4 ? ~0u : 0u,
+                               OFF & 8 ? ~0u : 0u};
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%6, %7, %8, %9}, p;\n\t}" ::"r"(
+            d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead), "r"(m[0]), "r"(m[1]),
+        "r"(m[2]), "r"(m[3])
+        : "memory");
+}
 // Arrives once on `bar` when every tcgen05 operation issued so far by the lane with
 // `lead` set has completed.
 __device__ __forceinline__ void mma_commit(uint64_t *bar, uint32_t lead) {

@@ -13,6 +13,11 @@
 //     same bytes at row shifts 0, 1, 2 (the fourth atom is a spare shift whose
 //     32 accumulator rows are not read).
 //   B (N = cout padded to 32): the row of g, one atom per 32 output channels.
+// Past the end of a row g is 0, but the dx = 0 rows still hold the row's last pixel
+// there, and an infinity times 0 is NaN.  So a row's last chunk stops at its last
+// pixel, and where that is inside a K step of 16 (W % 16 != 0) the step is two MMAs:
+// one that leaves out the dx = 0 lanes, one for them alone with the 8 pixels around
+// the edge from a box of the tensor without its last column (kEdgeBytes).
 // A CTA owns one block of 32 input channels, one dy and one share ("split") of
 // the pixel chunks of 64 pixels of a row; its 128 x N accumulator stays in TMEM
 // for the whole kernel and is written once as a partial sum.  A second kernel
@@ -61,6 +66,7 @@ constexpr int kLanes = 3 * kBlk;        // accumulator rows that are read: dx 0,
 constexpr int kXBytes = kHX * 64;                    // one x box
 constexpr int kXSlot = (kXBytes + 511) / 512 * 512;  // its slot (swizzle period)
 constexpr int kGBytes = kPX * 64;                    // one g box
+constexpr int kEdgeBytes = 8 * 64;                   // 8 pixels at the edge of a row
 constexpr int kHeader = 512;
 constexpr int kMaxStages = 3;
 constexpr int kBiasGroups = 8;          // pixel groups of a chunk in the bias sums
@@ -85,6 +91,10 @@ struct WKernelArgs {
     int nci, nco;    // 32-channel blocks of x and of g
     int n0;          // blocks of x that come from the first source
     int ns, nch;     // stages, chunks per stage
+    int steps, rem;  // whole K steps of a row's last chunk, and the pixels after them
+    // places in a chunk of its x box, its edge box (when rem > 0; it starts at pixel
+    // edge_x of the row) and its g boxes
+    int x_off, edge_off, edge_x, g_off;
     float *partial;  // [split][nci][dy][nco * 32][96 rows]
     float *pbias;    // [split][8][nco * 32]
     int32_t *status;
@@ -92,11 +102,11 @@ struct WKernelArgs {
 
 // MN-major operand in the 64-byte swizzle (layout type 4): atoms of 32
 // channels x 8 pixels; atoms along M / N are lbo bytes apart, groups of 8
-// pixels 512 bytes.  The swizzle follows the absolute address (boxes start on
+// pixels sbo bytes.  The swizzle follows the absolute address (boxes start on
 // its 512-byte period), so any pixel may be the first.
-__device__ __forceinline__ uint64_t desc_mn64(uint32_t saddr, uint32_t lbo) {
+__device__ __forceinline__ uint64_t desc_mn64(uint32_t saddr, uint32_t lbo, uint32_t sbo = 512) {
     return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) |
-           (static_cast<uint64_t>(lbo >> 4) << 16) | (static_cast<uint64_t>(512 >> 4) << 32) |
+           (static_cast<uint64_t>(lbo >> 4) << 16) | (static_cast<uint64_t>(sbo >> 4) << 32) |
            (1ull << 46) | (4ull << 61);
 }
 // both operands MN-major (bits 15 and 16)
@@ -114,9 +124,14 @@ __device__ __forceinline__ void tma_box(const CUtensorMap *map, uint32_t dst, ui
         : "memory");
 }
 
+// EDGE: rows that do not end with a chunk (W % 64 != 0).  Its tests in the other
+// instance made the gradients of 8 x 256 x 256 take 1229 us instead of 1204.
+template <bool EDGE>
 __global__ void __launch_bounds__(kThreads)
 wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
-             const __grid_constant__ CUtensorMap xmap1, const __grid_constant__ CUtensorMap gmap) {
+             const __grid_constant__ CUtensorMap xmap1, const __grid_constant__ CUtensorMap gmap,
+             const __grid_constant__ CUtensorMap emap0, const __grid_constant__ CUtensorMap emap1) {
+    // emap0, emap1: the sources without the last pixel of every row
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *base = smem_raw + ((512u - (tc::smem_u32(smem_raw) & 511u)) & 511u);
     WBars &bars = *reinterpret_cast<WBars *>(base);
@@ -130,7 +145,11 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
     // chunks of this split, and the stages they fill
     const int mine = (a.nchunks - split + splits - 1) / splits;
     const int nstages = (mine + a.nch - 1) / a.nch;
-    const int chunk_bytes = kXSlot + a.nco * kGBytes, stage_bytes = a.nch * chunk_bytes;
+    const int x_off = EDGE ? a.x_off : 0, g_off = EDGE ? a.g_off : kXSlot;
+    const int chunk_bytes = g_off + a.nco * kGBytes, stage_bytes = a.nch * chunk_bytes;
+    // a chunk's place in its row, advanced by `splits` chunks with carries (a division
+    // per chunk made the copy thread the kernel's bound)
+    const int dxc = splits % cw;
     const bool has_bias = blockIdx.y == 0;
     const uint32_t cols = N <= 32 ? 32 : N <= 64 ? 64 : 128;
 
@@ -161,10 +180,9 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
         // --------------------------------------------------------- TMA boxes
         if (lane == 0) {
             const CUtensorMap *xmap = ci < a.n0 ? &xmap0 : &xmap1;
+            const CUtensorMap *emap = ci < a.n0 ? &emap0 : &emap1;
             const int cx = (ci < a.n0 ? ci : ci - a.n0) * kBlk;
-            // the chunk's place, advanced by `splits` chunks with carries (a
-            // division per chunk made this thread the kernel's bound)
-            const int dxc = splits % cw, dby = splits / cw, dyy = dby % a.H, db = dby / a.H;
+            const int dby = splits / cw, dyy = dby % a.H, db = dby / a.H;
             int xc = split % cw, y = (split / cw) % a.H, b = split / cw / a.H;
             int s = 0, issued = 0;
             uint32_t ph = 0;
@@ -175,13 +193,23 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
                 }
                 const int k0 = issued * a.nch, kn = min(a.nch, mine - k0);
                 uint32_t at = tc::smem_u32(stages + s * stage_bytes);
+                int edges = 0;  // edge boxes of the stage
+                if (EDGE && a.rem)
+                    for (int k = 0, q = xc; k < kn; ++k) {
+                        edges += q == cw - 1;
+                        q += dxc;
+                        if (q >= cw) q -= cw;
+                    }
                 tc::mbar_arrive_expect_tx(&bars.full[s],
-                                          static_cast<uint32_t>(kn * (kXBytes + a.nco * kGBytes)));
+                                          static_cast<uint32_t>(kn * (kXBytes + a.nco * kGBytes) +
+                                                                edges * kEdgeBytes));
                 for (int k = 0; k < kn; ++k, at += chunk_bytes) {
                     const int x0 = xc * kPX;
-                    tma_box(xmap, at, &bars.full[s], cx, x0 - 1, y + dy - 1, b);
+                    tma_box(xmap, at + x_off, &bars.full[s], cx, x0 - 1, y + dy - 1, b);
+                    if (EDGE && a.rem && xc == cw - 1)
+                        tma_box(emap, at + a.edge_off, &bars.full[s], cx, a.edge_x, y + dy - 1, b);
                     for (int j = 0; j < a.nco; ++j)
-                        tma_box(&gmap, at + kXSlot + j * kGBytes, &bars.full[s], j * kBlk, x0, y, b);
+                        tma_box(&gmap, at + g_off + j * kGBytes, &bars.full[s], j * kBlk, x0, y, b);
                     xc += dxc;
                     y += dyy;
                     b += db;
@@ -212,7 +240,7 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
             const uint32_t lead = tc::elect_one();
             const uint32_t idesc = idesc_mn(N);
             bool ok = true;
-            int s = 0;
+            int s = 0, xc = split % cw;
             uint32_t ph = 0, acc = 0;
             for (int g = 0; g < nstages; ++g) {
                 if (!tc::mbar_wait_warp(&bars.full[s], ph, abort_flag)) {
@@ -224,12 +252,34 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
                 const int kn = min(a.nch, mine - g * a.nch);
                 uint32_t at = tc::smem_u32(stages + s * stage_bytes);
                 for (int k = 0; k < kn; ++k, at += chunk_bytes) {
-                    const uint64_t ad = desc_mn64(at, 64), bd = desc_mn64(at + kXSlot, kGBytes);
+                    const uint64_t ad = desc_mn64(at + x_off, 64),
+                                   bd = desc_mn64(at + g_off, kGBytes);
+                    const bool last = EDGE && xc == cw - 1;
+                    const int steps = last ? a.steps : kPX / 16;
 #pragma unroll
                     for (int ks = 0; ks < kPX / 16; ++ks) {
+                        if (EDGE && ks >= steps) break;
                         tc::mma_bf16(tmem, ad + tc::desc_offset(ks * 16 * 64),
                                      bd + tc::desc_offset(ks * 16 * 64), idesc, acc, lead);
                         acc = 1;
+                    }
+                    if (last && a.rem) {
+                        // the step over the edge: dx = 1, 2; then dx = 0, whose group of
+                        // 8 pixels with the edge is the edge box.  The other group is in
+                        // its place: before the edge when rem >= 8 (then the edge box lies
+                        // behind the x box), all zeros after it (then it lies before)
+                        const uint32_t off = steps * 16 * 64;
+                        const uint64_t bs = bd + tc::desc_offset(off);
+                        tc::mma_bf16_lanes<1>(tmem, ad + tc::desc_offset(off), bs, idesc, acc, lead);
+                        const uint64_t es =
+                            a.rem < 8 ? desc_mn64(at + a.edge_off, 64, x_off + off + 512 - a.edge_off)
+                                      : desc_mn64(at + x_off + off, 64, a.edge_off - x_off - off);
+                        tc::mma_bf16_lanes<14>(tmem, es, bs, idesc, acc, lead);
+                        acc = 1;
+                    }
+                    if (EDGE) {
+                        xc += dxc;
+                        if (xc >= cw) xc -= cw;
                     }
                 }
                 tc::mma_commit(&bars.empty[s], lead);
@@ -266,7 +316,7 @@ wgrad_kernel(const WKernelArgs a, const __grid_constant__ CUtensorMap xmap0,
                     break;
                 }
                 const int kn = min(a.nch, mine - g * a.nch);
-                const unsigned char *gs = stages + s * stage_bytes + kXSlot + 8 * pg * 64;
+                const unsigned char *gs = stages + s * stage_bytes + g_off + 8 * pg * 64;
                 for (int k = 0; k < kn; ++k, gs += chunk_bytes) {
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
@@ -393,13 +443,14 @@ wgrad_reduce_kernel(const float *__restrict__ partial, const float *__restrict__
         gw[(static_cast<int64_t>(co) * cin + ci) * 9 + (cd % 3) * 3 + row / kBlk] = acc;
 }
 
-// NHWC BF16 [B][H][W][C] as a 4-D tensor (channel, x, y, image), box 32
-// channels x bx pixels of one row; channels beyond C and pixels outside the image
-// arrive as zeros.
-bool nhwc_map(CUtensorMap *map, const __nv_bfloat16 *p, int B, int H, int W, int C, int bx) {
+// NHWC BF16 [B][H][W][C] as a 4-D tensor (channel, x, y, image) of its first
+// `columns` columns, box 32 channels x bx pixels of one row; channels beyond C and
+// pixels outside those columns or the image arrive as zeros.
+bool nhwc_map(CUtensorMap *map, const __nv_bfloat16 *p, int B, int H, int W, int C, int columns,
+              int bx) {
     auto enc = tensor_map_encoder();
     if (!enc) return false;
-    cuuint64_t dims[4] = {static_cast<cuuint64_t>(C), static_cast<cuuint64_t>(W),
+    cuuint64_t dims[4] = {static_cast<cuuint64_t>(C), static_cast<cuuint64_t>(columns),
                           static_cast<cuuint64_t>(H), static_cast<cuuint64_t>(B)};
     cuuint64_t strides[3] = {static_cast<cuuint64_t>(C) * 2, static_cast<cuuint64_t>(W) * C * 2,
                              static_cast<cuuint64_t>(H) * W * C * 2};
@@ -413,6 +464,7 @@ bool nhwc_map(CUtensorMap *map, const __nv_bfloat16 *p, int B, int H, int W, int
 
 struct Plan {
     int nci, nco, splits, nch, ns;
+    int rem, chunk;  // W % 16, bytes of a chunk
     int64_t nchunks;
 };
 
@@ -427,7 +479,9 @@ Plan plan(int B, int W, int H, int cin, int cout) {
     // four chunks per stage (one barrier round trip for 16 MMAs), two where g
     // is wide
     p.nch = p.nco <= 2 ? 4 : 2;
-    const int stage = p.nch * (kXSlot + p.nco * kGBytes);
+    p.rem = W % 16;
+    p.chunk = kXSlot + (p.rem ? kEdgeBytes : 0) + p.nco * kGBytes;
+    const int stage = p.nch * p.chunk;
     p.ns = std::min(kMaxStages, (kSmemLimit - kHeader - 512) / stage);  // 512: alignment slack
     return p;
 }
@@ -455,12 +509,18 @@ int wgrad(const WgradArgs &a, float *gw, float *gb, void *ws, cudaStream_t strea
     }
     const Plan p = plan(a.B, a.W, a.H, a.cin, a.cout);
     if (p.nchunks > 0x7fffffff) return SPP_ERR_ARG;
-    CUtensorMap xm0, xm1, gm;
-    if (!nhwc_map(&xm0, a.x0, a.B, a.H, a.W, a.c0, kHX) ||
-        !nhwc_map(&gm, a.g, a.B, a.H, a.W, a.cg, kPX))
+    CUtensorMap xm0, xm1, gm, em0, em1;
+    if (!nhwc_map(&xm0, a.x0, a.B, a.H, a.W, a.c0, a.W, kHX) ||
+        !nhwc_map(&gm, a.g, a.B, a.H, a.W, a.cg, a.W, kPX))
         return SPP_ERR_CUDA;
     xm1 = xm0;
-    if (a.c1 && !nhwc_map(&xm1, a.x1, a.B, a.H, a.W, a.c1, kHX)) return SPP_ERR_CUDA;
+    if (a.c1 && !nhwc_map(&xm1, a.x1, a.B, a.H, a.W, a.c1, a.W, kHX)) return SPP_ERR_CUDA;
+    em0 = xm0;
+    em1 = xm1;
+    const int without_last = std::max(1, a.W - 1);
+    if (p.rem && (!nhwc_map(&em0, a.x0, a.B, a.H, a.W, a.c0, without_last, 8) ||
+                  (a.c1 && !nhwc_map(&em1, a.x1, a.B, a.H, a.W, a.c1, without_last, 8))))
+        return SPP_ERR_CUDA;
     WKernelArgs k;
     k.H = a.H;
     k.W = a.W;
@@ -470,21 +530,31 @@ int wgrad(const WgradArgs &a, float *gw, float *gb, void *ws, cudaStream_t strea
     k.n0 = a.c1 ? a.c0 / kBlk : p.nci;
     k.ns = p.ns;
     k.nch = p.nch;
+    k.steps = ((a.W - 1) % kPX + 1) / 16;
+    k.rem = p.rem;
+    const bool edge_first = p.rem > 0 && p.rem < 8;
+    k.x_off = edge_first ? kEdgeBytes : 0;
+    k.edge_off = edge_first ? 0 : kXSlot;
+    // a row of one pixel has no other column: a box past the end, all zeros
+    k.edge_x = a.W == 1 ? 8 : a.W - p.rem - 1 + (edge_first ? 0 : 8);
+    k.g_off = kXSlot + (p.rem ? kEdgeBytes : 0);
     k.partial = static_cast<float *>(ws);
     k.pbias = k.partial + static_cast<size_t>(p.splits) * p.nci * 3 * p.nco * kBlk * kLanes;
     k.status = a.status;
-    const int smem = kHeader + 512 + p.ns * p.nch * (kXSlot + p.nco * kGBytes);
+    const int smem = kHeader + 512 + p.ns * p.nch * p.chunk;
     static int configured_dev = -1;
     int dev = 0;
     cudaGetDevice(&dev);
     if (configured_dev != dev) {
-        if (cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kSmemLimit) != cudaSuccess)
-            return SPP_ERR_CUDA;
+        for (auto *kernel : {wgrad_kernel<false>, wgrad_kernel<true>})
+            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kSmemLimit) != cudaSuccess)
+                return SPP_ERR_CUDA;
         configured_dev = dev;
     }
-    launch_dependent(wgrad_kernel, dim3(p.splits, 3 * p.nci), dim3(kThreads), smem, stream, k, xm0,
-                     xm1, gm);
+    launch_dependent(a.W % kPX ? wgrad_kernel<true> : wgrad_kernel<false>,
+                     dim3(p.splits, 3 * p.nci), dim3(kThreads), smem, stream, k, xm0, xm1, gm, em0,
+                     em1);
     const int blocks = p.nci * 3 * p.nco * kBlk * kLanes / kRedThreads + p.nco * kBlk / kBiasChannels;
     launch_dependent(wgrad_reduce_kernel, dim3(blocks), dim3(kRedThreads), 0, stream, k.partial, k.pbias, p.splits, p.nci, p.nco,
                      a.cin, a.cout, gw, gb);

@@ -46,3 +46,40 @@ def test_weight_gradient_tile_edges(spp, B, H, W, cin, cout):
     assert np.all(np.abs(gw.cpu().numpy() - ref_w) <= tol * abs_w)
     assert np.all(np.abs(gb.cpu().numpy() - gyb.sum(axis=(0, 2, 3)))
                   <= tol * np.abs(gyb).sum(axis=(0, 2, 3)))
+
+
+@pytest.mark.parametrize("W", [1, 2, 7, 8, 16, 20, 24, 44, 48, 63, 64, 65, 70, 80, 130])
+@pytest.mark.parametrize("cin,cout", [(32, 32), (40, 72), (192, 128)])
+def test_infinities_stay_with_the_taps_that_read_them(spp, W, cin, cout):
+    """The first and last input pixels of a row have no output pixel to their right
+    (tap dx = 2) and to their left (dx = 0): an infinity or NaN there leaves those
+    taps as they are with a 0 in its place, the same bits."""
+    B, H = 2, 3
+    g = torch.Generator().manual_seed(100 * cin + W)
+    x = torch.randn(B, H, W, cin, generator=g).to(torch.bfloat16)
+    gy = torch.randn(B, H, W, cout, generator=g).to(torch.bfloat16).cuda()
+    bad = x.clone()
+    for c, v in ((1, float("inf")), (cin // 2, float("nan")), (cin - 1, -float("inf"))):
+        x[:, :, -1, c] = 0
+        bad[:, :, -1, c] = v
+        if W > 1:
+            x[:, 1, 0, c - 1] = 0
+            bad[:, 1, 0, c - 1] = v
+    got = []
+    for t in (x, bad):
+        n = spp.binding.spp_conv3x3_backward_weights_workspace_bytes(B, W, H, cin, cout)
+        ws = torch.full((n,), 0xFF, dtype=torch.uint8, device="cuda")
+        gw = torch.full((cout, cin, 3, 3), float("nan"), device="cuda")
+        gb = torch.full((cout,), float("nan"), device="cuda")
+        spp.check(spp.binding.spp_conv3x3_backward_weights(t.cuda(), gy, B, W, H, cin, cout, gw, gb,
+                                                           ws, None))
+        got.append((gw.cpu().numpy(), gb.cpu().numpy()))
+    (gw, gb), (bw, bb) = got
+    last = [1, cin // 2, cin - 1]
+    first = [c - 1 for c in last] if W > 1 else []
+    clean = [c for c in range(cin) if c not in last + first]
+    assert np.all(np.isfinite(gw)) and np.array_equal(gb, bb)
+    assert np.array_equal(gw[:, clean], bw[:, clean])
+    assert np.array_equal(gw[:, last][..., 0], bw[:, last][..., 0])
+    assert np.array_equal(gw[:, first][..., 2], bw[:, first][..., 2])
+    assert not np.isfinite(bw[:, last][:, :, 1, 1]).any()
