@@ -19,6 +19,15 @@ import torch
 from . import _binding as B
 
 
+def _aligned(g):
+    """An incoming gradient as the library takes it: contiguous, from a 16-byte
+    boundary (a view into a larger tensor need not start at one); None stays None."""
+    if g is None:
+        return None
+    g = g.contiguous()
+    return g.clone() if g.data_ptr() % 16 else g
+
+
 class Reconstruct(torch.autograd.Function):
     """Coarse-to-fine gather pyramid (Appendix A) with the tone map of Sec. 5.
 
@@ -61,14 +70,10 @@ class Reconstruct(torch.autograd.Function):
         new = lambda ts: [torch.empty_like(x) for x in ts]
         g_layers, g_logits, g_hats = new(layers), new(logits), [None] + new(hats[1:])
         g_warped = torch.empty_like(hdr) if warped is not None else None
-        if g_hdr is not None:
-            g_hdr = g_hdr.contiguous()
-            if g_hdr.data_ptr() % 16:  # a view into a larger tensor
-                g_hdr = g_hdr.clone()
         B.check(B.spp_reconstruct_pyramid_backward(
-            layers, logits, hats, warped, mask, hdr, W, H, ctx.tm, g_hdr,
-            None if g_ldr is None else g_ldr.contiguous(), torch.empty_like(hdr), g_layers,
-            g_logits, g_hats, g_warped), "reconstruct backward")
+            layers, logits, hats, warped, mask, hdr, W, H, ctx.tm, _aligned(g_hdr),
+            _aligned(g_ldr), torch.empty_like(hdr), g_layers, g_logits, g_hats, g_warped),
+            "reconstruct backward")
         return (None, None, g_warped, None, *g_layers, *g_logits)
 
 
@@ -87,8 +92,9 @@ class WarpPrevious(torch.autograd.Function):
     def backward(ctx, g):
         (mv,) = ctx.saved_tensors
         _, H, W = g.shape
+        g = _aligned(g)
         gp = torch.zeros_like(g)
-        B.check(B.spp_warp_previous_backward(mv, W, H, g.contiguous(), gp), "warp backward")
+        B.check(B.spp_warp_previous_backward(mv, W, H, g, gp), "warp backward")
         return gp, None
 
 
@@ -127,7 +133,7 @@ class Splat(torch.autograd.Function):
         g0 = (g_layers[0].contiguous().clone() if g_layers[0] is not None
               else torch.zeros_like(fr.layers[0]))
         full = [g if g is not None else torch.zeros_like(x) for g, x in zip(g_layers, fr.layers)]
-        full = [x.contiguous() for x in full]
+        full = [_aligned(x) for x in full]
         B.check(B.spp_pyramid_backward(full, fr.W, fr.H, fr.L, g0), "pyramid backward")
         gs = torch.empty_like(fr.s)
         B.check(B.spp_splat_backward(fr.offsets, fr.counts, fr.rgb, fr.s, fr.layers[0], g0,
@@ -152,6 +158,6 @@ class DensityToS(torch.autograd.Function):
         gz = torch.empty_like(d)
         ws = torch.empty(max(B.spp_density_backward_workspace_bytes(), 16), dtype=torch.uint8,
                          device=d.device)
-        B.check(B.spp_density_backward(d, d.numel(), ctx.budget, ctx.phi, g.contiguous(), gz, ws),
+        B.check(B.spp_density_backward(d, d.numel(), ctx.budget, ctx.phi, _aligned(g), gz, ws),
                 "density backward")
         return None, None, None, None, gz.view_as(g)

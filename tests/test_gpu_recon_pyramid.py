@@ -90,3 +90,70 @@ def test_gradient_views_of_any_alignment(spp):
     one = torch.ones(1, device="cuda")
     for a, b in zip(grads(one.expand(3, H, W)), grads(torch.ones_like(hdr))):
         assert torch.equal(a, b)
+
+
+def test_ldr_gradient_views_of_any_alignment(spp):
+    """The same for the tone-mapped output, alone and joined to the HDR one by a
+    concatenation, whose backward hands out such views."""
+    from paper_2602_08642_gb300 import autograd
+    W, H, L = 30, 6, 2  # 3 W H is no multiple of 8
+    g = torch.Generator(device="cuda").manual_seed(6)
+    leaf = lambda *s: torch.randn(*s, generator=g, device="cuda").requires_grad_(True)
+    layers = [leaf(3, H >> l, W >> l) for l in range(L)]
+    logits = [leaf(29, H, W), leaf(25, H // 2, W // 2)]
+    hdr, ldr = autograd.Reconstruct.apply(L, spp.binding.make_tonemap(), None, None, *layers, *logits)
+    inputs = layers + logits
+    grads = lambda go: torch.autograd.grad(ldr, inputs, go, retain_graph=True)
+    buf = torch.randn(3 * H * W + 1, generator=g, device="cuda")
+    view = buf[1:].view(3, H, W)
+    assert view.data_ptr() % 16
+    for a, b in zip(grads(view), grads(view.clone())):
+        assert torch.equal(a, b)
+    n = 3 * H * W
+    both = torch.randn(2 * n + 1, generator=g, device="cuda")
+    cat = torch.cat([torch.zeros(1, device="cuda"), ldr.flatten(), hdr.flatten()])
+    got = torch.autograd.grad(cat, inputs, both, retain_graph=True)
+    want = torch.autograd.grad([ldr, hdr], inputs, [both[1:n + 1].view_as(ldr).clone(),
+                                                    both[n + 1:].view_as(hdr).clone()])
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+
+
+def test_gradient_views_of_any_alignment_elsewhere(spp):
+    """The warp, the splat and the density take such views too, and transposed ones.
+    The warp's backward adds with atomics: FP32 rounding of its few terms, 1e-5."""
+    from paper_2602_08642_gb300 import autograd
+    W, H, L = 36, 12, 2
+    g = torch.Generator(device="cuda").manual_seed(7)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+
+    def views(*shape):
+        """The same values as a plain tensor, from an odd offset, and transposed."""
+        plain = rnd(*shape)
+        buf = torch.zeros(plain.numel() + 1, device="cuda")
+        buf[1:] = plain.flatten()
+        odd = buf[1:].view(shape)
+        assert odd.data_ptr() % 16
+        return plain, odd, plain.transpose(-1, -2).contiguous().transpose(-1, -2)
+
+    prev = rnd(3, H, W).requires_grad_(True)
+    out = autograd.WarpPrevious.apply(prev, rnd(2, H, W))
+    got = [torch.autograd.grad(out, prev, v, retain_graph=True)[0] for v in views(3, H, W)]
+    assert all(torch.allclose(a, got[0], rtol=1e-5, atol=1e-5) for a in got)
+
+    fr = spp.Frame(W, H, L, max_budget=1.0)
+    params = spp.make_params(1.0, frame=1)
+    z = rnd(H, W)
+    d = (z - z.max()).exp()
+    fr.alloc(d, params)
+    fr.render(rnd(3, H, W).exp(), 5, 1)
+    fr.splat()
+    s = fr.s.clone().requires_grad_(True)
+    layers = autograd.Splat.apply(fr, params, s)
+    got = [torch.autograd.grad(layers, s, gs, retain_graph=True)[0]
+           for gs in zip(views(3, H, W), views(3, H // 2, W // 2))]
+    assert all(torch.equal(a, got[0]) for a in got)
+    zt = z.requires_grad_(True)
+    sz = autograd.DensityToS.apply(d, fr.s, 1.0, 0.125, zt)
+    got = [torch.autograd.grad(sz, zt, v, retain_graph=True)[0] for v in views(H, W)]
+    assert all(torch.equal(a, got[0]) for a in got)
