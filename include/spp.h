@@ -830,7 +830,9 @@ int spp_density_lowres(const float *d, int W, int H, int factor, float *out,
  *   - seeds and render_seeds are HOST arrays of B seeds (p->seed is not read);
  *   - the mask is shared.
  * With B > 1 every image's data starts on a 16-byte boundary: W*H, and for
- * logits C * Wl * Hl, are multiples of 4 (SPP_ERR_ALIGN otherwise). */
+ * logits C * Wl * Hl, are multiples of 4.  The sample map, the renderer, the
+ * reconstruction and its backward (for the logits) and the splat's backward answer
+ * SPP_ERR_ALIGN otherwise; the other entries read single values and take any size. */
 #define SPP_BATCH_OFFSETS_PAD 4
 int spp_assemble_features_batch(int B, const float *const *albedo, const float *const *normal,
                                 const float *const *depth, const float *const *mv,

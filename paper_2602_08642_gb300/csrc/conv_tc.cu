@@ -982,11 +982,10 @@ bool getenv_disable_tma_in() {
 // The rows of an upsampled chunk are shared too: halo row h reads coarse row
 // (h + 1) >> 1 of the box.
 //
-// The expansion (a thread per coarse piece, up to four 16-byte stores) bounded
-// these layers, the largest of the network: 96 -> 32 channels at 3840 x 2160
-// 550 -> 418 us, 192 -> 64 at 1920 x 1080 335 -> 308 us (of the same 4K forward; 317 us
-// with both phases handed over together), and 362 and 293 us with the issue from
-// warp-uniform code.
+// The expansion (a thread per coarse piece, up to four 16-byte stores) bounds these
+// layers, the largest of the network, in conv3x3_kernel: 96 -> 32 channels at
+// 3840 x 2160 take 554 us there and 360 us here, 192 -> 64 at 1920 x 1080 329 and
+// 289 us (of which handing the phases over one by one is 3 %).
 //
 // A tile is TR x 256 pixels.  Accumulators take 2 TR N columns: double-buffered
 // for N = 32, one set for N = 64 (half-height tiles with two sets would fetch the
@@ -1300,11 +1299,13 @@ conv3x3_up_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap omap0,
 template <int N, bool RES>
 bool launch_up(const ConvArgs &a, cudaStream_t stream, int *rc) {
     using C = Cfg<N, RES>;
-    // A tile of 256 columns took 1.5 (N = 32) or 1.77 (N = 64) times as long as one
-    // of 128 columns of the expanding kernel when this line was drawn (418 and 308 us
-    // against 550 and 335 us, over their tiles; with warp-uniform issue 362 and 293
-    // us), so the rounds of tiles per SM decide: padding columns and a last round that
-    // is nearly empty can cost more than the expansion.
+    // The rounds of tiles per SM decide: padding columns and a last round that is
+    // nearly empty can cost more than the expansion.  A round of tiles of 256 columns
+    // takes 1.23 to 1.30 (N = 32) or 1.49 to 1.58 (N = 64) times a round of 128 columns
+    // of the expanding kernel (both kernels on the network's layers at 3840 x 2160,
+    // 1920 x 1080, 1368 x 768, 1280 x 720 and 640 x 360: 360 us in 54 rounds against
+    // 554 us in 107 at N = 32, 289 us in 15 against 329 us in 27 at N = 64).  The line
+    // asks for 1.5 and 1.78 times the rounds, a margin of about an eighth.
     const int64_t rows = static_cast<int64_t>(a.B) * ((a.H + C::TR - 1) / C::TR), sms = sm_count();
     const int64_t ntiles = rows * ((a.W + 2 * kTileX - 1) / (2 * kTileX));
     const int64_t rounds = (ntiles + sms - 1) / sms;
