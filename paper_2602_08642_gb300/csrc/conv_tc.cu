@@ -33,7 +33,9 @@
 // SPP_ERR_TIMEOUT in the status word, the other roles leave at their next
 // wait, and TMEM is freed before the kernel returns.  On every path the MMA warp
 // waits for its issued MMAs and the copy thread for its last copies before they
-// leave: another role may have given up on them.
+// leave: another role may have given up on them.  (0.15 us a launch: 1080p forward
+// 714.0 -> 716.2 us.  The same waits behind the block's last barrier, only where a role
+// gave up, changed the roles' code: 735 us.)
 #include <cuda_bf16.h>
 
 #include <algorithm>
